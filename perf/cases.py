@@ -1,0 +1,200 @@
+"""What is timed of the expert-choice layer, and how far two correct implementations of it may differ.
+
+Five kinds of call, all through `paper_2202_09368_b200.binding`:
+
+  train    ec_moe_forward + ec_moe_backward: what a training step does with the layer
+  forward  ec_moe_forward(forward_only=True): what evaluation and serving do with it
+  route    ec_route, ec_shuffle, ec_unshuffle: the routing for a caller that runs experts of its own
+  assign   ec_capped_assignment: the solver of the capped variant (Section 3.3 of the paper)
+
+Sizes are in the paper's notation: n tokens per routing group, d model width, dff hidden width, E experts, capacity
+factor c.  Buffers that a program keeps from step to step (workspace, saved blob, gradients, outputs) are part of the
+prepared state; inputs are drawn from the seed with the distributions of `paper_2202_09368_b200.inputs`.
+"""
+import math
+
+import torch
+
+from paper_2202_09368_b200 import binding as B
+
+DTYPES = {"f32": torch.float32, "bf16": torch.bfloat16}
+
+
+def layer(kind, name, n, d, dff, E, c, dtype="bf16", groups=1, gelu="erf", bias=False, logit_scale=1.0):
+    case = {"kind": kind, "n": n, "d": d, "dff": dff, "E": E, "c": c, "dtype": dtype, "groups": groups, "gelu": gelu,
+            "bias": bias, "logit_scale": logit_scale}
+    return dict(case, name=name) if name else case
+
+
+def routing(name, n, d, E, c):
+    case = {"kind": "route", "n": n, "d": d, "E": E, "c": c, "dtype": "bf16"}
+    return dict(case, name=name) if name else case
+
+
+def assignment(name, n, E, c, b, iters):
+    case = {"kind": "assign", "n": n, "E": E, "c": c, "b": b, "iters": iters}
+    return dict(case, name=name) if name else case
+
+
+def listed():
+    return [
+        # the smallest layer anyone runs: a unit test or a toy model in fp32, all launches and latency
+        layer("forward", "forward_f32_tiny", 256, 64, 256, 4, 2.0, dtype="f32"),
+        # an fp32 training step of a small model (debugging, reference runs)
+        layer("train", "train_f32", 2048, 512, 2048, 16, 2.0, dtype="f32"),
+        # a bf16 training step that is over in a few hundred microseconds: launches count as much as kernels
+        layer("train", "train_small", 2048, 256, 512, 8, 2.0),
+        # one layer of the 100M-parameter model with 32 experts, eight sequences of 1024 tokens
+        layer("train", "train_100m32e", 8192, 768, 3072, 32, 2.0),
+        # nothing a multiple of a tile: ten experts, ragged widths, two routing groups, bias terms, the tanh GeLU
+        layer("train", "train_ragged", 3040, 1000, 2072, 10, 1.0, groups=2, gelu="tanh", bias=True),
+        # one layer of the 8B-parameter model with 64 experts, sixteen sequences of 1024 tokens: the largest step
+        layer("train", "train_8b64e", 16384, 4096, 16384, 64, 2.0),
+        # evaluation of the 100M model with 64 experts at a low capacity and a sharp gate: 64 rows per expert
+        layer("forward", "forward_100m64e_c05", 8192, 768, 3072, 64, 0.5, logit_scale=4.0),
+        # serving the 8B layer: one sequence of 1024 tokens, 32 rows per expert, the weights are what is read
+        layer("forward", "forward_8b64e_1k", 1024, 4096, 16384, 64, 2.0),
+        # the routing alone, from one short batch with few experts to the largest groups and expert counts
+        routing("route_4k_e8", 4096, 1024, 8, 2.0),
+        routing("route_64k_e256", 65536, 1024, 256, 2.0),
+        routing("route_256k_e32", 262144, 1024, 32, 2.0),
+        # the capped variant at the 8B layer's routing shape, at most two experts per token, the paper's 100 rounds
+        assignment("assign_16k_e64", 16384, 64, 2.0, 2, 100),
+    ]
+
+
+def _log(rng, lo, hi, mult=1):
+    """A size spread over the logarithm of [lo, hi], rounded to a multiple of `mult`."""
+    v = math.exp(rng.uniform(math.log(lo), math.log(hi)))
+    return max(mult, int(round(v / mult)) * mult)
+
+
+def draw(rng):
+    kind = rng.choices(["train", "forward", "f32", "route", "assign"], [30, 25, 15, 20, 10])[0]
+    if kind == "route":
+        n = _log(rng, 1024, 262144)
+        d = _log(rng, 256, min(2048, 2 ** 28 // n), 8)
+        return routing(None, n, d, rng.choice([8, 16, 32, 64, 128, 256]), rng.choice([1.0, 1.5, 2.0]))
+    if kind == "assign":
+        c = rng.choice([1.0, 1.5, 2.0])
+        return assignment(None, _log(rng, 512, 32768), rng.choice([8, 16, 32, 64, 100, 128, 256]), c,
+                          rng.choice([math.ceil(c), math.ceil(c) + 1]), 100)
+    E = rng.choice([4, 8, 10, 16, 24, 32, 48, 64])
+    c = rng.choice([0.5, 1.0, 1.25, 2.0])
+    gelu, bias, scale = rng.choice(["erf", "erf", "tanh"]), rng.random() < 0.25, rng.choice([1.0, 1.0, 4.0])
+    if kind == "f32":
+        n, d = _log(rng, 128, 4096), _log(rng, 32, 768, 4)
+        return layer(rng.choice(["train", "forward"]), None, n, d, int(d * rng.uniform(2, 4)) // 4 * 4, min(E, 32), c, "f32", 1, gelu,
+                     bias, scale)
+    mult = rng.choice([8, 64])
+    groups = rng.choice([1, 1, 1, 2, 4])
+    if kind == "train":
+        n, d = _log(rng, 512, 16384) // groups, _log(rng, 128, 2048, mult)
+    else:
+        n, d = max(128, _log(rng, 128, 16384) // groups), _log(rng, 128, 4096, mult)
+    return layer(kind, None, n, d, int(d * rng.uniform(2, 4)) // mult * mult, E, c, "bf16", groups, gelu, bias, scale)
+
+
+def config(case):
+    dtype = DTYPES[case.get("dtype", "bf16")]
+    if case["kind"] == "route":
+        return B.make_config(case["n"], case["d"], 8, case["E"], case["c"], dtype)
+    if case["kind"] == "assign":
+        return B.make_config(case["n"], 8, 8, case["E"], case["c"], dtype, cap_b=case["b"], cap_iters=case["iters"])
+    return B.make_config(case["n"], case["d"], case["dff"], case["E"], case["c"], dtype, gelu=case["gelu"], groups=case["groups"])
+
+
+def prepare(case, seed):
+    cfg, kind = config(case), case["kind"]
+    dtype = DTYPES[case.get("dtype", "bf16")]
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+
+    def normal(shape, std, dt=dtype):
+        return torch.empty(shape, dtype=dt, device="cuda").normal_(0.0, std, generator=gen)
+
+    N, k, E = B.total_tokens(cfg), B.slots_per_expert(cfg), case["E"]
+    s = {"kind": kind, "cfg": cfg, "ws": None}
+    if kind == "assign":
+        s["S"] = torch.softmax(normal((N, E), 1.0, torch.float32), dim=1)
+        s["A"] = torch.empty_like(s["S"])
+        s["ws"] = B.alloc_workspace(cfg)
+        return s
+    d = case["d"]
+    s["X"] = normal((N, d), 1.0)
+    s["Wg"] = normal((d, E), case.get("logit_scale", 1.0) / math.sqrt(d))
+    if kind == "route":
+        s["X_e"] = normal((E, k, d), 1.0, torch.float32)                # what the caller's experts return
+        s["X_in"] = torch.empty((E, k, d), dtype=dtype, device="cuda")
+        s["r"] = B.Routing(torch.empty(N, E, dtype=torch.float32, device="cuda"), torch.empty(E, k, dtype=torch.int32, device="cuda"),
+                           torch.empty(E, k, dtype=torch.float32, device="cuda"), torch.empty(N + 1, dtype=torch.int32, device="cuda"),
+                           torch.empty(E * k, dtype=torch.int32, device="cuda"))
+        s["X_out"] = torch.empty_like(s["X"])
+        s["ws"] = B.alloc_workspace(cfg)
+        return s
+    dff = case["dff"]
+    s["W1"] = normal((E, d, dff), 1.0 / math.sqrt(d))
+    s["W2"] = normal((E, d, dff), 1.0 / math.sqrt(dff))
+    s["b1"] = normal((E, dff), 0.5) if case["bias"] else None
+    s["b2"] = normal((E, d), 0.5) if case["bias"] else None
+    s["X_out"] = torch.empty_like(s["X"])
+    if kind == "train":
+        s["dX_out"] = normal((N, d), 1.0)
+        s["saved"], s["ws"] = B.alloc_saved(cfg), B.alloc_workspace(cfg)
+        s["grads"] = tuple(torch.empty_like(s[t]) for t in ("X", "Wg", "W1", "W2"))
+        s["bias_grads"] = (torch.empty_like(s["b1"]), torch.empty_like(s["b2"])) if case["bias"] else None
+    else:
+        s["ws"] = torch.empty(int(B.lib().ec_forward_only_workspace_bytes(cfg)), dtype=torch.uint8, device="cuda")
+    return s
+
+
+def run(s):
+    cfg, kind = s["cfg"], s["kind"]
+    if kind == "assign":
+        return B.ec_capped_assignment(cfg, s["S"], ws=s["ws"], A=s["A"])
+    X = s["X"]
+    if kind == "route":
+        r = B.ec_route(cfg, X, s["Wg"], ws=s["ws"], out=s["r"])
+        X_in = B.ec_shuffle(cfg, X, r.I, s["X_in"])
+        X_out = B.ec_unshuffle(cfg, s["X_e"], r.G, r.row_ptr, r.slots, s["X_out"])
+        return {"S": r.S, "I": r.I, "G": r.G, "row_ptr": r.row_ptr, "slots": r.slots, "X_in": X_in, "X_out": X_out}
+    Wg, W1, W2 = s["Wg"], s["W1"], s["W2"]
+    if kind == "forward":
+        return B.ec_moe_forward(cfg, X, Wg, W1, W2, s["X_out"], ws=s["ws"], forward_only=True, b1=s["b1"], b2=s["b2"])[0]
+    X_out, saved = B.ec_moe_forward(cfg, X, Wg, W1, W2, s["X_out"], s["saved"], s["ws"], b1=s["b1"], b2=s["b2"])
+    dX, dWg, dW1, dW2 = B.ec_moe_backward(cfg, X, Wg, W1, W2, s["dX_out"], saved, s["grads"], s["ws"], s["bias_grads"])
+    out = {"X_out": X_out, "dX": dX, "dWg": dWg, "dW1": dW1, "dW2": dW2}
+    if s["bias_grads"] is not None:
+        out["db1"], out["db2"] = s["bias_grads"]
+    return out
+
+
+def work(case):
+    """Inputs read once, outputs written once; the products of the layer and, for the solver, its rounds."""
+    n, E, kind = case["n"] * case.get("groups", 1), case["E"], case["kind"]
+    k = int(math.floor(case["n"] * case["c"] / E + 1e-9))
+    if kind == "assign":                                  # per round and entry: two exponentials, three scalings, the clip, two sums
+        return {"bytes": 2 * n * E * 4, "flops": 8.0 * case["iters"] * n * E}
+    b, d = (4 if case["dtype"] == "f32" else 2), case["d"]
+    slots = k * E * case.get("groups", 1)
+    gate = 2.0 * n * d * E
+    if kind == "route":
+        return {"bytes": (2 * n * d + d * E + slots * d) * b + n * E * 4 + 3 * slots * 4 + (n + 1) * 4 + slots * d * 4,
+                "flops": gate + 2.0 * slots * d}
+    dff = case["dff"]
+    weights, bias = 2 * E * d * dff + d * E, (E * (d + dff) if case["bias"] else 0)
+    product = 2.0 * slots * d * dff
+    if kind == "forward":
+        return {"bytes": (2 * n * d + weights + bias) * b, "flops": 2 * product + gate}
+    return {"bytes": (4 * n * d + 2 * weights + 2 * bias) * b, "flops": 6 * product + 3 * gate}
+
+
+def tolerance(case):
+    """About four times what the path itself shows against the same arithmetic in 64 bits on the listed cases, given the
+    same selection (seen: the solver rel 5e-6, max 2e-4; S and G rel 2e-6, X_out of the routing chain rel 1.7e-3, its
+    bf16 rounding; fp32 layers rel 1.1e-6, max 1.1e-5; bf16 layers rel 3.2e-3, max 0.03)."""
+    if case["kind"] == "assign":
+        return {"rel": 2e-5, "max": 8e-4}
+    if case["kind"] == "route":
+        # S in 64 bits puts up to 1.2 % of the entries of I elsewhere in their expert's list: scores that fp32 cannot order
+        return {"rel": 6e-3, "max": 0.02, "differ": 0.01}
+    return {"rel": 5e-6, "max": 5e-5} if case["dtype"] == "f32" else {"rel": 1e-2, "max": 0.12}
