@@ -168,6 +168,60 @@ def run(s):
     return out
 
 
+def exact(case, seed):
+    """What `run` returns, in 64 bits by plain torch.  Outputs that follow the order in which an expert lists its tokens
+    (I, X_in, and what the unshuffle makes of rows that already lie in slot order) have no such value: scores that fp32
+    cannot order come in either order."""
+    s, k, E = prepare(case, seed), int(math.floor(case["n"] * case["c"] / case["E"] + 1e-9)), case["E"]
+    if case["kind"] == "assign":
+        L = s["S"].double() / 1e-3
+        qb, qc = torch.zeros_like(L), torch.zeros_like(L[:, :1])
+        for _ in range(case["iters"]):
+            L = L + math.log(k) - torch.logsumexp(L, dim=0, keepdim=True)          # rows sum to k
+            L = L + qc
+            m = torch.clamp(math.log(case["b"]) - torch.logsumexp(L, dim=1, keepdim=True), max=0.0)
+            L, qc = L + m, -m                                                      # columns sum to at most b
+            box = L + qb
+            L = torch.clamp(box, max=0.0)                                          # entries at most 1
+            qb = box - L
+        return torch.exp(L)
+    X, Wg = s["X"].double(), s["Wg"].double()
+    S = torch.softmax(X @ Wg, dim=1)
+    if case["kind"] == "route":
+        G = torch.sort(S, dim=0, descending=True, stable=True)[0][:k].T.contiguous()
+        return {"S": S, "I": None, "G": G, "row_ptr": None, "slots": None, "X_in": None, "X_out": None}
+    first = [g * case["n"] for g in range(case["groups"])]
+    train, approx = case["kind"] == "train", "tanh" if case["gelu"] == "tanh" else "none"
+    out = {"X_out": torch.zeros_like(X)}
+    if train:
+        out.update(dX=torch.zeros_like(X), dWg=None, dW1=torch.empty_like(s["W1"], dtype=torch.float64),
+                   dW2=torch.empty_like(s["W2"], dtype=torch.float64))
+        if case["bias"]:
+            out.update(db1=torch.empty_like(s["b1"], dtype=torch.float64), db2=torch.empty_like(s["b2"], dtype=torch.float64))
+        dS, dX_out = torch.zeros_like(S), s["dX_out"].double()
+    for e in range(E):
+        rows = torch.cat([f + torch.sort(S[f:f + case["n"], e], descending=True, stable=True)[1][:k] for f in first])
+        W1, W2, x, g = s["W1"][e].double(), s["W2"][e].double(), X[rows], S[rows, e][:, None]
+        z = x @ W1 + (s["b1"][e].double() if case["bias"] else 0.0)
+        h = torch.nn.functional.gelu(z, approximate=approx)
+        y = h @ W2.T + (s["b2"][e].double() if case["bias"] else 0.0)
+        out["X_out"].index_add_(0, rows, g * y)
+        if train:
+            dy = g * dX_out[rows]
+            dS[rows, e] = (dX_out[rows] * y).sum(1)
+            dz = torch.ops.aten.gelu_backward(dy @ W2, z, approximate=approx)
+            out["dW1"][e], out["dW2"][e] = x.T @ dz, dy.T @ h
+            out["dX"].index_add_(0, rows, dz @ W1.T)
+            if case["bias"]:
+                out["db1"][e], out["db2"][e] = dz.sum(0), dy.sum(0)
+    if not train:
+        return out["X_out"]
+    dL = S * (dS - (dS * S).sum(1, keepdim=True))
+    out["dWg"] = X.T @ dL
+    out["dX"] += dL @ Wg.T
+    return out
+
+
 def work(case):
     """Inputs read once, outputs written once; the products of the layer and, for the solver, its rounds."""
     n, E, kind = case["n"] * case.get("groups", 1), case["E"], case["kind"]
