@@ -55,73 +55,169 @@ static inline unsigned grid_for(int64_t work, int threads, int64_t cap = 148 * 1
 
 // ------------------------------------------------------------------------------------------
 // Gate, Eq. 2: S = Softmax(X . Wg) over the experts of each token.  FMA version (fp32 path and
-// shapes the tensor-core kernel does not take).  One CTA handles TT tokens; the logits of the
-// TT x E (token, expert) pairs are spread over the threads.
+// shapes the tensor-core kernel does not take).
+//
+// A CTA computes the logits of 32 tokens.  Its eight warps are NG column groups of 32 experts times KS = 8 / NG slices of
+// the contraction: with few experts the work is a long sum per logit, and the slices keep all warps busy.  A chunk is 16
+// depths per slice; the next one travels to registers while the current one is multiplied (packed pairs, four tokens
+// times eight experts per thread).  The slices' sums join in ascending order, then a warp turns rows into their softmax.
+// Bound by the latency of a chunk (a CTA is alone on its SM at the layer's sizes).
 // ------------------------------------------------------------------------------------------
-constexpr int kGateTT = 8, kGateDC = 512, kGateThreads = 256, kGateMaxE = 256;
+constexpr int kGateTT = 32, kGateThreads = 256, kGateSlice = 16;
 
-template <typename T>
+__device__ __forceinline__ void gate_ld4(const float* p, float* f) {
+  const float4 v = *reinterpret_cast<const float4*>(p); f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
+}
+__device__ __forceinline__ void gate_ld4(const bf16* p, float* f) {
+  const uint2 v = *reinterpret_cast<const uint2*>(p);
+  f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xFFFF0000u);
+  f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xFFFF0000u);
+}
+__host__ __device__ constexpr int gate_smem_bytes(int NG) { return 2 * (8 / NG) * kGateSlice * (kGateTT + 32 * NG) * 4; }
+
+// WVEC: rows of Wg are whole 16-byte (fp32) or 8-byte (bf16) groups of four
+template <typename T, int NG, bool WVEC>
 __global__ void __launch_bounds__(kGateThreads)
-gate_softmax_simt_kernel(const T* __restrict__ X, const T* __restrict__ Wg, float* __restrict__ S,
-                         int64_t n, int d, int E) {
-  __shared__ float Xs[kGateTT][kGateDC];
-  __shared__ float Ls[kGateTT][kGateMaxE];
+gate_softmax_simt_kernel(const T* __restrict__ X, const T* __restrict__ Wg, float* __restrict__ S, int64_t n, int d, int E) {
+  constexpr int KS = 8 / NG, DK = KS * kGateSlice, C = 32 * NG;         // chunk: DK depths of 32 tokens and of C experts
+  constexpr int kX = DK * kGateTT, kW = DK * C, XQ = (kX / 4 + kGateThreads - 1) / kGateThreads, WQ = kW / 4 / kGateThreads;
+  extern __shared__ __align__(16) float gate_smem[];                    // [2][X chunk [DK][32] | W chunk [DK][C]]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t t0 = (int64_t)blockIdx.x * kGateTT;
-  const int tid = threadIdx.x;
-  constexpr int R = kGateTT * kGateMaxE / kGateThreads;
-  float acc[R];
+  float xv[XQ][4], wv[WQ][4];
+  // X quad q of this thread: four depths of one token; a warp covers 8 tokens x 64 bytes (fp32), and the XOR by 8 spreads
+  // the transposed stores over the banks.  W quad: four experts at one depth.
+  auto x_at = [&](int q, int& tok, int& k) {
+    const int w = warp + 8 * q;
+    tok = (w & 3) * 8 + (lane >> 2); k = ((w >> 2) * 4 + (lane & 3)) * 4;
+  };
+  auto fetch = [&](int d0) {
 #pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] = 0.f;
-  const int pairs = kGateTT * E;
-  for (int d0 = 0; d0 < d; d0 += kGateDC) {
-    const int dc = min(kGateDC, d - d0);
-    for (int idx = tid; idx < kGateTT * dc; idx += kGateThreads) {
-      const int tt = idx / dc, dd = idx % dc;
-      const int64_t t = t0 + tt;
-      Xs[tt][dd] = t < n ? ld_f(X, t * d + d0 + dd) : 0.f;
+    for (int q = 0; q < XQ; ++q) {
+      int tok, k; x_at(q, tok, k);
+      const int64_t t = min(t0 + tok, n - 1);
+      gate_ld4(X + t * d + (d0 + k < d ? d0 + k : 0), xv[q]);
     }
-    __syncthreads();
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int p = tid + r * kGateThreads;
-      if (p < pairs) {
-        const int tt = p / E, i = p % E;
-        float a = acc[r];
-        for (int dd = 0; dd < dc; ++dd) a = fmaf(Xs[tt][dd], ld_f(Wg, (int64_t)(d0 + dd) * E + i), a);
-        acc[r] = a;
+    for (int q = 0; q < WQ; ++q) {
+      const int idx = tid + q * kGateThreads, k = d0 + idx / (C / 4), c = (idx % (C / 4)) * 4;
+      const T* row = Wg + (int64_t)(k < d ? k : 0) * E;
+      if constexpr (WVEC) gate_ld4(row + (c < E ? c : 0), wv[q]);
+      else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) wv[q][j] = ld_f(row, c + j < E ? c + j : 0);
       }
     }
-    __syncthreads();
-  }
+  };
+  auto put = [&](float* buf, int d0) {                // what lies beyond d or E becomes zero here, after the loads have landed
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int p = tid + r * kGateThreads;
-    if (p < pairs) Ls[p / E][p % E] = acc[r];
+    for (int q = 0; q < XQ; ++q) {
+      int tok, k; x_at(q, tok, k);
+      if (k < DK) {
+        const bool ok = d0 + k < d;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) buf[(k + j) * kGateTT + (tok ^ (((k >> 2) & 3) * 8))] = ok ? xv[q][j] : 0.f;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < WQ; ++q) {
+      const int idx = tid + q * kGateThreads, kk = idx / (C / 4), c = (idx % (C / 4)) * 4;
+      const bool ok = d0 + kk < d;
+      float4 v;
+      v.x = ok && c < E ? wv[q][0] : 0.f; v.y = ok && c + 1 < E ? wv[q][1] : 0.f;
+      v.z = ok && c + 2 < E ? wv[q][2] : 0.f; v.w = ok && c + 3 < E ? wv[q][3] : 0.f;
+      *reinterpret_cast<float4*>(buf + kX + kk * C + c) = v;
+    }
+  };
+  const int cg = warp % NG, ks = warp / NG, tg = lane >> 2, cl = cg * 32 + (lane & 3) * 4;
+  unsigned long long acc[4][4];                       // token tg * 4 + i, experts cl, cl + 1 | cl + 2, cl + 3 | cl + 16 .. cl + 19
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  fetch(0);
+  put(gate_smem, 0);
+  __syncthreads();
+  int cur = 0;
+  for (int d0 = 0; d0 < d; d0 += DK, cur ^= 1) {
+    const float* xs = gate_smem + cur * (kX + kW) + ks * kGateSlice * kGateTT;
+    const float* ws = gate_smem + cur * (kX + kW) + kX + ks * kGateSlice * C;
+    if (d0 + DK < d) fetch(d0 + DK);
+#pragma unroll
+    for (int kk = 0; kk < kGateSlice; ++kk) {
+      const float4 a = *reinterpret_cast<const float4*>(xs + kk * kGateTT + ((tg * 4) ^ (((kk >> 2) & 3) * 8)));
+      const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(ws + kk * C + cl), b1 = *reinterpret_cast<const ulonglong2*>(ws + kk * C + cl + 16);
+      const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned long long aa = (unsigned long long)__float_as_uint(av[i]) | ((unsigned long long)__float_as_uint(av[i]) << 32);
+        const unsigned long long bb[4] = {b0.x, b0.y, b1.x, b1.y};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(aa), "l"(bb[j]));
+      }
+    }
+    if (d0 + DK < d) {                                // the other buffer was last read before the previous barrier
+      put(gate_smem + (cur ^ 1) * (kX + kW), d0 + DK);
+      __syncthreads();
+    }
   }
   __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31;     // one warp per token
-  const int64_t t = t0 + warp;
-  if (warp < kGateTT && t < n) {
-    float mx = -INFINITY;
-    for (int i = lane; i < E; i += 32) mx = fmaxf(mx, Ls[warp][i]);
+  float* part = gate_smem;                            // [KS][32 tokens][C]: 32 KiB, no more than the buffers
+  static_assert(KS * kGateTT * C <= 2 * (kX + kW), "the partial sums fit the buffers");
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float* row = part + (ks * kGateTT + tg * 4 + i) * C + cl;
+    *reinterpret_cast<ulonglong2*>(row) = make_ulonglong2(acc[i][0], acc[i][1]);
+    *reinterpret_cast<ulonglong2*>(row + 16) = make_ulonglong2(acc[i][2], acc[i][3]);
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int tok = warp; tok < kGateTT; tok += 8) {     // a warp per token
+    const int64_t t = t0 + tok;
+    if (t >= n) break;
+    float v[NG], mx = -INFINITY, sum = 0.f;
+#pragma unroll
+    for (int j = 0; j < NG; ++j) {
+      v[j] = 0.f;
+#pragma unroll
+      for (int q = 0; q < KS; ++q) v[j] += part[(q * kGateTT + tok) * C + j * 32 + lane];
+      if (j * 32 + lane < E) mx = fmaxf(mx, v[j]);
+    }
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float sum = 0.f;
-    for (int i = lane; i < E; i += 32) { const float e = expf(Ls[warp][i] - mx); Ls[warp][i] = e; sum += e; }
+#pragma unroll
+    for (int j = 0; j < NG; ++j) { v[j] = j * 32 + lane < E ? expf(v[j] - mx) : 0.f; sum += v[j]; }
     for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     const float inv = 1.f / sum;
-    for (int i = lane; i < E; i += 32) S[t * E + i] = Ls[warp][i] * inv;
+#pragma unroll
+    for (int j = 0; j < NG; ++j) if (j * 32 + lane < E) S[t * E + j * 32 + lane] = v[j] * inv;
   }
+}
+
+template <typename T, int NG>
+cudaError_t launch_gate_ng(const T* X, const T* Wg, float* S, int64_t n, int d, int E, cudaStream_t st) {
+  const unsigned grid = (unsigned)((n + kGateTT - 1) / kGateTT);
+  const bool wvec = E % 4 == 0;                       // Wg itself is 16-byte aligned
+  auto kern = wvec ? gate_softmax_simt_kernel<T, NG, true> : gate_softmax_simt_kernel<T, NG, false>;
+  constexpr int smem = gate_smem_bytes(NG);
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  count_launch();
+  kern<<<grid, kGateThreads, smem, st>>>(X, Wg, S, n, d, E);
+  return cudaGetLastError();
+}
+template <typename T>
+cudaError_t launch_gate_t(const T* X, const T* Wg, float* S, int64_t n, int d, int E, cudaStream_t st) {
+  if (E <= 32) return launch_gate_ng<T, 1>(X, Wg, S, n, d, E, st);
+  if (E <= 64) return launch_gate_ng<T, 2>(X, Wg, S, n, d, E, st);
+  if (E <= 128) return launch_gate_ng<T, 4>(X, Wg, S, n, d, E, st);
+  return launch_gate_ng<T, 8>(X, Wg, S, n, d, E, st);
 }
 
 cudaError_t launch_gate_softmax_simt(int dtype, const void* X, const void* Wg, float* S, int64_t n,
                                      int d, int E, cudaStream_t st) {
-  const unsigned grid = (unsigned)((n + kGateTT - 1) / kGateTT);
-  count_launch();
-  if (dtype == 0)
-    gate_softmax_simt_kernel<float><<<grid, kGateThreads, 0, st>>>((const float*)X, (const float*)Wg, S, n, d, E);
-  else
-    gate_softmax_simt_kernel<bf16><<<grid, kGateThreads, 0, st>>>((const bf16*)X, (const bf16*)Wg, S, n, d, E);
-  return cudaGetLastError();
+  if (E > 256) return cudaErrorInvalidValue;
+  return dtype == 0 ? launch_gate_t((const float*)X, (const float*)Wg, S, n, d, E, st)
+                    : launch_gate_t((const bf16*)X, (const bf16*)Wg, S, n, d, E, st);
 }
 
 // ------------------------------------------------------------------------------------------
