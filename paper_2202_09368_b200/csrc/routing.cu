@@ -1326,33 +1326,45 @@ cudaError_t launch_bwd_softmax(const float* S, const float* dG, const int32_t* r
 }
 
 // ------------------------------------------------------------------------------------------
-// Column sums per expert (gradients of the bias terms Eq. 3 leaves out): a thread owns a column and adds its rows in
-// order, so the result does not depend on scheduling; neighbouring threads read neighbouring columns.
+// Column sums per expert (gradients of the bias terms Eq. 3 leaves out).  A CTA owns 64 columns of one expert; its eight
+// warps take every eighth row, a lane two columns, and the eight sums join in ascending order, so the result does not
+// depend on scheduling.  Bound by the latency of the eight loads a warp has in flight.
 // ------------------------------------------------------------------------------------------
+__device__ __forceinline__ float2 ld_pair(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ float2 ld_pair(const bf16* p) {
+  const unsigned v = *reinterpret_cast<const unsigned*>(p);
+  return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
+}
 template <typename T>
 __global__ void __launch_bounds__(256) column_sums_kernel(const T* __restrict__ A, T* __restrict__ out, int64_t rows, int cols,
                                                           const int32_t* __restrict__ batch_rows) {
-  const int b = blockIdx.y, c = blockIdx.x * 256 + threadIdx.x;
-  if (c >= cols) return;
+  __shared__ float2 s_part[8][32];
+  const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, c = blockIdx.x * 64 + lane * 2;      // cols is a multiple of 4
   int64_t lim = rows;
   if (batch_rows != nullptr && batch_rows[b] < lim) lim = batch_rows[b];
-  const T* p = A + (int64_t)b * rows * cols + c;
-  float acc = 0.f;
-  int64_t r = 0;
-  for (; r + 8 <= lim; r += 8) {
-    float v[8];
+  const T* p = A + (int64_t)b * rows * cols + (c < cols ? c : 0);
+  float2 acc = make_float2(0.f, 0.f);
+  int64_t r = warp;
+  for (; r + 56 < lim; r += 64) {
+    float2 v[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = ld_f(p, (r + u) * cols);
+    for (int u = 0; u < 8; ++u) v[u] = ld_pair(p + (r + 8 * u) * cols);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) acc += v[u];
+    for (int u = 0; u < 8; ++u) { acc.x += v[u].x; acc.y += v[u].y; }
   }
-  for (; r < lim; ++r) acc += ld_f(p, r * cols);
-  if constexpr (sizeof(T) == 4) out[(int64_t)b * cols + c] = acc; else out[(int64_t)b * cols + c] = __float2bfloat16(acc);
+  for (; r < lim; r += 8) { const float2 v = ld_pair(p + r * cols); acc.x += v.x; acc.y += v.y; }
+  s_part[warp][lane] = acc;
+  __syncthreads();
+  if (warp != 0 || c >= cols) return;
+#pragma unroll
+  for (int w = 1; w < 8; ++w) { acc.x += s_part[w][lane].x; acc.y += s_part[w][lane].y; }
+  T* o = out + (int64_t)b * cols + c;
+  if constexpr (sizeof(T) == 4) { o[0] = acc.x; o[1] = acc.y; } else { o[0] = __float2bfloat16(acc.x); o[1] = __float2bfloat16(acc.y); }
 }
 
 cudaError_t launch_column_sums(int dtype, const void* A, void* out, int batches, int64_t rows, int cols,
                                const int32_t* batch_rows, cudaStream_t st) {
-  const dim3 grid((cols + 255) / 256, batches);
+  const dim3 grid((cols + 63) / 64, batches);
   count_launch();
   if (dtype == 0) column_sums_kernel<float><<<grid, 256, 0, st>>>((const float*)A, (float*)out, rows, cols, batch_rows);
   else column_sums_kernel<bf16><<<grid, 256, 0, st>>>((const bf16*)A, (bf16*)out, rows, cols, batch_rows);
