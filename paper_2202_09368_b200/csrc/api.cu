@@ -211,7 +211,7 @@ ec_status route_impl(const Dims& D, const void* X, const void* Wg, float* S, int
   if (D.cap_b) {                                    // Section 3.3: TopK(A, k) instead of TopK(S^T, k)
     float* A = (float*)(ws + W.cap_A);
     EC_CUDA(launch_capped_assignment(S, D.ng, D.E, D.kg, D.groups, D.cap_b, D.cap_iters, (float)D.cap_lambda, A,
-                                     ws + W.capped, st));
+                                     ws + W.capped, (int*)(ws + W.status), st));
     prof_mark("capped_assignment", st);
     keys = A;
   }
@@ -332,7 +332,7 @@ ec_status ec_capped_assignment(const ec_config* c, const float* S, float* A, voi
   EC_CUDA(cudaMemsetAsync(ws, 0, sizeof(StatusWord), st));
   prof_begin(st, 0);
   EC_CUDA(launch_capped_assignment(S, D.ng, D.E, D.kg, D.groups, D.cap_b, D.cap_iters, (float)D.cap_lambda, A,
-                                   (char*)ws + W.capped, st));
+                                   (char*)ws + W.capped, (int*)((char*)ws + W.status), st));
   prof_mark("capped_assignment", st);
   return EC_OK;
 }

@@ -16,29 +16,27 @@
 // of its tokens per expert, and the CTAs each combine those in a fixed order (so the result does not depend on
 // scheduling) before they touch their tokens.  Two forms:
 //   - resident: one cooperative launch for all rounds; a warp keeps log A and the factors of its (at most 8 /
-//     experts-per-lane) tokens in registers, the CTAs meet at a grid barrier once per round and only the row
-//     partials go through memory.  Used whenever the tokens fit (up to about 19 k tokens at 64 experts);
+//     experts-per-lane) tokens in registers, and only the row partials go through memory, as words that carry their
+//     round's number: a CTA waits for the words it needs, there is no grid barrier (see Exchange).  Used whenever the tokens
+//     fit (up to about 19 k tokens at 64 experts);
 //   - resident in shared memory: the same launch with the state in the CTA's shared memory, for up to about
 //     2.4 M entries per device (16384 tokens x 128 experts, 65536 x 32);
 //   - one launch per round with the state (2 x 4 bytes per entry) in global memory, where it stays in L2 at
 //     the layer sizes.  For everything else.
-// Either way a round costs latency (a barrier or a launch, one round trip for the partials, the reduction
-// trees), not bandwidth.  Routing groups are independent problems (grid.y).
+// Either way a round costs latency (one round trip for the partials or a launch, the reduction trees), not
+// bandwidth.  Routing groups are independent problems (grid.y).
 #include "internal.h"
 
-#include <cooperative_groups.h>
 #include <math.h>
 
 namespace ecmoe {
 
 namespace {
 
-namespace cg = cooperative_groups;
-
 constexpr int kCapThreads = 1024;
 constexpr int kCapWarps = kCapThreads / 32;
 constexpr int kCapMaxE = 256;
-constexpr int kCapLoads = 4;                         // partials a thread of the row step has in flight 
+constexpr int kRoundLoads = 4;                       // partials a thread of the row step has in flight (one launch per round)
 constexpr int kCapBatch = 4;                         // tokens of a warp whose loads are in flight together (fewer with many experts per lane)
 constexpr int kCapResident = 8;                      // (tokens per warp) x (experts per lane) the resident form holds:
                                                      // log A and the box factors of that many entries in a lane's registers
@@ -57,49 +55,186 @@ __device__ __forceinline__ void lse_butterfly(float& m, float& s, int width) {
   }
 }
 
-// Shared memory of a CTA: wpart [warps][E] float2 | shift [E] float
-__device__ __forceinline__ float* shift_of(float2* smem, int E) { return reinterpret_cast<float*>(smem + kCapWarps * E); }
+// ---- exchange of the row partials in the resident forms ---------------------------------------------
+// A word is 64 bits in global memory: a value in the low half, the number of the pass that wrote it in the high half.
+// Value and number are stored and loaded together, so a reader that sees the number has the value, without a barrier.
+// A round takes two hops: every CTA leaves its sums, one word per expert; the CTA an expert belongs to (expert i to CTA
+// i mod the group's CTAs, a warp per expert) adds them up and leaves the expert's shift in one word for every CTA.
+// Cycles of a round spent here at 16384 tokens x 64 experts on 148 CTAs: 14 k with a grid barrier and every CTA reading
+// all partials after it; 7.5 k with words in one hop, every CTA reading all CTAs' words, 11 MB per sweep; 6.9 k in two hops
+// with one copy of the shifts; 4.7 k like this.  Pass p uses the buffers p & 1; nobody can be two passes ahead of a
+// reader, since every pass waits for all CTAs' words of the one before.  The words start with the number 2^32 - 1 (the
+// launcher fills them).  All CTAs of a cooperative launch are on the device at once; a wait is nevertheless bounded:
+// after two seconds the status word says so and the CTAs leave.
+constexpr unsigned long long kCapWaitNs = 2000000000ull;
+__device__ __forceinline__ void word_store(unsigned long long* p, float v, unsigned pass) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"((unsigned long long)__float_as_uint(v) | ((unsigned long long)pass << 32)) : "memory");
+}
+__device__ __forceinline__ unsigned long long word_load(const unsigned long long* p) {
+  unsigned long long v; asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory"); return v;
+}
+__device__ __forceinline__ unsigned long long cap_timer() {
+  unsigned long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t;
+}
+// Fetches the words row[q], row[q + 32], ... of up to N CTAs (below bpg), all in flight together, until each carries
+// `pass`; 0 beyond the last CTA.  False when the wait ran out.
+constexpr int kCapLoads = 5;
+template <int N>
+__device__ __forceinline__ bool words_fetch(const unsigned long long* row, int q, int bpg, unsigned pass, float (&v)[N]) {
+  unsigned long long w[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) w[u] = q + u * 32 < bpg ? word_load(row + q + u * 32) : (unsigned long long)pass << 32;
+  unsigned long long t0 = 0;
+  for (unsigned spin = 0;; ++spin) {
+    bool ok = true;
+#pragma unroll
+    for (int u = 0; u < N; ++u) ok = ok && (unsigned)(w[u] >> 32) == pass;
+    if (ok) break;
+    if ((spin & 255u) == 255u) {
+      if (t0 == 0) t0 = cap_timer();
+      else if (cap_timer() - t0 > kCapWaitNs) return false;
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u)
+      if ((unsigned)(w[u] >> 32) != pass) w[u] = word_load(row + q + u * 32);
+  }
+#pragma unroll
+  for (int u = 0; u < N; ++u) v[u] = __uint_as_float((unsigned)w[u]);
+  return true;
+}
+// first_max, first_sum, even, odd: [groups * E][CTAs of a group]; shift_even, shift_odd: [groups][CTAs of a group][E], a copy
+// for each reader (148 CTAs waiting for the same four lines of L2 hold up the store they wait for)
+struct Exchange {
+  unsigned long long *first_max, *first_sum, *even, *odd, *shift_even, *shift_odd; int* status;
+  static size_t words(int bpg, int groups, int E) { return (size_t)6 * bpg * groups * E; }
+  static Exchange at(unsigned long long* p, int bpg, int groups, int E, int* status) {
+    const size_t n = (size_t)bpg * groups * E;
+    return {p, p + n, p + 2 * n, p + 3 * n, p + 4 * n, p + 5 * n, status};
+  }
+};
+
+// Shared memory of a CTA: wpart [warps][E + 1] float2 | shift [E] float
+__device__ __forceinline__ float* shift_of(float2* smem, int E) { return reinterpret_cast<float*>(smem + kCapWarps * (E + 1)); }
 
 // shift[i] = log k - log(sum over the group's tokens of exp L[:, i]) from the partials the CTAs of group g left.
-// P adjacent lanes share an expert: each combines every P-th CTA's partial in ascending order (loads several at
-// a time, kCapLoads in flight), a butterfly joins them.  Every thread of the CTA calls this.
-// The partials were written by other CTAs, in the resident forms by the same launch: they are read from L2
-// (ld.global.cg), never through a read-only or L1 path that could hold the values of two rounds ago.
+// P adjacent lanes share an expert: each combines every P-th CTA's partial in ascending order, a butterfly joins them.
+// Every thread of the CTA calls these.  The form of one launch per round reads (max, sum) pairs:
+__device__ __forceinline__ int row_lanes(int E) { int P = 32; while (P * E > kCapThreads) P >>= 1; return P; }       // E <= 256: P >= 4
 __device__ __forceinline__ void row_shifts(const float2* part_in, int g, int bpg, int E, float log_k, float* shift) {
-  int P = 32;
-  while (P * E > kCapThreads) P >>= 1;               // E <= 256: P >= 4
+  const int P = row_lanes(E);
   const int i = threadIdx.x / P, p0 = threadIdx.x % P;
   float m = 0.f, s = 0.f;
   if (i < E) {
-    for (int q = p0; q < bpg; q += kCapLoads * P) {
-      float2 v[kCapLoads];
+    for (int q = p0; q < bpg; q += kRoundLoads * P) {
+      float2 v[kRoundLoads];
 #pragma unroll
-      for (int u = 0; u < kCapLoads; ++u) {
+      for (int u = 0; u < kRoundLoads; ++u) {
         const int qq = q + u * P;
         v[u] = qq < bpg ? __ldcg(part_in + ((int64_t)g * E + i) * bpg + qq) : make_float2(0.f, 0.f);   // adjacent lanes, adjacent CTAs
       }
 #pragma unroll
-      for (int u = 0; u < kCapLoads; ++u) lse_add(m, s, v[u].x, v[u].y);
+      for (int u = 0; u < kRoundLoads; ++u) lse_add(m, s, v[u].x, v[u].y);
     }
   }
   lse_butterfly(m, s, P);                            // whole warps take part: P divides 32
   if (i < E && p0 == 0) shift[i] = log_k - (m + __logf(s));
   __syncthreads();
 }
+// The resident forms wait for words.  Pass 0 has a maximum and a sum per expert; from then on every entry is at most 1, the
+// maxima are taken as 0 and the sums are added as they are.  False when a wait ran out (for all threads of the CTA).
+__device__ __forceinline__ bool row_shifts(const Exchange& x, int pass, int g, int bpg, int blk, int E, float log_k, float* shift) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned long long* out = ((pass & 1) ? x.shift_odd : x.shift_even) + (int64_t)g * bpg * E;
+  bool ok = true;
+  for (int i = blk + warp * bpg; i < E; i += kCapWarps * bpg) {        // this CTA's experts: uniform across the warp
+    const int64_t row = ((int64_t)g * E + i) * bpg;
+    float m = 0.f, s = 0.f;
+    if (pass == 0) {
+      for (int q = lane; ok && q < bpg; q += 32) {
+        float mv[1], v[1];
+        ok = words_fetch(x.first_max + row, q, bpg, 0u, mv) && words_fetch(x.first_sum + row, q, bpg, 0u, v);
+        if (ok) lse_add(m, s, mv[0], v[0]);
+      }
+      lse_butterfly(m, s, 32);
+    } else {
+      for (int q = lane; ok && q < bpg; q += kCapLoads * 32) {
+        float v[kCapLoads];
+        ok = words_fetch(((pass & 1) ? x.odd : x.even) + row, q, bpg, (unsigned)pass, v);
+#pragma unroll
+        for (int u = 0; u < kCapLoads; ++u) s += ok ? v[u] : 0.f;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) break;
+    const float v = log_k - (m + __logf(s));
+    for (int q = lane; q < bpg; q += 32) word_store(out + (int64_t)q * E + i, v, (unsigned)pass);
+  }
+  if (ok && threadIdx.x < E) {
+    float v[1];
+    ok = words_fetch(out + (int64_t)blk * E + threadIdx.x, 0, 1, (unsigned)pass, v);
+    if (ok) shift[threadIdx.x] = v[0];
+  }
+  if (__syncthreads_and(ok)) return true;
+  if (threadIdx.x == 0) { atomicExch(x.status + 1, 8); atomicExch(x.status, 5 /* EC_ERR_TIMEOUT */); }
+  return false;
+}
 
-// The CTA's (max, sum of exp) per expert from the lanes' running values; warp w joins experts w, w + 32, ...
+// The CTA's (max, sum of exp) per expert from the lanes' running values; warp w joins experts w, w + 32, ...  A row of
+// wpart has a word to spare, which spreads the 32 warps' values of one expert over the banks.
 template <int EPL>
 __device__ __forceinline__ void publish_partials(const float (&pm)[EPL], const float (&ps)[EPL], float2* wpart, int E,
                                                  float2* __restrict__ part_out, int g, int bpg, int blk) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __syncthreads();                                   // the previous use of wpart and shift is over
 #pragma unroll
-  for (int j = 0; j < EPL; ++j) if (lane + 32 * j < E) wpart[warp * E + lane + 32 * j] = make_float2(pm[j], ps[j]);
+  for (int j = 0; j < EPL; ++j) if (lane + 32 * j < E) wpart[warp * (E + 1) + lane + 32 * j] = make_float2(pm[j], ps[j]);
   __syncthreads();
   for (int i = warp; i < E; i += kCapWarps) {
-    float2 v = wpart[lane * E + i];
+    float2 v = wpart[lane * (E + 1) + i];
     lse_butterfly(v.x, v.y, 32);
     if (lane == 0) part_out[((int64_t)g * E + i) * bpg + blk] = v;     // expert-major: the row step reads along the CTAs
+  }
+}
+// The same as words.  wpart was last read before the barrier of the row step in between, so one barrier is enough.
+template <int EPL>
+__device__ __forceinline__ void publish_words(const float (&pm)[EPL], const float (&ps)[EPL], float2* wpart, int E, const Exchange& x,
+                                              int pass, int g, int bpg, int blk) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (pass == 0) {
+#pragma unroll
+    for (int j = 0; j < EPL; ++j) if (lane + 32 * j < E) wpart[warp * (E + 1) + lane + 32 * j] = make_float2(pm[j], ps[j]);
+    __syncthreads();
+    for (int i = warp; i < E; i += kCapWarps) {
+      float2 v = wpart[lane * (E + 1) + i];
+      lse_butterfly(v.x, v.y, 32);
+      if (lane == 0) {
+        word_store(x.first_max + ((int64_t)g * E + i) * bpg + blk, v.x, 0u);
+        word_store(x.first_sum + ((int64_t)g * E + i) * bpg + blk, v.y, 0u);
+      }
+    }
+    return;
+  }
+  float* sums = reinterpret_cast<float*>(wpart);     // [warps][E + 1]; with E even the odd pitch keeps the banks apart
+  const int pitch = E | 1;
+#pragma unroll
+  for (int j = 0; j < EPL; ++j) if (lane + 32 * j < E) sums[warp * pitch + lane + 32 * j] = ps[j];
+  __syncthreads();
+  constexpr int kRows = EPL >= 8 ? 4 : EPL;          // experts a warp joins side by side (it has at most EPL of them)
+  for (int i0 = warp; i0 < E; i0 += kRows * kCapWarps) {
+    float v[kRows];
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) v[u] = i0 + u * kCapWarps < E ? sums[lane * pitch + i0 + u * kCapWarps] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) v[u] += __shfl_xor_sync(0xffffffffu, v[u], o);
+    if (lane == 0) {
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+        if (i0 + u * kCapWarps < E) word_store(((pass & 1) ? x.odd : x.even) + ((int64_t)g * E + i0 + u * kCapWarps) * bpg + blk, v[u], (unsigned)pass);
+    }
   }
 }
 
@@ -200,49 +335,93 @@ capped_round_kernel(const float* __restrict__ S, float* __restrict__ L, float* _
 }
 
 // ---- resident: all rounds in one cooperative launch ------------------------------------------------
-// Needs ng <= TPW * gridDim.x * warps per CTA; every CTA calls the grid barrier iters times.
+// exp and log without the denormal ranges' extra instructions: an entry below 2^-126 counts as 0 in the sums
+__device__ __forceinline__ float exp_ftz(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x * 1.4426950408889634f)); return y; }
+__device__ __forceinline__ float log_ftz(float x) { float y; asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y * 0.6931471805599453f; }
+
+// Sums of T values (a power of two) over the warp at once: lane l ends with the sum of value l mod T.  T - 1 + log2(32 / T)
+// shuffles where T butterflies take 5 T.
+template <int T>
+__device__ __forceinline__ float warp_sums(float (&v)[T]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int b = 1; b < T; b <<= 1) {
+    const bool up = (lane & b) != 0;
+#pragma unroll
+    for (int i = 0; i < T / (2 * b); ++i) {
+      const float give = up ? v[2 * i] : v[2 * i + 1], keep = up ? v[2 * i + 1] : v[2 * i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, b);
+    }
+  }
+  float s = v[0];
+#pragma unroll
+  for (int o = T; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// Needs ng <= TPW * gridDim.x * warps per CTA and all CTAs on the device at once.  A warp works on its TPW tokens side by
+// side: their column sums share one set of shuffles, lane l keeps the column factor of token l mod TPW and one
+// logarithm serves all of them.  exp(L) of the previous round times exp(shift) is exp(L) after the row step, so an entry costs one
+// exponential a round.  Places without a token or an expert hold kNowhere, whose exponential is 0 and stays 0.
+// 16384 tokens x 64 experts, cycles of a round: one token after the other with two exponentials an entry 4.1 k, this form 1.25 k.
+constexpr float kNowhere = -1e30f;
 template <int EPL, int TPW>
 __global__ void __launch_bounds__(kCapThreads)
-capped_resident_kernel(const float* __restrict__ S, float* __restrict__ A, float2* __restrict__ part0, float2* __restrict__ part1,
-                       int64_t ng, int E, float inv_lambda, float log_k, float log_b, int iters) {
+capped_resident_kernel(const float* __restrict__ S, float* __restrict__ A, const Exchange ex, int64_t ng, int E,
+                       float inv_lambda, float log_k, float log_b, int iters) {
   extern __shared__ float2 cap_smem[];
   float* shift = shift_of(cap_smem, E);
-  cg::grid_group grid = cg::this_grid();
   const int g = blockIdx.y, bpg = gridDim.x, blk = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)bpg * kCapWarps, t0 = (int64_t)blk * kCapWarps + warp;
-  float x[TPW][EPL], qb[TPW][EPL], qc[TPW], pm[EPL], ps[EPL];
+  float x[TPW][EPL], ea[TPW][EPL], qb[TPW][EPL], qc = 0.f, pm[EPL], ps[EPL];
 #pragma unroll
   for (int j = 0; j < EPL; ++j) { pm[j] = 0.f; ps[j] = 0.f; }
 #pragma unroll
   for (int u = 0; u < TPW; ++u) {
     const int64_t t = t0 + u * stride, row = ((int64_t)g * ng + t) * E;
-    qc[u] = 0.f;
 #pragma unroll
     for (int j = 0; j < EPL; ++j) {
       const int i = lane + 32 * j;
-      qb[u][j] = 0.f;
-      x[u][j] = (t < ng && i < E) ? S[row + i] * inv_lambda : -INFINITY;
+      qb[u][j] = 0.f; ea[u][j] = 0.f;
+      x[u][j] = (t < ng && i < E) ? S[row + i] * inv_lambda : kNowhere;
       if (t < ng && i < E) lse_add(pm[j], ps[j], x[u][j], 1.f);
     }
   }
-  publish_partials<EPL>(pm, ps, cap_smem, E, part0, g, bpg, blk);
+  publish_words<EPL>(pm, ps, cap_smem, E, ex, 0, g, bpg, blk);
   for (int it = 0; it < iters; ++it) {
-    grid.sync();                                     // every CTA's partials of the previous pass are in memory
-    row_shifts((it & 1) ? part1 : part0, g, bpg, E, log_k, shift);
+    if (!row_shifts(ex, it, g, bpg, blk, E, log_k, shift)) return;
+    float sh[EPL], es[EPL], sum[TPW];
 #pragma unroll
-    for (int j = 0; j < EPL; ++j) { pm[j] = 0.f; ps[j] = 0.f; }
+    for (int j = 0; j < EPL; ++j) { ps[j] = 0.f; sh[j] = lane + 32 * j < E ? shift[lane + 32 * j] : 0.f; es[j] = exp_ftz(sh[j]); }
 #pragma unroll
     for (int u = 0; u < TPW; ++u) {
-      if (t0 + u * stride < ng) {                    // uniform across the warp
+      sum[u] = 0.f;
 #pragma unroll
-        for (int j = 0; j < EPL; ++j) if (lane + 32 * j < E) x[u][j] += shift[lane + 32 * j];       // rows sum to k
-        token_round<EPL>(x[u], qb[u], qc[u], lane, E, log_b);
-#pragma unroll
-        for (int j = 0; j < EPL; ++j) if (lane + 32 * j < E) ps[j] += __expf(x[u][j]);      // entries at most 1
+      for (int j = 0; j < EPL; ++j) {
+        x[u][j] += sh[j];                            // rows sum to k
+        // After the row step every entry is at most k, so nothing overflows and the column sum needs no shift by the
+        // maximum; a column so small that the sum underflows is far below b and stays as it is.
+        sum[u] += it == 0 ? exp_ftz(x[u][j]) : ea[u][j] * es[j];
       }
     }
-    if (it + 1 < iters) publish_partials<EPL>(pm, ps, cap_smem, E, (it & 1) ? part0 : part1, g, bpg, blk);
+    const float total = warp_sums<TPW>(sum);
+    const float m = fminf(0.f, log_b - (log_ftz(total) + qc));         // a column above b is scaled down to b
+    const float mq = m + qc;
+    qc = -m;
+#pragma unroll
+    for (int u = 0; u < TPW; ++u) {
+      const float c = __shfl_sync(0xffffffffu, mq, u);
+#pragma unroll
+      for (int j = 0; j < EPL; ++j) {
+        const float Bv = x[u][j] + c + qb[u][j];
+        x[u][j] = fminf(Bv, 0.f);                    // entries above 1 are clipped
+        qb[u][j] = Bv - x[u][j];
+        ea[u][j] = exp_ftz(x[u][j]);
+        ps[j] += ea[u][j];
+      }
+    }
+    if (it + 1 < iters) publish_words<EPL>(pm, ps, cap_smem, E, ex, it + 1, g, bpg, blk);
   }
 #pragma unroll
   for (int u = 0; u < TPW; ++u) {
@@ -257,12 +436,10 @@ capped_resident_kernel(const float* __restrict__ S, float* __restrict__ A, float
 // factors ([warp][token]).  A warp touches only its own part, so no barrier guards it.
 template <int EPL>
 __global__ void __launch_bounds__(kCapThreads)
-capped_resident_smem_kernel(const float* __restrict__ S, float* __restrict__ A, float2* __restrict__ part0,
-                            float2* __restrict__ part1, int64_t ng, int E, float inv_lambda, float log_k, float log_b,
+capped_resident_smem_kernel(const float* __restrict__ S, float* __restrict__ A, const Exchange ex, int64_t ng, int E, float inv_lambda, float log_k, float log_b,
                             int iters, int tpw) {
   extern __shared__ float2 cap_smem[];
   float* shift = shift_of(cap_smem, E);
-  cg::grid_group grid = cg::this_grid();
   const int g = blockIdx.y, bpg = gridDim.x, blk = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)bpg * kCapWarps, t0 = (int64_t)blk * kCapWarps + warp;
@@ -286,10 +463,9 @@ capped_resident_smem_kernel(const float* __restrict__ S, float* __restrict__ A, 
       if (lane == 0) my_qc[u] = 0.f;
     }
   }
-  publish_partials<EPL>(pm, ps, cap_smem, E, part0, g, bpg, blk);
+  publish_words<EPL>(pm, ps, cap_smem, E, ex, 0, g, bpg, blk);
   for (int it = 0; it < iters; ++it) {
-    grid.sync();                                     // every CTA's partials of the previous pass are in memory
-    row_shifts((it & 1) ? part1 : part0, g, bpg, E, log_k, shift);
+    if (!row_shifts(ex, it, g, bpg, blk, E, log_k, shift)) return;
 #pragma unroll
     for (int j = 0; j < EPL; ++j) { pm[j] = 0.f; ps[j] = 0.f; }
     for (int u = 0; u < tpw; ++u) {
@@ -312,7 +488,7 @@ capped_resident_smem_kernel(const float* __restrict__ S, float* __restrict__ A, 
         }
       }
     }
-    if (it + 1 < iters) publish_partials<EPL>(pm, ps, cap_smem, E, (it & 1) ? part0 : part1, g, bpg, blk);
+    if (it + 1 < iters) publish_words<EPL>(pm, ps, cap_smem, E, ex, it + 1, g, bpg, blk);
   }
   for (int u = 0; u < tpw; ++u) {
     const int64_t t = t0 + u * stride, row = ((int64_t)g * ng + t) * E;
@@ -339,11 +515,15 @@ int blocks_per_group(int64_t ng, int groups, int sms) {
 constexpr int kCapMaxBlocks = 1024;
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
-size_t cap_smem_bytes(int E) { return (size_t)kCapWarps * E * 8 + (size_t)E * 4; }      // at most 65 KiB
+size_t cap_smem_bytes(int E) { return (size_t)kCapWarps * (E + 1) * 8 + (size_t)E * 4; }      // at most 65.3 KiB
 
 struct ResidentArgs {
-  const float* S; float* A; float2* part0; float2* part1; int64_t ng; int E; float inv_lambda, log_k, log_b; int iters;
+  const float* S; float* A; Exchange ex; int64_t ng; int E; float inv_lambda, log_k, log_b; int iters;
 };
+// no word carries a pass number: one left by an earlier call could carry a number this call waits for
+cudaError_t exchange_clear(const ResidentArgs& a, dim3 grid, cudaStream_t st) {
+  return cudaMemsetAsync(a.ex.first_max, 0xFF, Exchange::words(grid.x, grid.y, a.E) * sizeof(unsigned long long), st);
+}
 template <int EPL, int TPW>
 cudaError_t launch_resident(ResidentArgs a, dim3 grid, int sms, bool* fits, cudaStream_t st) {
   auto kern = capped_resident_kernel<EPL, TPW>;
@@ -352,9 +532,11 @@ cudaError_t launch_resident(ResidentArgs a, dim3 grid, int sms, bool* fits, cuda
     return cudaErrorInvalidValue;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCapThreads, smem) != cudaSuccess) return cudaErrorInvalidValue;
-  *fits = (int64_t)per_sm * sms >= (int64_t)grid.x * grid.y;         // a grid barrier needs every CTA on the device at once
+  *fits = (int64_t)per_sm * sms >= (int64_t)grid.x * grid.y;         // the CTAs wait for one another: all on the device at once
   if (!*fits) return cudaSuccess;
-  void* args[] = {&a.S, &a.A, &a.part0, &a.part1, &a.ng, &a.E, &a.inv_lambda, &a.log_k, &a.log_b, &a.iters};
+  const cudaError_t e = exchange_clear(a, grid, st);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&a.S, &a.A, &a.ex, &a.ng, &a.E, &a.inv_lambda, &a.log_k, &a.log_b, &a.iters};
   count_launch();
   return cudaLaunchCooperativeKernel((void*)kern, grid, dim3(kCapThreads), args, smem, st);
 }
@@ -380,7 +562,9 @@ cudaError_t launch_resident_smem(ResidentArgs a, int tpw, dim3 grid, int sms, bo
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCapThreads, smem) != cudaSuccess) return cudaErrorInvalidValue;
   *fits = (int64_t)per_sm * sms >= (int64_t)grid.x * grid.y;
   if (!*fits) return cudaSuccess;
-  void* args[] = {&a.S, &a.A, &a.part0, &a.part1, &a.ng, &a.E, &a.inv_lambda, &a.log_k, &a.log_b, &a.iters, &tpw};
+  const cudaError_t e = exchange_clear(a, grid, st);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&a.S, &a.A, &a.ex, &a.ng, &a.E, &a.inv_lambda, &a.log_k, &a.log_b, &a.iters, &tpw};
   count_launch();
   return cudaLaunchCooperativeKernel((void*)kern, grid, dim3(kCapThreads), args, smem, st);
 }
@@ -394,7 +578,7 @@ size_t capped_scratch_bytes(int64_t n, int E, int groups) {
 }
 
 cudaError_t launch_capped_assignment(const float* S, int64_t ng, int E, int64_t kg, int groups, int b, int iters,
-                                     float lambda, float* A, void* scratch, cudaStream_t st) {
+                                     float lambda, float* A, void* scratch, int* status, cudaStream_t st) {
   if (E > kCapMaxE || iters < 1 || b < 1 || !(lambda > 0.f)) return cudaErrorInvalidValue;
   const int64_t n = ng * groups;
   char* p = (char*)scratch;
@@ -410,11 +594,15 @@ cudaError_t launch_capped_assignment(const float* S, int64_t ng, int E, int64_t 
   int bpg = blocks_per_group(ng, groups, sms);
   if ((int64_t)bpg * groups > (int64_t)blocks) bpg = (int)(blocks / groups);
   const dim3 grid(bpg, groups);
+  // the words of the resident forms take the place of the two sets of partials
+  const size_t room = 2 * align256(blocks * E * sizeof(float2)) / sizeof(unsigned long long);
+  if (Exchange::words(bpg, groups, E) > room) coop = 0;
+  const Exchange ex = Exchange::at(reinterpret_cast<unsigned long long*>(part[0]), bpg, groups, E, status);
   const float inv_lambda = 1.f / lambda, log_k = logf((float)kg), log_b = logf((float)b);
   const int epl = E <= 32 ? 1 : (E <= 64 ? 2 : (E <= 128 ? 4 : 8));
   const int64_t tpw = (ng + (int64_t)bpg * kCapWarps - 1) / ((int64_t)bpg * kCapWarps);
   if (coop && tpw * epl <= kCapResident) {
-    ResidentArgs a{S, A, part[0], part[1], ng, E, inv_lambda, log_k, log_b, iters};
+    ResidentArgs a{S, A, ex, ng, E, inv_lambda, log_k, log_b, iters};
     bool fits = false;
     cudaError_t e = epl == 1 ? launch_resident_tpw<1>((int)tpw, a, grid, sms, &fits, st)
                   : epl == 2 ? launch_resident_tpw<2>((int)tpw, a, grid, sms, &fits, st)
@@ -424,7 +612,7 @@ cudaError_t launch_capped_assignment(const float* S, int64_t ng, int E, int64_t 
     if (fits) return cudaGetLastError();
   }
   if (coop && tpw * epl > kCapResident && tpw <= 1024) {             // too many entries for registers: try shared memory
-    ResidentArgs a{S, A, part[0], part[1], ng, E, inv_lambda, log_k, log_b, iters};
+    ResidentArgs a{S, A, ex, ng, E, inv_lambda, log_k, log_b, iters};
     bool fits = false;
     cudaError_t e = epl == 1 ? launch_resident_smem<1>(a, (int)tpw, grid, sms, &fits, st)
                   : epl == 2 ? launch_resident_smem<2>(a, (int)tpw, grid, sms, &fits, st)

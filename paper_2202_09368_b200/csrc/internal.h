@@ -97,7 +97,7 @@ cudaError_t launch_reduce_partials(int dtype, const float* part, void* out, int 
 // Kullback-Leibler projections, per routing group; entries in [0, 1].  E <= 256.
 size_t capped_scratch_bytes(int64_t n, int E, int groups);
 cudaError_t launch_capped_assignment(const float* S, int64_t ng, int E, int64_t kg, int groups, int b, int iters,
-                                     float lambda, float* A, void* scratch, cudaStream_t st);
+                                     float lambda, float* A, void* scratch, int* status, cudaStream_t st);
 // G[i, j] = S[I[i, j], i] for I, G of shape [E, k]
 cudaError_t launch_gather_gate(const float* S, const int32_t* I, float* G, int64_t slots_total, int64_t k, int E,
                                int64_t n, int* status, cudaStream_t st);
