@@ -499,6 +499,8 @@ capped_resident_smem_kernel(const float* __restrict__ S, float* __restrict__ A, 
 
 __global__ void gather_gate_kernel(const float* __restrict__ S, const int32_t* __restrict__ I, float* __restrict__ G,
                                    int64_t slots_total, int64_t k, int E, int64_t n, int* status) {
+  chain_enter();
+  S = after_enter(S); I = after_enter(I);
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < slots_total; s += (int64_t)gridDim.x * blockDim.x) {
     const int t = I[s];
     G[s] = idx_ok(t, 0, n, status) ? S[(int64_t)t * E + (int)(s / k)] : 0.f;
@@ -639,10 +641,8 @@ cudaError_t launch_capped_assignment(const float* S, int64_t ng, int E, int64_t 
 
 cudaError_t launch_gather_gate(const float* S, const int32_t* I, float* G, int64_t slots_total, int64_t k, int E,
                                int64_t n, int* status, cudaStream_t st) {
-  count_launch();
   const int64_t blocks = (slots_total + 255) / 256;
-  gather_gate_kernel<<<(unsigned)(blocks > 1184 ? 1184 : blocks), 256, 0, st>>>(S, I, G, slots_total, k, E, n, status);
-  return cudaGetLastError();
+  return launch_chained(gather_gate_kernel, dim3((unsigned)(blocks > 1184 ? 1184 : blocks)), dim3(256), 0, st, S, I, G, slots_total, k, E, n, status);
 }
 
 }  // namespace ecmoe

@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kern
   static_assert(TX % 8 == 0 && TM % 4 == 0 && TN % 4 == 0, "a warp covers 4 x 8 threads");
   using LA = TileLoader<TA, BM, BK, NT, VEC>;
   using LB = TileLoader<TB, BN, BK, NT, VEC>;
+  chain_enter();
   constexpr int kBuf = BK * (BM + BN);                // one k-tile of both operands
   extern __shared__ __align__(16) float simt_smem[];  // [KS groups][2 buffers][A | B]; after the main loop the other groups' sums
   const int b = blockIdx.z, grp = threadIdx.x / NT;
@@ -371,9 +372,7 @@ cudaError_t launch_tile(const GemmArgs& g, const Operand& oa, const Operand& ob,
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
-  count_launch();
-  kern<<<grid, BM / TM * (BN / TN) * KS, smem, st>>>(g, oa, ob, c_vec);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, dim3(BM / TM * (BN / TN) * KS), smem, st, g, oa, ob, c_vec);
 }
 
 // Operands whose groups of four straddle an edge (an expert count that is not a multiple of four, in the gate's gradients

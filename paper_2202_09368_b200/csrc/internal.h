@@ -40,9 +40,48 @@ __device__ __forceinline__ bool idx_ok(int64_t, int64_t, int64_t, int*) { return
 // 3 ties at the threshold were taken in token order.
 struct SelState { unsigned long long prefix; unsigned int k_rem, mode, shift, cand; unsigned int pad[2]; };
 
+// ---- chained launches ----------------------------------------------------------------------------
+// A layer call is a chain of kernels, most of them over in a few microseconds, on one stream.  launch_chained() lets the
+// next kernel of the chain be set up while the previous one drains (programmatic stream serialization).  The contract that
+// makes this safe, whatever runs before and after the call on the stream: every thread of a kernel launched this way
+// calls chain_enter() before its first access to global memory, which waits until everything before the kernel has
+// completed and is visible.  Completion is then transitive along the chain.  What may come before chain_enter(): shared
+// memory, barriers, tensor memory, descriptors in kernel parameters.
+// Pointers that are read through qualifiers a compiler may take for "never written" (const __restrict__ parameters)
+// pass through after_enter(), so that no load of theirs can be moved up past the wait.
+__device__ __forceinline__ void chain_enter() {
+#if defined(__CUDA_ARCH__)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+// Only the second half, for a kernel that is launched plainly (everything before it has completed when it starts).
+__device__ __forceinline__ void chain_next() {
+#if defined(__CUDA_ARCH__)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+template <typename T> __device__ __forceinline__ T* after_enter(T* p) {
+#if defined(__CUDA_ARCH__)
+  asm volatile("" : "+l"(p));
+#endif
+  return p;
+}
+
 // ---- bookkeeping (api.cu) ----------------------------------------------------------------------
 // Every kernel launch of the library goes through count_launch(); ec_launch_count() reports the sum.
 void count_launch(int n = 1);
+
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // ---- routing (routing.cu) -------------------------------------------------------------------
 cudaError_t launch_gate_softmax_simt(int dtype, const void* X, const void* Wg, float* S, int64_t n,

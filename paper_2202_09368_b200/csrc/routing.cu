@@ -79,6 +79,8 @@ __host__ __device__ constexpr int gate_smem_bytes(int NG) { return 2 * (8 / NG) 
 template <typename T, int NG, bool WVEC>
 __global__ void __launch_bounds__(kGateThreads)
 gate_softmax_simt_kernel(const T* __restrict__ X, const T* __restrict__ Wg, float* __restrict__ S, int64_t n, int d, int E) {
+  chain_enter();
+  X = after_enter(X); Wg = after_enter(Wg);
   constexpr int KS = 8 / NG, DK = KS * kGateSlice, C = 32 * NG;         // chunk: DK depths of 32 tokens and of C experts
   constexpr int kX = DK * kGateTT, kW = DK * C, XQ = (kX / 4 + kGateThreads - 1) / kGateThreads, WQ = kW / 4 / kGateThreads;
   extern __shared__ __align__(16) float gate_smem[];                    // [2][X chunk [DK][32] | W chunk [DK][C]]
@@ -201,9 +203,7 @@ cudaError_t launch_gate_ng(const T* X, const T* Wg, float* S, int64_t n, int d, 
   constexpr int smem = gate_smem_bytes(NG);
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  count_launch();
-  kern<<<grid, kGateThreads, smem, st>>>(X, Wg, S, n, d, E);
-  return cudaGetLastError();
+  return launch_chained(kern, dim3(grid), dim3(kGateThreads), smem, st, X, Wg, S, n, d, E);
 }
 template <typename T>
 cudaError_t launch_gate_t(const T* X, const T* Wg, float* S, int64_t n, int d, int E, cudaStream_t st) {
@@ -336,6 +336,8 @@ template <bool VEC>
 __global__ void __launch_bounds__(kHistThreads, 1)
 topk_hist_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, int pass, int rows_per_cta,
                  SelState* state, unsigned* hist, unsigned* counters) {
+  chain_enter();
+  S = after_enter(S);
   extern __shared__ unsigned sh[];                     // [bin][column]
   __shared__ unsigned long long s_prefix[kTopkChunk];
   __shared__ int s_active[kTopkChunk];
@@ -437,6 +439,8 @@ topk_hist_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, int 
 __global__ void __launch_bounds__(1024)
 topk_ties_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, int64_t kpad, SelState* state,
                  unsigned long long* keys) {
+  chain_enter();
+  S = after_enter(S);
   __shared__ unsigned s_warp[32];
   __shared__ unsigned s_total;
   const int e = blockIdx.x, grp = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -477,6 +481,8 @@ __global__ void __launch_bounds__(kHistThreads)
 topk_compact_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, int64_t kpad, int rows_per_cta,
                     const SelState* __restrict__ state, unsigned* cursor, unsigned long long* keys,
                     unsigned long long* cand) {
+  chain_enter();
+  S = after_enter(S); state = after_enter(state);
   __shared__ unsigned long long s_key[kCompactCap];
   __shared__ unsigned char s_tag[kCompactCap];         // column within the chunk, bit 7: candidate
   __shared__ unsigned s_cnt[2][kTopkChunk], s_base[2][kTopkChunk], s_n;
@@ -582,6 +588,8 @@ constexpr int kSortThreads = 1024;
 __global__ void __launch_bounds__(kSortThreads)
 topk_finish_tile_kernel(const unsigned long long* __restrict__ keys, const unsigned long long* __restrict__ cand,
                         const SelState* __restrict__ state, int64_t kpad, int64_t k, SlotMap map, int32_t* I, float* G) {
+  chain_enter();
+  keys = after_enter(keys); cand = after_enter(cand); state = after_enter(state);
   __shared__ unsigned long long sk[kSortTile];
   __shared__ unsigned long long sc[kCandCap];
   const int e = blockIdx.x;
@@ -602,6 +610,8 @@ topk_finish_tile_kernel(const unsigned long long* __restrict__ keys, const unsig
 __global__ void __launch_bounds__(kSortThreads)
 topk_resolve_kernel(unsigned long long* keys, const unsigned long long* __restrict__ cand,
                     const SelState* __restrict__ state, int64_t kpad, int64_t k) {
+  chain_enter();
+  cand = after_enter(cand); state = after_enter(state);
   __shared__ unsigned long long sc[kCandCap];
   const int e = blockIdx.x;
   const SelState st = state[e];
@@ -616,6 +626,7 @@ topk_resolve_kernel(unsigned long long* keys, const unsigned long long* __restri
 __global__ void __launch_bounds__(kSortThreads)
 topk_sort_tile_kernel(unsigned long long* keys, int64_t kpad, int64_t k, int64_t size_lo, int64_t size_hi,
                       int emit, SlotMap map, int32_t* I, float* G) {
+  chain_enter();
   __shared__ unsigned long long sk[kSortTile];
   const int64_t tiles_per_expert = (kpad + kSortTile - 1) / kSortTile;
   const int64_t expert = blockIdx.x / tiles_per_expert;
@@ -647,6 +658,7 @@ topk_sort_tile_kernel(unsigned long long* keys, int64_t kpad, int64_t k, int64_t
 // One compare-exchange step at a stride that spans tiles.
 __global__ void topk_sort_global_kernel(unsigned long long* keys, int64_t kpad, int64_t total_pairs,
                                         int64_t size, int64_t stride) {
+  chain_enter();
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < total_pairs;
        p += (int64_t)gridDim.x * blockDim.x) {
     const int64_t expert = p / (kpad >> 1), q = p % (kpad >> 1);
@@ -665,6 +677,8 @@ __global__ void topk_sort_global_kernel(unsigned long long* keys, int64_t kpad, 
 constexpr int kSmallN = 16384;
 __global__ void __launch_bounds__(1024)
 topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, SlotMap map, int32_t* I, float* G) {
+  chain_enter();
+  S = after_enter(S);
   extern __shared__ unsigned long long sm_keys[];      // [kpad] keys, then [n] values, then [kBins] histogram
   unsigned* val = reinterpret_cast<unsigned*>(sm_keys + kpad);
   unsigned* hist = val + n;
@@ -747,8 +761,7 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
     if (e0 != cudaSuccess) return e0;
     int threads = 128;                                 // about eight elements per thread
     while (threads < 1024 && threads * 8 < n) threads <<= 1;
-    count_launch();
-    topk_small_kernel<<<dim3(E, groups), threads, smem, st>>>(S, (int)n, E, (int)k, (int)L.kpad, smap, I, G);
+    launch_chained(topk_small_kernel, dim3(E, groups), dim3(threads), smem, st, S, (int)n, E, (int)k, (int)L.kpad, smap, I, G);
     return cudaGetLastError();
   }
   const int64_t VE = (int64_t)groups * E;              // independent columns: E per group
@@ -773,33 +786,25 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
   int64_t rows = (n + want - 1) / want; if (rows < 256) rows = 256;
   const dim3 grid((unsigned)((n + rows - 1) / rows), (unsigned)L.chunks, (unsigned)groups);
   for (int pass = 0; pass < kRadixPasses; ++pass) {
-    count_launch();
-    if (vec) topk_hist_kernel<true><<<grid, kHistThreads, kHistSmemBytes, st>>>(S, n, E, (unsigned)k, pass, (int)rows, state, hist, counters);
-    else topk_hist_kernel<false><<<grid, kHistThreads, kHistSmemBytes, st>>>(S, n, E, (unsigned)k, pass, (int)rows, state, hist, counters);
+    if (vec) launch_chained(topk_hist_kernel<true>, grid, dim3(kHistThreads), kHistSmemBytes, st, S, n, E, (unsigned)k, pass, (int)rows, state, hist, counters);
+    else launch_chained(topk_hist_kernel<false>, grid, dim3(kHistThreads), kHistSmemBytes, st, S, n, E, (unsigned)k, pass, (int)rows, state, hist, counters);
   }
-  count_launch();
-  topk_ties_kernel<<<dim3(E, groups), 1024, 0, st>>>(S, n, E, (unsigned)k, L.kpad, state, keys);
-  count_launch();
-  if (vec) topk_compact_kernel<true><<<grid, kHistThreads, 0, st>>>(S, n, E, (unsigned)k, L.kpad, (int)rows, state, cursor, keys, cand);
-  else topk_compact_kernel<false><<<grid, kHistThreads, 0, st>>>(S, n, E, (unsigned)k, L.kpad, (int)rows, state, cursor, keys, cand);
+  launch_chained(topk_ties_kernel, dim3(E, groups), dim3(1024), 0, st, S, n, E, (unsigned)k, L.kpad, state, keys);
+  if (vec) launch_chained(topk_compact_kernel<true>, grid, dim3(kHistThreads), 0, st, S, n, E, (unsigned)k, L.kpad, (int)rows, state, cursor, keys, cand);
+  else launch_chained(topk_compact_kernel<false>, grid, dim3(kHistThreads), 0, st, S, n, E, (unsigned)k, L.kpad, (int)rows, state, cursor, keys, cand);
   if (L.kpad <= kSortTile) {
-    count_launch();
-    topk_finish_tile_kernel<<<(unsigned)VE, kSortThreads, 0, st>>>(keys, cand, state, L.kpad, k, map, I, G);
+    launch_chained(topk_finish_tile_kernel, dim3((unsigned)VE), dim3(kSortThreads), 0, st, keys, cand, state, L.kpad, k, map, I, G);
   } else {
     const int64_t tiles = (L.kpad + kSortTile - 1) / kSortTile;
     const unsigned sort_grid = (unsigned)(VE * tiles);
-    count_launch();
-    topk_resolve_kernel<<<(unsigned)VE, kSortThreads, 0, st>>>(keys, cand, state, L.kpad, k);
-    count_launch();
-    topk_sort_tile_kernel<<<sort_grid, kSortThreads, 0, st>>>(keys, L.kpad, k, 2, kSortTile, 0, map, I, G);
+    launch_chained(topk_resolve_kernel, dim3((unsigned)VE), dim3(kSortThreads), 0, st, keys, cand, state, L.kpad, k);
+    launch_chained(topk_sort_tile_kernel, dim3(sort_grid), dim3(kSortThreads), 0, st, keys, L.kpad, k, 2, kSortTile, 0, map, I, G);
     const int64_t pairs = VE * (L.kpad >> 1);
     for (int64_t size = 2 * kSortTile; size <= L.kpad; size <<= 1) {
       for (int64_t stride = size >> 1; stride >= kSortTile; stride >>= 1) {
-        count_launch();
-        topk_sort_global_kernel<<<grid_for(pairs, 256), 256, 0, st>>>(keys, L.kpad, pairs, size, stride);
+        launch_chained(topk_sort_global_kernel, dim3(grid_for(pairs, 256)), dim3(256), 0, st, keys, L.kpad, pairs, size, stride);
       }
-      count_launch();
-      topk_sort_tile_kernel<<<sort_grid, kSortThreads, 0, st>>>(keys, L.kpad, k, size, size, size == L.kpad, map, I, G);
+      launch_chained(topk_sort_tile_kernel, dim3(sort_grid), dim3(kSortThreads), 0, st, keys, L.kpad, k, size, size, size == L.kpad, map, I, G);
     }
   }
   return cudaGetLastError();
@@ -811,6 +816,8 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
 // One warp per token row of S: the two largest scores, equal scores to the lower expert.  A score in [0, 1] orders
 // like its bit pattern; the key puts the inverted expert index below it so that one max decides both.
 __global__ void __launch_bounds__(256) token_top2_kernel(const float* __restrict__ S, int64_t rows, int E, int32_t* __restrict__ choice) {
+  chain_enter();
+  S = after_enter(S);
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < rows; t += warps) {
@@ -837,6 +844,8 @@ __global__ void __launch_bounds__(256) token_top2_kernel(const float* __restrict
 __global__ void __launch_bounds__(1024)
 token_admit_kernel(const float* __restrict__ S, const int32_t* __restrict__ choice, int n, int E, int k,
                    int32_t* __restrict__ I, float* __restrict__ G, int32_t* __restrict__ load, int32_t* __restrict__ requested) {
+  chain_enter();
+  S = after_enter(S); choice = after_enter(choice);
   __shared__ unsigned s_warp[33];
   const int e = blockIdx.x, grp = blockIdx.y, groups = gridDim.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t row0 = (int64_t)grp * n;
@@ -869,15 +878,13 @@ token_admit_kernel(const float* __restrict__ S, const int32_t* __restrict__ choi
 }
 
 cudaError_t launch_token_top2(const float* S, int64_t rows, int E, int32_t* choice, cudaStream_t st) {
-  count_launch();
-  token_top2_kernel<<<grid_for(rows * 32, 256, 148 * 8), 256, 0, st>>>(S, rows, E, choice);
+  launch_chained(token_top2_kernel, dim3(grid_for(rows * 32, 256, 148 * 8)), dim3(256), 0, st, S, rows, E, choice);
   return cudaGetLastError();
 }
 
 cudaError_t launch_token_admit(const float* S, const int32_t* choice, int64_t n, int E, int64_t k, int groups,
                                int32_t* I, float* G, int32_t* load, int32_t* requested, cudaStream_t st) {
-  count_launch();
-  token_admit_kernel<<<dim3(E, groups), 1024, 0, st>>>(S, choice, (int)n, E, (int)k, I, G, load, requested);
+  launch_chained(token_admit_kernel, dim3(E, groups), dim3(1024), 0, st, S, choice, (int)n, E, (int)k, I, G, load, requested);
   return cudaGetLastError();
 }
 
@@ -894,6 +901,8 @@ size_t inverse_scratch_bytes(int64_t n) {
 }
 
 __global__ void inv_count_kernel(const int32_t* __restrict__ I, int64_t total, int32_t* cnt, int64_t n, int* status) {
+  chain_enter();
+  I = after_enter(I);
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < total; s += (int64_t)gridDim.x * blockDim.x) {
     const int t = I[s];
     if (t >= 0 && idx_ok(t, 0, n, status)) atomicAdd(&cnt[t], 1);      // -1: an empty slot (token-choice routing only)
@@ -923,6 +932,8 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* s_warp, int& tot
 // Step 1: exclusive scan inside each tile of kScanTile counts (four per thread), tile sums aside.
 __global__ void __launch_bounds__(kScanThreads) inv_scan_tile_kernel(const int32_t* __restrict__ cnt, int64_t n,
                                                                       int32_t* row_ptr, int32_t* tile_sum) {
+  chain_enter();
+  cnt = after_enter(cnt);
   __shared__ int s_warp[33];
   const int64_t base = (int64_t)blockIdx.x * kScanTile + threadIdx.x * 4;
   int c[4];
@@ -938,6 +949,8 @@ __global__ void __launch_bounds__(kScanThreads) inv_scan_tile_kernel(const int32
 // Step 2: every tile adds the sum of the tiles before it; the last one also writes row_ptr[n].
 __global__ void __launch_bounds__(kScanThreads) inv_scan_add_kernel(const int32_t* __restrict__ tile_sum, int64_t n,
                                                                      int32_t* row_ptr) {
+  chain_enter();
+  tile_sum = after_enter(tile_sum);
   __shared__ int s_warp[33];
   int part = 0;
   for (int j = threadIdx.x; j < (int)blockIdx.x; j += kScanThreads) part += tile_sum[j];
@@ -952,6 +965,8 @@ __global__ void __launch_bounds__(kScanThreads) inv_scan_add_kernel(const int32_
 // Hands each slot a place in its token's list, counting the token's counter back down to zero.
 __global__ void inv_fill_kernel(const int32_t* __restrict__ I, int64_t total, const int32_t* __restrict__ row_ptr,
                                 int32_t* cnt, int32_t* slots, int64_t n) {
+  chain_enter();
+  I = after_enter(I); row_ptr = after_enter(row_ptr);
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < total; s += (int64_t)gridDim.x * blockDim.x) {
     const int t = I[s];
     if (t >= 0 && idx_ok(t, 0, n, nullptr)) slots[row_ptr[t] + atomicSub(&cnt[t], 1) - 1] = (int32_t)s;   // counted once, in inv_count
@@ -959,6 +974,8 @@ __global__ void inv_fill_kernel(const int32_t* __restrict__ I, int64_t total, co
 }
 
 __global__ void inv_sort_kernel(const int32_t* __restrict__ row_ptr, int64_t n, int32_t* slots) {
+  chain_enter();
+  row_ptr = after_enter(row_ptr);
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     const int a = row_ptr[t], b = row_ptr[t + 1];
     for (int i = a + 1; i < b; ++i) {
@@ -975,6 +992,8 @@ __global__ void inv_sort_kernel(const int32_t* __restrict__ row_ptr, int64_t n, 
 constexpr int kInvSmallN = 4096, kInvSmallSlots = 1 << 14;
 __global__ void __launch_bounds__(1024)
 inv_small_kernel(const int32_t* __restrict__ I, int n, int total, int32_t* row_ptr, int32_t* slots, int* status) {
+  chain_enter();
+  I = after_enter(I);
   extern __shared__ int s_cnt[];                       // [n] counts, then cursors
   __shared__ int s_warp[33];
   const int tid = threadIdx.x;
@@ -1013,6 +1032,8 @@ __device__ __forceinline__ void inv_cluster_sync() {
 }
 __global__ void __launch_bounds__(1024)
 inv_cluster_kernel(const int32_t* __restrict__ I, int n, int total, int32_t* row_ptr, int32_t* slots, int32_t* cnt, int* status) {
+  chain_enter();
+  I = after_enter(I);
   __shared__ int s_warp[33];
   __shared__ int s_tile;                               // sum of this CTA's part of the counts
   const int tid = threadIdx.x, rank = blockIdx.x, nc = gridDim.x;      // the grid is the one cluster
@@ -1058,10 +1079,12 @@ cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t total, int
   if (n > kInvSmallN && n <= kInvClusterN && total <= kInvClusterSlots) {
     cudaLaunchConfig_t cfg; memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(kInvClusterCtas); cfg.blockDim = dim3(1024); cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = kInvClusterCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_chained()
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
     count_launch();
     return cudaLaunchKernelEx(&cfg, inv_cluster_kernel, I, (int)n, (int)total, row_ptr, slots, (int32_t*)scratch, status);
   }
@@ -1069,8 +1092,7 @@ cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t total, int
     const int smem = (int)n * 4;
     cudaError_t e0 = cudaFuncSetAttribute(inv_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e0 != cudaSuccess) return e0;
-    count_launch();
-    inv_small_kernel<<<1, 1024, smem, st>>>(I, (int)n, (int)total, row_ptr, slots, status);
+    launch_chained(inv_small_kernel, dim3(1), dim3(1024), smem, st, I, (int)n, (int)total, row_ptr, slots, status);
     return cudaGetLastError();
   }
   int32_t* cnt = (int32_t*)scratch;
@@ -1078,16 +1100,11 @@ cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t total, int
   const unsigned tiles = (unsigned)((n + kScanTile - 1) / kScanTile);
   cudaError_t e;
   if ((e = cudaMemsetAsync(cnt, 0, (size_t)(n + 1) * 4, st)) != cudaSuccess) return e;
-  count_launch();
-  inv_count_kernel<<<grid_for(total, 256), 256, 0, st>>>(I, total, cnt, n, status);
-  count_launch();
-  inv_scan_tile_kernel<<<tiles, kScanThreads, 0, st>>>(cnt, n, row_ptr, tile_sum);
-  count_launch();
-  inv_scan_add_kernel<<<tiles, kScanThreads, 0, st>>>(tile_sum, n, row_ptr);
-  count_launch();
-  inv_fill_kernel<<<grid_for(total, 256), 256, 0, st>>>(I, total, row_ptr, cnt, slots, n);
-  count_launch();
-  inv_sort_kernel<<<grid_for(n, 256), 256, 0, st>>>(row_ptr, n, slots);
+  launch_chained(inv_count_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, I, total, cnt, n, status);
+  launch_chained(inv_scan_tile_kernel, dim3(tiles), dim3(kScanThreads), 0, st, cnt, n, row_ptr, tile_sum);
+  launch_chained(inv_scan_add_kernel, dim3(tiles), dim3(kScanThreads), 0, st, tile_sum, n, row_ptr);
+  launch_chained(inv_fill_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, I, total, row_ptr, cnt, slots, n);
+  launch_chained(inv_sort_kernel, dim3(grid_for(n, 256)), dim3(256), 0, st, row_ptr, n, slots);
   return cudaGetLastError();
 }
 
@@ -1155,6 +1172,8 @@ cudaError_t launch_validate_routing(const int32_t* I, const int32_t* row_ptr, co
 // ------------------------------------------------------------------------------------------
 __global__ void gather_kernel(const uint4* __restrict__ X, const int32_t* __restrict__ I, uint4* __restrict__ X_in,
                               int64_t total_vec, int vec_per_row, int64_t n, int* status) {
+  chain_enter();
+  X = after_enter(X); I = after_enter(I);
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total_vec; g += (int64_t)gridDim.x * blockDim.x) {
     const int64_t s = g / vec_per_row; const int v = (int)(g % vec_per_row);
     int t = I[s];                                      // -1: an empty slot (token-choice routing only) holds a zero row
@@ -1167,8 +1186,7 @@ cudaError_t launch_gather(int dtype, const void* X, const int32_t* I, void* X_in
                           cudaStream_t st) {
   const int vpr = d * (dtype == 0 ? 4 : 2) / 16;
   const int64_t tv = total * vpr;
-  count_launch();
-  gather_kernel<<<grid_for(tv, 256, 148 * 32), 256, 0, st>>>((const uint4*)X, I, (uint4*)X_in, tv, vpr, n, status);
+  launch_chained(gather_kernel, dim3(grid_for(tv, 256, 148 * 32)), dim3(256), 0, st, (const uint4*)X, I, (uint4*)X_in, tv, vpr, n, status);
   return cudaGetLastError();
 }
 
@@ -1197,6 +1215,8 @@ template <typename T>
 __global__ void combine_kernel(const float* __restrict__ X_e, const float* __restrict__ G,
                                const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ slots,
                                T* __restrict__ X_out, int64_t total_quads, int quads_per_row, int64_t slots_total, int* status) {
+  chain_enter();
+  X_e = after_enter(X_e); G = after_enter(G); row_ptr = after_enter(row_ptr); slots = after_enter(slots);
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total_quads; g += (int64_t)gridDim.x * blockDim.x) {
     const int64_t t = g / quads_per_row; const int v = (int)(g % quads_per_row);
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1233,20 +1253,22 @@ cudaError_t launch_combine(int dtype, const float* X_e, const float* G, const in
   const int qpr = d / 4;
   const int64_t tq = n * qpr;
   const unsigned grid = grid_for(tq, 256, 148 * 32);
-  if (dtype == 0) { count_launch(); combine_kernel<float><<<grid, 256, 0, st>>>(X_e, G, row_ptr, slots, (float*)X_out, tq, qpr, slots_total, status); }
-  else { count_launch(); combine_kernel<bf16><<<grid, 256, 0, st>>>(X_e, G, row_ptr, slots, (bf16*)X_out, tq, qpr, slots_total, status); }
+  if (dtype == 0) { launch_chained(combine_kernel<float>, grid, dim3(256), 0, st, X_e, G, row_ptr, slots, (float*)X_out, tq, qpr, slots_total, status); }
+  else { launch_chained(combine_kernel<bf16>, grid, dim3(256), 0, st, X_e, G, row_ptr, slots, (bf16*)X_out, tq, qpr, slots_total, status); }
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------
 // Backward of Eq. 4 per slot s = (i, j) holding token t:
 //   dX_e[s,:] = G[s] * dX_out[t,:],   dG[s] = <dX_out[t,:], X_e[s,:]>.   One warp per slot.
+// Launched plainly: a memset precedes it, and its loads are free to move above the previous piece's store.
 // ------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void bwd_combine_kernel(const T* __restrict__ dX_out, const float* __restrict__ X_e,
                                    const float* __restrict__ G, const int32_t* __restrict__ I,
                                    T* __restrict__ dX_e, float* __restrict__ dG, int64_t total, int quads_per_row, int64_t n,
                                    int* status) {
+  chain_next();
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < total; s += warps) {
@@ -1293,6 +1315,8 @@ template <typename TL>
 __global__ void bwd_softmax_kernel(const float* __restrict__ S, const float* __restrict__ dG,
                                    const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ slots,
                                    TL* __restrict__ dL, int64_t n, int E, int64_t k, int* status) {
+  chain_enter();
+  S = after_enter(S); dG = after_enter(dG); row_ptr = after_enter(row_ptr); slots = after_enter(slots);
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t slots_total = (int64_t)E * k;
@@ -1318,10 +1342,9 @@ __global__ void bwd_softmax_kernel(const float* __restrict__ S, const float* __r
 
 cudaError_t launch_bwd_softmax(const float* S, const float* dG, const int32_t* row_ptr, const int32_t* slots,
                                void* dL, int dl_bf16, int64_t n, int E, int64_t k, int* status, cudaStream_t st) {
-  count_launch();
   const unsigned grid = grid_for(n * 32, 256, 148 * 16);
-  if (dl_bf16) bwd_softmax_kernel<bf16><<<grid, 256, 0, st>>>(S, dG, row_ptr, slots, (bf16*)dL, n, E, k, status);
-  else bwd_softmax_kernel<float><<<grid, 256, 0, st>>>(S, dG, row_ptr, slots, (float*)dL, n, E, k, status);
+  if (dl_bf16) launch_chained(bwd_softmax_kernel<bf16>, grid, dim3(256), 0, st, S, dG, row_ptr, slots, (bf16*)dL, n, E, k, status);
+  else launch_chained(bwd_softmax_kernel<float>, grid, dim3(256), 0, st, S, dG, row_ptr, slots, (float*)dL, n, E, k, status);
   return cudaGetLastError();
 }
 
@@ -1338,6 +1361,8 @@ __device__ __forceinline__ float2 ld_pair(const bf16* p) {
 template <typename T>
 __global__ void __launch_bounds__(256) column_sums_kernel(const T* __restrict__ A, T* __restrict__ out, int64_t rows, int cols,
                                                           const int32_t* __restrict__ batch_rows) {
+  chain_enter();
+  A = after_enter(A); batch_rows = after_enter(batch_rows);
   __shared__ float2 s_part[8][32];
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, c = blockIdx.x * 64 + lane * 2;      // cols is a multiple of 4
   int64_t lim = rows;
@@ -1365,9 +1390,8 @@ __global__ void __launch_bounds__(256) column_sums_kernel(const T* __restrict__ 
 cudaError_t launch_column_sums(int dtype, const void* A, void* out, int batches, int64_t rows, int cols,
                                const int32_t* batch_rows, cudaStream_t st) {
   const dim3 grid((cols + 63) / 64, batches);
-  count_launch();
-  if (dtype == 0) column_sums_kernel<float><<<grid, 256, 0, st>>>((const float*)A, (float*)out, rows, cols, batch_rows);
-  else column_sums_kernel<bf16><<<grid, 256, 0, st>>>((const bf16*)A, (bf16*)out, rows, cols, batch_rows);
+  if (dtype == 0) launch_chained(column_sums_kernel<float>, grid, dim3(256), 0, st, (const float*)A, (float*)out, rows, cols, batch_rows);
+  else launch_chained(column_sums_kernel<bf16>, grid, dim3(256), 0, st, (const bf16*)A, (bf16*)out, rows, cols, batch_rows);
   return cudaGetLastError();
 }
 
@@ -1376,6 +1400,8 @@ cudaError_t launch_column_sums(int dtype, const void* A, void* out, int batches,
 // ------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void reduce_partials_kernel(const float* __restrict__ part, T* __restrict__ out, int P, int64_t elems) {
+  chain_enter();
+  part = after_enter(part);
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < elems; g += (int64_t)gridDim.x * blockDim.x) {
     float acc = 0.f;
     for (int p = 0; p < P; ++p) acc += part[(int64_t)p * elems + g];
@@ -1384,8 +1410,8 @@ __global__ void reduce_partials_kernel(const float* __restrict__ part, T* __rest
 }
 
 cudaError_t launch_reduce_partials(int dtype, const float* part, void* out, int P, int64_t elems, cudaStream_t st) {
-  if (dtype == 0) { count_launch(); reduce_partials_kernel<float><<<grid_for(elems, 256), 256, 0, st>>>(part, (float*)out, P, elems); }
-  else { count_launch(); reduce_partials_kernel<bf16><<<grid_for(elems, 256), 256, 0, st>>>(part, (bf16*)out, P, elems); }
+  if (dtype == 0) { launch_chained(reduce_partials_kernel<float>, dim3(grid_for(elems, 256)), dim3(256), 0, st, part, (float*)out, P, elems); }
+  else { launch_chained(reduce_partials_kernel<bf16>, dim3(grid_for(elems, 256)), dim3(256), 0, st, part, (bf16*)out, P, elems); }
   return cudaGetLastError();
 }
 
