@@ -700,9 +700,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                   }
                 }
               }
-              // both buffers are written: Z into the first, H = GeLU(Z) into the second
-              if (lane == 0) bulk_wait_read<0>();
-              __syncwarp();
+              // Z and H = GeLU(Z) are packed in registers first, so that the store of the previous chunk has the whole
+              // arithmetic to leave the two buffers: Z goes into the first, H into the second
+              uint4 zp[8], hp[8];
               // one uniform branch on the GeLU form around the whole chunk: inside it only that form is evaluated
               auto convert = [&](auto variant) {
 #pragma unroll
@@ -713,11 +713,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     z[e] = __uint_as_float(r[8 * j + e]); z[e + 1] = __uint_as_float(r[8 * j + e + 1]);
                     gelu_fwd2<decltype(variant)::value>(z[e], z[e + 1], h[e], h[e + 1]);
                   }
-                  if (!p.skip_c) *reinterpret_cast<uint4*>(stg + lane * 128 + ((j ^ sw) << 4)) = pack8(z);
-                  *reinterpret_cast<uint4*>(stg + 4096 + lane * 128 + ((j ^ sw) << 4)) = pack8(h);
+                  zp[j] = pack8(z); hp[j] = pack8(h);
                 }
               };
               if (p.gelu == 0) convert(std::integral_constant<int, 0>{}); else convert(std::integral_constant<int, 1>{});
+              if (lane == 0) bulk_wait_read<0>();
+              __syncwarp();
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                if (!p.skip_c) *reinterpret_cast<uint4*>(stg + lane * 128 + ((j ^ sw) << 4)) = zp[j];
+                *reinterpret_cast<uint4*>(stg + 4096 + lane * 128 + ((j ^ sw) << 4)) = hp[j];
+              }
               fence_async_smem();
               __syncwarp();
               if (lane == 0 && r0 < p.M) {
