@@ -183,6 +183,7 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, uint32_t src
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
                ::"l"(tm), "r"(src), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* tm) { asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory"); }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
@@ -345,6 +346,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int w = 0; w < kEpiWarps; ++w) published[w] = 0;
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (threadIdx.x == 32 * 2) {                       // the descriptors are on their way while the previous kernel drains
+    prefetch_map(&tmA); prefetch_map(&tmB); prefetch_map(&tmC);
+    if constexpr (EPI == EPI_GELU) prefetch_map(&tmC2);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
@@ -542,6 +547,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int nt = p.n_fast ? tile % p.tiles_n : (tile / p.tiles_m) % p.tiles_n;
       if (tile_kblocks(p, b, mt, TM) == 0) continue; // a tile of empty slots: nothing was accumulated, nothing is stored
       const int buf = kOneAcc ? 0 : it & 1; const uint32_t use = (uint32_t)(kOneAcc ? it : it >> 1);
+      // EPI_ADD_SLOTS: this thread's row of the index, fetched while the accumulator is made
+      int slot_a = 0, slot_b = 0, slot_first = 0;
+      if constexpr (EPI == EPI_ADD_SLOTS) {
+        const int m = mt * TM + (int)rank * BM + q * 32 + lane;
+        if (m < p.M) {
+          slot_a = p.row_ptr[m]; slot_b = p.row_ptr[m + 1];
+          if (!idx_ok(slot_a, 0, p.slots_total + 1, p.status) || !idx_ok(slot_b, slot_a, p.slots_total + 1, p.status)) slot_a = slot_b = 0;
+          if (slot_a < slot_b) slot_first = p.slots[slot_a];
+        }
+      }
       const bool ok = mbar_wait(tfull0 + 8 * buf, use & 1, abort_flag, p.status, 4);
       if constexpr (EPI == EPI_STORE) {
         // the four warps of a column half meet at named barriers below: they leave together or not at all (every one
@@ -646,7 +661,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int r0 = mt * TM + (int)rank * BM + q * 32;
         const int sw = lane & 7;
         constexpr int kColsPerWarp = BN >= 128 ? BN / 2 : BN;      // a 64-wide tile is drained by the first four warps alone
-        const bool active = half * kColsPerWarp < BN;
+        // (plain bf16 results: the four warps of a column half store together, whatever rows they have)
+        const bool active = half * kColsPerWarp < BN && (EPI == EPI_STORE || r0 < p.M);
         if constexpr (EPI == EPI_STORE_F32) {
 #pragma unroll 1
           for (int c0 = half * kColsPerWarp; active && c0 < (half + 1) * kColsPerWarp; c0 += 32, ++nchunk) {
@@ -757,14 +773,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (p.gelu == 0) scale(std::integral_constant<int, 0>{}); else scale(std::integral_constant<int, 1>{});
               }
               if constexpr (EPI == EPI_ADD_SLOTS) {
-                // this thread's row gains the rows of its slots (128 bytes of each), in slot order
-                if (row_ok) {
-                  int qa = p.row_ptr[row], qb = p.row_ptr[row + 1];
-                  if (!idx_ok(qa, 0, p.slots_total + 1, p.status) || !idx_ok(qb, qa, p.slots_total + 1, p.status)) qa = qb = 0;
-                  for (int qq = qa; qq < qb; ++qq) {
-                    const int sid = p.slots[qq];
-                    if (!idx_ok(sid, 0, p.slots_total, p.status)) continue;
-                    const bf16* src = p.rows + (int64_t)sid * p.ld_rows + n0 + c0;
+                // this thread's row gains the rows of its slots (128 bytes of each), in slot order; the next slot's id travels
+                // beside the row of the current one
+                {
+                  int sid = slot_first;
+                  for (int qq = slot_a; qq < slot_b; ++qq) {
+                    const int cur = sid;
+                    if (qq + 1 < slot_b) sid = p.slots[qq + 1];
+                    if (!idx_ok(cur, 0, p.slots_total, p.status)) continue;
+                    const bf16* src = p.rows + (int64_t)cur * p.ld_rows + n0 + c0;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                       if (n0 + c0 + 8 * j < p.N) {
@@ -900,7 +917,14 @@ int pick_bn(const TcGemmArgs& g, int pairs) {
     const int64_t narrow = (rows * ((g.N + 255) / 256) + pairs - 1) / pairs, wide = (rows * ((g.N + 511) / 512) + pairs - 1) / pairs;
     if (wide * 192 <= narrow * 100) return 512;
   }
-  return (g.N > 128 && g.M > BM) ? 256 : (g.N > 64 ? 128 : 64);
+  // A pair's 256-column tile halves to 128 columns where even then every tile has a pair to itself: half the epilogue
+  // per SM on twice the SMs (8 experts, 512
+  // rows, 256 x 512: GEMM-1 16.4 -> 14.3 us, dZ 20.5 -> 16.4 us)
+  if (g.M > BM && g.N > 128) {
+    const int64_t half = (int64_t)((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + 127) / 128) * g.batches;
+    return half <= pairs ? 128 : 256;
+  }
+  return g.N > 64 ? 128 : 64;
 }
 // Two CTAs per tile when a tile of 256 rows is not mostly padding and the pair's B halves are whole 64-wide blocks.
 int pick_ctas(const TcGemmArgs& g, int bn) { return (bn >= 128 && g.M > BM) ? 2 : 1; }
