@@ -83,7 +83,6 @@ struct TcParams {
   int tiles_m, tiles_n, total_tiles, kblocks;
   int n_fast;                                        // consecutive tiles run along N (else along M)
   int gelu;
-  const bf16* Zin;                                   // EPI_GELU_GRAD reads Z directly; every output leaves through a tensor map
   int64_t ldc, batch_c;
   int* status;
   int k_split;                                       // batches are cuts of one product along K
@@ -345,11 +344,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       int* published = (int*)(smem + S * kStage + kStaging + 256 + 2 * kEpiWarps * 32 * 8);
       for (int w = 0; w < kEpiWarps; ++w) published[w] = 0;
     }
+    if constexpr (EPI == EPI_GELU_GRAD) {
+      const uint32_t z0 = smem_u32(smem + S * kStage + kStaging + 256);
+      for (int i = 0; i < 2 * kEpiWarps; ++i) mbar_init(z0 + 8 * i, 1);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x == 32 * 2) {                       // the descriptors are on their way while the previous kernel drains
     prefetch_map(&tmA); prefetch_map(&tmB); prefetch_map(&tmC);
-    if constexpr (EPI == EPI_GELU) prefetch_map(&tmC2);
+    if constexpr (EPI == EPI_GELU || EPI == EPI_GELU_GRAD) prefetch_map(&tmC2);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
@@ -541,6 +544,36 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     int it = 0;
     uint32_t nchunk = 0;                           // chunks this warp has stored so far: picks the staging buffer
     const uint32_t tempty_leader = CTAS == 2 ? map_to_cta(tempty0, 0) : tempty0;
+    // EPI_GELU_GRAD: Z comes through the TMA unit, one chunk of 32 rows x 64 columns ahead of its use, into the staging
+    // buffer of that chunk (the two alternate), with a barrier per buffer.  (Each thread loading its own row of Z as it
+    // needed it left the wait in the open: 119-123 us for dZ at the 100M/32E shape, 113 us like this.  Loading it into registers a
+    // chunk ahead is worse, 141 us: the fence before every store waits for loads in flight.)
+    [[maybe_unused]] const uint32_t zbar0 = smem_u32(smem + S * kStage + kStaging + 256 + (warp - 2) * 16);
+    constexpr int kColsOfWarp = BN >= 128 ? BN / 2 : BN;
+    // first tile from `t` on, in this CTA's order, in which this warp has a chunk
+    [[maybe_unused]] auto z_tile_from = [&](int t) {
+      for (; t < p.total_tiles; t += tile_step) {
+        const int b = t / (p.tiles_m * p.tiles_n);
+        const int mt = p.n_fast ? (t / p.tiles_n) % p.tiles_m : t % p.tiles_m;
+        const int nt = p.n_fast ? t % p.tiles_n : (t / p.tiles_m) % p.tiles_n;
+        if (mt * TM + (int)rank * BM + q * 32 < p.M && nt * BN + half * kColsOfWarp < p.N && tile_kblocks(p, b, mt, TM) != 0) break;
+      }
+      return t;
+    };
+    [[maybe_unused]] auto z_issue = [&](uint32_t n, int t, int c0) {   // chunk number n of this warp; one lane
+      const int b = t / (p.tiles_m * p.tiles_n);
+      const int mt = p.n_fast ? (t / p.tiles_n) % p.tiles_m : t % p.tiles_m;
+      const int nt = p.n_fast ? t % p.tiles_n : (t / p.tiles_m) % p.tiles_n;
+      const uint32_t bar = zbar0 + 8 * (n & 1);
+      mbar_expect_tx(bar, 4096);
+      tma_load_3d(smem_u32(smem + S * kStage + (warp - 2) * kStagingPerWarp) + (n & 1) * 4096, &tmC2, bar, nt * BN + c0,
+                  mt * TM + (int)rank * BM + q * 32, b);
+    };
+    if constexpr (EPI == EPI_GELU_GRAD) {
+      const int t = half * kColsOfWarp < BN ? z_tile_from(first_tile) : p.total_tiles;
+      if (lane == 0 && t < p.total_tiles) z_issue(0, t, half * kColsOfWarp);
+      __syncwarp();
+    }
     for (int tile = first_tile; tile < p.total_tiles; tile += tile_step) {
       const int b = tile / (p.tiles_m * p.tiles_n);
       const int mt = p.n_fast ? (tile / p.tiles_n) % p.tiles_m : tile % p.tiles_m;
@@ -567,10 +600,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       tc_fence_after();
       const int row = mt * TM + (int)rank * BM + q * 32 + lane;
-      const bool row_ok = row < p.M;
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + buf * BN;
       const int n0 = nt * BN;
-      const int64_t obase = (int64_t)b * p.batch_c + (int64_t)row * p.ldc;
       if constexpr (EPI == EPI_SOFTMAX) {
         // Eq. 2: softmax over the N = E columns of each row; columns >= N are padding.  A thread owns one
         // row.  With BN >= 128 the two warps of a lane quarter take half of the columns each and exchange
@@ -749,18 +780,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               }
             } else {
               if constexpr (EPI == EPI_GELU_GRAD) {
-                // dZ = acc * GeLU'(Z): this thread's 64 values of Z (128 bytes of its row)
-                const bf16* zp = p.Zin + obase + n0 + c0;
-                uint4 zv[8];
+                // dZ = acc * GeLU'(Z).  The chunk of Z lies in the buffer that will take the chunk of dZ (see z_issue); a lane
+                // reads and rewrites its own row.  Half-way through the arithmetic the store of the previous chunk has read
+                // the other buffer, and the next chunk's Z is asked for.
+                const bool zok = mbar_wait(zbar0 + 8 * (nchunk & 1), (nchunk >> 1) & 1, abort_flag, p.status, 10);
+                if (!__all_sync(0xffffffffu, zok)) { gave_up = true; break; }
+                const uint8_t* zrow = stg + (nchunk & 1) * 4096 + lane * 128;
+                auto scale = [&](auto variant, int j0) {     // one uniform branch on the GeLU form, as above
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  zv[j] = make_uint4(0, 0, 0, 0);
-                  if (row_ok && n0 + c0 + 8 * j < p.N) zv[j] = *reinterpret_cast<const uint4*>(zp + 8 * j);
-                }
-                auto scale = [&](auto variant) {             // one uniform branch on the GeLU form, as above
-#pragma unroll
-                  for (int j = 0; j < 8; ++j) {
-                    const unsigned zw[4] = {zv[j].x, zv[j].y, zv[j].z, zv[j].w};
+                  for (int jj = 0; jj < 4; ++jj) {
+                    const int j = j0 + jj;
+                    const uint4 zv = *reinterpret_cast<const uint4*>(zrow + ((j ^ sw) << 4));
+                    const unsigned zw[4] = {zv.x, zv.y, zv.z, zv.w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                       float g0, g1;
@@ -770,7 +801,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     }
                   }
                 };
-                if (p.gelu == 0) scale(std::integral_constant<int, 0>{}); else scale(std::integral_constant<int, 1>{});
+                if (p.gelu == 0) scale(std::integral_constant<int, 0>{}, 0); else scale(std::integral_constant<int, 1>{}, 0);
+                {
+                  const bool more = c0 + 64 < (half + 1) * kColsPerWarp && n0 + c0 + 64 < p.N;
+                  const int zt = more ? tile : z_tile_from(tile + tile_step);
+                  if (lane == 0 && zt < p.total_tiles) { bulk_wait_read<0>(); z_issue(nchunk + 1, zt, more ? c0 + 64 : half * kColsPerWarp); }
+                  __syncwarp();
+                }
+                if (p.gelu == 0) scale(std::integral_constant<int, 0>{}, 4); else scale(std::integral_constant<int, 1>{}, 4);
               }
               if constexpr (EPI == EPI_ADD_SLOTS) {
                 // this thread's row gains the rows of its slots (128 bytes of each), in slot order; the next slot's id travels
@@ -818,8 +856,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (leader && rt0 < p.M) { tma_store_3d(&tmC, smem_u32(hb), n0 + c0, rt0, b); bulk_commit(); }
               } else {
                 uint8_t* bufp = stg + (nchunk & 1) * 4096;
-                if (lane == 0) bulk_wait_read<1>();  // the other buffer's store may still be in flight
-                __syncwarp();
+                if constexpr (EPI != EPI_GELU_GRAD) {  // there the buffer holds this chunk's Z
+                  if (lane == 0) bulk_wait_read<1>();  // the other buffer's store may still be in flight
+                  __syncwarp();
+                }
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                   float f[8];
@@ -835,6 +875,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
         }
       }
+      if constexpr (EPI == EPI_GELU_GRAD) { if (gave_up) break; }      // a wait for Z ran out
       tc_fence_before();
       __syncwarp();                                // every lane's tcgen05.ld has completed
       if (lane == 0) {                             // one arrival per warp frees the accumulator
@@ -933,7 +974,8 @@ template <int BN, int EPI, int CTAS>
 cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, const CUtensorMap& tc2,
                        const TcParams& p, cudaStream_t st) {
   // the split softmax trades one operand stage for its exchange area (4 KiB + counters), see the kernel
-  constexpr int smem = num_stages(BN / CTAS, staging_bytes(BN, EPI)) * stage_bytes(BN / CTAS) + staging_bytes(BN, EPI) + 1024 + 256;
+  constexpr int smem = num_stages(BN / CTAS, staging_bytes(BN, EPI)) * stage_bytes(BN / CTAS) + staging_bytes(BN, EPI) + 1024 + 256 +
+                       (EPI == EPI_GELU_GRAD ? 2 * kEpiWarps * 8 : 0);            // the barriers of Z
   auto kern = gemm_tc_kernel<BN, EPI, CTAS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -1032,6 +1074,7 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& g, cudaStream_t st) {
     // plain bf16 results are stored in boxes of 128 rows (a column half's four warps together), the rest in boxes of 32
     if (!make_map(&tc, cbase, g.N, g.M, g.batches, g.ldc, g.batch_c, g.c_f32 ? 32 : 64, (g.epi == EPI_STORE && !g.c_f32) ? 128 : 32,
                   g.c_f32 != 0)) return cudaErrorInvalidValue;
+    if (g.epi == EPI_GELU_GRAD && !make_map(&tc2, g.Zin, g.N, g.M, g.batches, g.ldc, g.batch_c, 64, 32)) return cudaErrorInvalidValue;
     if (g.epi == EPI_GELU && !make_map(&tc2, g.C2, g.N, g.M, g.batches, g.ldc, g.batch_c, 64, 32)) return cudaErrorInvalidValue;
   }
   TcParams p;
@@ -1039,7 +1082,6 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& g, cudaStream_t st) {
   p.tiles_m = (g.M + BM * ctas - 1) / (BM * ctas); p.tiles_n = (g.N + bn - 1) / bn;
   p.total_tiles = p.tiles_m * p.tiles_n * g.batches; p.kblocks = (g.K + BK - 1) / BK;
   p.gelu = g.gelu;
-  p.Zin = (const bf16*)g.Zin;
   p.ldc = g.ldc; p.batch_c = g.batch_c; p.status = g.status;
   p.k_split = g.k_split; p.skip_c = (g.epi == EPI_GELU && !g.C) ? 1 : 0;
   // Tile order.  Tiles running at the same time are consecutive ones.  Along M (default) they share the B tile,
