@@ -796,16 +796,23 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
   const unsigned thr = s_prefix, k_rem = s_rem, k_less = (unsigned)k - k_rem;      // k_rem keys equal to thr are wanted
   // winners in any order: the keys below the threshold, and those at it when all of them are wanted
   const bool all_eq = s_eq == k_rem;
-  for (int t0 = tid - lane; t0 < n; t0 += nt) {
-    const int t = t0 + lane;
-    const unsigned v = t < n ? val[t] : 0xFFFFFFFFu;
-    const bool m = t < n && (v < thr || (all_eq && v == thr));
-    const unsigned bal = __ballot_sync(0xffffffffu, m);
-    if (bal != 0) {
-      unsigned at = 0;
-      if (lane == 0) at = atomicAdd(&s_less, (unsigned)__popc(bal));
-      at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
-      if (m) sm_keys[at] = ((unsigned long long)v << 32) | (unsigned)t;
+  for (int t0 = tid - lane; t0 < n; t0 += 4 * nt) {    // uniform across the warp
+    unsigned v[4], bal[4], sum = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = t0 + u * nt + lane;
+      v[u] = t < n ? val[t] : 0xFFFFFFFFu;
+      bal[u] = __ballot_sync(0xffffffffu, t < n && (v[u] < thr || (all_eq && v[u] == thr)));
+      sum += __popc(bal[u]);
+    }
+    if (sum == 0) continue;
+    unsigned at = 0;
+    if (lane == 0) at = atomicAdd(&s_less, sum);
+    at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (bal[u] >> lane & 1u) sm_keys[at + __popc(bal[u] & ((1u << lane) - 1u))] = ((unsigned long long)v[u] << 32) | (unsigned)(t0 + u * nt + lane);
+      at += __popc(bal[u]);
     }
   }
   // else the first k_rem keys at the threshold in token order
@@ -1058,33 +1065,71 @@ __global__ void inv_fill_kernel(const int32_t* __restrict__ I, int64_t total, co
   }
 }
 
+// Sorts one token's list of slots (ascending).  Up to eight entries, which is nearly every token, are brought in together,
+// sorted in registers and written back: one round trip to memory where an insertion sort in place takes one per step.
+__device__ __forceinline__ void sort_list(int32_t* slots, int lo, int hi) {
+  const int len = hi - lo;
+  if (len <= 1) return;
+  if (len <= 8) {
+    int v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = i < len ? slots[lo + i] : 0x7FFFFFFF;
+    // odd-even transposition: eight rounds sort eight
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int i = r & 1; i + 1 < 8; i += 2) {
+        const int x = min(v[i], v[i + 1]), y = max(v[i], v[i + 1]);
+        v[i] = x; v[i + 1] = y;
+      }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) if (i < len) slots[lo + i] = v[i];
+    return;
+  }
+  for (int i = lo + 1; i < hi; ++i) {
+    const int v = slots[i]; int j = i - 1;
+    while (j >= lo && slots[j] > v) { slots[j + 1] = slots[j]; --j; }
+    slots[j + 1] = v;
+  }
+}
+
 __global__ void inv_sort_kernel(const int32_t* __restrict__ row_ptr, int64_t n, int32_t* slots) {
   chain_enter();
   row_ptr = after_enter(row_ptr);
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int a = row_ptr[t], b = row_ptr[t + 1];
-    for (int i = a + 1; i < b; ++i) {
-      const int v = slots[i]; int j = i - 1;
-      while (j >= a && slots[j] > v) { slots[j + 1] = slots[j]; --j; }
-      slots[j + 1] = v;
-    }
+    sort_list(slots, row_ptr[t], row_ptr[t + 1]);
   }
 }
 
 // Small inputs (n <= kInvSmallN tokens, at most kInvSmallSlots slots): the whole inverse index in one CTA and one
-// launch.  Counts and cursors live in shared memory; the order in which atomics hand out places does not
-// matter because every token's list is sorted at the end.
+// launch.  Counts, cursors and the lists themselves live in shared memory; the order in which atomics hand out places does
+// not matter because every token's list is sorted at the end.  A thread has eight entries of I in flight.
 constexpr int kInvSmallN = 4096, kInvSmallSlots = 1 << 14;
+template <typename F>
+__device__ __forceinline__ void for_slots(const int32_t* I, int first, int total, int step, int n, int* status, F&& f) {
+  for (int s0 = first; s0 < total; s0 += 8 * step) {
+    int t[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[u] = s0 + u * step < total ? I[s0 + u * step] : -1;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) if (t[u] >= 0 && !idx_ok(t[u], 0, n, status)) t[u] = -1;       // -1: an empty slot, or none
+    f(t, s0);
+  }
+}
 __global__ void __launch_bounds__(1024)
 inv_small_kernel(const int32_t* __restrict__ I, int n, int total, int32_t* row_ptr, int32_t* slots, int* status) {
   chain_enter();
   I = after_enter(I);
-  extern __shared__ int s_cnt[];                       // [n] counts, then cursors
+  extern __shared__ int s_cnt[];                       // [n] counts, then cursors; [total] the lists
+  int32_t* s_list = s_cnt + n;
   __shared__ int s_warp[33];
   const int tid = threadIdx.x;
   for (int t = tid; t < n; t += 1024) s_cnt[t] = 0;
   __syncthreads();
-  for (int s = tid; s < total; s += 1024) { const int t = I[s]; if (t >= 0 && idx_ok(t, 0, n, status)) atomicAdd(&s_cnt[t], 1); }
+  for_slots(I, tid, total, 1024, n, status, [&](const int (&t)[8], int) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) if (t[u] >= 0) atomicAdd(&s_cnt[t[u]], 1);
+  });
   __syncthreads();
   // exclusive scan over the tokens, 1024 * per at a time
   const int per = (n + 1023) / 1024, a = min(n, tid * per), b = min(n, a + per);
@@ -1095,17 +1140,14 @@ inv_small_kernel(const int32_t* __restrict__ I, int n, int total, int32_t* row_p
   for (int t = a; t < b; ++t) { const int c = s_cnt[t]; row_ptr[t] = run; s_cnt[t] = run; run += c; }   // s_cnt becomes the cursor
   if (tid == 0) row_ptr[n] = total_sum;
   __syncthreads();
-  for (int s = tid; s < total; s += 1024) { const int t = I[s]; if (t >= 0 && idx_ok(t, 0, n, nullptr)) slots[atomicAdd(&s_cnt[t], 1)] = s; }
+  for_slots(I, tid, total, 1024, n, nullptr, [&](const int (&t)[8], int s0) {      // bad entries were counted above
+#pragma unroll
+    for (int u = 0; u < 8; ++u) if (t[u] >= 0) s_list[atomicAdd(&s_cnt[t[u]], 1)] = s0 + u * 1024;
+  });
   __syncthreads();
-  __threadfence_block();
-  for (int t = tid; t < n; t += 1024) {                // after the fill s_cnt[t] is the end of token t's list
-    const int lo = t == 0 ? 0 : s_cnt[t - 1], hi = s_cnt[t];
-    for (int i = lo + 1; i < hi; ++i) {
-      const int v = slots[i]; int j = i - 1;
-      while (j >= lo && slots[j] > v) { slots[j + 1] = slots[j]; --j; }
-      slots[j + 1] = v;
-    }
-  }
+  for (int t = tid; t < n; t += 1024) sort_list(s_list, t == 0 ? 0 : s_cnt[t - 1], s_cnt[t]);          // after the fill s_cnt[t] is the end of token t's list
+  __syncthreads();
+  for (int s = tid; s < total_sum; s += 1024) slots[s] = s_list[s];
 }
 
 // Medium inputs (n <= kInvClusterN): one cluster of eight CTAs runs the five steps in one launch, with hardware
@@ -1125,7 +1167,10 @@ inv_cluster_kernel(const int32_t* __restrict__ I, int n, int total, int32_t* row
   const int gtid = rank * 1024 + tid, gsize = nc * 1024;
   for (int t = gtid; t < n; t += gsize) cnt[t] = 0;
   inv_cluster_sync();
-  for (int s = gtid; s < total; s += gsize) { const int t = I[s]; if (t >= 0 && idx_ok(t, 0, n, status)) atomicAdd(&cnt[t], 1); }
+  for_slots(I, gtid, total, gsize, n, status, [&](const int (&t)[8], int) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) if (t[u] >= 0) atomicAdd(&cnt[t[u]], 1);
+  });
   inv_cluster_sync();
   // exclusive scan: CTA `rank` takes tokens [lo, hi), a thread `per` consecutive ones of them
   const int per_cta = (n + nc - 1) / nc, lo = min(n, rank * per_cta), hi = min(n, lo + per_cta);
@@ -1147,16 +1192,15 @@ inv_cluster_kernel(const int32_t* __restrict__ I, int n, int total, int32_t* row
   for (int t = a; t < b; ++t) { const int c = cnt[t]; row_ptr[t] = run; cnt[t] = run; run += c; }      // cnt becomes the cursor
   if (rank == nc - 1 && tid == 0) row_ptr[n] = before + tile;
   inv_cluster_sync();
-  for (int s = gtid; s < total; s += gsize) { const int t = I[s]; if (t >= 0 && idx_ok(t, 0, n, nullptr)) slots[atomicAdd(&cnt[t], 1)] = s; }
+  for_slots(I, gtid, total, gsize, n, nullptr, [&](const int (&t)[8], int s0) {
+    int at[8];                                         // eight places asked for at once
+#pragma unroll
+    for (int u = 0; u < 8; ++u) at[u] = t[u] >= 0 ? atomicAdd(&cnt[t[u]], 1) : 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) if (t[u] >= 0) slots[at[u]] = s0 + u * gsize;
+  });
   inv_cluster_sync();
-  for (int t = gtid; t < n; t += gsize) {
-    const int p0 = row_ptr[t], p1 = row_ptr[t + 1];
-    for (int i = p0 + 1; i < p1; ++i) {
-      const int v = slots[i]; int j = i - 1;
-      while (j >= p0 && slots[j] > v) { slots[j + 1] = slots[j]; --j; }
-      slots[j + 1] = v;
-    }
-  }
+  for (int t = gtid; t < n; t += gsize) sort_list(slots, row_ptr[t], row_ptr[t + 1]);
 }
 
 cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t total, int32_t* row_ptr, int32_t* slots,
@@ -1174,7 +1218,7 @@ cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t total, int
     return cudaLaunchKernelEx(&cfg, inv_cluster_kernel, I, (int)n, (int)total, row_ptr, slots, (int32_t*)scratch, status);
   }
   if (n <= kInvSmallN && total <= kInvSmallSlots) {
-    const int smem = (int)n * 4;
+    const int smem = (int)(n + total) * 4;             // at most 80 KiB
     cudaError_t e0 = cudaFuncSetAttribute(inv_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e0 != cudaSuccess) return e0;
     launch_chained(inv_small_kernel, dim3(1), dim3(1024), smem, st, I, (int)n, (int)total, row_ptr, slots, status);
