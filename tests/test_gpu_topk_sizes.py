@@ -26,3 +26,24 @@ def test_selection_is_a_stable_sort(n, E, k, groups, levels):
         got = r.I[:, g * k:(g + 1) * k].long()
         assert torch.equal(got, want)
         assert torch.equal(r.G[:, g * k:(g + 1) * k], torch.gather(r.S.T, 1, got))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,d,E,c", [(130, 8, 4, 2.0), (777, 40, 3, 1.0), (3000, 296, 16, 2.0), (9000, 600, 64, 1.5), (2048, 1032, 8, 2.0)])
+def test_shuffle_and_unshuffle_at_odd_widths(n, d, E, c, dtype):
+    """Rows of 1 to 258 pieces: the shuffle copies bits, the unshuffle adds at most a few slots' rows per token in fp32."""
+    cfg = B.make_config(n, d, 8, E, c, dtype)
+    gen = torch.Generator(device="cuda").manual_seed(n + d)
+    X = torch.empty(n, d, dtype=dtype, device="cuda").normal_(generator=gen)
+    Wg = (torch.empty(d, E, device="cuda").normal_(generator=gen) / d ** 0.5).to(dtype)
+    r = B.ec_route(cfg, X, Wg)
+    assert torch.equal(B.ec_shuffle(cfg, X, r.I), X[r.I.long()])
+    k = B.slots_per_expert(cfg)
+    X_e = torch.empty(E, k, d, device="cuda").normal_(generator=gen)
+    Y = B.ec_unshuffle(cfg, X_e, r.G, r.row_ptr, r.slots).double()
+    terms = r.G.double()[..., None] * X_e.double()
+    want = torch.zeros(n, d, dtype=torch.float64, device="cuda").index_add_(0, r.I.flatten().long(), terms.flatten(0, 1))
+    size = torch.zeros_like(want).index_add_(0, r.I.flatten().long(), terms.abs().flatten(0, 1))
+    # at most E products and sums in fp32, then one rounding to the output's type
+    bound = (E + 1) * 2.0 ** -24 * size + (2.0 ** -8 if dtype == torch.bfloat16 else 2.0 ** -24) * want.abs()
+    assert ((Y - want).abs() <= bound + 1e-30).all()
