@@ -228,6 +228,8 @@ cudaError_t launch_gate_softmax_simt(int dtype, const void* X, const void* Wg, f
 // bit pattern is below 2^30 and monotone in its value: a smaller key is a larger score, and among
 // equal scores a lower token.  Keys of one expert are distinct, so "the k smallest keys, ascending"
 // is the unique answer with ties broken toward the lower token and slots listed by descending score.
+// What is not a score (NaN rows of a model that has diverged) counts as larger than any: the selection goes by
+// sel_bits(), which has both top bits set whatever the value, so every column has exactly k winners.
 //
 // Routing groups (several independent groups of n tokens) multiply the columns: every (group, expert) pair is
 // selected on its own and lands in its expert's row of I and G at the group's offset.
@@ -253,6 +255,12 @@ constexpr int kHistThreads = 1024;
 constexpr int kBins = 1 << kRadixBits;
 constexpr int kHistSmemBytes = (kBins + kBins / 32) * kTopkChunk * 4;   // [bin][column of the chunk]; the selection step re-uses it padded
 constexpr unsigned long long kKeyTop = 3ull << 62;              // the two always-set top bits of a key
+
+constexpr unsigned kScoreTop = 0xC0000000u;                     // the same two bits of ~bits(S)
+// What the selection orders by: ~bits(S) of a score, the largest one's place for anything else.  (The key of a winner keeps
+// the value's own bits.)
+__device__ __forceinline__ unsigned sel_bits(unsigned inverted) { return max(inverted, kScoreTop); }
+__device__ __forceinline__ unsigned sel_bits(float s) { return sel_bits(~__float_as_uint(s)); }
 
 __device__ __forceinline__ unsigned long long make_key(float s, int64_t t) {
   return ((unsigned long long)(~__float_as_uint(s)) << 32) | (unsigned long long)(unsigned)t;
@@ -365,7 +373,7 @@ topk_hist_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, int 
   const int64_t t0 = (int64_t)blockIdx.x * rows_per_cta;
   const int64_t t1 = min(n, t0 + rows_per_cta);
   {
-    // only the score half of the key matters here: v = ~bits(S), digit (v >> sh32) & 1023, and from the
+    // only the score half of the key matters here: v = sel_bits(S), digit (v >> sh32) & 1023, and from the
     // second pass on the bits above the digit have to equal the expert's prefix
     constexpr int NC = VEC ? 4 : 1;
     const int col0 = slab_first_col<VEC>(cw), sh32 = shift - 32;
@@ -376,7 +384,7 @@ topk_hist_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, int 
       want[j] = act[j] ? (unsigned)(s_prefix[col0 + j] >> 32) >> (sh32 + kRadixBits) : 0u;
     }
     for_slab<VEC>(S, E, c0, cw, t0, t1, [&](float s, int64_t, int j) {
-      const unsigned v = ~__float_as_uint(s);
+      const unsigned v = sel_bits(s);
       if (act[j] && (pass == 0 || (v >> (sh32 + kRadixBits)) == want[j]))
         atomicAdd(&sh[((v >> sh32) & (kBins - 1)) * kTopkChunk + col0 + j], 1u);
     });
@@ -452,7 +460,7 @@ topk_ties_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, int6
   for (int64_t base = 0; base < n && running < k_rem; base += 1024) {
     const int64_t t = base + tid;
     float s = 0.f; bool m = false;
-    if (t < n) { s = S[t * E + e]; m = ~__float_as_uint(s) == thr; }
+    if (t < n) { s = S[t * E + e]; m = sel_bits(s) == thr; }
     const unsigned bal = __ballot_sync(0xffffffffu, m);
     if (lane == 0) s_warp[warp] = __popc(bal);
     __syncthreads();
@@ -510,7 +518,7 @@ topk_compact_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, i
     if (kind == 0) { if (pos < k) keys[(size_t)(c0 + col) * kpad + pos] = key; }
     else if (pos < (unsigned)kCandCap) cand[(size_t)(c0 + col) * kCandCap + pos] = key;
   };
-  // per column of this thread: the decided score bits (thr, after dropping the low bits of v = ~bits(S) that
+  // per column of this thread: the decided score bits (thr, after dropping the low bits of sel_bits(S) that
   // are still open) and what happens to a key exactly at the threshold: 0 winner, 1 candidate, 2 nothing
   // (the tie walk has placed it)
   constexpr int NC = VEC ? 4 : 1;
@@ -523,7 +531,7 @@ topk_compact_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, i
     at_thr[j] = !ok ? 2 : (s_mode[col0 + j] == 1 ? 0 : (s_mode[col0 + j] == 2 ? 1 : 2));
   }
   for_slab<VEC>(S, E, c0, cw, t0, t1, [&](float s, int64_t t, int j) {
-    const unsigned hi = ~__float_as_uint(s) >> drop[j];
+    const unsigned hi = sel_bits(s) >> drop[j];
     if (hi > thr[j]) return;
     const int kind = hi < thr[j] ? 0 : at_thr[j];
     if (kind == 2) return;
@@ -754,13 +762,13 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
   for (int i = tid; i < kBins; i += nt) hist[i] = 0;
   if (tid == 0) { s_prefix = 0; s_rem = (unsigned)k; s_less = 0; }
   __syncthreads();
-  // v has its two top bits set (0 <= S <= 1); digits of 10 bits from bit 29 down
+  // sel_bits() has its two top bits set; digits of 10 bits from bit 29 down
   const int per = kBins / nt;                          // consecutive bins of a thread in the scan: 1 .. 8
   for (int pass = 0; pass < 3; ++pass) {
     const int sh = 20 - 10 * pass;
     const unsigned pre = s_prefix, rem = s_rem;
     for (int t = tid; t < n; t += nt) {
-      const unsigned v = val[t];
+      const unsigned v = sel_bits(val[t]);
       if (pass == 0 || (v >> (sh + 10)) == (pre >> (sh + 10))) atomicAdd(&hist[(v >> sh) & (kBins - 1)], 1u);
     }
     __syncthreads();
@@ -788,7 +796,7 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
           if (rem <= before + c[j]) { D = j; in = c[j]; found = true; } else before += c[j];
         }
       }
-      s_prefix = (pass == 0 ? 0xC0000000u : pre) | ((unsigned)(tid * per + D) << sh);
+      s_prefix = (pass == 0 ? kScoreTop : pre) | ((unsigned)(tid * per + D) << sh);
       s_rem = rem - before;
       s_eq = in;
     }
@@ -803,7 +811,8 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
     for (int u = 0; u < 4; ++u) {
       const int t = t0 + u * nt + lane;
       v[u] = t < n ? val[t] : 0xFFFFFFFFu;
-      bal[u] = __ballot_sync(0xffffffffu, t < n && (v[u] < thr || (all_eq && v[u] == thr)));
+      const unsigned sv = sel_bits(v[u]);
+      bal[u] = __ballot_sync(0xffffffffu, t < n && (sv < thr || (all_eq && sv == thr)));
       sum += __popc(bal[u]);
     }
     if (sum == 0) continue;
@@ -820,7 +829,7 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
   unsigned running = 0;
   for (int base = 0; !all_eq && base < n && running < k_rem; base += nt) {
     const int t = base + tid;
-    const bool m = t < n && val[t] == thr;
+    const bool m = t < n && sel_bits(val[t]) == thr;
     const unsigned bal = __ballot_sync(0xffffffffu, m);
     if (lane == 0) s_warp[warp] = __popc(bal);
     __syncthreads();
@@ -833,7 +842,7 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
     }
     __syncthreads();
     const unsigned idx = running + s_warp[warp] + __popc(bal & ((1u << lane) - 1u));
-    if (m && idx < k_rem) sm_keys[k_less + idx] = ((unsigned long long)thr << 32) | (unsigned)t;
+    if (m && idx < k_rem) sm_keys[k_less + idx] = ((unsigned long long)val[t] << 32) | (unsigned)t;
     running += s_warp[32];
     __syncthreads();
   }

@@ -28,6 +28,30 @@ def test_selection_is_a_stable_sort(n, E, k, groups, levels):
         assert torch.equal(r.G[:, g * k:(g + 1) * k], torch.gather(r.S.T, 1, got))
 
 
+# rows of NaN: fewer than k, more than k, more than the final sort chooses from, all
+@pytest.mark.parametrize("n,k,groups,nans", [(2048, 16, 1, 300), (2048, 512, 1, 100), (16384, 40, 1, 16384), (1000, 100, 3, 700), (20000, 300, 1, 100),
+                                             (20000, 300, 1, 400), (20000, 300, 2, 9000), (20000, 5000, 1, 20000)])
+def test_rows_that_are_not_numbers_leave_the_selection_whole(n, k, groups, nans):
+    """A model that has diverged hands in rows of NaN.  They count as the largest scores, so an expert still takes k tokens of its
+    group, NaN rows first (the lower tokens of them), then the best of the others."""
+    E = 4
+    cfg = B.make_config(n, E, 8, E, (k + 0.25) * E / n, torch.float32, groups=groups)
+    assert B.ec_capacity(cfg) == k
+    gen = torch.Generator(device="cuda").manual_seed(n + k + nans)
+    X = torch.empty(groups * n, E, device="cuda").normal_(generator=gen)
+    for g in range(groups):
+        X[g * n + torch.randperm(n, generator=gen, device="cuda")[:nans]] = float("nan")
+    r = B.ec_route(cfg, X, torch.eye(E, device="cuda"))
+    assert torch.equal(r.S.isnan().all(dim=1), X.isnan().any(dim=1))
+    for g in range(groups):
+        S = r.S[g * n:(g + 1) * n]
+        want = torch.sort(S.nan_to_num(nan=2.0), dim=0, descending=True, stable=True)[1][:k].T + g * n
+        assert torch.equal(r.I[:, g * k:(g + 1) * k].long(), want)
+    got = torch.gather(r.S.T, 1, r.I.long())
+    assert torch.equal(r.G.view(torch.int32), got.view(torch.int32))
+    assert B.ec_validate_routing(cfg, r.I, r.row_ptr, r.slots) == 0
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("n,d,E,c", [(130, 8, 4, 2.0), (777, 40, 3, 1.0), (3000, 296, 16, 2.0), (9000, 600, 64, 1.5), (2048, 1032, 8, 2.0)])
 def test_shuffle_and_unshuffle_at_odd_widths(n, d, E, c, dtype):
