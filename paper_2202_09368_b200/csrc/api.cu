@@ -590,6 +590,23 @@ ec_status ec_backward_view(const ec_config* c, void* ws, ec_backward_ptrs* out) 
   return EC_OK;
 }
 
+#ifdef EC_DEBUG
+// ec_capped_assignment in which one CTA of every group stays silent after the first pass and the others wait wait_ns for it:
+// what a wait that runs out leaves behind.  In the debug library only, for its test.
+ec_status ec_debug_capped_wait(const ec_config* c, const float* S, float* A, void* ws, size_t ws_bytes, long long wait_ns,
+                               int silent_cta, void* stream) {
+  Dims D; ec_status s = check_cfg(c, &D); if (s != EC_OK) return s;
+  if (!D.cap_b || !S || !A || !ws || misaligned(ws, kAlign) || wait_ns < 0) return EC_ERR_INVALID_ARG;
+  const WsLayout W = ws_layout(D);
+  if (ws_bytes < W.total) return EC_ERR_WORKSPACE;
+  cudaStream_t st = (cudaStream_t)stream;
+  EC_CUDA(cudaMemsetAsync(ws, 0, sizeof(StatusWord), st));
+  EC_CUDA(launch_capped_assignment(S, D.ng, D.E, D.kg, D.groups, D.cap_b, D.cap_iters, (float)D.cap_lambda, A, (char*)ws + W.capped,
+                                   (int*)((char*)ws + W.status), st, (unsigned long long)wait_ns, silent_cta));
+  return EC_OK;
+}
+#endif
+
 int ec_debug_build(void) {
 #ifdef EC_DEBUG
   return 1;

@@ -65,8 +65,8 @@ __device__ __forceinline__ void lse_butterfly(float& m, float& s, int width) {
 // with one copy of the shifts; 4.7 k like this.  Pass p uses the buffers p & 1; nobody can be two passes ahead of a
 // reader, since every pass waits for all CTAs' words of the one before.  The words start with the number 2^32 - 1 (the
 // launcher fills them).  All CTAs of a cooperative launch are on the device at once; a wait is nevertheless bounded:
-// after two seconds the status word says so and the CTAs leave.
-constexpr unsigned long long kCapWaitNs = 2000000000ull;
+// after kCapWaitNs the status word says so and the CTAs leave, with zeros in their part of A: what follows on the stream
+// reads A before anyone has looked at the status.
 __device__ __forceinline__ void word_store(unsigned long long* p, float v, unsigned pass) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"((unsigned long long)__float_as_uint(v) | ((unsigned long long)pass << 32)) : "memory");
 }
@@ -80,7 +80,7 @@ __device__ __forceinline__ unsigned long long cap_timer() {
 // `pass`; 0 beyond the last CTA.  False when the wait ran out.
 constexpr int kCapLoads = 5;
 template <int N>
-__device__ __forceinline__ bool words_fetch(const unsigned long long* row, int q, int bpg, unsigned pass, float (&v)[N]) {
+__device__ __forceinline__ bool words_fetch(const unsigned long long* row, int q, int bpg, unsigned pass, unsigned long long wait_ns, float (&v)[N]) {
   unsigned long long w[N];
 #pragma unroll
   for (int u = 0; u < N; ++u) w[u] = q + u * 32 < bpg ? word_load(row + q + u * 32) : (unsigned long long)pass << 32;
@@ -92,7 +92,7 @@ __device__ __forceinline__ bool words_fetch(const unsigned long long* row, int q
     if (ok) break;
     if ((spin & 255u) == 255u) {
       if (t0 == 0) t0 = cap_timer();
-      else if (cap_timer() - t0 > kCapWaitNs) return false;
+      else if (cap_timer() - t0 > wait_ns) return false;
     }
 #pragma unroll
     for (int u = 0; u < N; ++u)
@@ -106,10 +106,12 @@ __device__ __forceinline__ bool words_fetch(const unsigned long long* row, int q
 // for each reader (148 CTAs waiting for the same four lines of L2 hold up the store they wait for)
 struct Exchange {
   unsigned long long *first_max, *first_sum, *even, *odd, *shift_even, *shift_odd; int* status;
+  unsigned long long wait_ns;
+  int silent;                                        // debug build: this CTA of a group leaves no words after the first pass (-1: none)
   static size_t words(int bpg, int groups, int E) { return (size_t)6 * bpg * groups * E; }
-  static Exchange at(unsigned long long* p, int bpg, int groups, int E, int* status) {
+  static Exchange at(unsigned long long* p, int bpg, int groups, int E, int* status, unsigned long long wait_ns, int silent) {
     const size_t n = (size_t)bpg * groups * E;
-    return {p, p + n, p + 2 * n, p + 3 * n, p + 4 * n, p + 5 * n, status};
+    return {p, p + n, p + 2 * n, p + 3 * n, p + 4 * n, p + 5 * n, status, wait_ns, silent};
   }
 };
 
@@ -152,14 +154,14 @@ __device__ __forceinline__ bool row_shifts(const Exchange& x, int pass, int g, i
     if (pass == 0) {
       for (int q = lane; ok && q < bpg; q += 32) {
         float mv[1], v[1];
-        ok = words_fetch(x.first_max + row, q, bpg, 0u, mv) && words_fetch(x.first_sum + row, q, bpg, 0u, v);
+        ok = words_fetch(x.first_max + row, q, bpg, 0u, x.wait_ns, mv) && words_fetch(x.first_sum + row, q, bpg, 0u, x.wait_ns, v);
         if (ok) lse_add(m, s, mv[0], v[0]);
       }
       lse_butterfly(m, s, 32);
     } else {
       for (int q = lane; ok && q < bpg; q += kCapLoads * 32) {
         float v[kCapLoads];
-        ok = words_fetch(((pass & 1) ? x.odd : x.even) + row, q, bpg, (unsigned)pass, v);
+        ok = words_fetch(((pass & 1) ? x.odd : x.even) + row, q, bpg, (unsigned)pass, x.wait_ns, v);
 #pragma unroll
         for (int u = 0; u < kCapLoads; ++u) s += ok ? v[u] : 0.f;
       }
@@ -173,7 +175,7 @@ __device__ __forceinline__ bool row_shifts(const Exchange& x, int pass, int g, i
   }
   if (ok && threadIdx.x < E) {
     float v[1];
-    ok = words_fetch(out + (int64_t)blk * E + threadIdx.x, 0, 1, (unsigned)pass, v);
+    ok = words_fetch(out + (int64_t)blk * E + threadIdx.x, 0, 1, (unsigned)pass, x.wait_ns, v);
     if (ok) shift[threadIdx.x] = v[0];
   }
   if (__syncthreads_and(ok)) return true;
@@ -202,6 +204,9 @@ template <int EPL>
 __device__ __forceinline__ void publish_words(const float (&pm)[EPL], const float (&ps)[EPL], float2* wpart, int E, const Exchange& x,
                                               int pass, int g, int bpg, int blk) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#ifdef EC_DEBUG
+  if (pass > 0 && blk == x.silent) return;
+#endif
   if (pass == 0) {
 #pragma unroll
     for (int j = 0; j < EPL; ++j) if (lane + 32 * j < E) wpart[warp * (E + 1) + lane + 32 * j] = make_float2(pm[j], ps[j]);
@@ -389,8 +394,9 @@ capped_resident_kernel(const float* __restrict__ S, float* __restrict__ A, const
     }
   }
   publish_words<EPL>(pm, ps, cap_smem, E, ex, 0, g, bpg, blk);
+  bool whole = true;                                 // no wait ran out
   for (int it = 0; it < iters; ++it) {
-    if (!row_shifts(ex, it, g, bpg, blk, E, log_k, shift)) return;
+    if (!(whole = row_shifts(ex, it, g, bpg, blk, E, log_k, shift))) break;
     float sh[EPL], es[EPL], sum[TPW];
 #pragma unroll
     for (int j = 0; j < EPL; ++j) { ps[j] = 0.f; sh[j] = lane + 32 * j < E ? shift[lane + 32 * j] : 0.f; es[j] = exp_ftz(sh[j]); }
@@ -427,7 +433,7 @@ capped_resident_kernel(const float* __restrict__ S, float* __restrict__ A, const
   for (int u = 0; u < TPW; ++u) {
     const int64_t t = t0 + u * stride, row = ((int64_t)g * ng + t) * E;
 #pragma unroll
-    for (int j = 0; j < EPL; ++j) if (t < ng && lane + 32 * j < E) A[row + lane + 32 * j] = __expf(x[u][j]);
+    for (int j = 0; j < EPL; ++j) if (t < ng && lane + 32 * j < E) A[row + lane + 32 * j] = whole ? __expf(x[u][j]) : 0.f;
   }
 }
 
@@ -464,8 +470,9 @@ capped_resident_smem_kernel(const float* __restrict__ S, float* __restrict__ A, 
     }
   }
   publish_words<EPL>(pm, ps, cap_smem, E, ex, 0, g, bpg, blk);
+  bool whole = true;                                 // no wait ran out
   for (int it = 0; it < iters; ++it) {
-    if (!row_shifts(ex, it, g, bpg, blk, E, log_k, shift)) return;
+    if (!(whole = row_shifts(ex, it, g, bpg, blk, E, log_k, shift))) break;
 #pragma unroll
     for (int j = 0; j < EPL; ++j) { pm[j] = 0.f; ps[j] = 0.f; }
     for (int u = 0; u < tpw; ++u) {
@@ -493,7 +500,7 @@ capped_resident_smem_kernel(const float* __restrict__ S, float* __restrict__ A, 
   for (int u = 0; u < tpw; ++u) {
     const int64_t t = t0 + u * stride, row = ((int64_t)g * ng + t) * E;
 #pragma unroll
-    for (int j = 0; j < EPL; ++j) if (t < ng && lane + 32 * j < E) A[row + lane + 32 * j] = __expf(mine[(2 * u) * E + lane + 32 * j]);
+    for (int j = 0; j < EPL; ++j) if (t < ng && lane + 32 * j < E) A[row + lane + 32 * j] = whole ? __expf(mine[(2 * u) * E + lane + 32 * j]) : 0.f;
   }
 }
 
@@ -580,7 +587,8 @@ size_t capped_scratch_bytes(int64_t n, int E, int groups) {
 }
 
 cudaError_t launch_capped_assignment(const float* S, int64_t ng, int E, int64_t kg, int groups, int b, int iters,
-                                     float lambda, float* A, void* scratch, int* status, cudaStream_t st) {
+                                     float lambda, float* A, void* scratch, int* status, cudaStream_t st, unsigned long long wait_ns,
+                                     int silent_cta) {
   if (E > kCapMaxE || iters < 1 || b < 1 || !(lambda > 0.f)) return cudaErrorInvalidValue;
   const int64_t n = ng * groups;
   char* p = (char*)scratch;
@@ -599,7 +607,7 @@ cudaError_t launch_capped_assignment(const float* S, int64_t ng, int E, int64_t 
   // the words of the resident forms take the place of the two sets of partials
   const size_t room = 2 * align256(blocks * E * sizeof(float2)) / sizeof(unsigned long long);
   if (Exchange::words(bpg, groups, E) > room) coop = 0;
-  const Exchange ex = Exchange::at(reinterpret_cast<unsigned long long*>(part[0]), bpg, groups, E, status);
+  const Exchange ex = Exchange::at(reinterpret_cast<unsigned long long*>(part[0]), bpg, groups, E, status, wait_ns, silent_cta);
   const float inv_lambda = 1.f / lambda, log_k = logf((float)kg), log_b = logf((float)b);
   const int epl = E <= 32 ? 1 : (E <= 64 ? 2 : (E <= 128 ? 4 : 8));
   const int64_t tpw = (ng + (int64_t)bpg * kCapWarps - 1) / ((int64_t)bpg * kCapWarps);

@@ -134,9 +134,13 @@ cudaError_t launch_reduce_partials(int dtype, const float* part, void* out, int 
 // ---- capped expert choice, Section 3.3 (capped.cu) ---------------------------------------------
 // A [n, E] (token-major, n = groups * ng): the assignment after `iters` rounds of Dykstra's algorithm with
 // Kullback-Leibler projections, per routing group; entries in [0, 1].  E <= 256.
+// When a wait for another CTA takes longer than wait_ns, EC_ERR_TIMEOUT goes into the status word and the CTAs whose
+// waits ran out leave zeros in A.  silent_cta (debug build only): a CTA of every group that stays silent after the first pass.
+constexpr unsigned long long kCapWaitNs = 2000000000ull;
 size_t capped_scratch_bytes(int64_t n, int E, int groups);
 cudaError_t launch_capped_assignment(const float* S, int64_t ng, int E, int64_t kg, int groups, int b, int iters,
-                                     float lambda, float* A, void* scratch, int* status, cudaStream_t st);
+                                     float lambda, float* A, void* scratch, int* status, cudaStream_t st,
+                                     unsigned long long wait_ns = kCapWaitNs, int silent_cta = -1);
 // G[i, j] = S[I[i, j], i] for I, G of shape [E, k]
 cudaError_t launch_gather_gate(const float* S, const int32_t* I, float* G, int64_t slots_total, int64_t k, int E,
                                int64_t n, int* status, cudaStream_t st);

@@ -4,6 +4,7 @@ The debug build stands in for a memory checker: every index a kernel reads from 
 its range first, a bad one is recorded (EC_ERR_INDEX) and the access it would have addressed is skipped.  It must
 give the same bits as the normal build on valid inputs, and survive corrupted index structures, which only it is given.
 """
+import ctypes
 import importlib.util
 import os
 
@@ -120,3 +121,23 @@ def test_debug_build_survives_and_reports_corrupted_indices(D, dtype, fuse):
     out = D.ec_unshuffle(cfg, X_in.float(), r.G, rp, sl)
     assert torch.isfinite(out.float()).all()
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("n,E,groups", [(130, 8, 1), (4736, 32, 1), (9000, 64, 1), (1500, 16, 3), (16384, 128, 1)])
+def test_a_solver_wait_that_runs_out_is_reported_and_leaves_a_defined_assignment(D, n, E, groups):
+    """Registers and shared memory, one group and three.  One CTA of a group leaves no words from the second pass on and the others
+    wait 5 ms: the call ends, the status says so, A holds numbers that a selection can work on, and the next call on the same
+    workspace is the right one."""
+    cfg = D.make_config(n, 8, 8, E, 2.0, BF16, groups=groups, cap_b=3, cap_iters=20, cap_lambda=1e-2)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    S = torch.softmax(torch.empty(n * groups, E, device="cuda").normal_(generator=gen), dim=1)
+    want = D.ec_capped_assignment(cfg, S)
+    ws = D.alloc_workspace(cfg)
+    A = torch.full_like(S, float("nan"))
+    call = D.lib().ec_debug_capped_wait
+    call.argtypes = [ctypes.POINTER(D.ec_config)] + [ctypes.c_void_p] * 3 + [ctypes.c_size_t, ctypes.c_longlong, ctypes.c_int, ctypes.c_void_p]
+    assert call(ctypes.byref(cfg), S.data_ptr(), A.data_ptr(), ws.data_ptr(), ws.numel(), 5_000_000, 1, D._stream()) == D.EC_OK
+    assert D.ec_read_status(ws) == D.EC_ERR_TIMEOUT
+    assert bool(((A >= 0) & (A <= 1)).all())
+    again = D.ec_capped_assignment(cfg, S, ws=ws)
+    assert D.ec_read_status(ws) == D.EC_OK and torch.equal(again, want)
