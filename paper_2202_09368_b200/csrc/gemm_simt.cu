@@ -159,7 +159,7 @@ struct TileLoader {
 };
 
 template <typename TA, typename TB, typename TC, int EPI, int BM, int BN, int BK, int TM, int TN, int KS, int MINB, bool VEC>
-__global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kernel(const GemmArgs g, const Operand oa, const Operand ob, int c_vec) {
+__global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kernel(const GemmArgs g, const Operand oa, const Operand ob, int c_vec, int col0) {
   constexpr int NT = BM / TM * (BN / TN), TX = BN / TN, GM = TM / 4, GN = TN / 4;
   static_assert(TX % 8 == 0 && TM % 4 == 0 && TN % 4 == 0, "a warp covers 4 x 8 threads");
   using LA = TileLoader<TA, BM, BK, NT, VEC>;
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kern
   extern __shared__ __align__(16) float simt_smem[];  // [KS groups][2 buffers][A | B]; after the main loop the other groups' sums
   const int b = blockIdx.z, grp = threadIdx.x / NT;
   float* bufs = simt_smem + grp * 2 * kBuf;
-  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;     // row tiles on grid.x: M (tokens) is the dimension without a limit
+  const int m0 = blockIdx.x * BM, n0 = (col0 + blockIdx.y) * BN;     // row tiles on grid.x: M (tokens) is the longer dimension as a rule
   const int warp = (threadIdx.x % NT) >> 5, lane = threadIdx.x & 31;
   const int tx = (lane & 7) + 8 * (warp % (TX / 8)), ty = (lane >> 3) + 4 * (warp / (TX / 8));
   unsigned long long acc[TM][TN / 2];
@@ -353,7 +353,7 @@ Tile pick_tile(const GemmArgs& g, int sms) {
   constexpr double kLatency = 1000.;                  // cycles of a k-tile nobody hides
   Tile best = TILE_64x32; double least = 0.;
   for (const Form& f : forms) {
-    const int64_t tiles = (int64_t)((g.M + f.bm - 1) / f.bm) * ((g.N + f.bn - 1) / f.bn) * g.batches, q = (tiles + sms - 1) / sms;
+    const int64_t tiles = (((int64_t)g.M + f.bm - 1) / f.bm) * ((g.N + f.bn - 1) / f.bn) * g.batches, q = (tiles + sms - 1) / sms;
     const double work = (double)q * f.bm * f.bn * g.K / 128. / (q >= f.per_sm ? f.full : f.alone);
     const double steps = (double)((q + f.per_sm - 1) / f.per_sm) * ((g.K + f.kstep - 1) / f.kstep) * kLatency;
     const double t = work > steps ? work : steps;
@@ -364,15 +364,22 @@ Tile pick_tile(const GemmArgs& g, int sms) {
 
 template <typename TA, typename TB, typename TC, int EPI, int BM, int BN, int BK, int TM, int TN, int KS, int MINB, bool VEC>
 cudaError_t launch_tile(const GemmArgs& g, const Operand& oa, const Operand& ob, int c_vec, cudaStream_t st) {
-  const dim3 grid((g.M + BM - 1) / BM, (g.N + BN - 1) / BN, g.batches);
-  if (grid.y > 65535u || grid.z > 65535u) return cudaErrorInvalidConfiguration;
+  constexpr int kMaxCols = 65535;                     // column tiles of one launch (grid.y): wider results take several
+  if (g.batches > 65535) return cudaErrorInvalidConfiguration;
   auto kern = gemm_simt_kernel<TA, TB, TC, EPI, BM, BN, BK, TM, TN, KS, MINB, VEC>;
   constexpr int bufs = KS * 2 * BK * (BM + BN) * 4, sums = KS > 1 ? BM * BN * 4 : 0, smem = bufs > sums ? bufs : sums;
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
-  return launch_chained(kern, grid, dim3(BM / TM * (BN / TN) * KS), smem, st, g, oa, ob, c_vec);
+  const unsigned rows = (unsigned)(((int64_t)g.M + BM - 1) / BM);
+  const int cols = (g.N + BN - 1) / BN;
+  for (int col0 = 0; col0 < cols; col0 += kMaxCols) {
+    const dim3 grid(rows, cols - col0 < kMaxCols ? cols - col0 : kMaxCols, g.batches);
+    const cudaError_t e = launch_chained(kern, grid, dim3(BM / TM * (BN / TN) * KS), smem, st, g, oa, ob, c_vec, col0);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Operands whose groups of four straddle an edge (an expert count that is not a multiple of four, in the gate's gradients

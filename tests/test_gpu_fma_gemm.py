@@ -28,3 +28,36 @@ def test_fp32_products_match_64_bits(k, d, dff, E):
         # a chain of `terms` fused multiply-adds in fp32: at most terms * 2^-24 of the sum of the terms' sizes
         bound = (terms + 1) * 2.0 ** -24 * (a.abs() @ b.abs())
         assert ((C.double() - a @ b).abs() <= bound).all(), kind
+
+
+@pytest.mark.parametrize("dtype,E", [(torch.float32, 2), (torch.float32, 4), (torch.bfloat16, 2)])
+def test_rows_wider_than_one_grid_of_column_tiles(dtype, E):
+    """d = 2^21 + 8: 65537 column tiles of 32, more than a grid has places for, in dX = dL . Wg^T + slot rows when the number
+    of experts is not a multiple of four (fp32) or eight (bf16); beside it the same width on wider tiles."""
+    n, d, dff = 8, (1 << 21) + 8, 8
+    cfg = B.make_config(n, d, dff, E, 1.0, dtype)
+    gen = torch.Generator(device="cuda").manual_seed(E)
+
+    def normal(scale, *shape):
+        return (torch.empty(shape, device="cuda").normal_(generator=gen) * scale).to(dtype)
+
+    X, Wg, W1, W2, dY = normal(1, n, d), normal(d ** -0.5, d, E), normal(d ** -0.5, E, d, dff), normal(dff ** -0.5, E, d, dff), normal(1, n, d)
+    ws = B.alloc_workspace(cfg)
+    Y, saved = B.ec_moe_forward(cfg, X, Wg, W1, W2, ws=ws)
+    v = {name: t.clone() for name, t in B.saved_view(cfg, saved).items()}
+    dX = B.ec_moe_backward(cfg, X, Wg, W1, W2, dY, saved, ws=ws)[0]
+    assert B.ec_read_status(ws) == B.EC_OK
+    w = B.backward_view(cfg, ws)
+    eps = 2.0 ** -24 if dtype == torch.float32 else 2.0 ** -8          # of one rounding to the result's type; the sums are fp32
+
+    def check(got, a, b, rows=None):
+        want, size = a.double() @ b.double(), a.double().abs() @ b.double().abs()
+        if rows is not None:                            # each token's slot rows, and the sizes of what is added up
+            want.index_add_(0, v["I"].flatten().long(), rows.double().flatten(0, 1))
+            size.index_add_(0, v["I"].flatten().long(), rows.double().abs().flatten(0, 1))
+        bound = (a.shape[-1] + E + 1) * 2.0 ** -24 * size + eps * want.abs() + 1e-30
+        assert ((got.double() - want).abs() <= bound).all()
+
+    check(v["X_e"], v["H"], W2.transpose(1, 2))
+    check(w["dX_in"], w["dZ"], W1.transpose(1, 2))
+    check(dX, w["dL"], Wg.T, w["dX_in"])
