@@ -383,7 +383,8 @@ cudaError_t launch_tile(const GemmArgs& g, const Operand& oa, const Operand& ob,
 }
 
 // Operands whose groups of four straddle an edge (an expert count that is not a multiple of four, in the gate's gradients
-// only) are loaded one element at a time, in the small tile.
+// only) are loaded one element at a time, in the small tile.  No list (a_rows) and no GeLU comes here: the products that
+// have them contract rows of whole 16-byte vectors.
 template <typename TA, typename TB, typename TC, int EPI>
 cudaError_t launch_odd(const GemmArgs& g, const Operand& oa, const Operand& ob, int c_vec, cudaStream_t st) {
   return launch_tile<TA, TB, TC, EPI, 64, 32, 32, 4, 4, 1, 4, false>(g, oa, ob, c_vec, st);
@@ -425,6 +426,7 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st) {
   const int c_vec = g.N % 4 == 0 && g.ldc % 4 == 0 && (g.batches == 1 || g.batch_c % 4 == 0) && out4(g.C) && out4(g.C2) && out4(g.Zin) &&
                     out4(g.rows) && g.ld_rows % 4 == 0;
   if (g.bias && g.bias_dtype != g.c_dtype) return cudaErrorInvalidValue;
+  if (g.a_rows && !(oa.vec && ob.vec)) return cudaErrorInvalidValue;         // the scalar tile does not read through a list
   if (g.a_dtype == 0 && g.b_dtype == 0 && g.c_dtype == 0) {
     if (oa.vec && ob.vec) {
       const Tile tile = pick_tile(g, sms);
@@ -437,8 +439,6 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st) {
     } else {
       switch (g.epi) {
         case EPI_STORE: return launch_odd<float, float, float, EPI_STORE>(g, oa, ob, c_vec, st);
-        case EPI_GELU: return launch_odd<float, float, float, EPI_GELU>(g, oa, ob, c_vec, st);
-        case EPI_GELU_GRAD: return launch_odd<float, float, float, EPI_GELU_GRAD>(g, oa, ob, c_vec, st);
         case EPI_ADD_SLOTS: return launch_odd<float, float, float, EPI_ADD_SLOTS>(g, oa, ob, c_vec, st);
       }
     }

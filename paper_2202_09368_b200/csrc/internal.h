@@ -163,7 +163,8 @@ struct GemmArgs {
   const void* bias; int bias_dtype;    // not null: bias[b * N + n] is added to the accumulator before the epilogue's function
   // a_rows != null: A is a row selection of one matrix (Eq. 3's X_in = P . X without the copy).  The index along M
   // (a_rows_k = 0) or along K (a_rows_k = 1) is replaced by a_rows[b * a_rows_batch + index], which must lie in
-  // [0, a_rows_total); batch_a is unused.
+  // [0, a_rows_total); batch_a is unused.  Both operands must allow loads of four elements (see launch_gemm_simt), else
+  // the product is refused.
   const int32_t* a_rows; int64_t a_rows_batch, a_rows_total; int a_rows_k;
 };
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);

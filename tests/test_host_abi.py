@@ -3,6 +3,7 @@ symbol the header declares, and its size / validation functions follow Eq. 1."""
 import ctypes
 import os
 import re
+import subprocess
 
 import pytest
 import torch
@@ -89,3 +90,28 @@ def test_capped_config_checks():
                 B.make_config(256, 64, 128, 8, 2.0, torch.bfloat16, cap_b=2, cap_lambda=0.0),
                 B.make_config(256, 64, 128, 8, 2.0, torch.bfloat16, cap_b=-1)):
         assert B.ec_workspace_bytes(bad) == 0
+
+
+def test_fma_gemm_refuses_a_row_list_it_would_not_read(tmp_path):
+    """The FMA GEMM reads A through a row list only with four-element loads.  Any other operand with a list (a pitch that is no
+    multiple of four, a list along the contiguous direction) is an invalid value before anything is launched."""
+    src = tmp_path / "list.cu"
+    src.write_text("""
+#include "internal.h"
+#include <stdio.h>
+#include <string.h>
+int main() {
+  ecmoe::GemmArgs g; memset(&g, 0, sizeof(g));
+  g.A = g.B = g.C = (void*)256; g.a_rows = (const int32_t*)256; g.a_rows_batch = 8; g.a_rows_total = 8;
+  g.M = 8; g.N = 8; g.K = 8; g.batches = 1; g.sam = 9; g.sak = 1; g.sbk = 8; g.sbn = 1; g.ldc = 8;
+  const int odd_pitch = ecmoe::launch_gemm_simt(g, 0);
+  g.sam = 8; g.a_rows_k = 1;
+  const int contiguous = ecmoe::launch_gemm_simt(g, 0);
+  printf("%d %d %d", odd_pitch, contiguous, (int)cudaErrorInvalidValue);
+}
+""")
+    exe, pkg = str(tmp_path / "list"), os.path.dirname(BUILD.OUT)
+    subprocess.check_call([BUILD.NVCC] + BUILD.FLAGS[:2] + ["-std=c++17", "-I", BUILD.CSRC, str(src), BUILD.OUT, "-o", exe, "-Xlinker", "-rpath", "-Xlinker", pkg])
+    env = dict(os.environ, CUDA_VISIBLE_DEVICES="")    # nothing is to reach a device
+    a, b, invalid = subprocess.run([exe], stdout=subprocess.PIPE, text=True, check=True, env=env).stdout.split()
+    assert a == b == invalid
