@@ -384,6 +384,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     int stage = 0; uint32_t phase = 0;
     const uint32_t leader_full0 = CTAS == 2 ? map_to_cta(full0, 0) : full0;
     const int nidx = p.a_mn ? p.K : p.M;               // stored rows of A per batch
+    const int32_t* a_rows = after_enter(p.a_rows);
     auto pick = [&](const int32_t* list, int pos) {
       const int r = __ldg(list + min(pos, nidx - 1));
       return idx_ok(r, 0, p.a_rows_total, p.status) ? r : 0;
@@ -393,7 +394,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int mt = p.n_fast ? (tile / p.tiles_n) % p.tiles_m : tile % p.tiles_m;
       const int nt = p.n_fast ? tile % p.tiles_n : (tile / p.tiles_m) % p.tiles_n;
       const int m0 = mt * TM + (int)rank * BM, n0 = nt * BN + (int)rank * kBHalf;
-      const int32_t* rows_b = p.a_rows + (int64_t)b * p.a_rows_batch;
+      const int32_t* rows_b = a_rows + (int64_t)b * p.a_rows_batch;
       int ri[4];
       const int rbase = p.a_mn ? 4 * (lane & 15) : m0 + 4 * lane;
 #pragma unroll
@@ -700,7 +701,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (n0 + c0 >= p.N) break;             // uniform across the warp
             uint32_t r[32]; tc_ld32(taddr + c0, r);
             if (p.bias != nullptr) {               // the bias term of Eq. 3's second product: the same 32 values for every row
-              const bf16* bp = p.bias + (int64_t)b * p.N + n0 + c0;
+              const bf16* bp = after_enter(p.bias) + (int64_t)b * p.N + n0 + c0;
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
                 if (n0 + c0 + 8 * j < p.N) {
@@ -733,7 +734,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             tc_ld32_issue(taddr + c0, r); tc_ld32_issue(taddr + c0 + 32, r + 32); tc_ld_wait();
             if constexpr (EPI == EPI_GELU) {
               if (p.bias != nullptr) {             // Z = X_in . W1 + b1: the same 64 values for every row
-                const bf16* bp = p.bias + (int64_t)b * p.N + n0 + c0;
+                const bf16* bp = after_enter(p.bias) + (int64_t)b * p.N + n0 + c0;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                   if (n0 + c0 + 8 * j < p.N) {

@@ -47,7 +47,7 @@ struct SelState { unsigned long long prefix; unsigned int k_rem, mode, shift, ca
 // calls chain_enter() before its first access to global memory, which waits until everything before the kernel has
 // completed and is visible.  Completion is then transitive along the chain.  What may come before chain_enter(): shared
 // memory, barriers, tensor memory, descriptors in kernel parameters.
-// Pointers that are read through qualifiers a compiler may take for "never written" (const __restrict__ parameters)
+// Pointers that are read in ways a compiler may take for "never written" (const __restrict__ parameters, __ldg())
 // pass through after_enter(), so that no load of theirs can be moved up past the wait.
 __device__ __forceinline__ void chain_enter() {
 #if defined(__CUDA_ARCH__)
