@@ -858,7 +858,9 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
     const SlotMap smap = {E, groups, k, n};
     const int kpad = L.kpad < 32 ? 32 : (int)L.kpad;   // the sort works on whole warps of keys
     const int smem = (int)(kpad * 8 + n * 4 + kBins * 4);
-    cudaError_t e0 = cudaFuncSetAttribute(topk_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the attribute is one per device, whatever threads launch: always the most that any call needs, never less than another's
+    constexpr int kMostSmem = kSortTile * 8 + kSmallN * 4 + kBins * 4;
+    cudaError_t e0 = cudaFuncSetAttribute(topk_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
     if (e0 != cudaSuccess) return e0;
     int threads = 128;                                 // at most four keys per thread for the sort (kpad < 2 n)
     while (threads < 1024 && threads * 4 < n) threads <<= 1;
@@ -1228,8 +1230,9 @@ cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t total, int
     return cudaLaunchKernelEx(&cfg, inv_cluster_kernel, I, (int)n, (int)total, row_ptr, slots, (int32_t*)scratch, status);
   }
   if (n <= kInvSmallN && total <= kInvSmallSlots) {
-    const int smem = (int)(n + total) * 4;             // at most 80 KiB
-    cudaError_t e0 = cudaFuncSetAttribute(inv_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int smem = (int)(n + total) * 4;
+    constexpr int kMostSmem = (kInvSmallN + kInvSmallSlots) * 4;         // as for topk_small_kernel: 80 KiB, not this call's
+    cudaError_t e0 = cudaFuncSetAttribute(inv_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
     if (e0 != cudaSuccess) return e0;
     launch_chained(inv_small_kernel, dim3(1), dim3(1024), smem, st, I, (int)n, (int)total, row_ptr, slots, status);
     return cudaGetLastError();
