@@ -1,4 +1,5 @@
-"""The fp32 expert products at the edges of the FMA kernel's tiles, against the same products in 64 bits."""
+"""The FMA kernels at the edges of their tiles, against the same arithmetic in 64 bits: the fp32 expert products, the gate gradients
+and products of very wide layers, the gate."""
 import pytest
 import torch
 
@@ -61,3 +62,22 @@ def test_rows_wider_than_one_grid_of_column_tiles(dtype, E):
     check(v["X_e"], v["H"], W2.transpose(1, 2))
     check(w["dX_in"], w["dZ"], W1.transpose(1, 2))
     check(dX, w["dL"], Wg.T, w["dX_in"])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,d,E", [(33, 136, 36), (100, 1000, 60), (65, 72, 33), (31, 264, 70), (200, 520, 100), (64, 8, 130), (40, 640, 132), (97, 200, 253),
+                                   (500, 40, 252), (32, 128, 30)])
+def test_gate_widths_of_the_fma_kernel(n, d, E, dtype):
+    """Expert counts the tensor-core gate does not take (no multiple of eight) from one to eight column groups, in whole groups of
+    four and not, tokens and depths that end inside a chunk: against the softmax in 64 bits."""
+    cfg = B.make_config(n, d, 8, E, 4.0 * E / n, dtype)
+    gen = torch.Generator(device="cuda").manual_seed(n + E)
+    X = torch.empty(n, d, device="cuda").normal_(generator=gen).to(dtype)
+    Wg = (torch.empty(d, E, device="cuda").normal_(generator=gen) / d ** 0.5).to(dtype)
+    r = B.ec_route(cfg, X, Wg)
+    want = torch.softmax(X.double() @ Wg.double(), dim=1)
+    # a logit is off by at most d * 2^-24 of the sum of its terms' sizes, twice that (with the largest one) in the exponent; expf, the
+    # sum and the quotient add at most (E + 8) roundings
+    logit = d * 2.0 ** -24 * (X.double().abs() @ Wg.double().abs()).amax(dim=1, keepdim=True)
+    assert ((r.S.double() - want).abs() <= (2 * logit + (E + 8) * 2.0 ** -23) * want).all()
+    assert B.ec_validate_routing(cfg, r.I, r.row_ptr, r.slots) == 0

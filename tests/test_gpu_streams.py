@@ -54,3 +54,41 @@ def test_routing_of_several_sizes_from_several_threads():
     _together([j for j, _ in jobs], 2000)
     for _, check in jobs:
         check()
+
+
+def _layer(n, d, dff, E, dtype, seed, **kw):
+    cfg = B.make_config(n, d, dff, E, 2.0, dtype, **kw)
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+
+    def normal(scale, *shape):
+        return (torch.empty(shape, device="cuda").normal_(generator=gen) * scale).to(dtype)
+
+    X, Wg, W1, W2, dY = normal(1, n, d), normal(d ** -0.5, d, E), normal(d ** -0.5, E, d, dff), normal(dff ** -0.5, E, d, dff), normal(1, n, d)
+    ws, saved, Y = B.alloc_workspace(cfg), B.alloc_saved(cfg), torch.empty_like(X)
+    grads = tuple(torch.empty_like(t) for t in (X, Wg, W1, W2))
+
+    def step():
+        B.ec_moe_forward(cfg, X, Wg, W1, W2, X_out=Y, saved=saved, ws=ws)
+        assert not kw.get("cap_b") or B.ec_read_status(ws) == B.EC_OK         # the solver's waits, before the backward pass clears the word
+        B.ec_moe_backward(cfg, X, Wg, W1, W2, dY, saved, grads=grads, ws=ws)
+
+    step()
+    want = [t.clone() for t in (Y,) + grads]
+
+    def check():
+        assert B.ec_read_status(ws) == B.EC_OK
+        for got, ref in zip((Y,) + grads, want):
+            assert torch.equal(got, ref)
+
+    return step, check
+
+
+def test_layers_on_several_streams_at_once():
+    """Kernels that are set up while their predecessor drains, products that fill every SM, and the solver, whose CTAs wait for one
+    another, two of it among them."""
+    bf16, f32 = torch.bfloat16, torch.float32
+    jobs = [_layer(4096, 256, 512, 32, bf16, 1, cap_b=3, cap_iters=20), _layer(2048, 128, 256, 16, bf16, 2, cap_b=3, cap_iters=20),
+            _layer(2048, 256, 1024, 8, bf16, 3), _layer(512, 128, 256, 10, f32, 4), _layer(20000, 64, 64, 8, bf16, 5)]
+    _together([j for j, _ in jobs], 100)
+    for _, check in jobs:
+        check()
