@@ -251,7 +251,7 @@ ec_status ec_moe_forward(const ec_config* cfg, const void* X, const void* Wg, co
  *   dX_out [n, d] in, `saved` as filled by ec_moe_forward with the same cfg and inputs;
  *   dX [n, d], dWg [d, E], dW1, dW2 [E, d, d'] out, overwritten (not accumulated);
  *   db1 [E, d'], db2 [E, d] out, the gradients of the bias terms (sums of dZ and of dX_e over an expert's slots,
- *   in slot order, fp32, rounded once); either may be NULL (not wanted).  The biases themselves are not needed here:
+ *   fp32 in a fixed order, rounded once); either may be NULL (not wanted).  The biases themselves are not needed here:
  *   the saved Z already contains b1.
  */
 ec_status ec_moe_backward(const ec_config* cfg, const void* X, const void* Wg, const void* W1,

@@ -960,8 +960,7 @@ int pick_bn(const TcGemmArgs& g, int pairs) {
     if (wide * 192 <= narrow * 100) return 512;
   }
   // A pair's 256-column tile halves to 128 columns where even then every tile has a pair to itself: half the epilogue
-  // per SM on twice the SMs (8 experts, 512
-  // rows, 256 x 512: GEMM-1 16.4 -> 14.3 us, dZ 20.5 -> 16.4 us)
+  // per SM on twice the SMs (8 experts of 512 rows, 256 x 512: GEMM-1 16.4 -> 14.3 us, dZ 20.5 -> 16.4 us)
   if (g.M > BM && g.N > 128) {
     const int64_t half = (int64_t)((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + 127) / 128) * g.batches;
     return half <= pairs ? 128 : 256;

@@ -123,7 +123,8 @@ cudaError_t launch_bwd_combine(int dtype, const void* dX_out, const float* X_e, 
 cudaError_t launch_bwd_softmax(const float* S, const float* dG, const int32_t* row_ptr,
                                const int32_t* slots, void* dL, int dl_bf16, int64_t n, int E, int64_t k,
                                int* status, cudaStream_t st);
-// out[b, c] = sum over the rows r < min(rows, batch_rows[b]) of A[b, r, c], in ascending r, fp32, cast to dtype
+// out[b, c] = sum over the rows r < min(rows, batch_rows[b]) of A[b, r, c], fp32, cast to dtype; in a fixed order: eight chains
+// (the rows with r mod 8 = 0, 1, ..., each in ascending r), joined in that order
 // (gradients of the bias terms: column sums of dZ and dX_e per expert); batch_rows may be null
 cudaError_t launch_column_sums(int dtype, const void* A, void* out, int batches, int64_t rows, int cols,
                                const int32_t* batch_rows, cudaStream_t st);

@@ -1,4 +1,5 @@
-"""Calls from several host threads, each on a stream of its own, at the same time: every one gives the bits it gives alone."""
+"""Calls from several host threads and streams at the same time, and results handed from one stream to another: every call gives
+the bits it gives alone."""
 import threading
 
 import pytest
@@ -92,3 +93,39 @@ def test_layers_on_several_streams_at_once():
     _together([j for j, _ in jobs], 100)
     for _, check in jobs:
         check()
+
+
+def test_results_handed_from_stream_to_stream():
+    """The steps of the routing chain alternate between two streams that wait for each other's events, on new inputs every time: a kernel
+    that is set up early still reads what the other stream wrote before the event."""
+    n, d, E = 8192, 512, 16
+    cfg = B.make_config(n, d, 8, E, 2.0, torch.bfloat16)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    Xs = [torch.empty(n, d, dtype=torch.bfloat16, device="cuda").normal_(generator=gen) for _ in range(4)]
+    Wg = (torch.empty(d, E, device="cuda").normal_(generator=gen) / d ** 0.5).to(torch.bfloat16)
+    k, ws = B.slots_per_expert(cfg), B.alloc_workspace(cfg)
+    wants = []
+    for X in Xs:
+        r = B.ec_route(cfg, X, Wg, ws=ws)
+        X_in = B.ec_shuffle(cfg, X, r.I)
+        wants.append((X_in, B.ec_unshuffle(cfg, X_in.float(), r.G, r.row_ptr, r.slots)))
+    X, r = torch.zeros_like(Xs[0]), B.ec_route(cfg, Xs[0], Wg, ws=ws)
+    X_in, X_e = torch.empty(E, k, d, dtype=torch.bfloat16, device="cuda"), torch.empty(E, k, d, device="cuda")
+    outs = [torch.empty_like(w[1]) for w in wants * 10]
+    one, two = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def on(stream, other, f):
+        stream.wait_stream(other)
+        with torch.cuda.stream(stream):
+            f()
+
+    for i, out in enumerate(outs):
+        on(one, two, lambda: X.copy_(Xs[i % 4]))
+        on(two, one, lambda: B.ec_route(cfg, X, Wg, ws=ws, out=r))
+        on(one, two, lambda: B.ec_shuffle(cfg, X, r.I, X_in))
+        on(two, one, lambda: X_e.copy_(X_in))
+        on(one, two, lambda: B.ec_unshuffle(cfg, X_e, r.G, r.row_ptr, r.slots, out))
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        assert torch.equal(out, wants[i % 4][1])
