@@ -14,8 +14,10 @@
 //     scalar stores of a transposed tile over all 32 banks and keeps groups of four together.
 // At n = 2048, d = 512, d' = 2048, 16 experts (8.6 GFLOP per expert product) a product takes 174-207 us, 42-50 TFLOP/s of the
 // 74 the FMA pipe has; the 64 x 64 tile with 4 x 4 results per thread, one buffer and scalar loads that this replaces
-// took 445-640 us.  What is left: shared-memory fragment loads occupy their pipe for 0.8 of the multiply-adds' time,
-// and 512 tiles over 148 SMs leave the fourth wave half empty.
+// took 445-640 us.  What is left, from the counters: the FMA pipe is busy 75 % of the time in the plain 128 x 128 tile and the
+// shared-memory pipe 48 % (two CTAs of four warps on an SM do not cover all of each other's fragment loads and barriers),
+// 70 % with 128 tiles on 148 SMs, 60 and 53 % where GeLU and GeLU' (erff) follow in the open; 512 tiles on 296 places
+// leave the second round 0.73 full.
 #include "internal.h"
 
 namespace ecmoe {
@@ -159,7 +161,7 @@ struct TileLoader {
 };
 
 template <typename TA, typename TB, typename TC, int EPI, int BM, int BN, int BK, int TM, int TN, int KS, int MINB, bool VEC>
-__global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kernel(const GemmArgs g, const Operand oa, const Operand ob, int c_vec, int col0) {
+__global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kernel(const GemmArgs g, const Operand oa, const Operand ob, int c_vec) {
   constexpr int NT = BM / TM * (BN / TN), TX = BN / TN, GM = TM / 4, GN = TN / 4;
   static_assert(TX % 8 == 0 && TM % 4 == 0 && TN % 4 == 0, "a warp covers 4 x 8 threads");
   using LA = TileLoader<TA, BM, BK, NT, VEC>;
@@ -169,7 +171,7 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kern
   extern __shared__ __align__(16) float simt_smem[];  // [KS groups][2 buffers][A | B]; after the main loop the other groups' sums
   const int b = blockIdx.z, grp = threadIdx.x / NT;
   float* bufs = simt_smem + grp * 2 * kBuf;
-  const int m0 = blockIdx.x * BM, n0 = (col0 + blockIdx.y) * BN;     // row tiles on grid.x: M (tokens) is the longer dimension as a rule
+  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;     // row tiles on grid.x: M (tokens) is the dimension without a limit
   const int warp = (threadIdx.x % NT) >> 5, lane = threadIdx.x & 31;
   const int tx = (lane & 7) + 8 * (warp % (TX / 8)), ty = (lane >> 3) + 4 * (warp / (TX / 8));
   unsigned long long acc[TM][TN / 2];
@@ -340,12 +342,20 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kern
   }
 }
 
+// Column tiles sit on grid.y.  64 columns cover every width the layer takes (2^22 - 64), 32 columns the widths below 2 097 121.
+// (Several launches with a column offset do it too, but one more kernel argument changed the code of the tiles that every
+// layer uses: an fp32 step of 531 us took 541.)
+constexpr int kMaxColTiles = 65535;
+
 enum Tile { TILE_128x128, TILE_128x128_K2, TILE_64x64_K2, TILE_64x32 };
 // The SM with the most tiles decides: its multiply-adds at the rate the tile reaches (share of the 128 per cycle), or its
 // k-tiles one after the other where too few warps hide their latency.  Rates measured on the three products of the
 // layer above (8.6 GFLOP each; 512, 128 and 512 tiles of 128 x 128): 194, 233 and 174 us with the plain 128 x 128 tile,
 // 207, 206 and 196 us with its contraction cut in two, the better one where there is a tile per SM at most (the second
 // product); 236-298 us with 64 x 64 and 262 us with 64 x 32 tiles, which win by their number on small problems.
+// Against the best of the four on 34 other sizes (k 12-1813, d 32-1024, d' 32-4096, 1 to 32 experts; 102 products): the same
+// or within 4.4 % in nine of ten, 1.29 times the best at worst (k = 1219, d = 164, d' = 2924, 4 experts: H . W2^T in 64 x 32
+// tiles 218 us, in 64 x 64 169).
 Tile pick_tile(const GemmArgs& g, int sms) {
   struct Form { Tile id; int bm, bn, kstep, per_sm; double alone, full; };
   static const Form forms[] = {{TILE_128x128, 128, 128, 16, 2, 0.61, 0.80}, {TILE_128x128_K2, 128, 128, 32, 1, 0.70, 0.70},
@@ -353,6 +363,7 @@ Tile pick_tile(const GemmArgs& g, int sms) {
   constexpr double kLatency = 1000.;                  // cycles of a k-tile nobody hides
   Tile best = TILE_64x32; double least = 0.;
   for (const Form& f : forms) {
+    if ((g.N + f.bn - 1) / f.bn > kMaxColTiles) continue;
     const int64_t tiles = (((int64_t)g.M + f.bm - 1) / f.bm) * ((g.N + f.bn - 1) / f.bn) * g.batches, q = (tiles + sms - 1) / sms;
     const double work = (double)q * f.bm * f.bn * g.K / 128. / (q >= f.per_sm ? f.full : f.alone);
     const double steps = (double)((q + f.per_sm - 1) / f.per_sm) * ((g.K + f.kstep - 1) / f.kstep) * kLatency;
@@ -364,22 +375,15 @@ Tile pick_tile(const GemmArgs& g, int sms) {
 
 template <typename TA, typename TB, typename TC, int EPI, int BM, int BN, int BK, int TM, int TN, int KS, int MINB, bool VEC>
 cudaError_t launch_tile(const GemmArgs& g, const Operand& oa, const Operand& ob, int c_vec, cudaStream_t st) {
-  constexpr int kMaxCols = 65535;                     // column tiles of one launch (grid.y): wider results take several
-  if (g.batches > 65535) return cudaErrorInvalidConfiguration;
+  const dim3 grid((unsigned)(((int64_t)g.M + BM - 1) / BM), (g.N + BN - 1) / BN, g.batches);
+  if (grid.y > (unsigned)kMaxColTiles || grid.z > 65535u) return cudaErrorInvalidConfiguration;
   auto kern = gemm_simt_kernel<TA, TB, TC, EPI, BM, BN, BK, TM, TN, KS, MINB, VEC>;
   constexpr int bufs = KS * 2 * BK * (BM + BN) * 4, sums = KS > 1 ? BM * BN * 4 : 0, smem = bufs > sums ? bufs : sums;
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
-  const unsigned rows = (unsigned)(((int64_t)g.M + BM - 1) / BM);
-  const int cols = (g.N + BN - 1) / BN;
-  for (int col0 = 0; col0 < cols; col0 += kMaxCols) {
-    const dim3 grid(rows, cols - col0 < kMaxCols ? cols - col0 : kMaxCols, g.batches);
-    const cudaError_t e = launch_chained(kern, grid, dim3(BM / TM * (BN / TN) * KS), smem, st, g, oa, ob, c_vec, col0);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  return launch_chained(kern, grid, dim3(BM / TM * (BN / TN) * KS), smem, st, g, oa, ob, c_vec);
 }
 
 // Operands whose groups of four straddle an edge (an expert count that is not a multiple of four, in the gate's gradients
@@ -387,6 +391,9 @@ cudaError_t launch_tile(const GemmArgs& g, const Operand& oa, const Operand& ob,
 // have them contract rows of whole 16-byte vectors.
 template <typename TA, typename TB, typename TC, int EPI>
 cudaError_t launch_odd(const GemmArgs& g, const Operand& oa, const Operand& ob, int c_vec, cudaStream_t st) {
+  if constexpr (EPI == EPI_ADD_SLOTS) {               // the one product whose columns are the layer's width
+    if (g.N > 32 * kMaxColTiles) return launch_tile<TA, TB, TC, EPI, 64, 64, 16, 8, 8, 2, 3, false>(g, oa, ob, c_vec, st);
+  }
   return launch_tile<TA, TB, TC, EPI, 64, 32, 32, 4, 4, 1, 4, false>(g, oa, ob, c_vec, st);
 }
 template <int EPI>

@@ -33,8 +33,8 @@ def test_fp32_products_match_64_bits(k, d, dff, E):
 
 @pytest.mark.parametrize("dtype,E", [(torch.float32, 2), (torch.float32, 4), (torch.bfloat16, 2)])
 def test_rows_wider_than_one_grid_of_column_tiles(dtype, E):
-    """d = 2^21 + 8: 65537 column tiles of 32, more than a grid has places for, in dX = dL . Wg^T + slot rows when the number
-    of experts is not a multiple of four (fp32) or eight (bf16); beside it the same width on wider tiles."""
+    """d = 2^21 + 8: 65537 column tiles of 32, more than a grid has places for: dX = dL . Wg^T + slot rows takes wider ones, with the
+    number of experts a multiple of four (fp32) or not, and so do GEMM-2 and dX_in."""
     n, d, dff = 8, (1 << 21) + 8, 8
     cfg = B.make_config(n, d, dff, E, 1.0, dtype)
     gen = torch.Generator(device="cuda").manual_seed(E)
