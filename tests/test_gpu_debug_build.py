@@ -141,3 +141,22 @@ def test_a_solver_wait_that_runs_out_is_reported_and_leaves_a_defined_assignment
     assert bool(((A >= 0) & (A <= 1)).all())
     again = D.ec_capped_assignment(cfg, S, ws=ws)
     assert D.ec_read_status(ws) == D.EC_OK and torch.equal(again, want)
+
+
+@pytest.mark.parametrize("n,E,dtype,kw", [(2048, 8, BF16, {}), (20000, 8, BF16, {}), (2048, 8, F32, dict(fuse_gather=True)), (2048, 8, BF16, dict(fuse_gather=True)),
+                                          (2048, 8, BF16, dict(router="token")), (2048, 8, BF16, dict(cap_b=3, cap_iters=5)),
+                                          (20000, 65, BF16, dict(cap_b=3, cap_iters=5)), (1000, 10, F32, dict(groups=2))])
+def test_a_layer_with_rows_of_nan_stays_inside_its_buffers(D, n, E, dtype, kw):
+    """Half of the tokens are NaN, many more than an expert takes: whatever the values, no index is out of range."""
+    d, dff, g = 64, 64, kw.get("groups", 1)
+    cfg = D.make_config(n, d, dff, E, 1.0, dtype, **kw)
+    li = IN.make_layer_inputs(n * g, d, dff, E, dtype, seed=n)
+    X, Wg, W1, W2, dY = (t.cuda() for t in (li.X, li.Wg, li.W1, li.W2, li.dX_out))
+    X[::2] = float("nan")
+    ws = D.alloc_workspace(cfg)
+    Y, saved = D.ec_moe_forward(cfg, X, Wg, W1, W2, ws=ws)
+    assert D.ec_read_status(ws) == D.EC_OK
+    v = D.saved_view(cfg, saved)
+    assert D.ec_validate_routing(cfg, v["I"], v["row_ptr"], v["slots"]) == 0
+    D.ec_moe_backward(cfg, X, Wg, W1, W2, dY, saved, ws=ws)
+    assert D.ec_read_status(ws) == D.EC_OK
