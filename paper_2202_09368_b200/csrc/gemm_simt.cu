@@ -1,7 +1,7 @@
 // Plain FMA batched GEMM with arbitrary element strides and the layer's fused epilogues.
-// It is the arithmetic of the fp32 path (the 1e-4 tolerance rules out TF32 tensor cores) and, with one bf16 operand, of
-// the gate gradients whose expert count the tcgen05 kernel does not take.  fp32 accumulation throughout: every result
-// is one chain of fused multiply-adds in ascending k, or, where a tile's contraction is shared by two groups of threads
+// It is the arithmetic of the fp32 path's gate gradients and of its small expert products (the others run on the tensor cores
+// in three bf16 pieces, gemm_f32_tc.cu) and, with one bf16 operand, of the gate gradients whose expert count the tcgen05
+// kernel does not take.  fp32 accumulation throughout: every result is one chain of fused multiply-adds in ascending k, or, where a tile's contraction is shared by two groups of threads
 // (KS = 2: they take its k-tiles in turn), the sum of two such chains.
 //
 // A CTA computes a BM x BN tile, a thread TM x TN results of it (groups of four rows and four columns, so that every
@@ -12,7 +12,7 @@
 //     of two shared buffers: one barrier per k-tile, no load latency in the open;
 //   - both tiles lie [k][m] and [k][n], whatever the storage order.  A column is XOR-ed with a function of k that spreads the
 //     scalar stores of a transposed tile over all 32 banks and keeps groups of four together.
-// At n = 2048, d = 512, d' = 2048, 16 experts (8.6 GFLOP per expert product) a product takes 174-207 us, 42-50 TFLOP/s of the
+// At n = 2048, d = 512, d' = 2048, 16 experts (8.6 GFLOP per expert product) a product takes 174-207 us here, 42-50 TFLOP/s of the
 // 74 the FMA pipe has; the 64 x 64 tile with 4 x 4 results per thread, one buffer and scalar loads that this replaces
 // took 445-640 us.  What is left, from the counters: the FMA pipe is busy 75 % of the time in the plain 128 x 128 tile and the
 // shared-memory pipe 48 % (two CTAs of four warps on an SM do not cover all of each other's fragment loads and barriers),
@@ -50,22 +50,6 @@ __device__ __forceinline__ unsigned long long pair2(float a, float b) {
 }
 __device__ __forceinline__ unsigned long long fma_pair(unsigned long long a, unsigned long long b, unsigned long long c) {
   unsigned long long d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d;
-}
-
-__device__ __forceinline__ float gelu_fwd(float z, int variant) {
-  if (variant == 0) return 0.5f * z * (1.f + erff(z * 0.70710678118654752f));
-  const float u = 0.7978845608028654f * (z + 0.044715f * z * z * z);
-  return 0.5f * z * (1.f + tanhf(u));
-}
-__device__ __forceinline__ float gelu_bwd(float z, int variant) {
-  if (variant == 0) {
-    const float Phi = 0.5f * (1.f + erff(z * 0.70710678118654752f));
-    const float phi = 0.3989422804014327f * expf(-0.5f * z * z);
-    return Phi + z * phi;
-  }
-  const float a = 0.7978845608028654f;
-  const float th = tanhf(a * (z + 0.044715f * z * z * z));
-  return 0.5f * (1.f + th) + 0.5f * z * (1.f - th * th) * a * (1.f + 3.f * 0.044715f * z * z);
 }
 
 // How an operand's tile is fetched: which storage direction is contiguous and whether four elements along it can be
@@ -356,7 +340,7 @@ enum Tile { TILE_128x128, TILE_128x128_K2, TILE_64x64_K2, TILE_64x32 };
 // Against the best of the four on 34 other sizes (k 12-1813, d 32-1024, d' 32-4096, 1 to 32 experts; 102 products): the same
 // or within 4.4 % in nine of ten, 1.29 times the best at worst (k = 1219, d = 164, d' = 2924, 4 experts: H . W2^T in 64 x 32
 // tiles 218 us, in 64 x 64 169).
-Tile pick_tile(const GemmArgs& g, int sms) {
+Tile pick_tile(const GemmArgs& g, int sms, double* cycles) {
   struct Form { Tile id; int bm, bn, kstep, per_sm; double alone, full; };
   static const Form forms[] = {{TILE_128x128, 128, 128, 16, 2, 0.61, 0.80}, {TILE_128x128_K2, 128, 128, 32, 1, 0.70, 0.70},
                                {TILE_64x64_K2, 64, 64, 32, 3, 0.45, 0.60}, {TILE_64x32, 64, 32, 32, 4, 0.35, 0.52}};
@@ -370,6 +354,7 @@ Tile pick_tile(const GemmArgs& g, int sms) {
     const double t = work > steps ? work : steps;
     if (least == 0. || t < least) { least = t; best = f.id; }
   }
+  *cycles = least;
   return best;
 }
 
@@ -436,7 +421,13 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st) {
   if (g.a_rows && !(oa.vec && ob.vec)) return cudaErrorInvalidValue;         // the scalar tile does not read through a list
   if (g.a_dtype == 0 && g.b_dtype == 0 && g.c_dtype == 0) {
     if (oa.vec && ob.vec) {
-      const Tile tile = pick_tile(g, sms);
+      double fma_cycles; int cols = 0;
+      const Tile tile = pick_tile(g, sms, &fma_cycles);
+      // The tensor cores where their estimate is the lower one.  They win from a few k-blocks and tiles on: 205 against 67 us at
+      // 256 x 512 x 2048 (16 experts), 14.7 against 12.9 at 58 x 584 x 180 (10); with few rows or a short or lonely contraction
+      // a tile of multiply-adds is over sooner: 16.3 against 17.0 at 8 x 128 x 384 (24), 21.0 against 23.1 at 40 x 200 x 600 (16).
+      const double tc_cycles = c_vec ? plan_gemm_f32_tc(g, sms, &cols) : -1.;
+      if (tc_cycles >= 0. && tc_cycles < fma_cycles) return launch_gemm_f32_tc(g, cols, sms, st);
       switch (g.epi) {
         case EPI_STORE: return launch_f32<EPI_STORE>(g, tile, oa, ob, c_vec, st);
         case EPI_GELU: return launch_f32<EPI_GELU>(g, tile, oa, ob, c_vec, st);

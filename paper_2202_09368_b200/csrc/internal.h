@@ -149,6 +149,23 @@ cudaError_t launch_gather_gate(const float* S, const int32_t* I, float* G, int64
 // ---- plain FMA GEMM (gemm_simt.cu) -------------------------------------------------------------
 enum Epilogue { EPI_STORE = 0, EPI_GELU = 1, EPI_GELU_GRAD = 2, EPI_ADD_SLOTS = 3 };
 
+// GeLU and its derivative as the fp32 path takes them (variant 0: z Phi(z), 1: the tanh form)
+__device__ __forceinline__ float gelu_fwd(float z, int variant) {
+  if (variant == 0) return 0.5f * z * (1.f + erff(z * 0.70710678118654752f));
+  const float u = 0.7978845608028654f * (z + 0.044715f * z * z * z);
+  return 0.5f * z * (1.f + tanhf(u));
+}
+__device__ __forceinline__ float gelu_bwd(float z, int variant) {
+  if (variant == 0) {
+    const float Phi = 0.5f * (1.f + erff(z * 0.70710678118654752f));
+    const float phi = 0.3989422804014327f * expf(-0.5f * z * z);
+    return Phi + z * phi;
+  }
+  const float a = 0.7978845608028654f;
+  const float th = tanhf(a * (z + 0.044715f * z * z * z));
+  return 0.5f * (1.f + th) + 0.5f * z * (1.f - th * th) * a * (1.f + 3.f * 0.044715f * z * z);
+}
+
 struct GemmArgs {
   const void* A; const void* B; void* C;
   int a_dtype, b_dtype, c_dtype;       // ec_dtype values; accumulation is always fp32
@@ -169,6 +186,11 @@ struct GemmArgs {
   const int32_t* a_rows; int64_t a_rows_batch, a_rows_total; int a_rows_k;
 };
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
+// ---- fp32 products on the tensor cores (gemm_f32_tc.cu): launch_gemm_simt takes them where they are the faster ones.  Operands
+// and results fp32, every row a whole number of 16-byte groups at a 16-byte aligned address.  The plan gives the columns per
+// tile (64 or 128) and the estimated cycles, or a negative number for a product that this kernel does not take.
+double plan_gemm_f32_tc(const GemmArgs& g, int sms, int* cols);
+cudaError_t launch_gemm_f32_tc(const GemmArgs& g, int cols, int sms, cudaStream_t st);
 
 // ---- tcgen05 GEMM (gemm_tc.cu) ---------------------------------------------------------------------
 struct TcGemmArgs {
