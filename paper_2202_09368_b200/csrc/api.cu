@@ -189,21 +189,26 @@ ec_status route_impl(const Dims& D, const void* X, const void* Wg, float* S, int
                      int32_t* row_ptr, int32_t* slots, char* ws, const WsLayout& W, cudaStream_t st,
                      int32_t* load = nullptr, int32_t* requested = nullptr) {
   bool done = false;
+  int* status = (int*)(ws + W.status);
+  const bool selects = D.router != EC_ROUTER_TOKEN_TOP2;
+  const IndexPlan plan = plan_index(D.ng, D.E, D.kg, D.groups, selects, ws + W.topk, ws + W.inverse);
+  // the gate's kernel clears the status block and the slot marks
   if (D.dtype == EC_BF16) {
     TcGemmArgs t; memset(&t, 0, sizeof(t));
     t.A = X; t.B = Wg; t.a_mn_major = 0; t.b_mn_major = 1;
     t.M = (int)D.n; t.N = D.E; t.K = D.d; t.batches = 1; t.lda = D.d; t.ldb = D.E;
-    t.epi = EPI_SOFTMAX; t.S = S; t.ldc = D.E; t.status = (int*)(ws + W.status);
+    t.epi = EPI_SOFTMAX; t.S = S; t.ldc = D.E; t.status = status;
+    t.clear = plan.marks.words; t.clear_words = plan.marks.per_token ? plan.marks.per_token : 1;
     if (tc_gemm_supported(t)) { EC_CUDA(launch_gemm_tc(t, st)); done = true; }
   }
-  if (!done) EC_CUDA(launch_gate_softmax_simt(D.dtype, X, Wg, S, D.n, D.d, D.E, st));
+  if (!done) EC_CUDA(launch_gate_softmax_simt(D.dtype, X, Wg, S, D.n, D.d, D.E, plan.marks, status, st));
   prof_mark("gate_softmax", st);
-  if (D.router == EC_ROUTER_TOKEN_TOP2) {            // Section 3.1's token choice as a contrast: tokens pick, experts have buffers
+  if (!selects) {                                    // Section 3.1's token choice as a contrast: tokens pick, experts have buffers
     int32_t* choice = (int32_t*)(ws + W.choice);
     EC_CUDA(launch_token_top2(S, D.n, D.E, choice, st));
-    EC_CUDA(launch_token_admit(S, choice, D.ng, D.E, D.kg, D.groups, I, G, load, requested, st));
+    EC_CUDA(launch_token_admit(S, choice, D.ng, D.E, D.kg, D.groups, I, G, load, requested, plan.marks, st));
     prof_mark("token_choice", st);
-    EC_CUDA(launch_inverse_index(I, D.n, D.slots, row_ptr, slots, ws + W.inverse, (int*)(ws + W.status), st));
+    EC_CUDA(launch_inverse_index(I, D.n, D.slots, D.k, plan, row_ptr, slots, ws + W.inverse, status, st));
     prof_mark("inverse_index", st);
     return EC_OK;
   }
@@ -211,14 +216,15 @@ ec_status route_impl(const Dims& D, const void* X, const void* Wg, float* S, int
   if (D.cap_b) {                                    // Section 3.3: TopK(A, k) instead of TopK(S^T, k)
     float* A = (float*)(ws + W.cap_A);
     EC_CUDA(launch_capped_assignment(S, D.ng, D.E, D.kg, D.groups, D.cap_b, D.cap_iters, (float)D.cap_lambda, A,
-                                     ws + W.capped, (int*)(ws + W.status), st));
+                                     ws + W.capped, status, st));
     prof_mark("capped_assignment", st);
     keys = A;
   }
-  EC_CUDA(launch_topk(keys, D.ng, D.E, D.kg, D.groups, I, G, ws + W.topk, st));
-  if (D.cap_b) EC_CUDA(launch_gather_gate(S, I, G, D.slots, D.k, D.E, D.n, (int*)(ws + W.status), st));      // the gate weights stay S at I
-  prof_mark("topk", st);
-  EC_CUDA(launch_inverse_index(I, D.n, D.slots, row_ptr, slots, ws + W.inverse, (int*)(ws + W.status), st));
+  EC_CUDA(launch_topk(keys, D.ng, D.E, D.kg, D.groups, I, G, plan, row_ptr, slots, ws + W.topk, status, st));
+  if (D.cap_b) EC_CUDA(launch_gather_gate(S, I, G, D.slots, D.k, D.E, D.n, status, st));      // the gate weights stay S at I
+  prof_mark(plan.fused ? "topk_index" : "topk", st);
+  if (plan.fused) return EC_OK;
+  EC_CUDA(launch_inverse_index(I, D.n, D.slots, D.k, plan, row_ptr, slots, ws + W.inverse, status, st));
   prof_mark("inverse_index", st);
   return EC_OK;
 }
@@ -300,7 +306,6 @@ ec_status ec_route(const ec_config* c, const void* X, const void* Wg, float* S, 
   const WsLayout W = ws_layout(D);
   if (ws_bytes < W.total) return EC_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
-  EC_CUDA(cudaMemsetAsync(ws, 0, sizeof(StatusWord), st));
   prof_begin(st, 0);
   return route_impl(D, X, Wg, S, I, G, row_ptr, slots, (char*)ws, W, st);
 }
@@ -317,7 +322,6 @@ ec_status ec_route_token_choice(const ec_config* c, const void* X, const void* W
   const WsLayout W = ws_layout(D);
   if (ws_bytes < W.total) return EC_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
-  EC_CUDA(cudaMemsetAsync(ws, 0, sizeof(StatusWord), st));
   prof_begin(st, 0);
   return route_impl(D, X, Wg, S, I, G, row_ptr, slots, (char*)ws, W, st, load, requested);
 }
@@ -378,9 +382,8 @@ ec_status ec_route_static(const ec_config* c, const void* X, const void* Wg, flo
   void* ws = nullptr;
   if ((s = static_scratch(&ws)) != EC_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
-  // The array keeps whatever the previous call left: the status word is cleared here, and the
-  // routing stages clear their own counters, histograms and cursors before they use them.
-  EC_CUDA(cudaMemsetAsync(ws, 0, sizeof(StatusWord), st));
+  // The array keeps whatever the previous call left: the routing stages clear the status word and their own
+  // counters, marks, histograms and cursors before they use them.
   prof_begin(st, 0);
   return route_impl(D, X, Wg, S, I, G, row_ptr, slots, (char*)ws, W, st);
 }
@@ -402,7 +405,6 @@ ec_status ec_moe_forward(const ec_config* c, const void* X, const void* Wg, cons
   int32_t* row_ptr = (int32_t*)(sv + L.row_ptr); int32_t* slots = (int32_t*)(sv + L.slots);
   void* X_in = sv + L.X_in; void* Z = keep ? sv + L.Z : nullptr; void* H = sv + L.H; float* X_e = (float*)(sv + L.X_e);
   int* status = (int*)(w + W.status);
-  EC_CUDA(cudaMemsetAsync(ws, 0, sizeof(StatusWord), st));
   prof_begin(st, 0);
   // token-choice contrast: slots filled per expert; with one routing group they are a prefix of the expert's buffer and
   // the tensor-core GEMMs skip what lies beyond
@@ -410,14 +412,17 @@ ec_status ec_moe_forward(const ec_config* c, const void* X, const void* Wg, cons
   int32_t* requested = D.router ? (int32_t*)(sv + L.requested) : nullptr;
   const int32_t* rag = D.router && D.groups == 1 ? load : nullptr;
   if ((s = route_impl(D, X, Wg, S, I, G, row_ptr, slots, w, W, st, load, requested)) != EC_OK) return s;
-  if (!D.fuse) {
+  // The fp32 kernels pick rows of X through I as fast as they read rows of X_in: where nothing is kept, X_in is not made.
+  // (bf16 does not: its row-indexed loads are the slower ones.)
+  const bool in_place = D.fuse || (!keep && D.dtype == EC_F32 && D.router == EC_ROUTER_EXPERT_CHOICE);
+  if (!in_place) {
     EC_CUDA(launch_gather(D.dtype, X, I, X_in, D.slots, D.d, D.n, status, st));
     prof_mark("gather", st);
   }
   const int64_t kd = D.k * D.d, kf = D.k * D.dff, df = (int64_t)D.d * D.dff;
-  // Z = X_in[i] . W1[i],  H = GeLU(Z); with fuse_gather X_in[i] is rows I[i, :] of X read in place
+  // Z = X_in[i] . W1[i],  H = GeLU(Z); in place, X_in[i] is rows I[i, :] of X
   BatchedGemm g1 = {X_in, 0, D.d, kd, W1, 1, D.dff, df, Z, D.dff, kf, (int)D.k, D.dff, D.d, D.E, EPI_GELU, H, nullptr, 0, rag, 1, b1};
-  if (D.fuse) { g1.A = X; g1.batch_a = 0; g1.a_rows = I; g1.a_rows_batch = D.k; g1.a_rows_total = D.n; }
+  if (in_place) { g1.A = X; g1.batch_a = 0; g1.a_rows = I; g1.a_rows_batch = D.k; g1.a_rows_total = D.n; }
   if ((s = run_gemm(D, g1, status, st)) != EC_OK) return s;
   prof_mark("gemm1_gelu", st);
   // X_e = H[i] . W2[i]^T, kept in fp32

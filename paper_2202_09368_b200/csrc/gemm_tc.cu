@@ -85,6 +85,7 @@ struct TcParams {
   int64_t ldc, batch_c;
   int* status;
   int k_split;                                       // batches are cuts of one product along K
+  unsigned* clear; int clear_words;                  // EPI_SOFTMAX: words per row to zero
   int skip_c;                                        // EPI_GELU: only H = GeLU(acc) is stored, the accumulator itself is not
   const int32_t* row_ptr; const int32_t* slots; const bf16* rows; int64_t ld_rows;   // EPI_ADD_SLOTS
   int64_t slots_total;                               // rows of `rows`: what the debug build checks the slot ids against
@@ -407,6 +408,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int q = warp & 3;                        // TMEM lane quarter this warp may read
     const int half = (warp - 2) >> 2;              // which half of the tile's columns this warp handles
     int it = 0;
+    if constexpr (EPI == EPI_SOFTMAX) {            // the first kernel of a call: its status block starts at zero
+      if (p.clear != nullptr && blockIdx.x == 0) for (int i = threadIdx.x - 64; i < kStatusWords; i += kEpiWarps * 32) p.status[i] = 0;
+    }
     uint32_t nchunk = 0;                           // chunks this warp has stored so far: picks the staging buffer
     const uint32_t tempty_leader = CTAS == 2 ? map_to_cta(tempty0, 0) : tempty0;
     // EPI_GELU_GRAD: Z comes through the TMA unit, one chunk of 32 rows x 64 columns ahead of its use, into the staging
@@ -526,6 +530,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         const float inv = 1.f / sum;
         const int sw = lane & 7;
+        if (half == 0 && p.clear != nullptr && r0 + lane < p.M)
+          for (int w = 0; w < p.clear_words; ++w) p.clear[(int64_t)(r0 + lane) * p.clear_words + w] = 0u;
         if (active) {
 #pragma unroll 1
           for (int c0 = cbeg; c0 < cbeg + kColsPerWarp && c0 < p.N; c0 += 32, ++nchunk) {
@@ -769,16 +775,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // ---------------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------------
+void* driver_entry(const char* name) {
+  void* p = nullptr; cudaDriverEntryPointQueryResult qr;
+  return cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &qr) == cudaSuccess && qr == cudaDriverEntryPointSuccess ? p : nullptr;
+}
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr; cudaDriverEntryPointQueryResult qr;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qr) == cudaSuccess &&
-        qr == cudaDriverEntryPointSuccess)
-      fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-  });
+  std::call_once(once, [] { fn = (PFN_cuTensorMapEncodeTiled_v12000)driver_entry("cuTensorMapEncodeTiled"); });
   return fn;
+}
+// The tensor maps are encoded by the driver, which wants a context; a host thread whose first CUDA call this is has none yet.
+cudaError_t bind_context(int dev) {
+  static PFN_cuCtxGetCurrent_v4000 current = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] { current = (PFN_cuCtxGetCurrent_v4000)driver_entry("cuCtxGetCurrent"); });
+  CUcontext ctx = nullptr;
+  if (current != nullptr && current(&ctx) == CUDA_SUCCESS && ctx != nullptr) return cudaSuccess;
+  return cudaSetDevice(dev);
 }
 
 // Tensor map over a matrix stored [batches][rows][inner] with row pitch ld and batch pitch bs (elements).
@@ -915,6 +929,8 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& g, cudaStream_t st) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const cudaError_t bound = bind_context(dev);
+  if (bound != cudaSuccess) return bound;
   const int bn = pick_bn(g, sms / 2);
   const int ctas = pick_ctas(g, bn);
   const int bnl = bn / ctas;                         // rows of B one CTA loads
@@ -956,6 +972,7 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& g, cudaStream_t st) {
   p.row_ptr = g.row_ptr; p.slots = g.slots; p.rows = (const bf16*)g.rows; p.ld_rows = g.ld_rows; p.slots_total = g.slots_total;
   p.batch_rows = g.batch_rows; p.ragged = g.ragged;
   p.bias = (const bf16*)g.bias;
+  p.clear = g.clear; p.clear_words = g.clear_words;
   p.a_rows = g.a_rows; p.a_rows_batch = g.a_rows_batch; p.a_rows_total = (int)g.a_rows_total;
   switch (g.epi) {
     case EPI_STORE: return g.c_f32 ? launch_bn<EPI_STORE_F32>(bn, ctas, ta, tb, tc, tc2, p, st)

@@ -19,6 +19,8 @@ constexpr int kSortTile = 4096;    // 64-bit keys sorted in shared memory by one
 // Word 0 of the workspace: status written by kernels (0 = fine, 5 = a bounded wait expired, 6 = an index read from
 // I, row_ptr or slots was out of range); word 2 counts such indices.
 struct StatusWord { int code; int where; int bad_indices; int pad[61]; };
+constexpr int kStatusWords = sizeof(StatusWord) / 4;
+constexpr int kSelectCounter = 16;                   // word of the status block: CTAs of the selection that are done
 
 // Debug build (-DEC_DEBUG): every index read from I, row_ptr or slots is checked against its range before it is used;
 // a bad one is recorded in the status word and the access it would have addressed is skipped.  In the normal build
@@ -72,35 +74,53 @@ template <typename T> __device__ __forceinline__ T* after_enter(T* p) {
 // Every kernel launch of the library goes through count_launch(); ec_launch_count() reports the sum.
 void count_launch(int n = 1);
 
+// cluster: CTAs of a cluster along x, 1 for none
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
-  cudaLaunchAttribute attr[1];
+inline cudaError_t launch_chained_cluster(int cluster, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
   count_launch();
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  return launch_chained_cluster(1, kern, grid, block, smem, st, args...);
+}
 
 // ---- routing (routing.cu) -------------------------------------------------------------------
+// What the selection leaves for the token -> slot index.  per_token > 0: that many words per token, bit e % 32 of word e / 32 set
+// when expert e took the token: the number of bits is the length of the token's list, the number below e the place of e's slot
+// in it.  per_token = 0: one word per token, the length alone.  The gate's kernel clears them.
+struct SlotMarks { unsigned* words; int per_token; };
+// marks: n tokens of them are cleared, and the status block with them (the gate is the first kernel of a call)
 cudaError_t launch_gate_softmax_simt(int dtype, const void* X, const void* Wg, float* S, int64_t n,
-                                     int d, int E, cudaStream_t st);
+                                     int d, int E, const SlotMarks& marks, int* status, cudaStream_t st);
 // scratch layout for the selection is described in routing.cu; bytes needed:
 // `groups` independent routing groups of n tokens each (S has groups * n rows); I and G are [E, groups * k],
 // group g of an expert at positions g * k .. g * k + k - 1, with global token indices
 size_t topk_scratch_bytes(int64_t n, int E, int64_t k, int groups);
+size_t inverse_scratch_bytes(int64_t n);
+// The marks of a call and whether the selection's own kernel also builds the index (`selects` = false: there is no selection,
+// the marks come from token_admit_kernel).  ng, k: per group.
+struct IndexPlan { SlotMarks marks; bool fused, small; };       // small: one launch, ranks from the marks
+IndexPlan plan_index(int64_t ng, int E, int64_t k, int groups, bool selects, void* topk_scratch, void* inverse_scratch);
+// With plan.fused, row_ptr and slots are written too.
 cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups, int32_t* I, float* G,
-                        void* scratch, cudaStream_t st);
+                        const IndexPlan& plan, int32_t* row_ptr, int32_t* slots, void* scratch, int* status, cudaStream_t st);
 // Token-choice contrast (Section 3.1): every token's two best experts (ties: lower expert) into choice [rows, 2];
 // then, per expert and group, the requests in token order fill a buffer of k slots: I (-1 = empty), G (0 = empty),
 // load and requested [groups, E].
 cudaError_t launch_token_top2(const float* S, int64_t rows, int E, int32_t* choice, cudaStream_t st);
 cudaError_t launch_token_admit(const float* S, const int32_t* choice, int64_t n, int E, int64_t k, int groups,
-                               int32_t* I, float* G, int32_t* load, int32_t* requested, cudaStream_t st);
-size_t inverse_scratch_bytes(int64_t n);
+                               int32_t* I, float* G, int32_t* load, int32_t* requested, const SlotMarks& marks, cudaStream_t st);
+// row_ptr and slots from I and the marks (k_row slots per expert, all groups)
 // (`status`: the workspace's status word, for the index checks of the debug build; may be null)
-cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t slots_total, int32_t* row_ptr,
+cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t slots_total, int64_t k_row, const IndexPlan& plan, int32_t* row_ptr,
                                  int32_t* slots, void* scratch, int* status, cudaStream_t st);
 cudaError_t launch_gather(int dtype, const void* X, const int32_t* I, void* X_in, int64_t slots_total,
                           int d, int64_t n, int* status, cudaStream_t st);
@@ -206,6 +226,7 @@ struct TcGemmArgs {
                                                                       // EPI_GELU with C null writes only C2 = GeLU(acc)
   int c_f32;
   float* S;         // EPI_SOFTMAX: fp32 row softmax of the N columns, [M, N]
+  unsigned* clear; int clear_words;  // EPI_SOFTMAX: words per row that are set to zero (the slot marks), and the status block with them
   int* status;      // device status word
   // k_split != 0: one matrix product cut along K.  A and B are single matrices (batch strides unused),
   // `batches` is the number of cuts and K the length of one (a multiple of 64); cut b contracts rows

@@ -46,6 +46,14 @@ template <> struct Vec<bf16> {
   }
 };
 
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// this CTA's shared-memory address as CTA `rank` of the cluster has it
+__device__ __forceinline__ unsigned cluster_address(const void* p, int rank) {
+  unsigned r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank)); return r;
+}
+
 static inline unsigned grid_for(int64_t work, int threads, int64_t cap = 148 * 16) {
   int64_t b = (work + threads - 1) / threads;
   if (b < 1) b = 1;
@@ -79,8 +87,10 @@ __host__ __device__ constexpr int gate_smem_bytes(int NG) { return 2 * (8 / NG) 
 // WVEC: rows of Wg are whole 16-byte (fp32) or 8-byte (bf16) groups of four
 template <typename T, int NG, bool WVEC>
 __global__ void __launch_bounds__(kGateThreads)
-gate_softmax_simt_kernel(const T* __restrict__ X, const T* __restrict__ Wg, float* __restrict__ S, int64_t n, int d, int E) {
+gate_softmax_simt_kernel(const T* __restrict__ X, const T* __restrict__ Wg, float* __restrict__ S, int64_t n, int d, int E,
+                         const SlotMarks marks, int* status) {
   chain_enter();
+  if (blockIdx.x == 0) for (int i = threadIdx.x; i < kStatusWords; i += kGateThreads) status[i] = 0;     // the first kernel of a call
   X = after_enter(X); Wg = after_enter(Wg);
   constexpr int KS = 8 / NG, DK = KS * kGateSlice, C = 32 * NG;         // chunk: DK depths of 32 tokens and of C experts
   constexpr int kX = DK * kGateTT, kW = DK * C, XQ = (kX / 4 + kGateThreads - 1) / kGateThreads, WQ = kW / 4 / kGateThreads;
@@ -178,6 +188,8 @@ gate_softmax_simt_kernel(const T* __restrict__ X, const T* __restrict__ Wg, floa
   for (int tok = warp; tok < kGateTT; tok += 8) {     // a warp per token
     const int64_t t = t0 + tok;
     if (t >= n) break;
+    const int words = max(1, marks.per_token);
+    if (lane < words) marks.words[t * words + lane] = 0u;
     float v[NG], mx = -INFINITY, sum = 0.f;
 #pragma unroll
     for (int j = 0; j < NG; ++j) {
@@ -197,28 +209,28 @@ gate_softmax_simt_kernel(const T* __restrict__ X, const T* __restrict__ Wg, floa
 }
 
 template <typename T, int NG>
-cudaError_t launch_gate_ng(const T* X, const T* Wg, float* S, int64_t n, int d, int E, cudaStream_t st) {
+cudaError_t launch_gate_ng(const T* X, const T* Wg, float* S, int64_t n, int d, int E, const SlotMarks& marks, int* status, cudaStream_t st) {
   const unsigned grid = (unsigned)((n + kGateTT - 1) / kGateTT);
   const bool wvec = E % 4 == 0;                       // Wg itself is 16-byte aligned
   auto kern = wvec ? gate_softmax_simt_kernel<T, NG, true> : gate_softmax_simt_kernel<T, NG, false>;
   constexpr int smem = gate_smem_bytes(NG);
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  return launch_chained(kern, dim3(grid), dim3(kGateThreads), smem, st, X, Wg, S, n, d, E);
+  return launch_chained(kern, dim3(grid), dim3(kGateThreads), smem, st, X, Wg, S, n, d, E, marks, status);
 }
 template <typename T>
-cudaError_t launch_gate_t(const T* X, const T* Wg, float* S, int64_t n, int d, int E, cudaStream_t st) {
-  if (E <= 32) return launch_gate_ng<T, 1>(X, Wg, S, n, d, E, st);
-  if (E <= 64) return launch_gate_ng<T, 2>(X, Wg, S, n, d, E, st);
-  if (E <= 128) return launch_gate_ng<T, 4>(X, Wg, S, n, d, E, st);
-  return launch_gate_ng<T, 8>(X, Wg, S, n, d, E, st);
+cudaError_t launch_gate_t(const T* X, const T* Wg, float* S, int64_t n, int d, int E, const SlotMarks& marks, int* status, cudaStream_t st) {
+  if (E <= 32) return launch_gate_ng<T, 1>(X, Wg, S, n, d, E, marks, status, st);
+  if (E <= 64) return launch_gate_ng<T, 2>(X, Wg, S, n, d, E, marks, status, st);
+  if (E <= 128) return launch_gate_ng<T, 4>(X, Wg, S, n, d, E, marks, status, st);
+  return launch_gate_ng<T, 8>(X, Wg, S, n, d, E, marks, status, st);
 }
 
 cudaError_t launch_gate_softmax_simt(int dtype, const void* X, const void* Wg, float* S, int64_t n,
-                                     int d, int E, cudaStream_t st) {
+                                     int d, int E, const SlotMarks& marks, int* status, cudaStream_t st) {
   if (E > 256) return cudaErrorInvalidValue;
-  return dtype == 0 ? launch_gate_t((const float*)X, (const float*)Wg, S, n, d, E, st)
-                    : launch_gate_t((const bf16*)X, (const bf16*)Wg, S, n, d, E, st);
+  return dtype == 0 ? launch_gate_t((const float*)X, (const float*)Wg, S, n, d, E, marks, status, st)
+                    : launch_gate_t((const bf16*)X, (const bf16*)Wg, S, n, d, E, marks, status, st);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -560,12 +572,18 @@ topk_compact_kernel(const float* __restrict__ S, int64_t n, int E, unsigned k, i
 
 // Slot j of virtual expert ve = group * E + expert lands in row `expert` of I and G (each groups * k long) at
 // position group * k + j, and the token index becomes global (group * n + token within the group).
-struct SlotMap { int E, groups; int64_t k, n; };
+struct SlotMap { int E, groups; int64_t k, n; SlotMarks marks; };
+__device__ __forceinline__ void mark_slot(const SlotMarks& m, int64_t token, int e) {
+  if (m.per_token > 0) atomicOr(m.words + token * m.per_token + (e >> 5), 1u << (e & 31));
+  else atomicAdd(m.words + token, 1u);
+}
 __device__ __forceinline__ void emit_slot(unsigned long long key, int32_t* I, float* G, const SlotMap& m, int64_t ve, int64_t j) {
   const int64_t grp = ve / m.E, e = ve % m.E;
   const int64_t o = (e * m.groups + grp) * m.k + j;
-  I[o] = (int32_t)((unsigned)(key & 0xFFFFFFFFull) + (unsigned)(grp * m.n));
+  const unsigned t = (unsigned)(key & 0xFFFFFFFFull) + (unsigned)(grp * m.n);
+  I[o] = (int32_t)t;
   G[o] = __uint_as_float(~(unsigned)(key >> 32));
+  mark_slot(m.marks, t, (int)e);
 }
 
 // Bitonic sorting of keys in shared memory by the whole CTA.  The steps whose stride spans a warp's keys work on shared memory
@@ -732,6 +750,73 @@ __global__ void topk_sort_global_kernel(unsigned long long* keys, int64_t kpad, 
   }
 }
 
+// Exclusive scan of the CTA's per-thread values (any thread count that is a multiple of 32, at most 1024);
+// returns the thread's offset and, in `total`, the sum over the CTA.
+__device__ __forceinline__ int block_exclusive_scan(int v, int* s_warp, int& total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  int inc = v;
+  for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += u; }
+  if (lane == 31) s_warp[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    const int w = lane < nwarps ? s_warp[lane] : 0;
+    int winc = w;
+    for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(0xffffffffu, winc, o); if (lane >= o) winc += u; }
+    s_warp[lane] = winc - w;
+    if (lane == 31) s_warp[32] = winc;
+  }
+  __syncthreads();
+  total = s_warp[32];
+  return s_warp[warp] + inc - v;
+}
+
+// The token -> slot index by one CTA, from the marks: the lists' lengths are numbers of bits, a scan gives their starts, and a
+// slot's place in its token's list is the number of experts below its own that took the token.  No atomics, no sorting.  Marks,
+// starts and lists lie in shared memory (index_smem_bytes): what goes to a token's place in global memory costs an SM a cycle
+// per word, and one CTA has all of it to do.  A thread has eight slots in flight.  What other CTAs wrote is read past L1.
+__host__ __device__ __forceinline__ int64_t index_smem_words(int64_t N, int64_t total, int W) { return N * W + N + total; }
+__device__ __forceinline__ void build_index(const int32_t* I, int N, int total, int k_row, const SlotMarks& m, int32_t* row_ptr,
+                                            int32_t* slots, int* smem, int* s_warp, int* status) {
+  const int tid = threadIdx.x, nt = blockDim.x, W = m.per_token;
+  unsigned* marks = reinterpret_cast<unsigned*>(smem);                 // [N][W]
+  int *start = smem + N * W, *list = start + N;                        // [N], [total]
+  for (int i0 = tid; i0 < N * W; i0 += 8 * nt) {
+    unsigned v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = i0 + u * nt < N * W ? __ldcg(m.words + i0 + u * nt) : 0u;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) if (i0 + u * nt < N * W) marks[i0 + u * nt] = v[u];
+  }
+  __syncthreads();
+  const int per = (N + nt - 1) / nt, a = min(N, tid * per), b = min(N, a + per);
+  int sum = 0;
+  for (int i = a * W; i < b * W; ++i) sum += __popc(marks[i]);
+  int filled;
+  int run = block_exclusive_scan(sum, s_warp, filled);
+  for (int t = a; t < b; ++t) {
+    start[t] = run;
+    for (int w = 0; w < W; ++w) run += __popc(marks[t * W + w]);
+  }
+  __syncthreads();
+  for (int t = tid; t < N; t += nt) row_ptr[t] = start[t];
+  if (tid == 0) row_ptr[N] = filled;
+  for (int s0 = tid; s0 < total; s0 += 8 * nt) {
+    int t[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[u] = s0 + u * nt < total ? __ldcg(I + s0 + u * nt) : -1;     // -1: an empty slot (token-choice routing only), or none
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (t[u] < 0 || !idx_ok(t[u], 0, N, status)) continue;
+      const int e = (s0 + u * nt) / k_row;
+      int at = start[t[u]] + __popc(marks[t[u] * W + (e >> 5)] & ((1u << (e & 31)) - 1u));
+      for (int w = 0; w < e >> 5; ++w) at += __popc(marks[t[u] * W + w]);
+      list[at] = s0 + u * nt;
+    }
+  }
+  __syncthreads();
+  for (int s = tid; s < filled; s += nt) slots[s] = list[s];
+}
+
 // Small groups (n <= kSmallN tokens, k <= kSortTile): the whole selection of one expert in one CTA.  The
 // column is brought into shared memory once (as v = ~bits(S)), three 10-bit histogram passes over it find
 // the value of the k-th key exactly, keys below it are winners, keys equal to it win in token order, and the
@@ -739,9 +824,16 @@ __global__ void topk_sort_global_kernel(unsigned long long* keys, int64_t kpad, 
 // A CTA per expert leaves most SMs idle, so a CTA's own latency is what counts: about four keys per thread, eight loads of
 // a thread in flight, every thread takes part in a pass's scan, and the walk in token order is taken only when
 // not all keys at the threshold are wanted.  2048 tokens, k = 512: 33.5 k cycles before that, 17 k now.
+// With row_ptr, the last CTA to finish also builds the token -> slot index (build_index; `done` counts the CTAs).
+// CLUSTER: a column alone costs a CTA a request per token, of which it uses 4 of 32 bytes (8192 tokens: 10.5 k cycles, 16384:
+// 33 k; with the third pass, which is hardly ever needed, 24.5 us at 8192 tokens and 32 experts, 22.5 now).  The CTAs of eight experts form a cluster: each reads an eighth of the tokens, all eight scores of a token together, and sends every
+// score to its expert's CTA.
 constexpr int kSmallN = 16384;
+template <bool CLUSTER>
 __global__ void __launch_bounds__(1024)
-topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, SlotMap map, int32_t* I, float* G) {
+topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, const SlotMap map, int32_t* I, float* G, int32_t* row_ptr,
+                  int32_t* slots, int* done, int* status) {
+  if constexpr (CLUSTER) cluster_barrier();            // every CTA of the cluster has started: its shared memory may be written
   chain_enter();
   S = after_enter(S);
   extern __shared__ unsigned long long sm_keys[];      // [kpad] keys (kpad >= 32), then [n] values, then [kBins] histogram
@@ -750,13 +842,39 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
   __shared__ unsigned s_prefix, s_rem, s_eq, s_less, s_warp[33];
   const int e = blockIdx.x, grp = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nt = blockDim.x, nwarps = nt >> 5;         // 128 .. 1024 threads (a power of two), by the size of the group
-  const float* col = S + (size_t)grp * n * E + e;
-  for (int t0 = tid; t0 < n; t0 += 8 * nt) {
-    float x[8];
+  if constexpr (CLUSTER) {
+    const int rank = e & 7, e0 = e - rank, ne = min(8, E - e0);
+    const int per = (n + 7) / 8, t1 = min(n, (rank + 1) * per);
+    unsigned dst[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = col[(size_t)min(t0 + u * nt, n - 1) * E];
+    for (int j = 0; j < 8; ++j) dst[j] = cluster_address(val, j);
+    const bool vec = E % 4 == 0;                       // rows of S are whole 16-byte groups, and so is e0
+    for (int t = rank * per + tid; t < t1; t += nt) {
+      const float* p = S + ((size_t)grp * n + t) * E + e0;
+      float x[8];
+      if (vec) {
+        const float4 a = *reinterpret_cast<const float4*>(p);
+        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+        if (ne > 4) { const float4 b = *reinterpret_cast<const float4*>(p + 4); x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w; }
+      } else {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) if (t0 + u * nt < n) val[t0 + u * nt] = ~__float_as_uint(x[u]);
+        for (int j = 0; j < 8; ++j) x[j] = j < ne ? p[j] : 0.f;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j < ne) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(dst[j] + 4u * (unsigned)t), "r"(~__float_as_uint(x[j])) : "memory");
+    }
+    cluster_barrier();
+    if (e >= E) return;
+  } else {
+    const float* col = S + (size_t)grp * n * E + e;
+    for (int t0 = tid; t0 < n; t0 += 8 * nt) {
+      float x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = col[(size_t)min(t0 + u * nt, n - 1) * E];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) if (t0 + u * nt < n) val[t0 + u * nt] = ~__float_as_uint(x[u]);
+    }
   }
   for (int i = tid; i < kpad; i += nt) sm_keys[i] = ~0ull;
   for (int i = tid; i < kBins; i += nt) hist[i] = 0;
@@ -764,8 +882,9 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
   __syncthreads();
   // sel_bits() has its two top bits set; digits of 10 bits from bit 29 down
   const int per = kBins / nt;                          // consecutive bins of a thread in the scan: 1 .. 8
+  int sh = 20;
   for (int pass = 0; pass < 3; ++pass) {
-    const int sh = 20 - 10 * pass;
+    sh = 20 - 10 * pass;
     const unsigned pre = s_prefix, rem = s_rem;
     for (int t = tid; t < n; t += nt) {
       const unsigned v = sel_bits(val[t]);
@@ -801,8 +920,9 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
       s_eq = in;
     }
     __syncthreads();
+    if (s_eq == s_rem) break;                          // the whole bucket is wanted: nearly always after 20 of the 30 bits
   }
-  const unsigned thr = s_prefix, k_rem = s_rem, k_less = (unsigned)k - k_rem;      // k_rem keys equal to thr are wanted
+  const unsigned thr = s_prefix >> sh, k_rem = s_rem, k_less = (unsigned)k - k_rem;      // k_rem keys equal to thr are wanted
   // winners in any order: the keys below the threshold, and those at it when all of them are wanted
   const bool all_eq = s_eq == k_rem;
   for (int t0 = tid - lane; t0 < n; t0 += 4 * nt) {    // uniform across the warp
@@ -811,7 +931,7 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
     for (int u = 0; u < 4; ++u) {
       const int t = t0 + u * nt + lane;
       v[u] = t < n ? val[t] : 0xFFFFFFFFu;
-      const unsigned sv = sel_bits(v[u]);
+      const unsigned sv = sel_bits(v[u]) >> sh;
       bal[u] = __ballot_sync(0xffffffffu, t < n && (sv < thr || (all_eq && sv == thr)));
       sum += __popc(bal[u]);
     }
@@ -825,7 +945,7 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
       at += __popc(bal[u]);
     }
   }
-  // else the first k_rem keys at the threshold in token order
+  // else (all 30 bits are decided) the first k_rem keys at the threshold in token order
   unsigned running = 0;
   for (int base = 0; !all_eq && base < n && running < k_rem; base += nt) {
     const int t = base + tid;
@@ -849,24 +969,55 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, Sl
   __syncthreads();
   sort_keys(sm_keys, kpad, 0, (unsigned)kpad);
   for (int i = tid; i < k; i += nt) emit_slot(sm_keys[i], I, G, map, (int64_t)grp * E + e, i);
+  if (row_ptr == nullptr) return;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_less = atomicAdd(done, 1) == E * map.groups - 1 ? 1u : 0u;
+  __syncthreads();
+  if (!s_less) return;
+  __threadfence();
+  build_index(I, n * map.groups, E * k * map.groups, k * map.groups, map.marks, row_ptr, slots, reinterpret_cast<int*>(sm_keys),
+              reinterpret_cast<int*>(s_warp), status);
+}
+
+// Dynamic shared memory of a launch: the attribute is one per device, whatever threads launch, so it is always set to the most
+// that any call needs, never less than another's
+constexpr int kMostSelectSmem = kSortTile * 8 + kSmallN * 4 + kBins * 4;
+constexpr int kIndexClusterTokens = 16384, kIndexClusterSlots = 1 << 17;
+IndexPlan plan_index(int64_t ng, int E, int64_t k, int groups, bool selects, void* topk_scratch, void* inverse_scratch) {
+  const int64_t N = ng * groups, total = (int64_t)E * k * groups;
+  const int words = (E + 31) / 32;
+  IndexPlan p;
+  // The selection's last CTA builds the index where everything fits its shared memory (2048 tokens, 8 experts: 24.5 us with two
+  // launches that counted, filled and sorted, 20.5 so); a cluster of eight CTAs up to 16384 tokens (8192 tokens, 32 experts: 18.4 us with
+  // atomics and sorting, 14.4 from the marks; one CTA alone takes 22).  Their marks may take the place of the large selection's
+  // scratch, which such a call does not use.
+  const bool one_launch = selects && ng <= kSmallN && k <= kSortTile;
+  p.fused = one_launch && N <= 4096 && index_smem_words(N, total, words) * 4 <= kMostSelectSmem;
+  p.small = p.fused || (N <= kIndexClusterTokens && total <= kIndexClusterSlots && (one_launch || !selects));
+  p.marks.per_token = p.small || words == 1 ? words : 0;
+  p.marks.words = (unsigned*)(p.marks.per_token > 1 ? topk_scratch : inverse_scratch);
+  return p;
 }
 
 cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups, int32_t* I, float* G,
-                        void* scratch, cudaStream_t st) {
+                        const IndexPlan& plan, int32_t* row_ptr, int32_t* slots, void* scratch, int* status, cudaStream_t st) {
   const TopkLayout L = topk_layout(n, E, k, groups);
   if (n <= kSmallN && L.kpad <= kSortTile) {
-    const SlotMap smap = {E, groups, k, n};
+    const SlotMap smap = {E, groups, k, n, plan.marks};
     const int kpad = L.kpad < 32 ? 32 : (int)L.kpad;   // the sort works on whole warps of keys
-    const int smem = (int)(kpad * 8 + n * 4 + kBins * 4);
-    // the attribute is one per device, whatever threads launch: always the most that any call needs, never less than another's
-    constexpr int kMostSmem = kSortTile * 8 + kSmallN * 4 + kBins * 4;
-    cudaError_t e0 = cudaFuncSetAttribute(topk_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
+    int smem = (int)(kpad * 8 + n * 4 + kBins * 4);
+    if (plan.fused) smem = max(smem, (int)index_smem_words(n * groups, (int64_t)E * k * groups, plan.marks.per_token) * 4);
+    const bool cluster = n > 4096 && E >= 8;
+    auto kern = cluster ? topk_small_kernel<true> : topk_small_kernel<false>;
+    cudaError_t e0 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSelectSmem);
     if (e0 != cudaSuccess) return e0;
     int threads = 128;                                 // at most four keys per thread for the sort (kpad < 2 n)
     while (threads < 1024 && threads * 4 < n) threads <<= 1;
     while (threads < 1024 && threads * 4 < kpad) threads <<= 1;
-    launch_chained(topk_small_kernel, dim3(E, groups), dim3(threads), smem, st, S, (int)n, E, (int)k, kpad, smap, I, G);
-    return cudaGetLastError();
+    while (plan.fused && threads < 1024 && threads * 8 < (int64_t)E * k * groups) threads <<= 1;
+    return launch_chained_cluster(cluster ? 8 : 1, kern, dim3(cluster ? (E + 7) / 8 * 8 : E, groups), dim3(threads), smem, st, S, (int)n, E, (int)k, kpad, smap, I, G,
+                                  plan.fused ? row_ptr : nullptr, slots, status + kSelectCounter, status);
   }
   const int64_t VE = (int64_t)groups * E;              // independent columns: E per group
   char* base = (char*)scratch;
@@ -876,7 +1027,7 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
   unsigned* cursor = (unsigned*)(base + L.off_cursor);
   unsigned long long* cand = (unsigned long long*)(base + L.off_cand);
   unsigned long long* keys = (unsigned long long*)(base + L.off_keys);
-  const SlotMap map = {E, groups, k, n};
+  const SlotMap map = {E, groups, k, n, plan.marks};
   cudaError_t e;
   const bool vec = E % 4 == 0 && ((uintptr_t)S & 15) == 0;
   // the histogram kernels use 132 KiB of dynamic shared memory
@@ -947,7 +1098,7 @@ __global__ void __launch_bounds__(256) token_top2_kernel(const float* __restrict
 // the token order.  Empty slots get -1 / 0.
 __global__ void __launch_bounds__(1024)
 token_admit_kernel(const float* __restrict__ S, const int32_t* __restrict__ choice, int n, int E, int k,
-                   int32_t* __restrict__ I, float* __restrict__ G, int32_t* __restrict__ load, int32_t* __restrict__ requested) {
+                   int32_t* __restrict__ I, float* __restrict__ G, int32_t* __restrict__ load, int32_t* __restrict__ requested, const SlotMarks marks) {
   chain_enter();
   S = after_enter(S); choice = after_enter(choice);
   __shared__ unsigned s_warp[33];
@@ -972,7 +1123,7 @@ token_admit_kernel(const float* __restrict__ S, const int32_t* __restrict__ choi
     }
     __syncthreads();
     const unsigned pos = running + s_warp[warp] + __popc(bal & ((1u << lane) - 1u));
-    if (m && pos < (unsigned)k) { Ie[pos] = (int32_t)(row0 + t); Ge[pos] = S[(row0 + t) * E + e]; }
+    if (m && pos < (unsigned)k) { Ie[pos] = (int32_t)(row0 + t); Ge[pos] = S[(row0 + t) * E + e]; mark_slot(marks, row0 + t, e); }
     running += s_warp[32];
     __syncthreads();
   }
@@ -987,16 +1138,17 @@ cudaError_t launch_token_top2(const float* S, int64_t rows, int E, int32_t* choi
 }
 
 cudaError_t launch_token_admit(const float* S, const int32_t* choice, int64_t n, int E, int64_t k, int groups,
-                               int32_t* I, float* G, int32_t* load, int32_t* requested, cudaStream_t st) {
-  launch_chained(token_admit_kernel, dim3(E, groups), dim3(1024), 0, st, S, choice, (int)n, E, (int)k, I, G, load, requested);
+                               int32_t* I, float* G, int32_t* load, int32_t* requested, const SlotMarks& marks, cudaStream_t st) {
+  launch_chained(token_admit_kernel, dim3(E, groups), dim3(1024), 0, st, S, choice, (int)n, E, (int)k, I, G, load, requested, marks);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------
-// Index form of P = Onehot(I) (Eq. 2) read by token: row_ptr / slots.
-// Integer atomics only count and hand out positions; each token's short list is then sorted,
-// so the result does not depend on the order in which threads ran.
-// scratch: [cnt n+1 int32][tile sums ceil(n / kScanTile) int32]
+// Index form of P = Onehot(I) (Eq. 2) read by token: row_ptr / slots, from I and the marks the selection left (SlotMarks).
+// Up to 4096 tokens the selection's last CTA does it (build_index, above), up to 16384 a cluster.  Beyond, a scan of the lists' lengths in two steps, then every slot goes to its place: with up to 32 experts its rank is read from the
+// marks; with more (a word per token: the masks would outgrow the scratch) places are handed out by atomics and each token's
+// list is sorted, so the result does not depend on the order in which threads ran.
+// scratch: [marks n+1 words][tile sums ceil(n / kScanTile) int32]
 // ------------------------------------------------------------------------------------------
 constexpr int kScanTile = 4096, kScanThreads = 1024;
 static size_t inv_cnt_bytes(int64_t n) { return ((size_t)(n + 1) * 4 + 255) & ~(size_t)255; }
@@ -1004,45 +1156,14 @@ size_t inverse_scratch_bytes(int64_t n) {
   return inv_cnt_bytes(n) + ((((size_t)(n + kScanTile - 1) / kScanTile) * 4 + 255) & ~(size_t)255);
 }
 
-__global__ void inv_count_kernel(const int32_t* __restrict__ I, int64_t total, int32_t* cnt, int64_t n, int* status) {
-  chain_enter();
-  I = after_enter(I);
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < total; s += (int64_t)gridDim.x * blockDim.x) {
-    const int t = I[s];
-    if (t >= 0 && idx_ok(t, 0, n, status)) atomicAdd(&cnt[t], 1);      // -1: an empty slot (token-choice routing only)
-  }
-}
-
-// Exclusive scan of the CTA's per-thread values (any thread count that is a multiple of 32, at most 1024);
-// returns the thread's offset and, in `total`, the sum over the CTA.
-__device__ __forceinline__ int block_exclusive_scan(int v, int* s_warp, int& total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  int inc = v;
-  for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += u; }
-  if (lane == 31) s_warp[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    const int w = lane < nwarps ? s_warp[lane] : 0;
-    int winc = w;
-    for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(0xffffffffu, winc, o); if (lane >= o) winc += u; }
-    s_warp[lane] = winc - w;
-    if (lane == 31) s_warp[32] = winc;
-  }
-  __syncthreads();
-  total = s_warp[32];
-  return s_warp[warp] + inc - v;
-}
-
 // Step 1: exclusive scan inside each tile of kScanTile counts (four per thread), tile sums aside.
-__global__ void __launch_bounds__(kScanThreads) inv_scan_tile_kernel(const int32_t* __restrict__ cnt, int64_t n,
-                                                                      int32_t* row_ptr, int32_t* tile_sum) {
+__global__ void __launch_bounds__(kScanThreads) inv_scan_tile_kernel(const SlotMarks m, int64_t n, int32_t* row_ptr, int32_t* tile_sum) {
   chain_enter();
-  cnt = after_enter(cnt);
   __shared__ int s_warp[33];
   const int64_t base = (int64_t)blockIdx.x * kScanTile + threadIdx.x * 4;
   int c[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) c[j] = base + j < n ? cnt[base + j] : 0;
+  for (int j = 0; j < 4; ++j) { const unsigned v = base + j < n ? m.words[base + j] : 0u; c[j] = m.per_token ? __popc(v) : (int)v; }
   int total;
   int run = block_exclusive_scan(c[0] + c[1] + c[2] + c[3], s_warp, total);
 #pragma unroll
@@ -1066,14 +1187,16 @@ __global__ void __launch_bounds__(kScanThreads) inv_scan_add_kernel(const int32_
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) row_ptr[n] = before + tile_sum[blockIdx.x];
 }
 
-// Hands each slot a place in its token's list, counting the token's counter back down to zero.
-__global__ void inv_fill_kernel(const int32_t* __restrict__ I, int64_t total, const int32_t* __restrict__ row_ptr,
-                                int32_t* cnt, int32_t* slots, int64_t n) {
+// Puts each slot into its token's list: where its rank says, or at a place handed out by counting the token's word down to zero.
+__global__ void inv_fill_kernel(const int32_t* __restrict__ I, int64_t total, int64_t k_row, const int32_t* __restrict__ row_ptr,
+                                const SlotMarks m, int32_t* slots, int64_t n, int* status) {
   chain_enter();
   I = after_enter(I); row_ptr = after_enter(row_ptr);
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < total; s += (int64_t)gridDim.x * blockDim.x) {
-    const int t = I[s];
-    if (t >= 0 && idx_ok(t, 0, n, nullptr)) slots[row_ptr[t] + atomicSub(&cnt[t], 1) - 1] = (int32_t)s;   // counted once, in inv_count
+    const int t = I[s];                                // -1: an empty slot (token-choice routing only)
+    if (t < 0 || !idx_ok(t, 0, n, status)) continue;
+    const int at = m.per_token ? __popc(m.words[t] & ((1u << (int)(s / k_row)) - 1u)) : (int)atomicSub(m.words + t, 1u) - 1;
+    slots[row_ptr[t] + at] = (int32_t)s;
   }
 }
 
@@ -1113,140 +1236,76 @@ __global__ void inv_sort_kernel(const int32_t* __restrict__ row_ptr, int64_t n, 
   }
 }
 
-// Small inputs (n <= kInvSmallN tokens, at most kInvSmallSlots slots): the whole inverse index in one CTA and one
-// launch.  Counts, cursors and the lists themselves live in shared memory; the order in which atomics hand out places does
-// not matter because every token's list is sorted at the end.  A thread has eight entries of I in flight.
-constexpr int kInvSmallN = 4096, kInvSmallSlots = 1 << 14;
-template <typename F>
-__device__ __forceinline__ void for_slots(const int32_t* I, int first, int total, int step, int n, int* status, F&& f) {
-  for (int s0 = first; s0 < total; s0 += 8 * step) {
-    int t[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) t[u] = s0 + u * step < total ? I[s0 + u * step] : -1;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) if (t[u] >= 0 && !idx_ok(t[u], 0, n, status)) t[u] = -1;       // -1: an empty slot, or none
-    f(t, s0);
-  }
-}
+// Up to kIndexClusterTokens tokens: one cluster of eight CTAs, each an eighth of the tokens in the scan (the eight sums are read from
+// the other CTAs' shared memory) and an eighth of the slots in the fill.
 __global__ void __launch_bounds__(1024)
-inv_small_kernel(const int32_t* __restrict__ I, int n, int total, int32_t* row_ptr, int32_t* slots, int* status) {
-  chain_enter();
-  I = after_enter(I);
-  extern __shared__ int s_cnt[];                       // [n] counts, then cursors; [total] the lists
-  int32_t* s_list = s_cnt + n;
-  __shared__ int s_warp[33];
-  const int tid = threadIdx.x;
-  for (int t = tid; t < n; t += 1024) s_cnt[t] = 0;
-  __syncthreads();
-  for_slots(I, tid, total, 1024, n, status, [&](const int (&t)[8], int) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) if (t[u] >= 0) atomicAdd(&s_cnt[t[u]], 1);
-  });
-  __syncthreads();
-  // exclusive scan over the tokens, 1024 * per at a time
-  const int per = (n + 1023) / 1024, a = min(n, tid * per), b = min(n, a + per);
-  int sum = 0;
-  for (int t = a; t < b; ++t) sum += s_cnt[t];
-  int total_sum;
-  int run = block_exclusive_scan(sum, s_warp, total_sum);
-  for (int t = a; t < b; ++t) { const int c = s_cnt[t]; row_ptr[t] = run; s_cnt[t] = run; run += c; }   // s_cnt becomes the cursor
-  if (tid == 0) row_ptr[n] = total_sum;
-  __syncthreads();
-  for_slots(I, tid, total, 1024, n, nullptr, [&](const int (&t)[8], int s0) {      // bad entries were counted above
-#pragma unroll
-    for (int u = 0; u < 8; ++u) if (t[u] >= 0) s_list[atomicAdd(&s_cnt[t[u]], 1)] = s0 + u * 1024;
-  });
-  __syncthreads();
-  for (int t = tid; t < n; t += 1024) sort_list(s_list, t == 0 ? 0 : s_cnt[t - 1], s_cnt[t]);          // after the fill s_cnt[t] is the end of token t's list
-  __syncthreads();
-  for (int s = tid; s < total_sum; s += 1024) slots[s] = s_list[s];
-}
-
-// Medium inputs (n <= kInvClusterN): one cluster of eight CTAs runs the five steps in one launch, with hardware
-// cluster barriers between them (counts and cursors in global memory, the eight tile sums of the scan read
-// from the other CTAs' shared memory).
-constexpr int kInvClusterN = 16384, kInvClusterSlots = 1 << 17, kInvClusterCtas = 8;
-__device__ __forceinline__ void inv_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__global__ void __launch_bounds__(1024)
-inv_cluster_kernel(const int32_t* __restrict__ I, int n, int total, int32_t* row_ptr, int32_t* slots, int32_t* cnt, int* status) {
+index_cluster_kernel(const int32_t* __restrict__ I, int n, int total, int k_row, const SlotMarks m, int32_t* row_ptr, int32_t* slots, int* status) {
   chain_enter();
   I = after_enter(I);
   __shared__ int s_warp[33];
   __shared__ int s_tile;                               // sum of this CTA's part of the counts
-  const int tid = threadIdx.x, rank = blockIdx.x, nc = gridDim.x;      // the grid is the one cluster
-  const int gtid = rank * 1024 + tid, gsize = nc * 1024;
-  for (int t = gtid; t < n; t += gsize) cnt[t] = 0;
-  inv_cluster_sync();
-  for_slots(I, gtid, total, gsize, n, status, [&](const int (&t)[8], int) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) if (t[u] >= 0) atomicAdd(&cnt[t[u]], 1);
-  });
-  inv_cluster_sync();
-  // exclusive scan: CTA `rank` takes tokens [lo, hi), a thread `per` consecutive ones of them
-  const int per_cta = (n + nc - 1) / nc, lo = min(n, rank * per_cta), hi = min(n, lo + per_cta);
+  const int tid = threadIdx.x, rank = blockIdx.x, W = m.per_token;     // the grid is the one cluster
+  // exclusive scan: CTA `rank` takes tokens [lo, hi), a thread `per` consecutive ones of them (at most two)
+  const int per_cta = (n + 7) / 8, lo = min(n, rank * per_cta), hi = min(n, lo + per_cta);
   const int per = (per_cta + 1023) / 1024, a = min(hi, lo + tid * per), b = min(hi, a + per);
-  int sum = 0;
-  for (int t = a; t < b; ++t) sum += cnt[t];
+  int len[kIndexClusterTokens / 8192], sum = 0;
+#pragma unroll
+  for (int j = 0; j < kIndexClusterTokens / 8192; ++j) {
+    len[j] = 0;
+    if (a + j < b) for (int w = 0; w < W; ++w) len[j] += __popc(m.words[(int64_t)(a + j) * W + w]);
+    sum += len[j];
+  }
   int tile;
   int run = block_exclusive_scan(sum, s_warp, tile);
   if (tid == 0) s_tile = tile;
-  inv_cluster_sync();
+  cluster_barrier();
   int before = 0;
   for (int r = 0; r < rank; ++r) {
-    unsigned remote; int v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"((unsigned)__cvta_generic_to_shared(&s_tile)), "r"(r));
-    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote));
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_address(&s_tile, r)));
     before += v;
   }
   run += before;
-  for (int t = a; t < b; ++t) { const int c = cnt[t]; row_ptr[t] = run; cnt[t] = run; run += c; }      // cnt becomes the cursor
-  if (rank == nc - 1 && tid == 0) row_ptr[n] = before + tile;
-  inv_cluster_sync();
-  for_slots(I, gtid, total, gsize, n, nullptr, [&](const int (&t)[8], int s0) {
-    int at[8];                                         // eight places asked for at once
 #pragma unroll
-    for (int u = 0; u < 8; ++u) at[u] = t[u] >= 0 ? atomicAdd(&cnt[t[u]], 1) : 0;
+  for (int j = 0; j < kIndexClusterTokens / 8192; ++j) if (a + j < b) { row_ptr[a + j] = run; run += len[j]; }
+  if (rank == 7 && tid == 0) row_ptr[n] = before + tile;
+  cluster_barrier();                                   // row_ptr is visible to the cluster, and nobody reads s_tile any more
+  for (int s0 = rank * 1024 + tid; s0 < total; s0 += 8 * 8192) {
+    int t[8], at[8], e[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) if (t[u] >= 0) slots[at[u]] = s0 + u * gsize;
-  });
-  inv_cluster_sync();
-  for (int t = gtid; t < n; t += gsize) sort_list(slots, row_ptr[t], row_ptr[t + 1]);
+    for (int u = 0; u < 8; ++u) {
+      const int s = s0 + u * 8192;
+      t[u] = s < total ? I[s] : -1;                    // -1: an empty slot (token-choice routing only), or none
+      e[u] = s / k_row;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (t[u] >= 0 && !idx_ok(t[u], 0, n, status)) t[u] = -1;
+      at[u] = t[u] >= 0 ? __ldcg(row_ptr + t[u]) : 0;
+    }
+    for (int w = 0; w < W; ++w) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (t[u] >= 0 && w <= e[u] >> 5) {
+          const unsigned bits = m.words[(int64_t)t[u] * W + w];
+          at[u] += __popc(w == e[u] >> 5 ? bits & ((1u << (e[u] & 31)) - 1u) : bits);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) if (t[u] >= 0) slots[at[u]] = s0 + u * 8192;
+  }
 }
 
-cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t total, int32_t* row_ptr, int32_t* slots,
-                                 void* scratch, int* status, cudaStream_t st) {
-  if (n > kInvSmallN && n <= kInvClusterN && total <= kInvClusterSlots) {
-    cudaLaunchConfig_t cfg; memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(kInvClusterCtas); cfg.blockDim = dim3(1024); cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kInvClusterCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_chained()
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 2;
-    count_launch();
-    return cudaLaunchKernelEx(&cfg, inv_cluster_kernel, I, (int)n, (int)total, row_ptr, slots, (int32_t*)scratch, status);
-  }
-  if (n <= kInvSmallN && total <= kInvSmallSlots) {
-    const int smem = (int)(n + total) * 4;
-    constexpr int kMostSmem = (kInvSmallN + kInvSmallSlots) * 4;         // as for topk_small_kernel: 80 KiB, not this call's
-    cudaError_t e0 = cudaFuncSetAttribute(inv_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
-    if (e0 != cudaSuccess) return e0;
-    launch_chained(inv_small_kernel, dim3(1), dim3(1024), smem, st, I, (int)n, (int)total, row_ptr, slots, status);
-    return cudaGetLastError();
-  }
-  int32_t* cnt = (int32_t*)scratch;
+cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t total, int64_t k_row, const IndexPlan& plan, int32_t* row_ptr,
+                                 int32_t* slots, void* scratch, int* status, cudaStream_t st) {
+  if (plan.small)
+    return launch_chained_cluster(8, index_cluster_kernel, dim3(8), dim3(1024), 0, st, I, (int)n, (int)total, (int)k_row, plan.marks, row_ptr, slots, status);
   int32_t* tile_sum = (int32_t*)((char*)scratch + inv_cnt_bytes(n));
   const unsigned tiles = (unsigned)((n + kScanTile - 1) / kScanTile);
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(cnt, 0, (size_t)(n + 1) * 4, st)) != cudaSuccess) return e;
-  launch_chained(inv_count_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, I, total, cnt, n, status);
-  launch_chained(inv_scan_tile_kernel, dim3(tiles), dim3(kScanThreads), 0, st, cnt, n, row_ptr, tile_sum);
+  launch_chained(inv_scan_tile_kernel, dim3(tiles), dim3(kScanThreads), 0, st, plan.marks, n, row_ptr, tile_sum);
   launch_chained(inv_scan_add_kernel, dim3(tiles), dim3(kScanThreads), 0, st, tile_sum, n, row_ptr);
-  launch_chained(inv_fill_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, I, total, row_ptr, cnt, slots, n);
-  launch_chained(inv_sort_kernel, dim3(grid_for(n, 256)), dim3(256), 0, st, row_ptr, n, slots);
+  launch_chained(inv_fill_kernel, dim3(grid_for(total, 256)), dim3(256), 0, st, I, total, k_row, row_ptr, plan.marks, slots, n, status);
+  if (!plan.marks.per_token) launch_chained(inv_sort_kernel, dim3(grid_for(n, 256)), dim3(256), 0, st, row_ptr, n, slots);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,36 @@
+"""The token -> slot index against a stable sort of I: one CTA's limits (16384 tokens, 65536 slots), mark words of 1 to 8 per token,
+the scan beyond them with and without ranks, routing groups, empty slots."""
+import pytest
+import torch
+
+from paper_2202_09368_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,E,c,groups,router", [
+    (256, 4, 2.0, 1, "expert"), (1, 1, 1.0, 1, "expert"), (31, 31, 3.0, 1, "expert"), (2048, 8, 2.0, 1, "expert"), (4096, 32, 2.0, 1, "expert"),
+    (4096, 33, 2.0, 1, "expert"), (16384, 64, 2.0, 1, "expert"), (8192, 256, 8.0, 1, "expert"), (16384, 128, 4.0, 1, "expert"),
+    (8191, 104, 9.0, 1, "expert"), (16385, 32, 2.0, 1, "expert"), (16385, 40, 2.0, 1, "expert"), (20000, 256, 2.0, 1, "expert"),
+    (16384, 4, 2.0, 1, "expert"), (1000, 16, 1.5, 5, "expert"), (1000, 72, 1.5, 16, "expert"), (3000, 16, 1.0, 9, "expert"),
+    (3000, 48, 1.0, 9, "expert"), (4096, 16, 2.0, 1, "token"), (1024, 40, 2.0, 3, "token"), (20000, 16, 2.0, 1, "token"), (9000, 64, 1.0, 2, "token")])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_index_is_a_stable_sort(n, E, c, groups, router, dtype):
+    d, N = 16, n * groups
+    cfg = B.make_config(n, d, 8, E, c, dtype, groups=groups, router=router)
+    gen = torch.Generator(device="cuda").manual_seed(n + E)
+    X = torch.empty((N, d), device="cuda").normal_(generator=gen).to(dtype)
+    Wg = (torch.empty((d, E), device="cuda").normal_(generator=gen) / 4).to(dtype)
+    ws = B.alloc_workspace(cfg)
+    ws.fill_(0xA5)                                      # whatever an earlier call left
+    route = B.ec_route if router == "expert" else B.ec_route_token_choice
+    for _ in range(2):
+        r = route(cfg, X, Wg, ws=ws)
+        assert B.ec_read_status(ws) == B.EC_OK
+        I = r.I.flatten().long()
+        filled = (I >= 0).nonzero().flatten()
+        order = torch.sort(I[filled], stable=True)[1]
+        lengths = torch.bincount(I[filled], minlength=N)
+        assert torch.equal(r.row_ptr.long(), torch.cat([lengths.new_zeros(1), lengths.cumsum(0)]))
+        assert torch.equal(r.slots.flatten()[:filled.numel()].long(), filled[order])
+        assert B.ec_validate_routing(cfg, r.I, r.row_ptr, r.slots, ws) == 0
