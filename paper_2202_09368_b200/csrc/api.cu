@@ -454,11 +454,33 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
   void* dL = w + W.dL; float* part = (float*)(w + W.dWg_part);
   int* status = (int*)(w + W.status);
   const int32_t* rag = D.router && D.groups == 1 ? (const int32_t*)(sv + L.load) : nullptr;   // see ec_moe_forward
-  EC_CUDA(cudaMemsetAsync(ws, 0, sizeof(StatusWord), st));
   const int64_t kd = D.k * D.d, kf = D.k * D.dff, df = (int64_t)D.d * D.dff;
-  // Eq. 4 backward: dX_e, dG
+  // the two gate-gradient products; on tensor cores dL [n, E] is bf16
+  const int P = dwg_splits(D);
+  TcGemmArgs tw; memset(&tw, 0, sizeof(tw));          // dWg = X^T . dL, cut along the tokens
+  const int64_t cut = (((D.n + P - 1) / P) + 63) / 64 * 64;
+  tw.A = X; tw.a_mn_major = 1; tw.lda = D.d; tw.B = dL; tw.b_mn_major = 1; tw.ldb = D.E;
+  tw.M = D.d; tw.N = D.E; tw.K = (int)cut; tw.batches = P; tw.k_split = 1; tw.k_total = D.n;
+  tw.epi = EPI_STORE; tw.c_f32 = 1; tw.C = part; tw.ldc = D.E; tw.batch_c = (int64_t)D.d * D.E; tw.status = status;
+  TcGemmArgs tx; memset(&tx, 0, sizeof(tx));          // dX = dL . Wg^T + rows of dX_in
+  tx.A = dL; tx.a_mn_major = 0; tx.lda = D.E; tx.B = Wg; tx.b_mn_major = 0; tx.ldb = D.E;
+  tx.M = (int)D.n; tx.N = D.d; tx.K = D.E; tx.batches = 1;
+  tx.epi = EPI_ADD_SLOTS; tx.C = dX; tx.ldc = D.d; tx.status = status;
+  tx.row_ptr = row_ptr; tx.slots = slots; tx.rows = dX_in; tx.ld_rows = D.d; tx.slots_total = D.slots;
+  const bool tc_gate = D.dtype == EC_BF16 && tc_gemm_supported(tw) && tc_gemm_supported(tx);     // mirrored by gate_grads_on_tc()
+  // Eq. 4 backward: dX_e, dG; then the softmax's: dL.  In the debug build, whose kernels may record a bad index in the status
+  // block as soon as they start, it is cleared before, else by this first kernel; and a slot that a bad list leaves out has zeros.
+#ifdef EC_DEBUG
+  EC_CUDA(cudaMemsetAsync(ws, 0, sizeof(StatusWord), st));
+  EC_CUDA(cudaMemsetAsync(dX_e, 0, (size_t)D.slots * D.d * D.eb, st));
+  EC_CUDA(cudaMemsetAsync(dG, 0, (size_t)D.slots * 4, st));
+  const int clear = 0;
+#else
+  const int clear = 1;
+#endif
   prof_begin(st, 1);
-  EC_CUDA(launch_bwd_combine(D.dtype, dX_out, X_e, G, I, dX_e, dG, D.slots, D.d, D.n, status, st));
+  EC_CUDA(launch_bwd_tokens(D.dtype, dX_out, X_e, G, S, row_ptr, slots, D.router ? I : nullptr, dX_e, dG, dL, tc_gate ? 1 : 0, D.n, D.d, D.E, D.k, clear,
+                            status, st));
   prof_mark("bwd_combine", st);
   // dZ = (dX_e[i] . W2[i]) * GeLU'(Z)
   BatchedGemm g3 = {dX_e, 0, D.d, kd, W2, 1, D.dff, df, dZ, D.dff, kf, (int)D.k, D.dff, D.d, D.E, EPI_GELU_GRAD, nullptr, Z, 0, rag, 1, nullptr};
@@ -482,21 +504,6 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
   BatchedGemm g6 = {dZ, 0, D.dff, kf, W1, 0, D.dff, df, dX_in, D.d, kd, (int)D.k, D.d, D.dff, D.E, EPI_STORE, nullptr, nullptr, 0, rag, 1, nullptr};
   if ((s = run_gemm(D, g6, status, st)) != EC_OK) return s;
   prof_mark("gemm_dXin", st);
-  // softmax backward: dL [n, E]; bf16 when the two gate-gradient products below run on tensor cores
-  const int P = dwg_splits(D);
-  TcGemmArgs tw; memset(&tw, 0, sizeof(tw));          // dWg = X^T . dL, cut along the tokens
-  const int64_t cut = (((D.n + P - 1) / P) + 63) / 64 * 64;
-  tw.A = X; tw.a_mn_major = 1; tw.lda = D.d; tw.B = dL; tw.b_mn_major = 1; tw.ldb = D.E;
-  tw.M = D.d; tw.N = D.E; tw.K = (int)cut; tw.batches = P; tw.k_split = 1; tw.k_total = D.n;
-  tw.epi = EPI_STORE; tw.c_f32 = 1; tw.C = part; tw.ldc = D.E; tw.batch_c = (int64_t)D.d * D.E; tw.status = status;
-  TcGemmArgs tx; memset(&tx, 0, sizeof(tx));          // dX = dL . Wg^T + rows of dX_in
-  tx.A = dL; tx.a_mn_major = 0; tx.lda = D.E; tx.B = Wg; tx.b_mn_major = 0; tx.ldb = D.E;
-  tx.M = (int)D.n; tx.N = D.d; tx.K = D.E; tx.batches = 1;
-  tx.epi = EPI_ADD_SLOTS; tx.C = dX; tx.ldc = D.d; tx.status = status;
-  tx.row_ptr = row_ptr; tx.slots = slots; tx.rows = dX_in; tx.ld_rows = D.d; tx.slots_total = D.slots;
-  const bool tc_gate = D.dtype == EC_BF16 && tc_gemm_supported(tw) && tc_gemm_supported(tx);     // mirrored by gate_grads_on_tc()
-  EC_CUDA(launch_bwd_softmax(S, dG, row_ptr, slots, dL, tc_gate ? 1 : 0, D.n, D.E, D.k, status, st));
-  prof_mark("bwd_softmax", st);
   if (tc_gate) {
     EC_CUDA(launch_gemm_tc(tw, st));
     EC_CUDA(launch_reduce_partials(D.dtype, part, dWg, P, (int64_t)D.d * D.E, st));

@@ -134,15 +134,12 @@ cudaError_t launch_combine(int dtype, const float* X_e, const float* G, const in
 cudaError_t launch_validate_routing(const int32_t* I, const int32_t* row_ptr, const int32_t* slots, int64_t n, int64_t ng,
                                     int E, int64_t k_total, int64_t kg, int groups, int allow_empty, int* violations,
                                     cudaStream_t st);
-// dX_e[s,:] = G[s] * dX_out[I[s],:],  dG[s] = <dX_out[I[s],:], X_e[s,:]>
-cudaError_t launch_bwd_combine(int dtype, const void* dX_out, const float* X_e, const float* G,
-                               const int32_t* I, void* dX_e, float* dG, int64_t slots_total, int d, int64_t n,
-                               int* status, cudaStream_t st);
-// dL[t,i] = S[t,i] * (dS[t,i] - sum_i' dS[t,i'] S[t,i']),  dS scattered from dG through the inverse index;
-// dL is stored as bf16 when dl_bf16 (operand of the tensor-core dWg / dX products), else fp32
-cudaError_t launch_bwd_softmax(const float* S, const float* dG, const int32_t* row_ptr,
-                               const int32_t* slots, void* dL, int dl_bf16, int64_t n, int E, int64_t k,
-                               int* status, cudaStream_t st);
+// dX_e[s,:] = G[s] * dX_out[t,:] and dG[s] = <dX_out[t,:], X_e[s,:]> for the slots s of every token t; then
+// dL[t,i] = S[t,i] * (dS[t,i] - sum_i' dS[t,i'] S[t,i']) with dS = dG at the token's slots, stored as bf16 when dl_bf16 (operand of
+// the tensor-core dWg / dX products), else fp32.  empty: I where slots may be empty, else null.  clear: the status block starts at zero.
+cudaError_t launch_bwd_tokens(int dtype, const void* dX_out, const float* X_e, const float* G, const float* S, const int32_t* row_ptr, const int32_t* slots,
+                              const int32_t* empty, void* dX_e, float* dG, void* dL, int dl_bf16, int64_t n, int d, int E, int64_t k, int clear, int* status,
+                              cudaStream_t st);
 // out[b, c] = sum over the rows r < min(rows, batch_rows[b]) of A[b, r, c], fp32, cast to dtype; in a fixed order: eight chains
 // (the rows with r mod 8 = 0, 1, ..., each in ascending r), joined in that order
 // (gradients of the bias terms: column sums of dZ and dX_e per expert); batch_rows may be null
