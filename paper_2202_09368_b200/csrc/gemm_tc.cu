@@ -66,10 +66,13 @@ constexpr int kWideMinK = 2048;                      // contraction length from 
 // bn = rows of B one CTA loads per k-block (BN / CTAS)
 __host__ __device__ constexpr int stage_bytes(int bn) { return kABytes + bn * BK * 2; }
 // Staging for the epilogue: every warp's when the tile is split between the warp pairs, else (a 64-wide tile with
-// the softmax, drained by the first four warps alone) only theirs, which leaves room for more stages.
-__host__ __device__ constexpr int staging_bytes(int bn_tile, int epi) { return (epi == EPI_SOFTMAX && bn_tile < 128 ? 4 : kEpiWarps) * kStagingPerWarp; }
+// the softmax, drained by the first four warps alone) only theirs, which leaves room for more stages.  A turned product has none.
+__host__ __device__ constexpr int staging_bytes(int bn_tile, int epi, bool turned) {
+  return turned ? 0 : (epi == EPI_SOFTMAX && bn_tile < 128 ? 4 : kEpiWarps) * kStagingPerWarp;
+}
 __host__ __device__ constexpr int num_stages(int bn, int staging) {
-  return (kSmemBudget - staging) / stage_bytes(bn) > 8 ? 8 : (kSmemBudget - staging) / stage_bytes(bn);
+  const int fit = (kSmemBudget - staging) / stage_bytes(bn), most = staging == 0 ? 12 : 8;
+  return fit > most ? most : fit;
 }
 // Two accumulators of BN columns (a power of two for BN = 64, 128, 256), or one of 512.  A CTA pair takes all 512
 // columns, so both CTAs are certain to get base address 0: one tcgen05.mma writes the same
@@ -83,6 +86,7 @@ struct TcParams {
   int n_fast;                                        // consecutive tiles run along N (else along M)
   int gelu;
   int64_t ldc, batch_c;
+  void* c; void* c2; const bf16* zin;                // turned products, which store without the TMA unit
   int* status;
   int k_split;                                       // batches are cuts of one product along K
   unsigned* clear; int clear_words;                  // EPI_SOFTMAX: words per row to zero
@@ -173,7 +177,7 @@ __device__ __forceinline__ int tile_kblocks(const TcParams& p, int b, int mt, in
 // ---------------------------------------------------------------------------------------------
 // The kernel
 // ---------------------------------------------------------------------------------------------
-template <int BN, int EPI, int CTAS>
+template <int BN, int EPI, int CTAS, bool TURNED>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmC2, const TcParams p) {
@@ -184,7 +188,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   static_assert(BN <= 256 || CTAS == 2, "512-wide tiles are for CTA pairs");
   constexpr int TM = BM * CTAS;                     // rows of the tile the CTA (pair) works on
   constexpr bool kXchg = EPI == EPI_SOFTMAX && BN >= 128;            // the softmax epilogue's exchange area replaces a stage
-  constexpr int kStaging = staging_bytes(BN, EPI);
+  static_assert(!TURNED || (CTAS == 1 && BN <= 64 && EPI != EPI_SOFTMAX && EPI != EPI_ADD_SLOTS), "turned: one CTA, all tokens in one tile");
+  constexpr int kStaging = staging_bytes(BN, EPI, TURNED);
   constexpr int S = num_stages(BNL, kStaging) - (kXchg ? 1 : 0);
   constexpr int kBBytes = BNL * BK * 2;
   constexpr int kStage = kABytes + kBBytes;
@@ -209,15 +214,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       int* published = (int*)(smem + S * kStage + kStaging + 256 + 2 * kEpiWarps * 32 * 8);
       for (int w = 0; w < kEpiWarps; ++w) published[w] = 0;
     }
-    if constexpr (EPI == EPI_GELU_GRAD) {
+    if constexpr (EPI == EPI_GELU_GRAD && !TURNED) {
       const uint32_t z0 = smem_u32(smem + S * kStage + kStaging + 256);
       for (int i = 0; i < 2 * kEpiWarps; ++i) mbar_init(z0 + 8 * i, 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x == 32 * 2) {                       // the descriptors are on their way while the previous kernel drains
-    prefetch_map(&tmA); prefetch_map(&tmB); prefetch_map(&tmC);
-    if constexpr (EPI == EPI_GELU || EPI == EPI_GELU_GRAD) prefetch_map(&tmC2);
+    prefetch_map(&tmA); prefetch_map(&tmB);
+    if constexpr (!TURNED) prefetch_map(&tmC);
+    if constexpr (!TURNED && (EPI == EPI_GELU || EPI == EPI_GELU_GRAD)) prefetch_map(&tmC2);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
@@ -402,6 +408,74 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           if constexpr (CTAS == 2) tc_commit_pair(tfull0 + 8 * buf); else tc_commit(tfull0 + 8 * buf);
         }
       }
+    }
+  } else if constexpr (TURNED) {
+    // ------------------------------------------------------------------ epilogue of a turned product
+    // A lane of tensor memory is a column of the result (one of the weights' 128), a column of it a token: a warp holds 32
+    // neighbouring columns of a token's row and stores them as they are, 128 or 64 bytes at a time.
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    constexpr int kTokens = BN / 2, kChunk = 16;     // of a warp; at a time
+    int it = 0;
+    for (int tile = first_tile; tile < p.total_tiles; tile += tile_step, ++it) {
+      const int b = tile / (p.tiles_m * p.tiles_n);
+      const int mt = p.n_fast ? (tile / p.tiles_n) % p.tiles_m : tile % p.tiles_m;
+      const int buf = it & 1; const uint32_t use = (uint32_t)(it >> 1);
+      const int col = mt * TM + q * 32 + lane;
+      float bias = 0.f;
+      if constexpr (EPI == EPI_GELU || EPI == EPI_STORE_F32)
+        if (p.bias != nullptr && col < p.M) bias = __bfloat162float(__ldg(after_enter(p.bias) + (int64_t)b * p.M + col));
+      const bool ok = mbar_wait(tfull0 + 8 * buf, use & 1, abort_flag, p.status, 4);
+      if (!__all_sync(0xffffffffu, ok)) { gave_up = true; break; }
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + buf * BN + half * kTokens;
+      const int64_t out0 = (int64_t)b * p.batch_c + col;
+#pragma unroll 1
+      for (int c = 0; c < kTokens && half * kTokens + c < p.N; c += kChunk) {       // uniform across the warp
+        uint32_t r[kChunk]; tc_ld16(taddr + c, r);
+        const int t0 = half * kTokens + c;
+        auto inside = [&](int j) { return col < p.M && t0 + j < p.N; };
+        auto at = [&](int j) { return out0 + (int64_t)(t0 + j) * p.ldc; };
+        if constexpr (EPI == EPI_STORE_F32) {
+#pragma unroll
+          for (int j = 0; j < kChunk; ++j) if (inside(j)) ((float*)p.c)[at(j)] = __uint_as_float(r[j]) + bias;
+        } else if constexpr (EPI == EPI_STORE) {
+#pragma unroll
+          for (int j = 0; j < kChunk; ++j) if (inside(j)) ((bf16*)p.c)[at(j)] = __float2bfloat16(__uint_as_float(r[j]));
+        } else if constexpr (EPI == EPI_GELU) {
+          auto convert = [&](auto variant) {
+#pragma unroll
+            for (int j = 0; j < kChunk; j += 2) {
+              const float z0 = __uint_as_float(r[j]) + bias, z1 = __uint_as_float(r[j + 1]) + bias;
+              float h0, h1;
+              gelu_fwd2<decltype(variant)::value>(z0, z1, h0, h1);
+              if (!p.skip_c) {
+                if (inside(j)) ((bf16*)p.c)[at(j)] = __float2bfloat16(z0);
+                if (inside(j + 1)) ((bf16*)p.c)[at(j + 1)] = __float2bfloat16(z1);
+              }
+              if (inside(j)) ((bf16*)p.c2)[at(j)] = __float2bfloat16(h0);
+              if (inside(j + 1)) ((bf16*)p.c2)[at(j + 1)] = __float2bfloat16(h1);
+            }
+          };
+          if (p.gelu == 0) convert(std::integral_constant<int, 0>{}); else convert(std::integral_constant<int, 1>{});
+        } else {
+          bf16 z[kChunk];
+#pragma unroll
+          for (int j = 0; j < kChunk; ++j) z[j] = inside(j) ? p.zin[at(j)] : __float2bfloat16(0.f);
+          auto scale = [&](auto variant) {
+#pragma unroll
+            for (int j = 0; j < kChunk; j += 2) {
+              float g0, g1;
+              gelu_bwd2<decltype(variant)::value>(__bfloat162float(z[j]), __bfloat162float(z[j + 1]), g0, g1);
+              if (inside(j)) ((bf16*)p.c)[at(j)] = __float2bfloat16(__uint_as_float(r[j]) * g0);
+              if (inside(j + 1)) ((bf16*)p.c)[at(j + 1)] = __float2bfloat16(__uint_as_float(r[j + 1]) * g1);
+            }
+          };
+          if (p.gelu == 0) scale(std::integral_constant<int, 0>{}); else scale(std::integral_constant<int, 1>{});
+        }
+      }
+      tc_fence_before();
+      __syncwarp();                                  // every lane's tcgen05.ld has completed
+      if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
     }
   } else {
     // ------------------------------------------------------------------ epilogue, one tile row per thread
@@ -848,13 +922,14 @@ int pick_bn(const TcGemmArgs& g, int pairs) {
 // Two CTAs per tile when a tile of 256 rows is not mostly padding and the pair's B halves are whole 64-wide blocks.
 int pick_ctas(const TcGemmArgs& g, int bn) { return (bn >= 128 && g.M > BM) ? 2 : 1; }
 
-template <int BN, int EPI, int CTAS>
+template <int BN, int EPI, int CTAS, bool TURNED = false>
 cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, const CUtensorMap& tc2,
                        const TcParams& p, cudaStream_t st) {
   // the split softmax trades one operand stage for its exchange area (4 KiB + counters), see the kernel
-  constexpr int smem = num_stages(BN / CTAS, staging_bytes(BN, EPI)) * stage_bytes(BN / CTAS) + staging_bytes(BN, EPI) + 1024 + 256 +
-                       (EPI == EPI_GELU_GRAD ? 2 * kEpiWarps * 8 : 0);            // the barriers of Z
-  auto kern = gemm_tc_kernel<BN, EPI, CTAS>;
+  constexpr int staging = staging_bytes(BN, EPI, TURNED);
+  constexpr int smem = num_stages(BN / CTAS, staging) * stage_bytes(BN / CTAS) + staging + 1024 + 256 +
+                       (EPI == EPI_GELU_GRAD && !TURNED ? 2 * kEpiWarps * 8 : 0);            // the barriers of Z
+  auto kern = gemm_tc_kernel<BN, EPI, CTAS, TURNED>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 148;
@@ -891,6 +966,11 @@ cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tb, const CUten
 }
 
 template <int EPI>
+cudaError_t launch_turned(int bn, const CUtensorMap& ta, const CUtensorMap& tb, const TcParams& p, cudaStream_t st) {
+  return bn == 32 ? launch_one<32, EPI, 1, true>(ta, tb, ta, ta, p, st) : launch_one<64, EPI, 1, true>(ta, tb, ta, ta, p, st);
+}
+
+template <int EPI>
 cudaError_t launch_bn(int bn, int ctas, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, const CUtensorMap& tc2,
                       const TcParams& p, cudaStream_t st) {
   {
@@ -902,9 +982,11 @@ cudaError_t launch_bn(int bn, int ctas, const CUtensorMap& ta, const CUtensorMap
       return launch_one<128, EPI, 2>(ta, tb, tc, tc2, p, st);
     }
   }
-  if (bn == 256) return launch_one<256, EPI, 1>(ta, tb, tc, tc2, p, st);
+  if constexpr (EPI == EPI_SOFTMAX) {
+    if (bn == 256) return launch_one<256, EPI, 1>(ta, tb, tc, tc2, p, st);
+  }
   if (bn == 128) return launch_one<128, EPI, 1>(ta, tb, tc, tc2, p, st);
-  return launch_one<64, EPI, 1>(ta, tb, tc, tc2, p, st);
+  return bn == 64 ? launch_one<64, EPI, 1>(ta, tb, tc, tc2, p, st) : cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -925,12 +1007,44 @@ bool tc_gemm_supported(const TcGemmArgs& g) {
   return true;
 }
 
+// Few rows per expert (M <= 64): the product streams the weights, and a tile of 128 rows is mostly fill.  Turned, the weights'
+// columns are the 128 rows of the MMA and the tokens its 32 or 64 columns: no multiply-adds on fill, whose energy the 1000 W
+// cap turns into time (32 rows, 64 experts of 4096 x 16384: 1690 and 1560 us a product, 5.3 TB/s of weights, turned 1350 and
+// 1285, 6.7 TB/s; the same on a cold GPU, 1340), and 9 or 11 stages of weights on their way instead of five (64 rows, 64 experts of
+// 768 x 3072: the forward pass 171 -> 165 us).  Beyond 64 rows the fill saved is less than what stores without the TMA unit cost (80
+// rows, 48 experts of 1136 x 2304: a step of 509 us takes 525).
+static bool turns(const TcGemmArgs& g) {
+  return g.M <= 64 && !g.a_mn_major && !g.a_rows && !g.k_split && (!g.batch_rows || g.ragged == 1) &&
+         (g.epi == EPI_STORE || g.epi == EPI_GELU || g.epi == EPI_GELU_GRAD);
+}
+
+cudaError_t launch_gemm_turned(const TcGemmArgs& g, cudaStream_t st) {
+  const int bn = g.M <= 32 ? 32 : 64;
+  CUtensorMap ta, tb;
+  const bool oka = g.b_mn_major ? make_map(&ta, g.B, g.N, g.K, g.batches, g.ldb, g.batch_b, 64, BK)
+                                : make_map(&ta, g.B, g.K, g.N, g.batches, g.ldb, g.batch_b, BK, BM);
+  if (!oka || !make_map(&tb, g.A, g.K, g.M, g.batches, g.lda, g.batch_a, BK, bn)) return cudaErrorInvalidValue;
+  TcParams p; memset(&p, 0, sizeof(p));
+  p.M = g.N; p.N = g.M; p.K = g.K; p.batches = g.batches; p.a_mn = g.b_mn_major; p.b_mn = 0;
+  p.tiles_m = (g.N + BM - 1) / BM; p.tiles_n = 1;
+  p.total_tiles = p.tiles_m * g.batches; p.kblocks = (g.K + BK - 1) / BK;
+  p.gelu = g.gelu; p.ldc = g.ldc; p.batch_c = g.batch_c; p.status = g.status; p.bias = (const bf16*)g.bias;
+  p.c = g.C; p.c2 = g.C2; p.zin = (const bf16*)g.Zin; p.skip_c = (g.epi == EPI_GELU && !g.C) ? 1 : 0;
+  switch (g.epi) {
+    case EPI_STORE: return g.c_f32 ? launch_turned<EPI_STORE_F32>(bn, ta, tb, p, st) : launch_turned<EPI_STORE>(bn, ta, tb, p, st);
+    case EPI_GELU: return launch_turned<EPI_GELU>(bn, ta, tb, p, st);
+    case EPI_GELU_GRAD: return launch_turned<EPI_GELU_GRAD>(bn, ta, tb, p, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
 cudaError_t launch_gemm_tc(const TcGemmArgs& g, cudaStream_t st) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const cudaError_t bound = bind_context(dev);
   if (bound != cudaSuccess) return bound;
+  if (turns(g)) return launch_gemm_turned(g, st);
   const int bn = pick_bn(g, sms / 2);
   const int ctas = pick_ctas(g, bn);
   const int bnl = bn / ctas;                         // rows of B one CTA loads
@@ -957,7 +1071,7 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& g, cudaStream_t st) {
     if (g.epi == EPI_GELU_GRAD && !make_map(&tc2, g.Zin, g.N, g.M, g.batches, g.ldc, g.batch_c, 64, 32)) return cudaErrorInvalidValue;
     if (g.epi == EPI_GELU && !make_map(&tc2, g.C2, g.N, g.M, g.batches, g.ldc, g.batch_c, 64, 32)) return cudaErrorInvalidValue;
   }
-  TcParams p;
+  TcParams p; memset(&p, 0, sizeof(p));
   p.M = g.M; p.N = g.N; p.K = g.K; p.batches = g.batches; p.a_mn = g.a_mn_major; p.b_mn = g.b_mn_major;
   p.tiles_m = (g.M + BM * ctas - 1) / (BM * ctas); p.tiles_n = (g.N + bn - 1) / bn;
   p.total_tiles = p.tiles_m * p.tiles_n * g.batches; p.kblocks = (g.K + BK - 1) / BK;
