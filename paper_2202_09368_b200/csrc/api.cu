@@ -156,6 +156,7 @@ struct BatchedGemm {
   // A's stored rows are rows of the matrix at A (a_rows_total rows, pitch lda) picked through a_rows (Eq. 3's
   // X_in = P . X read in place): row r of batch b is matrix row a_rows[b * a_rows_batch + r]
   const int32_t* a_rows; int64_t a_rows_batch, a_rows_total;
+  int early;                                         // see chain_enter()
 };
 
 ec_status run_gemm(const Dims& D, const BatchedGemm& b, int* status_word, cudaStream_t st) {
@@ -167,7 +168,7 @@ ec_status run_gemm(const Dims& D, const BatchedGemm& b, int* status_word, cudaSt
     t.epi = b.epi; t.gelu = D.gelu; t.C = b.C; t.C2 = b.C2; t.Zin = b.Zin; t.ldc = b.ldc; t.batch_c = b.batch_c; t.c_f32 = b.c_f32;
     t.status = status_word;
     t.batch_rows = b.batch_rows; t.ragged = b.ragged; t.bias = b.bias;
-    t.a_rows = b.a_rows; t.a_rows_batch = b.a_rows_batch; t.a_rows_total = b.a_rows_total;
+    t.a_rows = b.a_rows; t.a_rows_batch = b.a_rows_batch; t.a_rows_total = b.a_rows_total; t.early = b.early;
     if (tc_gemm_supported(t)) { EC_CUDA(launch_gemm_tc(t, st)); return EC_OK; }
   }
   GemmArgs g; memset(&g, 0, sizeof(g));
@@ -180,7 +181,7 @@ ec_status run_gemm(const Dims& D, const BatchedGemm& b, int* status_word, cudaSt
   g.epi = b.epi; g.gelu = D.gelu; g.C2 = b.C2; g.Zin = b.Zin;
   g.bias = b.bias; g.bias_dtype = D.dtype;
   g.a_rows = b.a_rows; g.a_rows_batch = b.a_rows_batch; g.a_rows_total = b.a_rows_total; g.a_rows_k = b.a_mn;   // the stored rows of A run along K when it is MN-major
-  g.status = status_word;
+  g.status = status_word; g.early = b.early;
   EC_CUDA(launch_gemm_simt(g, st));
   return EC_OK;
 }
@@ -461,11 +462,11 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
   const int64_t cut = (((D.n + P - 1) / P) + 63) / 64 * 64;
   tw.A = X; tw.a_mn_major = 1; tw.lda = D.d; tw.B = dL; tw.b_mn_major = 1; tw.ldb = D.E;
   tw.M = D.d; tw.N = D.E; tw.K = (int)cut; tw.batches = P; tw.k_split = 1; tw.k_total = D.n;
-  tw.epi = EPI_STORE; tw.c_f32 = 1; tw.C = part; tw.ldc = D.E; tw.batch_c = (int64_t)D.d * D.E; tw.status = status;
+  tw.epi = EPI_STORE; tw.c_f32 = 1; tw.C = part; tw.ldc = D.E; tw.batch_c = (int64_t)D.d * D.E; tw.status = status; tw.early = 1;
   TcGemmArgs tx; memset(&tx, 0, sizeof(tx));          // dX = dL . Wg^T + rows of dX_in
   tx.A = dL; tx.a_mn_major = 0; tx.lda = D.E; tx.B = Wg; tx.b_mn_major = 0; tx.ldb = D.E;
   tx.M = (int)D.n; tx.N = D.d; tx.K = D.E; tx.batches = 1;
-  tx.epi = EPI_ADD_SLOTS; tx.C = dX; tx.ldc = D.d; tx.status = status;
+  tx.epi = EPI_ADD_SLOTS; tx.C = dX; tx.ldc = D.d; tx.status = status; tx.early = 1;
   tx.row_ptr = row_ptr; tx.slots = slots; tx.rows = dX_in; tx.ld_rows = D.d; tx.slots_total = D.slots;
   const bool tc_gate = D.dtype == EC_BF16 && tc_gemm_supported(tw) && tc_gemm_supported(tx);     // mirrored by gate_grads_on_tc()
   // Eq. 4 backward: dX_e, dG; then the softmax's: dL.  In the debug build, whose kernels may record a bad index in the status
@@ -491,8 +492,10 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
     if (db2) EC_CUDA(launch_column_sums(D.dtype, dX_e, db2, D.E, D.k, D.d, rag, st));
     prof_mark("bias_grads", st);
   }
-  // dW2[i] = dX_e[i]^T . H[i]
+  // dW2[i] = dX_e[i]^T . H[i].  Early (see chain_enter(); here and below): what it reads is older than the last kernel that waits, as
+  // it is for dX_in and dWg behind dW1, which does, and for dX behind the sum of the partials
   BatchedGemm g4 = {dX_e, 1, D.d, kd, H, 1, D.dff, kf, dW2, D.dff, df, D.d, D.dff, (int)D.k, D.E, EPI_STORE, nullptr, nullptr, 0, rag, 2, nullptr};
+  g4.early = 1;
   if ((s = run_gemm(D, g4, status, st)) != EC_OK) return s;
   prof_mark("gemm_dW2", st);
   // dW1[i] = X_in[i]^T . dZ[i]
@@ -502,6 +505,7 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
   prof_mark("gemm_dW1", st);
   // dX_in[i] = dZ[i] . W1[i]^T
   BatchedGemm g6 = {dZ, 0, D.dff, kf, W1, 0, D.dff, df, dX_in, D.d, kd, (int)D.k, D.d, D.dff, D.E, EPI_STORE, nullptr, nullptr, 0, rag, 1, nullptr};
+  g6.early = 1;
   if ((s = run_gemm(D, g6, status, st)) != EC_OK) return s;
   prof_mark("gemm_dXin", st);
   if (tc_gate) {
@@ -520,7 +524,7 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
     g.M = D.d; g.N = D.E; g.K = (int)chunk; g.batches = P; g.k_limit = D.n;
     g.sam = 1; g.sak = D.d; g.sbk = D.E; g.sbn = 1; g.ldc = D.E;
     g.batch_a = chunk * D.d; g.batch_b = chunk * D.E; g.batch_c = (int64_t)D.d * D.E;
-    g.epi = EPI_STORE;
+    g.epi = EPI_STORE; g.early = 1;
     EC_CUDA(launch_gemm_simt(g, st));
     EC_CUDA(launch_reduce_partials(D.dtype, part, dWg, P, (int64_t)D.d * D.E, st));
     prof_mark("dWg", st);
@@ -532,7 +536,7 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
     g.M = (int)D.n; g.N = D.d; g.K = D.E; g.batches = 1;
     g.sam = D.E; g.sak = 1; g.sbk = 1; g.sbn = D.E; g.ldc = D.d;
     g.epi = EPI_ADD_SLOTS; g.row_ptr = row_ptr; g.slots = slots; g.rows = dX_in; g.ld_rows = D.d;
-    g.slots_total = D.slots; g.status = status;
+    g.slots_total = D.slots; g.status = status; g.early = 1;
     EC_CUDA(launch_gemm_simt(g, st));
     prof_mark("dX", st);
   }

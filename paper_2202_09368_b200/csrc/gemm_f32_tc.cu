@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) gemm_f32_tc_kernel(const __gri
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  chain_enter();
+  chain_enter(g.early);
   const uint32_t tmem_base = *tmem_slot;
   const int kblocks = (g.K + FK - 1) / FK;
   auto place = [&](int tile, int& b, int& m0, int& n0) {               // row tiles fastest: CTAs that run together share columns of B
@@ -297,6 +297,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) gemm_f32_tc_kernel(const __gri
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
   }
+  chain_leave(g.early);
 }
 
 template <int EPI, int FN, bool A_K, bool B_K, bool LIST>

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kern
   static_assert(TX % 8 == 0 && TM % 4 == 0 && TN % 4 == 0, "a warp covers 4 x 8 threads");
   using LA = TileLoader<TA, BM, BK, NT, VEC>;
   using LB = TileLoader<TB, BN, BK, NT, VEC>;
-  chain_enter();
+  chain_enter(g.early);
   constexpr int kBuf = BK * (BM + BN);                // one k-tile of both operands
   extern __shared__ __align__(16) float simt_smem[];  // [KS groups][2 buffers][A | B]; after the main loop the other groups' sums
   const int b = blockIdx.z, grp = threadIdx.x / NT;
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kern
       }
       __syncthreads();
     }
-    if (grp != 0) return;
+    if (grp != 0) { chain_leave(g.early); return; }
   }
   TC* C = g.C ? (TC*)g.C + (int64_t)b * g.batch_c : nullptr;
   // EPI_ADD_SLOTS: the lists of a thread's four rows are walked side by side, so that four rows of `rows` are in flight
@@ -324,6 +324,7 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN) * KS, MINB) gemm_simt_kern
       }
     }
   }
+  chain_leave(g.early);
 }
 
 // Column tiles sit on grid.y.  64 columns cover every width the layer takes (2^22 - 64), 32 columns the widths below 2 097 121.

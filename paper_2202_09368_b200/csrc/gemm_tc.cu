@@ -94,6 +94,7 @@ struct TcParams {
   const int32_t* row_ptr; const int32_t* slots; const bf16* rows; int64_t ld_rows;   // EPI_ADD_SLOTS
   int64_t slots_total;                               // rows of `rows`: what the debug build checks the slot ids against
   const int32_t* batch_rows; int ragged;             // meaningful rows per batch along M (1) or K (2), zeros beyond
+  int early;                                         // see chain_enter()
   const bf16* bias;                                  // EPI_GELU, EPI_STORE_F32: bias[b * N + n] joins every row of the accumulator
   const int32_t* a_rows; int64_t a_rows_batch; int a_rows_total;   // A's stored rows come from one matrix through this index list (tmA is then 2-D)
 };
@@ -233,7 +234,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   __syncthreads();
   if constexpr (CTAS == 2) cluster_sync_all();     // the peer's barriers exist before anything is sent to them
   tc_fence_after();
-  chain_enter();                                   // the barriers and tensor memory above are set up while the previous kernel drains
+  chain_enter(p.early);                            // the barriers and tensor memory above are set up while the previous kernel drains
   const uint32_t tmem_base = *tmem_slot;
   const uint32_t smem_base = smem_u32(smem);
   bool gave_up = false;
@@ -844,6 +845,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kCols) : "memory");
   }
+  chain_leave(p.early);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1028,7 +1030,7 @@ cudaError_t launch_gemm_turned(const TcGemmArgs& g, cudaStream_t st) {
   p.M = g.N; p.N = g.M; p.K = g.K; p.batches = g.batches; p.a_mn = g.b_mn_major; p.b_mn = 0;
   p.tiles_m = (g.N + BM - 1) / BM; p.tiles_n = 1;
   p.total_tiles = p.tiles_m * g.batches; p.kblocks = (g.K + BK - 1) / BK;
-  p.gelu = g.gelu; p.ldc = g.ldc; p.batch_c = g.batch_c; p.status = g.status; p.bias = (const bf16*)g.bias;
+  p.gelu = g.gelu; p.ldc = g.ldc; p.batch_c = g.batch_c; p.status = g.status; p.bias = (const bf16*)g.bias; p.early = g.early;
   p.c = g.C; p.c2 = g.C2; p.zin = (const bf16*)g.Zin; p.skip_c = (g.epi == EPI_GELU && !g.C) ? 1 : 0;
   switch (g.epi) {
     case EPI_STORE: return g.c_f32 ? launch_turned<EPI_STORE_F32>(bn, ta, tb, p, st) : launch_turned<EPI_STORE>(bn, ta, tb, p, st);
@@ -1085,7 +1087,7 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& g, cudaStream_t st) {
   p.n_fast = (int64_t)g.M * g.N > ((int64_t)g.M + g.N) * g.K ? 1 : 0;
   p.row_ptr = g.row_ptr; p.slots = g.slots; p.rows = (const bf16*)g.rows; p.ld_rows = g.ld_rows; p.slots_total = g.slots_total;
   p.batch_rows = g.batch_rows; p.ragged = g.ragged;
-  p.bias = (const bf16*)g.bias;
+  p.bias = (const bf16*)g.bias; p.early = g.early;
   p.clear = g.clear; p.clear_words = g.clear_words;
   p.a_rows = g.a_rows; p.a_rows_batch = g.a_rows_batch; p.a_rows_total = (int)g.a_rows_total;
   switch (g.epi) {

@@ -57,10 +57,19 @@ __device__ __forceinline__ void chain_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #endif
 }
-// Only the second half, for a kernel that is launched plainly (everything before it has completed when it starts).
-__device__ __forceinline__ void chain_next() {
+// A kernel that reads nothing its predecessor in the chain writes, and writes nothing that one touches, may run beside its tail
+// (`early`): it starts where SMs fall idle and waits for the predecessor at its end instead, so that completion stays transitive.
+// What it does read must be complete when it starts.  It starts when every CTA of its predecessor has passed chain_enter(); so
+// with K the last kernel before it that is not early, everything before K is complete, and K and the early ones since may run.
+__device__ __forceinline__ void chain_enter(int early) {
 #if defined(__CUDA_ARCH__)
+  if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+__device__ __forceinline__ void chain_leave(int early) {               // every thread, at the kernel's end
+#if defined(__CUDA_ARCH__)
+  if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
 #endif
 }
 template <typename T> __device__ __forceinline__ T* after_enter(T* p) {
@@ -201,6 +210,7 @@ struct GemmArgs {
   // [0, a_rows_total); batch_a is unused.  Both operands must allow loads of four elements (see launch_gemm_simt), else
   // the product is refused.
   const int32_t* a_rows; int64_t a_rows_batch, a_rows_total; int a_rows_k;
+  int early;                           // see chain_enter()
 };
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
 // ---- fp32 products on the tensor cores (gemm_f32_tc.cu): launch_gemm_simt takes them where they are the faster ones.  Operands
@@ -246,6 +256,7 @@ struct TcGemmArgs {
   // is matrix row a_rows[b * a_rows_batch + r] (every entry in [0, a_rows_total)).  batch_a is unused; not with
   // k_split or batch_rows.
   const int32_t* a_rows; int64_t a_rows_batch, a_rows_total;
+  int early;         // see chain_enter()
 };
 constexpr int EPI_SOFTMAX = 4;
 bool tc_gemm_supported(const TcGemmArgs& g);
