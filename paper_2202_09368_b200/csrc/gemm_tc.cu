@@ -70,8 +70,10 @@ __host__ __device__ constexpr int stage_bytes(int bn) { return kABytes + bn * BK
 __host__ __device__ constexpr int staging_bytes(int bn_tile, int epi, bool turned) {
   return turned ? 0 : (epi == EPI_SOFTMAX && bn_tile < 128 ? 4 : kEpiWarps) * kStagingPerWarp;
 }
+// There 96 to 112 KiB of weights on their way are the most that pays (64 tokens, 1920 x 5064, products with W1 and W2: 4 stages 240 and
+// 233 us, 6: 213 and 213, 7: 229 and 211, 9: 252 and 221; 32 tokens, 4096 x 16384: 4 stages 1443 us, 6: 1291, 7: 1256, 11: 1433).
 __host__ __device__ constexpr int num_stages(int bn, int staging) {
-  const int fit = (kSmemBudget - staging) / stage_bytes(bn), most = staging == 0 ? 12 : 8;
+  const int fit = (kSmemBudget - staging) / stage_bytes(bn), most = staging == 0 ? (bn <= 32 ? 7 : 6) : 8;
   return fit > most ? most : fit;
 }
 // Two accumulators of BN columns (a power of two for BN = 64, 128, 256), or one of 512.  A CTA pair takes all 512
@@ -1011,9 +1013,9 @@ bool tc_gemm_supported(const TcGemmArgs& g) {
 
 // Few rows per expert (M <= 64): the product streams the weights, and a tile of 128 rows is mostly fill.  Turned, the weights'
 // columns are the 128 rows of the MMA and the tokens its 32 or 64 columns: no multiply-adds on fill, whose energy the 1000 W
-// cap turns into time (32 rows, 64 experts of 4096 x 16384: 1690 and 1560 us a product, 5.3 TB/s of weights, turned 1350 and
-// 1285, 6.7 TB/s; the same on a cold GPU, 1340), and 9 or 11 stages of weights on their way instead of five (64 rows, 64 experts of
-// 768 x 3072: the forward pass 171 -> 165 us).  Beyond 64 rows the fill saved is less than what stores without the TMA unit cost (80
+// cap turns into time (32 rows, 64 experts of 4096 x 16384: 1371 and 1328 us a product, 6.3 TB/s of weights, turned 1256 each,
+// 6.8 TB/s; on a box with a lower cap 1690 and 1560, and 1350 and 1285), and more weights on their way than five stages hold (64 rows,
+// 64 experts of 768 x 3072: the forward pass 171 -> 162 us).  Beyond 64 rows the fill saved is less than what stores without the TMA unit cost (80
 // rows, 48 experts of 1136 x 2304: a step of 509 us takes 525).
 static bool turns(const TcGemmArgs& g) {
   return g.M <= 64 && !g.a_mn_major && !g.a_rows && !g.k_split && (!g.batch_rows || g.ragged == 1) &&
