@@ -2,6 +2,7 @@
 // and the element-wise parts of its backward pass.  Everything here is bandwidth- or
 // latency-bound integer / fp32 work; the dense contractions live in gemm_*.cu.
 #include "internal.h"
+#include "tc_ptx.cuh"
 
 #include <string.h>
 
@@ -1467,15 +1468,162 @@ __global__ void combine_kernel(const float* __restrict__ X_e, const float* __res
   }
 }
 
-cudaError_t launch_combine(int dtype, const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots,
-                           void* X_out, int64_t n, int d, int64_t slots_total, int* status, cudaStream_t st) {
+// The same for many rows: a producer warp streams the rows of X_e that a CTA's tokens need (consecutive tokens' slots are one run
+// of `slots`) into a ring in shared memory with bulk copies, GROUP / 32 warps take a token's rows from it in slot order.  The
+// plain kernel holds a row piece per thread behind two dependent loads of indices; here some 190 KiB per SM are on their way at
+// all times.  A ring entry has a barrier for its bytes (and its weight, stored before them) and one for its readers.
+// 262144 x 1024, two slots a token: 490 -> 404 us, 6.6 TB/s; 16384 x 4096: 137 -> 119.
+// floats of X_e from which the ring is taken: beyond L2.  Below it a CTA's start-up is not won back (16384 slots of 768: 18.5 -> 20.5 us,
+// 8192 of 1024: the routing chain 49.2 -> 50.6)
+constexpr int64_t kRingFrom = 32 << 20;
+constexpr int kRingWarps = 8, kRingBytes = 192 * 1024, kRingMost = 96;
+constexpr unsigned long long kRingWaitNs = 2000000000ull;
+struct Ring { uint64_t full[kRingMost], empty[kRingMost]; float weight[kRingMost]; int row[kRingMost]; int gave_up; };
+// bounded, like every wait: false when it ran out, or when another warp's did
+__device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatile int* gave_up) {
+  if (mbar_try(bar, parity)) return true;
+  const unsigned long long t0 = globaltimer();
+  for (uint32_t spin = 1;; ++spin) {
+    if (mbar_try(bar, parity)) return true;
+    if ((spin & 63u) == 0 && (*gave_up || globaltimer() - t0 > kRingWaitNs)) { *gave_up = 1; return false; }
+  }
+}
+// Waits for row number `row` of the CTA in entry `at`.  A group whose tokens have no slots runs ahead of the others and may come to an
+// entry a whole round early, when the parity of its barrier says nothing yet: the entry's own row number, written before its bytes
+// are asked for, has to be the wanted one first.
+__device__ __forceinline__ bool ring_take(Ring& ring, uint32_t full, int at, int row, uint32_t parity) {
+  volatile int* held = &ring.row[at];
+  if (*held != row) {
+    const unsigned long long t0 = globaltimer();
+    for (uint32_t spin = 1; *held != row; ++spin)
+      if ((spin & 63u) == 0 && (*(volatile int*)&ring.gave_up || globaltimer() - t0 > kRingWaitNs)) { *(volatile int*)&ring.gave_up = 1; return false; }
+  }
+  return ring_wait(full, parity, &ring.gave_up);
+}
+template <typename T, int GROUP, int NQ>
+__global__ void __launch_bounds__(32 * (kRingWarps + 1), 1)
+combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d, int depth,
+                    int64_t per_cta, int* status) {
+  extern __shared__ __align__(128) uint8_t ring_smem[];                // [depth][d] fp32
+  __shared__ Ring ring;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t full0 = smem_u32(ring.full), empty0 = smem_u32(ring.empty);
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < depth; ++i) { mbar_init(full0 + 8 * i, 1); mbar_init(empty0 + 8 * i, GROUP / 32); ring.row[i] = -1; }
+    ring.gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  chain_enter();
+  const int64_t t0 = (int64_t)blockIdx.x * per_cta, t1 = min(n, t0 + per_cta);
+  if (t0 >= t1) return;
+  const int64_t qa = row_ptr[t0];
+  if (warp == kRingWarps) {                            // ---- producer: entry by entry, up to 32 at a time
+    const int64_t qb = row_ptr[t1];
+    const int step = min(32, depth);                   // a lane never waits for another of the same step
+    const uint32_t bytes = (uint32_t)d * 4u;
+    int64_t q = qa + lane;
+    int id = lane < step && q < qb ? slots[q] : -1;
+    float w = id >= 0 ? G[id] : 0.f;
+    int at = lane % depth; uint32_t phase = 1;         // lane < step <= depth
+    for (; q - lane < qb; q += step) {
+      const int idn = lane < step && q + step < qb ? slots[q + step] : -1;
+      bool ok = true;
+      if (id >= 0) {
+        ok = ring_wait(empty0 + 8 * at, phase, &ring.gave_up);
+        if (ok) {
+          ring.weight[at] = w;
+          *(volatile int*)&ring.row[at] = (int)(q - qa);
+          mbar_expect_tx(full0 + 8 * at, bytes);
+          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                       ::"r"(smem_u32(ring_smem) + (uint32_t)at * bytes), "l"(X_e + (int64_t)id * d), "r"(bytes), "r"(full0 + 8 * at) : "memory");
+        }
+      }
+      if (!__all_sync(0xffffffffu, ok)) break;
+      id = idn; w = id >= 0 ? G[id] : 0.f;
+      at += step;
+      if (at >= depth) { at -= depth; phase ^= 1; }
+    }
+  } else {                                             // ---- consumers: a group per token
+    constexpr int kGroups = kRingWarps * 32 / GROUP;
+    const int grp = threadIdx.x / GROUP, gl = threadIdx.x % GROUP;
+    int64_t t = t0 + grp;
+    int64_t a = t < t1 ? row_ptr[t] : 0, b = t < t1 ? row_ptr[t + 1] : 0;
+    bool ok = true;
+    for (; ok && t < t1; t += kGroups) {
+      const int64_t an = t + kGroups < t1 ? row_ptr[t + kGroups] : 0, bn = t + kGroups < t1 ? row_ptr[t + kGroups + 1] : 0;
+      float acc[NQ][4];
+#pragma unroll
+      for (int j = 0; j < NQ; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+      int at = (int)((a - qa) % depth); uint32_t phase = (uint32_t)((a - qa) / depth) & 1u;
+      for (int64_t q = a; q < b; ++q) {
+        ok = ring_take(ring, full0 + 8 * at, at, (int)(q - qa), phase);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        const float w = ring.weight[at];
+        const float4* x = reinterpret_cast<const float4*>(ring_smem) + (int64_t)at * (d / 4);
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) {
+          const int v = gl + j * GROUP;
+          if (v < d / 4) {
+            const float4 f = x[v];
+            acc[j][0] = fmaf(w, f.x, acc[j][0]); acc[j][1] = fmaf(w, f.y, acc[j][1]);
+            acc[j][2] = fmaf(w, f.z, acc[j][2]); acc[j][3] = fmaf(w, f.w, acc[j][3]);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty0 + 8 * at);
+        if (++at == depth) { at = 0; phase ^= 1; }
+      }
+      if (ok) {
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) if (gl + j * GROUP < d / 4) store4(X_out + t * d + 4 * (gl + j * GROUP), acc[j]);
+      }
+      a = an; b = bn;
+    }
+  }
+  __syncthreads();
+  if (ring.gave_up) {                                  // copies in flight land before the shared memory goes
+    const unsigned long long s0 = globaltimer();
+    while (globaltimer() - s0 < 200000ull) __nanosleep(1000);
+    if (threadIdx.x == 0 && status != nullptr) { atomicExch(status + 1, 11); atomicExch(status, 5 /* EC_ERR_TIMEOUT */); }
+  }
+}
+
+template <typename T, int GROUP, int NQ>
+cudaError_t launch_combine_ring(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d,
+                                int* status, int sms, cudaStream_t st) {
+  auto kern = combine_ring_kernel<T, GROUP, NQ>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+  if (e != cudaSuccess) return e;
+  const int fit = kRingBytes / (d * 4), depth = fit < kRingMost ? fit : kRingMost;
+  const int64_t per_cta = (n + sms - 1) / sms;
+  return launch_chained(kern, dim3((unsigned)((n + per_cta - 1) / per_cta)), dim3(32 * (kRingWarps + 1)), (size_t)depth * d * 4, st, X_e, G, row_ptr, slots,
+                        X_out, n, d, depth, per_cta, status);
+}
+template <typename T>
+cudaError_t launch_combine_t(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d,
+                             int64_t slots_total, int* status, cudaStream_t st) {
+#ifndef EC_DEBUG                                       // the debug build's lists may be anything: the plain kernel checks every index
+  if (slots_total * d >= kRingFrom && d <= 8192) {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (d <= 512) return launch_combine_ring<T, 32, 4>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
+    if (d <= 1024) return launch_combine_ring<T, 32, 8>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
+    if (d <= 2048) return launch_combine_ring<T, 64, 8>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
+    if (d <= 4096) return launch_combine_ring<T, 128, 8>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
+    return launch_combine_ring<T, 256, 8>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
+  }
+#endif
   const int qpr = d / 4;
   const int64_t tq = n * qpr;
-  const unsigned grid = grid_for(tq, 256, 148 * 32);
-  const RowOf row = row_of(tq, qpr);
-  if (dtype == 0) { launch_chained(combine_kernel<float>, grid, dim3(256), 0, st, X_e, G, row_ptr, slots, (float*)X_out, tq, qpr, row, slots_total, status); }
-  else { launch_chained(combine_kernel<bf16>, grid, dim3(256), 0, st, X_e, G, row_ptr, slots, (bf16*)X_out, tq, qpr, row, slots_total, status); }
-  return cudaGetLastError();
+  return launch_chained(combine_kernel<T>, dim3(grid_for(tq, 256, 148 * 32)), dim3(256), 0, st, X_e, G, row_ptr, slots, X_out, tq, qpr, row_of(tq, qpr),
+                        slots_total, status);
+}
+cudaError_t launch_combine(int dtype, const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots,
+                           void* X_out, int64_t n, int d, int64_t slots_total, int* status, cudaStream_t st) {
+  return dtype == 0 ? launch_combine_t(X_e, G, row_ptr, slots, (float*)X_out, n, d, slots_total, status, st)
+                    : launch_combine_t(X_e, G, row_ptr, slots, (bf16*)X_out, n, d, slots_total, status, st);
 }
 
 // ------------------------------------------------------------------------------------------
