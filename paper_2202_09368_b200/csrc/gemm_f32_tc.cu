@@ -24,6 +24,7 @@
 // 1.7 k.  At 2048 tokens, 512 x 2048, 16 experts (8.6 GFLOP a product): 67-71 us a product, 166-206 us with multiply-adds.
 #include "internal.h"
 #include "tc_ptx.cuh"
+#include "gelu.cuh"
 
 namespace ecmoe {
 
@@ -262,21 +263,24 @@ __global__ void __launch_bounds__(kF32Threads, 1) gemm_f32_tc_kernel(const __gri
         auto z_at = [&](int i) {
           return mr + 4 * i < g.M && n < g.N ? *reinterpret_cast<const float4*>((const float*)g.Zin + o0 + 4 * i * g.ldc) : make_float4(0.f, 0.f, 0.f, 0.f);
         };
-        float4 zn = make_float4(0.f, 0.f, 0.f, 0.f);
-        if constexpr (EPI == EPI_GELU_GRAD) zn = z_at(0);
-#pragma unroll 1
+        float4 zn[2];                                // Z of the next two rows
+        if constexpr (EPI == EPI_GELU_GRAD) { zn[0] = z_at(0); zn[1] = z_at(1); }
+#pragma unroll 2
         for (int i = 0; i < 8; ++i) {
           const int r = 4 * i + (lane >> 3);
-          const float4 z = zn;
-          if constexpr (EPI == EPI_GELU_GRAD) if (i < 7) zn = z_at(i + 1);
+          float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+          if constexpr (EPI == EPI_GELU_GRAD) { z = zn[i & 1]; if (i < 6) zn[i & 1] = z_at(i + 2); }
           float4 v = *reinterpret_cast<const float4*>(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
           if (mr + 4 * i >= g.M || n >= g.N) continue;
           const int64_t o = o0 + 4 * i * g.ldc;
           v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
           if constexpr (EPI == EPI_GELU) {
-            *reinterpret_cast<float4*>((float*)g.C2 + o) = make_float4(gelu_fwd(v.x, g.gelu), gelu_fwd(v.y, g.gelu), gelu_fwd(v.z, g.gelu), gelu_fwd(v.w, g.gelu));
+            float4 h = v;
+            gelu_fwd2_fine(g.gelu, h.x, h.y); gelu_fwd2_fine(g.gelu, h.z, h.w);
+            *reinterpret_cast<float4*>((float*)g.C2 + o) = h;
           } else if constexpr (EPI == EPI_GELU_GRAD) {
-            v.x *= gelu_bwd(z.x, g.gelu); v.y *= gelu_bwd(z.y, g.gelu); v.z *= gelu_bwd(z.z, g.gelu); v.w *= gelu_bwd(z.w, g.gelu);
+            gelu_bwd2_fine(g.gelu, z.x, z.y, z.x, z.y); gelu_bwd2_fine(g.gelu, z.z, z.w, z.z, z.w);
+            v.x *= z.x; v.y *= z.y; v.z *= z.z; v.w *= z.w;
           }
           if (g.C) *reinterpret_cast<float4*>((float*)g.C + o) = v;
         }
