@@ -685,7 +685,7 @@ topk_finish_tile_kernel(const unsigned long long* __restrict__ keys, const unsig
   const int e = blockIdx.x;
   const SelState st = state[e];
   const int len = max(32, (int)kpad);
-  for (int i = threadIdx.x; i < len; i += kSortThreads) sk[i] = i < kpad ? keys[(size_t)e * kpad + i] : ~0ull;
+  for (int i = threadIdx.x; i < len; i += kSortThreads) sk[i] = i < k ? keys[(size_t)e * kpad + i] : ~0ull;      // padding sorts last
   __syncthreads();
   if (st.mode == 2) {
     load_sorted_candidates(cand, e, st.cand, sc);
@@ -724,7 +724,7 @@ topk_sort_tile_kernel(unsigned long long* keys, int64_t kpad, int64_t k, int64_t
   const int64_t base = (blockIdx.x % tiles_per_expert) * kSortTile;   // index inside the expert
   const int len = (int)min((int64_t)kSortTile, kpad - base);          // power of two
   unsigned long long* src = keys + expert * kpad + base;
-  for (int i = threadIdx.x; i < len; i += kSortThreads) sk[i] = src[i];
+  for (int i = threadIdx.x; i < len; i += kSortThreads) sk[i] = size_lo > 2 || base + i < k ? src[i] : ~0ull;    // padding sorts last
   __syncthreads();
   if (size_lo == 2) sort_keys(sk, len, (unsigned)base, (unsigned)size_hi);
   else sort_one_size<kSortTile / kSortThreads>(sk, len, (unsigned)base, (unsigned)size_lo);
@@ -1035,7 +1035,6 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
   if ((e = vec ? cudaFuncSetAttribute(topk_hist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistSmemBytes)
                : cudaFuncSetAttribute(topk_hist_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistSmemBytes)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(base, 0, L.zero_bytes, st)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(keys, 0xFF, (size_t)VE * L.kpad * 8, st)) != cudaSuccess) return e;
   // rows per CTA: one CTA per SM fits (the histogram takes 132 KiB of shared memory), so one wave over all
   // chunks and groups; at least 256 rows each
   int64_t want = (int64_t)148 / ((int64_t)L.chunks * groups); if (want < 1) want = 1;
