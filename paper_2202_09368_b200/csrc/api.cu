@@ -456,17 +456,21 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
   int* status = (int*)(w + W.status);
   const int32_t* rag = D.router && D.groups == 1 ? (const int32_t*)(sv + L.load) : nullptr;   // see ec_moe_forward
   const int64_t kd = D.k * D.d, kf = D.k * D.dff, df = (int64_t)D.d * D.dff;
+  // Products that may start beside their predecessor's tail (see chain_enter()) do, up to a TFLOP each: 2048 x 256 step 100.9 -> 88.6 us,
+  // 8192 x 768 x 3072 (77 GFLOP) 673 -> 659.  Products of milliseconds win nothing at their tails and two at a time share L2 and the
+  // power cap worse: the 8B step (4.4 TFLOP) takes 28.1 ms without and 28.8 with.
+  const int early = 2.0 * (double)D.slots * D.d * D.dff < 1e12 ? 1 : 0;
   // the two gate-gradient products; on tensor cores dL [n, E] is bf16
   const int P = dwg_splits(D);
   TcGemmArgs tw; memset(&tw, 0, sizeof(tw));          // dWg = X^T . dL, cut along the tokens
   const int64_t cut = (((D.n + P - 1) / P) + 63) / 64 * 64;
   tw.A = X; tw.a_mn_major = 1; tw.lda = D.d; tw.B = dL; tw.b_mn_major = 1; tw.ldb = D.E;
   tw.M = D.d; tw.N = D.E; tw.K = (int)cut; tw.batches = P; tw.k_split = 1; tw.k_total = D.n;
-  tw.epi = EPI_STORE; tw.c_f32 = 1; tw.C = part; tw.ldc = D.E; tw.batch_c = (int64_t)D.d * D.E; tw.status = status; tw.early = 1;
+  tw.epi = EPI_STORE; tw.c_f32 = 1; tw.C = part; tw.ldc = D.E; tw.batch_c = (int64_t)D.d * D.E; tw.status = status; tw.early = early;
   TcGemmArgs tx; memset(&tx, 0, sizeof(tx));          // dX = dL . Wg^T + rows of dX_in
   tx.A = dL; tx.a_mn_major = 0; tx.lda = D.E; tx.B = Wg; tx.b_mn_major = 0; tx.ldb = D.E;
   tx.M = (int)D.n; tx.N = D.d; tx.K = D.E; tx.batches = 1;
-  tx.epi = EPI_ADD_SLOTS; tx.C = dX; tx.ldc = D.d; tx.status = status; tx.early = 1;
+  tx.epi = EPI_ADD_SLOTS; tx.C = dX; tx.ldc = D.d; tx.status = status; tx.early = early;
   tx.row_ptr = row_ptr; tx.slots = slots; tx.rows = dX_in; tx.ld_rows = D.d; tx.slots_total = D.slots;
   const bool tc_gate = D.dtype == EC_BF16 && tc_gemm_supported(tw) && tc_gemm_supported(tx);     // mirrored by gate_grads_on_tc()
   // Eq. 4 backward: dX_e, dG; then the softmax's: dL.  In the debug build, whose kernels may record a bad index in the status
@@ -492,10 +496,10 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
     if (db2) EC_CUDA(launch_column_sums(D.dtype, dX_e, db2, D.E, D.k, D.d, rag, st));
     prof_mark("bias_grads", st);
   }
-  // dW2[i] = dX_e[i]^T . H[i].  Early (see chain_enter(); here and below): what it reads is older than the last kernel that waits, as
-  // it is for dX_in and dWg behind dW1, which does, and for dX behind the sum of the partials
+  // dW2[i] = dX_e[i]^T . H[i].  Early (here and below): what it reads is older than the last kernel that waits, as it is for dX_in and
+  // dWg behind dW1, which does, and for dX behind the sum of the partials
   BatchedGemm g4 = {dX_e, 1, D.d, kd, H, 1, D.dff, kf, dW2, D.dff, df, D.d, D.dff, (int)D.k, D.E, EPI_STORE, nullptr, nullptr, 0, rag, 2, nullptr};
-  g4.early = 1;
+  g4.early = early;
   if ((s = run_gemm(D, g4, status, st)) != EC_OK) return s;
   prof_mark("gemm_dW2", st);
   // dW1[i] = X_in[i]^T . dZ[i]
@@ -505,7 +509,7 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
   prof_mark("gemm_dW1", st);
   // dX_in[i] = dZ[i] . W1[i]^T
   BatchedGemm g6 = {dZ, 0, D.dff, kf, W1, 0, D.dff, df, dX_in, D.d, kd, (int)D.k, D.d, D.dff, D.E, EPI_STORE, nullptr, nullptr, 0, rag, 1, nullptr};
-  g6.early = 1;
+  g6.early = early;
   if ((s = run_gemm(D, g6, status, st)) != EC_OK) return s;
   prof_mark("gemm_dXin", st);
   if (tc_gate) {
@@ -524,7 +528,7 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
     g.M = D.d; g.N = D.E; g.K = (int)chunk; g.batches = P; g.k_limit = D.n;
     g.sam = 1; g.sak = D.d; g.sbk = D.E; g.sbn = 1; g.ldc = D.E;
     g.batch_a = chunk * D.d; g.batch_b = chunk * D.E; g.batch_c = (int64_t)D.d * D.E;
-    g.epi = EPI_STORE; g.early = 1;
+    g.epi = EPI_STORE; g.early = early;
     EC_CUDA(launch_gemm_simt(g, st));
     EC_CUDA(launch_reduce_partials(D.dtype, part, dWg, P, (int64_t)D.d * D.E, st));
     prof_mark("dWg", st);
@@ -536,7 +540,7 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
     g.M = (int)D.n; g.N = D.d; g.K = D.E; g.batches = 1;
     g.sam = D.E; g.sak = 1; g.sbk = 1; g.sbn = D.E; g.ldc = D.d;
     g.epi = EPI_ADD_SLOTS; g.row_ptr = row_ptr; g.slots = slots; g.rows = dX_in; g.ld_rows = D.d;
-    g.slots_total = D.slots; g.status = status; g.early = 1;
+    g.slots_total = D.slots; g.status = status; g.early = early;
     EC_CUDA(launch_gemm_simt(g, st));
     prof_mark("dX", st);
   }
