@@ -19,6 +19,13 @@ __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigne
 __device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
 __device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
 
+// z within [-Z, Z]; NaN stays NaN (fminf and fmaxf answer the other operand), so that a derivative taken there is NaN too
+__device__ __forceinline__ float clamp_nan(float z, float Z) {
+  float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(z), "f"(-Z));
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(r), "f"(Z));
+  return r;
+}
+
 // Phi(z) = (1 + erf(z / sqrt 2)) / 2 for two values at once, without special-function instructions:
 // erf(u) = u Q(t) with t = 2 u^2 / U^2 - 1 in [-1, 1], U = 3.4, u clamped to [-U, U] (erf(3.4) = 1 - 1.5e-6), and Q
 // the degree-11 polynomial that interpolates erf(u) / u at the Chebyshev nodes in t (fitted for this file; the
@@ -67,7 +74,7 @@ __device__ __forceinline__ void gelu_bwd2(float z0, float z1, float& g0, float& 
   unsigned long long g;
   if constexpr (VARIANT == 0) {
     constexpr float Z = 5.5f;
-    const unsigned long long z = pk2(fminf(fmaxf(z0, -Z), Z), fminf(fmaxf(z1, -Z), Z));
+    const unsigned long long z = pk2(clamp_nan(z0, Z), clamp_nan(z1, Z));
     const unsigned long long t = fma2(mul2(z, z), pk2(2.f / (Z * Z), 2.f / (Z * Z)), pk2(-1.f, -1.f));
     constexpr float c[16] = {1.287591376e-01f, -6.573985250e-02f, 5.367434234e-02f, -5.373902109e-02f, 6.012413464e-02f, -6.868787701e-02f,
                              7.575927955e-02f, -7.385357749e-02f, 5.931453062e-02f, -5.048873522e-02f, 5.172561041e-02f, -3.163604518e-02f,
@@ -90,7 +97,7 @@ __device__ __forceinline__ void gelu_bwd2(float z0, float z1, float& g0, float& 
 // experts); 84 and 96 like this
 template <int N>
 __device__ __forceinline__ unsigned long long odd_poly2(float z0, float z1, float Z, const float (&c)[N], unsigned long long& zc) {
-  zc = pk2(fminf(fmaxf(z0, -Z), Z), fminf(fmaxf(z1, -Z), Z));
+  zc = pk2(clamp_nan(z0, Z), clamp_nan(z1, Z));
   const unsigned long long t = fma2(mul2(zc, zc), pk2(2.f / (Z * Z), 2.f / (Z * Z)), pk2(-1.f, -1.f));
   unsigned long long acc = pk2(c[N - 1], c[N - 1]);
 #pragma unroll
