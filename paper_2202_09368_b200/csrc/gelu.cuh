@@ -1,4 +1,5 @@
-// GeLU and its derivative in the epilogues of the tensor-core products, on packed pairs of fp32 values and without branches.
+// GeLU and its derivative in the epilogues of the bf16 products, on packed pairs of fp32 values and without branches.  (The fp32 products
+// take gelu_fwd and gelu_bwd of internal.h.)
 #pragma once
 #include <stdint.h>
 
@@ -89,48 +90,6 @@ __device__ __forceinline__ void gelu_bwd2(float z0, float z1, float& g0, float& 
     g = fma2(mul2(mul2(z, s), fma2(s, pk2(-1.f, -1.f), pk2(1.f, 1.f))), fma2(zz, pk2(w1, w1), pk2(w0, w0)), s);
   }
   g0 = lo2(g); g1 = hi2(g);
-}
-
-// The same for fp32 results (the epilogues of the fp32 products on tensor cores): Phi and GeLU' of the erf form by polynomials of
-// degree 15 on [-5.3, 5.3] (|error| 8.4e-8) and 17 on [-5.8, 5.8] (2.3e-7).  Beside the splitting warps every instruction of an
-// epilogue counts: with erff and expf GEMM-1 took 92 us where the product without an epilogue takes 72, dZ 115 (256 x 512 x 2048, 16
-// experts); 84 and 96 like this
-template <int N>
-__device__ __forceinline__ unsigned long long odd_poly2(float z0, float z1, float Z, const float (&c)[N], unsigned long long& zc) {
-  zc = pk2(clamp_nan(z0, Z), clamp_nan(z1, Z));
-  const unsigned long long t = fma2(mul2(zc, zc), pk2(2.f / (Z * Z), 2.f / (Z * Z)), pk2(-1.f, -1.f));
-  unsigned long long acc = pk2(c[N - 1], c[N - 1]);
-#pragma unroll
-  for (int i = N - 2; i >= 0; --i) acc = fma2(acc, t, pk2(c[i], c[i]));
-  return acc;
-}
-__device__ __forceinline__ void gelu_fwd2_fine(int variant, float& z0, float& z1) {
-  const unsigned long long z = pk2(z0, z1);
-  unsigned long long gate;
-  if (variant == 0) {
-    constexpr float c[16] = {1.333925591e-01f, -6.651843254e-02f, 4.926455599e-02f, -3.959193226e-02f, 3.207243618e-02f, -2.526302165e-02f,
-                             1.897313267e-02f, -1.336712550e-02f, 8.679343655e-03f, -5.372115350e-03f, 3.373292434e-03f, -1.764693291e-03f,
-                             5.441169150e-04f, -2.895659743e-04f, 3.415073814e-04f, -1.344471650e-04f};
-    unsigned long long zc;
-    const unsigned long long q = odd_poly2(z0, z1, 5.3f, c, zc);
-    gate = fma2(zc, q, pk2(0.5f, 0.5f));
-  } else {
-    gate = tanh_gate2(z, mul2(z, z));
-  }
-  const unsigned long long h = mul2(z, gate);
-  z0 = lo2(h); z1 = hi2(h);
-}
-__device__ __forceinline__ void gelu_bwd2_fine(int variant, float z0, float z1, float& g0, float& g1) {
-  if (variant == 0) {
-    constexpr float c[18] = {1.219987794e-01f, -6.165751869e-02f, 4.863529830e-02f, -4.619428565e-02f, 5.017595275e-02f, -5.776049435e-02f,
-                             6.495053381e-02f, -6.935448228e-02f, 7.035347965e-02f, -6.151823790e-02f, 4.235884695e-02f, -3.399980956e-02f,
-                             3.672469116e-02f, -2.090521005e-02f, -7.978317807e-04f, -1.036321868e-03f, 7.645974817e-03f, -3.412456848e-03f};
-    unsigned long long zc;
-    const unsigned long long q = odd_poly2(z0, z1, 5.8f, c, zc), g = fma2(zc, q, pk2(0.5f, 0.5f));
-    g0 = lo2(g); g1 = hi2(g);
-  } else {
-    gelu_bwd2<1>(z0, z1, g0, g1);
-  }
 }
 
 }  // namespace
