@@ -2,23 +2,11 @@
 // take gelu_fwd and gelu_bwd of internal.h.)
 #pragma once
 #include <stdint.h>
+#include "tc_ptx.cuh"
 
 namespace ecmoe {
 
 namespace {
-
-// Packed fp32 pairs: two lanes of arithmetic per instruction (fma.rn.f32x2 and friends).
-__device__ __forceinline__ unsigned long long pk2(float a, float b) {
-  return (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(b) << 32);
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
-  unsigned long long d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
-}
-__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
-__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
 
 // z within [-Z, Z]; NaN stays NaN (fminf and fmaxf answer the other operand), so that a derivative taken there is NaN too
 __device__ __forceinline__ float clamp_nan(float z, float Z) {

@@ -1,8 +1,10 @@
 // fp32 expert products on the tensor cores.
 //
 // An fp32 value is the sum of three bf16 values, x = h + m + l: h is x rounded to bf16, m what is left rounded, l the rest,
-// which fits eight bits.  (Exact from 2^-110 up; below that l loses what lies under 2^-133.  A value that is not finite, or
-// that rounds to infinity in bf16, leaves a NaN.)  A product of two such sums is taken as six of its nine terms,
+// which fits eight bits.  The pieces are those of 2^24 x, so that the lowest bit of the smallest x is still a normal bf16 number, and
+// the sums are multiplied by 2^-48 at the end: both exact.  What this range does not hold at the other end (|x| from 2^104, sums
+// from 2^80, infinities) comes out infinite or NaN, and every such element is taken again by multiply-adds from global memory
+// (take_again): the result is then the multiply-add kernel's.  A product of two such sums is taken as six of its nine terms,
 //
 //     a b  =  ah bh + (ah bm + am bh) + (am bm + ah bl + al bh)  +  terms below 2^-26 of |a b|,
 //
@@ -43,12 +45,16 @@ __host__ __device__ constexpr int f32_smem_bytes(int fn) { return kStages * f32_
 // index that ld multiplies.
 struct Side { const float* p; int64_t ld; int rows, kb; const int32_t* list; int64_t list_total; int* status; };
 
-// x = h + m + l for two values, packed
+constexpr float kScaleIn = 16777216.f, kScaleOut = 1.f / 281474976710656.f;          // 2^24, 2^-48
+
+// 2^24 x = h + m + l for two values, packed
 __device__ __forceinline__ unsigned bf2(float a, float b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const unsigned*>(&v);
 }
 __device__ __forceinline__ void split2(float a, float b, unsigned& h, unsigned& m, unsigned& l) {
+  const unsigned long long x = mul2(pk2(a, b), pk2(kScaleIn, kScaleIn));
+  a = lo2(x); b = hi2(x);
   h = bf2(a, b);
   a -= __uint_as_float(h << 16); b -= __uint_as_float(h & 0xFFFF0000u);
   m = bf2(a, b);
@@ -140,6 +146,39 @@ __device__ __forceinline__ void issue_terms(uint32_t st, uint32_t d_tmem, int le
 #pragma unroll
     for (int kk = 0; kk < FK / 16; ++kk)
       if (kk == 0 || kk * 16 < left) tc_mma(d_tmem, a0 + ((kTermA[t] * kAP + kk * a_step) >> 4), b0 + ((kTermB[t] * kBP + kk * b_step) >> 4), idesc, (t | kk) != 0);
+}
+
+// What the pieces could not hold: the marked elements of row `row`, bit j for column n0 + j, by multiply-adds in ascending k, four columns
+// at a time.  NaN four times ends a sum.  Not inlined: in the epilogue's own loop it costs a step 20 us, like this 4.
+template <int EPI, bool A_K, bool B_K, bool LIST>
+__device__ __noinline__ void take_again(const GemmArgs& g, int b, int row, int n0, unsigned long long bad) {
+  if (row >= g.M) return;
+  const float* A = (const float*)g.A + (LIST ? 0 : (int64_t)b * g.batch_a);
+  const int32_t* list = LIST ? g.a_rows + (int64_t)b * g.a_rows_batch : nullptr;
+  const int64_t lda = A_K ? g.sam : g.sak, ldb = B_K ? g.sbn : g.sbk;
+  for (; bad != 0; bad >>= 4, n0 += 4) {
+    if ((bad & 15ull) == 0 || n0 >= g.N) continue;
+    const float* B = (const float*)g.B + (int64_t)b * g.batch_b + (B_K ? n0 * ldb : n0);
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int k = 0; k < g.K; ++k) {
+      int64_t line = A_K ? row : k;
+      bool ok = true;
+      if constexpr (LIST) { line = list[line]; ok = idx_ok(line, 0, g.a_rows_total, g.status); }
+      const float a = ok ? A[line * lda + (A_K ? k : row)] : 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[j] = fmaf(a, B_K ? B[j * ldb + k] : B[k * ldb + j], acc[j]);
+      if ((k & 63) == 63 && isnan(acc[0]) && isnan(acc[1]) && isnan(acc[2]) && isnan(acc[3])) break;
+    }
+    for (int j = 0; j < 4; ++j) {
+      if (!(bad >> j & 1ull)) continue;
+      const int64_t o = (int64_t)b * g.batch_c + (int64_t)row * g.ldc + n0 + j;
+      float v = acc[j] + (g.bias ? ((const float*)g.bias)[(int64_t)b * g.N + n0 + j] : 0.f);
+      if constexpr (EPI == EPI_GELU) ((float*)g.C2)[o] = gelu_fwd(v, g.gelu);
+      if constexpr (EPI == EPI_GELU_GRAD) v *= gelu_bwd(((const float*)g.Zin)[o], g.gelu);
+      if (g.C) ((float*)g.C)[o] = v;
+    }
+  }
 }
 
 template <int EPI, int FN, bool A_K, bool B_K, bool LIST>
@@ -248,6 +287,14 @@ __global__ void __launch_bounds__(kF32Threads, 1) gemm_f32_tc_kernel(const __gri
         if (++buf == kRing) { buf = 0; tphase ^= 1; }
       }
       if (gave_up) break;
+      unsigned long long zero = 0ull, bad = 0ull;    // zero: NaN as soon as one of this lane's elements is not finite; bad: which ones
+#pragma unroll
+      for (int j = 0; j < kCols; j += 2) zero = fma2(pk2(acc[j], acc[j + 1]), pk2(0.f, 0.f), zero);
+      const bool redo = __any_sync(0xffffffffu, lo2(zero) + hi2(zero) != 0.f);
+      if (redo) {
+#pragma unroll
+        for (int j = 0; j < kCols; ++j) bad |= (unsigned long long)!isfinite(acc[j]) << j;
+      }
 #pragma unroll
       for (int c = 0; c < kCols; c += 32) {
         // rows of 32 columns into the staging buffer (swizzled: no bank conflicts either way), back as lines: eight lanes a row
@@ -272,7 +319,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) gemm_f32_tc_kernel(const __gri
           float4 v = *reinterpret_cast<const float4*>(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
           if (mr + 4 * i >= g.M || n >= g.N) continue;
           const int64_t o = o0 + 4 * i * g.ldc;
-          v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
+          v.x = fmaf(v.x, kScaleOut, bias.x); v.y = fmaf(v.y, kScaleOut, bias.y); v.z = fmaf(v.z, kScaleOut, bias.z); v.w = fmaf(v.w, kScaleOut, bias.w);
           // GeLU as the multiply-add kernel takes it, exact at both ends.  (Packed polynomials save 19 us of a 530 us step at 2048 x 512 x
           // 2048, 16 experts, but their gate is off by 5e-8 for every z beyond 5.3 and by 1.0e-7 before, where erff's is within 6e-8.)
           if constexpr (EPI == EPI_GELU) {
@@ -286,6 +333,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) gemm_f32_tc_kernel(const __gri
         }
         __syncwarp();
       }
+      if (redo) take_again<EPI, A_K, B_K, LIST>(g, b, m0 + q * 32 + lane, n0 + half * kCols, bad);
     }
   }
 

@@ -1,4 +1,4 @@
-// PTX of the tensor-core kernels: mbarriers with bounded waits, TMA copies, tensor memory, tcgen05.mma and its descriptors.
+// PTX of the tensor-core kernels: mbarriers with bounded waits, TMA copies, tensor memory, tcgen05.mma and its descriptors, packed fp32 pairs.
 #pragma once
 #include <cuda.h>
 #include <stdint.h>
@@ -149,6 +149,19 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
          (1ull << 46) | (2ull << 61);
 }
+
+// Packed fp32 pairs: two lanes of arithmetic per instruction (fma.rn.f32x2 and friends).
+__device__ __forceinline__ unsigned long long pk2(float a, float b) {
+  return (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(b) << 32);
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
+}
+__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
 
 }  // namespace
 

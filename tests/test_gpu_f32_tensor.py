@@ -62,3 +62,53 @@ def test_layer_matches_64_bits(gelu, fuse):
     for got, want in zip((dW1, dW2, *bias_grads), (w1.grad, w2.grad, c1.grad, c2.grad)):
         # sums of at most 1332 terms in fp32: measured 2e-6 of the root mean square at most
         assert (got.double() - want).abs().max() <= 1e-5 * want.pow(2).mean().sqrt()
+
+
+def _three_products(cfg, k, d, dff, E, make):
+    """The three kinds with operands made by make(kind, which, shape): (result, A as it multiplies, B as it multiplies) in 64 bits."""
+    for kind, sa, sb in ((B.EC_GEMM_XW1, (E, k, d), (E, d, dff)), (B.EC_GEMM_HW2T, (E, k, dff), (E, d, dff)), (B.EC_GEMM_ATB, (E, k, d), (E, k, dff))):
+        A, Bm = make(kind, 0, sa), make(kind, 1, sb)
+        out = B.ec_expert_gemm(cfg, kind, A, Bm)
+        yield out.double(), A.double().transpose(1, 2) if kind == B.EC_GEMM_ATB else A.double(), Bm.double().transpose(1, 2) if kind == B.EC_GEMM_HW2T else Bm.double()
+
+
+# operands of 2^a and 2^b: subnormal numbers, products near both ends of the range and beyond the middle of it
+@pytest.mark.parametrize("a,b", [(-120, 10), (10, -120), (-140, 100), (100, -100), (-60, -60), (60, 60), (120, -10)])
+def test_products_over_the_range_of_fp32(a, b):
+    k, d, dff, E = 260, 316, 1028, 8
+    cfg = B.make_config(k * E, d, dff, E, 1.0, torch.float32)
+    gen = torch.Generator(device="cuda").manual_seed(a + 1000)
+    for out, A, Bm in _three_products(cfg, k, d, dff, E, lambda kind, which, shape: torch.ldexp(torch.empty(shape, device="cuda").normal_(generator=gen),
+                                                                                              torch.tensor(b if which else a, device="cuda"))):
+        terms = A.shape[2]
+        # as above; elements taken by multiply-adds have a rounding per term instead, and results below 2^-126 one of 2^-149 on top
+        units = 16 + 20 * 4 / 256 + (terms + 63) // 64 + 0.75 if a + b < 100 else terms
+        assert ((out - A @ Bm).abs() <= units * 2.0 ** -24 * (A.abs() @ Bm.abs()) + 2.0 ** -148).all()
+
+
+def test_infinities_huge_values_and_nan_stay_in_their_rows_and_columns():
+    """One infinity, one finite value that bf16 would round to infinity, one overflowing pair and one NaN: what 64 bits say they make
+    of their rows and columns, and nothing elsewhere."""
+    k, d, dff, E = 260, 316, 1028, 8
+    cfg = B.make_config(k * E, d, dff, E, 1.0, torch.float32)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+
+    def make(kind, which, shape):
+        t = torch.empty(shape, device="cuda").normal_(generator=gen)
+        if which == 0:
+            t[0, 5, 7], t[1, 131, 3], t[2, 9, 11], t[3, 200, 100] = float("inf"), 3.396e38, 1e30, float("nan")
+        else:
+            t[4, 17, 19] = -float("inf")
+            t[1] *= 1e-6                               # the huge value's products are finite
+            t[2, 3:5, 21:25] = 1e30
+            if kind != B.EC_GEMM_HW2T:
+                t[2, 11 if kind == B.EC_GEMM_XW1 else 9, 30] = 3e30
+        return t
+
+    for out, A, Bm in _three_products(cfg, k, d, dff, E, make):
+        want = (A @ Bm).float().double()               # rounded to fp32: sums beyond its range are infinite
+        assert torch.equal(torch.isnan(out), torch.isnan(want))
+        assert torch.equal(torch.isinf(out), torch.isinf(want)) and torch.equal(out[torch.isinf(out)], want[torch.isinf(want)])
+        fine = torch.isfinite(want)
+        size = A.abs().nan_to_num(0, 0) @ Bm.abs().nan_to_num(0, 0)
+        assert ((out - want).abs()[fine] <= A.shape[2] * 2.0 ** -24 * size[fine]).all()
