@@ -133,9 +133,10 @@ cudaError_t launch_inverse_index(const int32_t* I, int64_t n, int64_t slots_tota
                                  int32_t* slots, void* scratch, int* status, cudaStream_t st);
 cudaError_t launch_gather(int dtype, const void* X, const int32_t* I, void* X_in, int64_t slots_total,
                           int d, int64_t n, int* status, cudaStream_t st);
+constexpr unsigned long long kRingWaitNs = 2000000000ull;    // of the combine's ring; silent_cta: see ec_debug_unshuffle_wait (debug build)
 cudaError_t launch_combine(int dtype, const float* X_e, const float* G, const int32_t* row_ptr,
                            const int32_t* slots, void* X_out, int64_t n, int d, int64_t slots_total, int* status,
-                           cudaStream_t st);
+                           cudaStream_t st, unsigned long long wait_ns = kRingWaitNs, int silent_cta = -1);
 // Counts what is wrong with an index structure (every access range-checked): I entries outside [0, n) (or [-1, n) when
 // empty slots are allowed) or outside their routing group, row_ptr not starting at 0 / decreasing / not ending at
 // the number of filled slots, slots entries out of range, not ascending within a token, or pointing at a slot that

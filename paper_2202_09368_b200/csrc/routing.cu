@@ -1476,33 +1476,33 @@ __global__ void combine_kernel(const float* __restrict__ X_e, const float* __res
 // 8192 of 1024: the routing chain 49.2 -> 50.6)
 constexpr int64_t kRingFrom = 32 << 20;
 constexpr int kRingWarps = 8, kRingBytes = 192 * 1024, kRingMost = 96;
-constexpr unsigned long long kRingWaitNs = 2000000000ull;
 struct Ring { uint64_t full[kRingMost], empty[kRingMost]; float weight[kRingMost]; int row[kRingMost]; int gave_up; };
-// bounded, like every wait: false when it ran out, or when another warp's did
-__device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatile int* gave_up) {
+// bounded, like every wait: false when it ran out, or when another warp's did.  The clock also runs while another process has the
+// device, so this is not a fault: the warps then read what is left of their rows from global memory.
+__device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatile int* gave_up, unsigned long long wait_ns) {
   if (mbar_try(bar, parity)) return true;
   const unsigned long long t0 = globaltimer();
   for (uint32_t spin = 1;; ++spin) {
     if (mbar_try(bar, parity)) return true;
-    if ((spin & 63u) == 0 && (*gave_up || globaltimer() - t0 > kRingWaitNs)) { *gave_up = 1; return false; }
+    if ((spin & 63u) == 0 && (*gave_up || globaltimer() - t0 > wait_ns)) { *gave_up = 1; return false; }
   }
 }
 // Waits for row number `row` of the CTA in entry `at`.  A group whose tokens have no slots runs ahead of the others and may come to an
 // entry a whole round early, when the parity of its barrier says nothing yet: the entry's own row number, written before its bytes
 // are asked for, has to be the wanted one first.
-__device__ __forceinline__ bool ring_take(Ring& ring, uint32_t full, int at, int row, uint32_t parity) {
+__device__ __forceinline__ bool ring_take(Ring& ring, uint32_t full, int at, int row, uint32_t parity, unsigned long long wait_ns) {
   volatile int* held = &ring.row[at];
   if (*held != row) {
     const unsigned long long t0 = globaltimer();
     for (uint32_t spin = 1; *held != row; ++spin)
-      if ((spin & 63u) == 0 && (*(volatile int*)&ring.gave_up || globaltimer() - t0 > kRingWaitNs)) { *(volatile int*)&ring.gave_up = 1; return false; }
+      if ((spin & 63u) == 0 && (*(volatile int*)&ring.gave_up || globaltimer() - t0 > wait_ns)) { *(volatile int*)&ring.gave_up = 1; return false; }
   }
-  return ring_wait(full, parity, &ring.gave_up);
+  return ring_wait(full, parity, &ring.gave_up, wait_ns);
 }
 template <typename T, int GROUP, int NQ>
 __global__ void __launch_bounds__(32 * (kRingWarps + 1), 1)
 combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d, int depth,
-                    int64_t per_cta, int* status) {
+                    int64_t per_cta, unsigned long long wait_ns, int silent) {
   extern __shared__ __align__(128) uint8_t ring_smem[];                // [depth][d] fp32
   __shared__ Ring ring;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1528,8 +1528,11 @@ combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, co
     for (; q - lane < qb; q += step) {
       const int idn = lane < step && q + step < qb ? slots[q + step] : -1;
       bool ok = true;
+#ifdef EC_DEBUG
+      if ((int)blockIdx.x == silent && q - lane > qa) break;           // asks for no more rows than the first few
+#endif
       if (id >= 0) {
-        ok = ring_wait(empty0 + 8 * at, phase, &ring.gave_up);
+        ok = ring_wait(empty0 + 8 * at, phase, &ring.gave_up, wait_ns);
         if (ok) {
           ring.weight[at] = w;
           *(volatile int*)&ring.row[at] = (int)(q - qa);
@@ -1548,35 +1551,36 @@ combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, co
     const int grp = threadIdx.x / GROUP, gl = threadIdx.x % GROUP;
     int64_t t = t0 + grp;
     int64_t a = t < t1 ? row_ptr[t] : 0, b = t < t1 ? row_ptr[t + 1] : 0;
-    bool ok = true;
-    for (; ok && t < t1; t += kGroups) {
+    bool ok = true;                                    // until a wait runs out
+    for (; t < t1; t += kGroups) {
       const int64_t an = t + kGroups < t1 ? row_ptr[t + kGroups] : 0, bn = t + kGroups < t1 ? row_ptr[t + kGroups + 1] : 0;
       float acc[NQ][4];
 #pragma unroll
       for (int j = 0; j < NQ; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
       int at = (int)((a - qa) % depth); uint32_t phase = (uint32_t)((a - qa) / depth) & 1u;
-      for (int64_t q = a; q < b; ++q) {
-        ok = ring_take(ring, full0 + 8 * at, at, (int)(q - qa), phase);
-        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      auto add = [&](int j, float w, const float4& f) {
+        acc[j][0] = fmaf(w, f.x, acc[j][0]); acc[j][1] = fmaf(w, f.y, acc[j][1]);
+        acc[j][2] = fmaf(w, f.z, acc[j][2]); acc[j][3] = fmaf(w, f.w, acc[j][3]);
+      };
+      int64_t q = a;
+      for (; ok && q < b; ++q) {
+        ok = __all_sync(0xffffffffu, ring_take(ring, full0 + 8 * at, at, (int)(q - qa), phase, wait_ns));
+        if (!ok) break;
         const float w = ring.weight[at];
         const float4* x = reinterpret_cast<const float4*>(ring_smem) + (int64_t)at * (d / 4);
 #pragma unroll
-        for (int j = 0; j < NQ; ++j) {
-          const int v = gl + j * GROUP;
-          if (v < d / 4) {
-            const float4 f = x[v];
-            acc[j][0] = fmaf(w, f.x, acc[j][0]); acc[j][1] = fmaf(w, f.y, acc[j][1]);
-            acc[j][2] = fmaf(w, f.z, acc[j][2]); acc[j][3] = fmaf(w, f.w, acc[j][3]);
-          }
-        }
+        for (int j = 0; j < NQ; ++j) if (gl + j * GROUP < d / 4) add(j, w, x[gl + j * GROUP]);
         __syncwarp();
         if (lane == 0) mbar_arrive(empty0 + 8 * at);
         if (++at == depth) { at = 0; phase ^= 1; }
       }
-      if (ok) {
+      for (; q < b; ++q) {                             // without the ring
+        const int64_t id = slots[q];
 #pragma unroll
-        for (int j = 0; j < NQ; ++j) if (gl + j * GROUP < d / 4) store4(X_out + t * d + 4 * (gl + j * GROUP), acc[j]);
+        for (int j = 0; j < NQ; ++j) if (gl + j * GROUP < d / 4) add(j, G[id], reinterpret_cast<const float4*>(X_e + id * d)[gl + j * GROUP]);
       }
+#pragma unroll
+      for (int j = 0; j < NQ; ++j) if (gl + j * GROUP < d / 4) store4(X_out + t * d + 4 * (gl + j * GROUP), acc[j]);
       a = an; b = bn;
     }
   }
@@ -1584,45 +1588,48 @@ combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, co
   if (ring.gave_up) {                                  // copies in flight land before the shared memory goes
     const unsigned long long s0 = globaltimer();
     while (globaltimer() - s0 < 200000ull) __nanosleep(1000);
-    if (threadIdx.x == 0 && status != nullptr) { atomicExch(status + 1, 11); atomicExch(status, 5 /* EC_ERR_TIMEOUT */); }
   }
 }
 
 template <typename T, int GROUP, int NQ>
 cudaError_t launch_combine_ring(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d,
-                                int* status, int sms, cudaStream_t st) {
+                                int sms, unsigned long long wait_ns, int silent, cudaStream_t st) {
   auto kern = combine_ring_kernel<T, GROUP, NQ>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
   if (e != cudaSuccess) return e;
   const int fit = kRingBytes / (d * 4), depth = fit < kRingMost ? fit : kRingMost;
   const int64_t per_cta = (n + sms - 1) / sms;
   return launch_chained(kern, dim3((unsigned)((n + per_cta - 1) / per_cta)), dim3(32 * (kRingWarps + 1)), (size_t)depth * d * 4, st, X_e, G, row_ptr, slots,
-                        X_out, n, d, depth, per_cta, status);
+                        X_out, n, d, depth, per_cta, wait_ns, silent);
 }
 template <typename T>
 cudaError_t launch_combine_t(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d,
-                             int64_t slots_total, int* status, cudaStream_t st) {
-#ifndef EC_DEBUG                                       // the debug build's lists may be anything: the plain kernel checks every index
-  if (slots_total * d >= kRingFrom && d <= 8192) {
+                             int64_t slots_total, int* status, cudaStream_t st, unsigned long long wait_ns, int silent) {
+#ifdef EC_DEBUG                                        // the debug build's lists may be anything: the plain kernel checks every index
+  const bool ring = silent >= 0;
+#else
+  const bool ring = slots_total * d >= kRingFrom;
+#endif
+  if (ring && d <= 8192) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (d <= 512) return launch_combine_ring<T, 32, 4>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
-    if (d <= 1024) return launch_combine_ring<T, 32, 8>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
-    if (d <= 2048) return launch_combine_ring<T, 64, 8>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
-    if (d <= 4096) return launch_combine_ring<T, 128, 8>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
-    return launch_combine_ring<T, 256, 8>(X_e, G, row_ptr, slots, X_out, n, d, status, sms, st);
+    if (d <= 512) return launch_combine_ring<T, 32, 4>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
+    if (d <= 1024) return launch_combine_ring<T, 32, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
+    if (d <= 2048) return launch_combine_ring<T, 64, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
+    if (d <= 4096) return launch_combine_ring<T, 128, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
+    return launch_combine_ring<T, 256, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
   }
-#endif
   const int qpr = d / 4;
   const int64_t tq = n * qpr;
   return launch_chained(combine_kernel<T>, dim3(grid_for(tq, 256, 148 * 32)), dim3(256), 0, st, X_e, G, row_ptr, slots, X_out, tq, qpr, row_of(tq, qpr),
                         slots_total, status);
 }
 cudaError_t launch_combine(int dtype, const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots,
-                           void* X_out, int64_t n, int d, int64_t slots_total, int* status, cudaStream_t st) {
-  return dtype == 0 ? launch_combine_t(X_e, G, row_ptr, slots, (float*)X_out, n, d, slots_total, status, st)
-                    : launch_combine_t(X_e, G, row_ptr, slots, (bf16*)X_out, n, d, slots_total, status, st);
+                           void* X_out, int64_t n, int d, int64_t slots_total, int* status, cudaStream_t st,
+                           unsigned long long wait_ns, int silent) {
+  return dtype == 0 ? launch_combine_t(X_e, G, row_ptr, slots, (float*)X_out, n, d, slots_total, status, st, wait_ns, silent)
+                    : launch_combine_t(X_e, G, row_ptr, slots, (bf16*)X_out, n, d, slots_total, status, st, wait_ns, silent);
 }
 
 // ------------------------------------------------------------------------------------------

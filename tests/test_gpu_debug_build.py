@@ -143,6 +143,24 @@ def test_a_solver_wait_that_runs_out_is_reported_and_leaves_a_defined_assignment
     assert D.ec_read_status(ws) == D.EC_OK and torch.equal(again, want)
 
 
+@pytest.mark.parametrize("n,d,E,dtype", [(3000, 512, 8, BF16), (2000, 1024, 16, F32), (1500, 2048, 8, BF16), (1000, 4096, 8, F32), (700, 8192, 4, BF16)])
+def test_an_unshuffle_whose_waits_run_out_is_finished_all_the_same(D, n, d, E, dtype):
+    """One CTA of the ring gets its first rows only and its warps wait 2 ms for the others: nobody can tell from the result."""
+    cfg = D.make_config(n, d, 8, E, 2.0, dtype)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    I = torch.stack([torch.randperm(n, device="cuda", generator=gen)[:D.ec_capacity(cfg)] for _ in range(E)]).flatten()
+    slots = torch.sort(I, stable=True)[1].int()
+    row_ptr = torch.cat([I.new_zeros(1), torch.bincount(I, minlength=n).cumsum(0)]).int()
+    X_e = torch.empty((I.numel(), d), device="cuda").normal_(generator=gen)
+    G = torch.rand(I.numel(), device="cuda", generator=gen)
+    want = D.ec_unshuffle(cfg, X_e, G, row_ptr, slots)
+    out = torch.full_like(want, float("nan"))
+    call = D.lib().ec_debug_unshuffle_wait
+    call.argtypes = [ctypes.POINTER(D.ec_config)] + [ctypes.c_void_p] * 5 + [ctypes.c_longlong, ctypes.c_int, ctypes.c_void_p]
+    assert call(ctypes.byref(cfg), X_e.data_ptr(), G.data_ptr(), row_ptr.data_ptr(), slots.data_ptr(), out.data_ptr(), 2_000_000, 1, D._stream()) == D.EC_OK
+    assert torch.equal(out, want)
+
+
 @pytest.mark.parametrize("n,E,dtype,kw", [(2048, 8, BF16, {}), (20000, 8, BF16, {}), (2048, 8, F32, dict(fuse_gather=True)), (2048, 8, BF16, dict(fuse_gather=True)),
                                           (2048, 8, BF16, dict(router="token")), (2048, 8, BF16, dict(cap_b=3, cap_iters=5)),
                                           (20000, 65, BF16, dict(cap_b=3, cap_iters=5)), (1000, 10, F32, dict(groups=2))])
