@@ -1499,10 +1499,23 @@ __device__ __forceinline__ bool ring_take(Ring& ring, uint32_t full, int at, int
   }
   return ring_wait(full, parity, &ring.gave_up, wait_ns);
 }
+// The first token at which `slot_weight` per slot and `token_weight` per token before it add up to `work` or more: where a CTA's share
+// begins.  One warp, 32 candidates a step.
+__device__ __forceinline__ int64_t share_start(const int32_t* row_ptr, int64_t n, int slot_weight, int token_weight, int64_t work) {
+  int64_t lo = 0, hi = n;                              // every token before lo is short of it, hi is not (or is n)
+  while (lo < hi) {
+    const int64_t step = (hi - lo + 31) / 32, t = min(hi - 1, lo + ((threadIdx.x & 31) + 1) * step - 1);
+    const int below = __popc(__ballot_sync(0xffffffffu, (int64_t)row_ptr[t] * slot_weight + t * token_weight < work));     // candidates ascend
+    if (below < 32) hi = min(hi - 1, lo + (below + 1) * step - 1);
+    lo = min(hi, lo + below * step);
+  }
+  return lo;
+}
+
 template <typename T, int GROUP, int NQ>
 __global__ void __launch_bounds__(32 * (kRingWarps + 1), 1)
 combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d, int depth,
-                    int64_t per_cta, unsigned long long wait_ns, int silent) {
+                    unsigned long long wait_ns, int silent) {
   extern __shared__ __align__(128) uint8_t ring_smem[];                // [depth][d] fp32
   __shared__ Ring ring;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1512,9 +1525,18 @@ combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, co
     ring.gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
   chain_enter();
-  const int64_t t0 = (int64_t)blockIdx.x * per_cta, t1 = min(n, t0 + per_cta);
+  // A CTA's tokens: shares of equal bytes, a row of fp32 read per slot and a row written per token, wherever the slots lie.  (Equal
+  // numbers of tokens leave the work to a few CTAs when all experts take the same ones: 65536 x 1024, 64 experts: 4260 us, 176 so,
+  // where the plain kernel takes 123: with 64 slots a token, one group at a time has the ring to itself.)
+  __shared__ int64_t share[2];
+  if (warp < 2) {
+    const int64_t work = (int64_t)row_ptr[n] * 4 + n * (int64_t)sizeof(T);
+    const int64_t t = share_start(row_ptr, n, 4, sizeof(T), work * (blockIdx.x + warp) / gridDim.x);
+    if (lane == 0) share[warp] = t;
+  }
+  __syncthreads();
+  const int64_t t0 = share[0], t1 = share[1];
   if (t0 >= t1) return;
   const int64_t qa = row_ptr[t0];
   if (warp == kRingWarps) {                            // ---- producer: entry by entry, up to 32 at a time
@@ -1549,11 +1571,14 @@ combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, co
   } else {                                             // ---- consumers: a group per token
     constexpr int kGroups = kRingWarps * 32 / GROUP;
     const int grp = threadIdx.x / GROUP, gl = threadIdx.x % GROUP;
+    // the bounds of the group's next 32 lists, a lane each, and of the 32 after them: tokens without slots cost a row of zeros, no round trip
+    auto bound = [&](int64_t t, int end) { return t < t1 ? row_ptr[t + end] : 0; };
     int64_t t = t0 + grp;
-    int64_t a = t < t1 ? row_ptr[t] : 0, b = t < t1 ? row_ptr[t + 1] : 0;
+    int la = 0, lb = 0, la2 = bound(t + lane * kGroups, 0), lb2 = bound(t + lane * kGroups, 1);
     bool ok = true;                                    // until a wait runs out
-    for (; t < t1; t += kGroups) {
-      const int64_t an = t + kGroups < t1 ? row_ptr[t + kGroups] : 0, bn = t + kGroups < t1 ? row_ptr[t + kGroups + 1] : 0;
+    for (int i = 0; t < t1; t += kGroups, i = (i + 1) & 31) {
+      if (i == 0) { la = la2; lb = lb2; la2 = bound(t + (32 + lane) * kGroups, 0); lb2 = bound(t + (32 + lane) * kGroups, 1); }
+      const int64_t a = __shfl_sync(0xffffffffu, la, i), b = __shfl_sync(0xffffffffu, lb, i);
       float acc[NQ][4];
 #pragma unroll
       for (int j = 0; j < NQ; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
@@ -1581,7 +1606,6 @@ combine_ring_kernel(const float* X_e, const float* G, const int32_t* row_ptr, co
       }
 #pragma unroll
       for (int j = 0; j < NQ; ++j) if (gl + j * GROUP < d / 4) store4(X_out + t * d + 4 * (gl + j * GROUP), acc[j]);
-      a = an; b = bn;
     }
   }
   __syncthreads();
@@ -1598,9 +1622,8 @@ cudaError_t launch_combine_ring(const float* X_e, const float* G, const int32_t*
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
   if (e != cudaSuccess) return e;
   const int fit = kRingBytes / (d * 4), depth = fit < kRingMost ? fit : kRingMost;
-  const int64_t per_cta = (n + sms - 1) / sms;
-  return launch_chained(kern, dim3((unsigned)((n + per_cta - 1) / per_cta)), dim3(32 * (kRingWarps + 1)), (size_t)depth * d * 4, st, X_e, G, row_ptr, slots,
-                        X_out, n, d, depth, per_cta, wait_ns, silent);
+  return launch_chained(kern, dim3((unsigned)(n < sms ? n : sms)), dim3(32 * (kRingWarps + 1)), (size_t)depth * d * 4, st, X_e, G, row_ptr, slots, X_out, n, d,
+                        depth, wait_ns, silent);
 }
 template <typename T>
 cudaError_t launch_combine_t(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d,

@@ -35,3 +35,28 @@ def test_combine_through_the_ring(n, d, E, c, dtype, crowded):
     eps = 2.0 ** -24 if dtype == torch.float32 else 2.0 ** -8          # of the rounding to the result's type; at most E sums in fp32
     assert ((out.double() - want).abs() <= eps * want.abs() + (E + 1) * 2.0 ** -24 * size).all()
     assert torch.equal(out, B.ec_unshuffle(cfg, X_e, G, row_ptr, order.int()))
+
+
+@pytest.mark.parametrize("n,d,E", [(16384, 1024, 64), (16384, 4096, 64)])
+def test_tokens_with_many_slots_side_by_side_cost_no_more(n, d, E):
+    """Every expert takes the same first tokens (as with padding rows that are all alike: ties go to the lowest): the same bytes as
+    anywhere, and all SMs have to share them.  Times vary by some percent; one SM in thirty at work is a factor of twenty."""
+    cfg = B.make_config(n, d, 8, E, 2.0, torch.bfloat16)
+    k = B.ec_capacity(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    X_e = torch.empty((E, k, d), device="cuda").normal_(generator=gen)
+    G, out = torch.rand((E, k), device="cuda", generator=gen), torch.empty((n, d), device="cuda", dtype=torch.bfloat16)
+    took = []
+    for I in (torch.stack([torch.randperm(n, device="cuda", generator=gen)[:k] for _ in range(E)]), torch.arange(k, device="cuda").repeat(E, 1)):
+        slots = torch.sort(I.flatten(), stable=True)[1].int()
+        row_ptr = torch.cat([I.new_zeros(1), torch.bincount(I.flatten(), minlength=n).cumsum(0)]).int()
+        times = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            B.ec_unshuffle(cfg, X_e, G, row_ptr, slots, out)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        took.append(sorted(times)[6])
+    assert took[1] <= 3 * took[0]
