@@ -625,7 +625,7 @@ ec_status ec_debug_capped_wait(const ec_config* c, const float* S, float* A, voi
                                    (int*)((char*)ws + W.status), st, (unsigned long long)wait_ns, silent_cta));
   return EC_OK;
 }
-// ec_unshuffle through the ring whatever the size, in which one CTA asks for a few rows only and its waits run out after wait_ns.
+// ec_unshuffle through the ring whatever the number of slots (where the width takes it), in which one CTA asks for a few rows only and its waits run out after wait_ns.
 ec_status ec_debug_unshuffle_wait(const ec_config* c, const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, void* X_out,
                                   long long wait_ns, int silent_cta, void* stream) {
   Dims D; ec_status s = check_cfg(c, &D); if (s != EC_OK) return s;

@@ -1471,11 +1471,17 @@ __global__ void combine_kernel(const float* __restrict__ X_e, const float* __res
 // of `slots`) into a ring in shared memory with bulk copies, GROUP / 32 warps take a token's rows from it in slot order.  The
 // plain kernel holds a row piece per thread behind two dependent loads of indices; here some 190 KiB per SM are on their way at
 // all times.  A ring entry has a barrier for its bytes (and its weight, stored before them) and one for its readers.
-// 262144 x 1024, two slots a token: 490 -> 404 us, 6.6 TB/s; 16384 x 4096: 137 -> 119.
-// floats of X_e from which the ring is taken: beyond L2.  Below it a CTA's start-up is not won back (16384 slots of 768: 18.5 -> 20.5 us,
-// 8192 of 1024: the routing chain 49.2 -> 50.6)
-constexpr int64_t kRingFrom = 32 << 20;
-constexpr int kRingWarps = 8, kRingBytes = 192 * 1024, kRingMost = 96;
+// 262144 x 1024, two slots a token: 490 -> 420 us from a flushed L2, 16384 x 4096: 121 -> 119.
+// Where the ring is taken, from both sides measured (us plain / ring, L2 flushed, E k d in millions of floats).
+//   Rows from 768 floats on: a row costs the producer and its readers a fixed time, and below it a warp cannot ask for them fast
+//   enough: bf16 results 1024 wide, 512 M: 490 / 420; 768, 384 M: 332 / 326; 640, 320 M: 281 / 294; 512, 256 M: 242 / 266; 256, 64 M: 72 / 115; 64, 32 M: 49 / 213.
+//   X_e beyond L2: below it a CTA's start-up is not won back (16384 slots of 768: 18.5 / 20.5; 8192 of 1024: the routing chain 49.2 / 50.6).
+//   fp32 results, whose stores weigh as much as half of the loads: up to 2048 wide and from 256 M on (1024, 512 M: 557 / 513; 1024, 256 M:
+//   377 / 364; 2048, 512 M: 545 / 528); else 1024, 128 M: 138 / 139; 768, 192 M: 272 / 279; 4096, 256 M: 257 / 270; 8192, 512 M: 500 / 516.
+constexpr int kRingBytes = 192 * 1024, kRingFrom = 768, kRingTo = 8192, kRingToF32 = 2048, kRingWarps = 8, kRingMost = kRingBytes / (4 * kRingFrom);
+template <typename T> constexpr bool takes_ring(int64_t floats, int d) {
+  return sizeof(T) == 2 ? floats >= 32 << 20 && d >= kRingFrom && d <= kRingTo : floats >= 256 << 20 && d >= kRingFrom && d <= kRingToF32;
+}
 struct Ring { uint64_t full[kRingMost], empty[kRingMost]; float weight[kRingMost]; int row[kRingMost]; int gave_up; };
 // bounded, like every wait: false when it ran out, or when another warp's did.  The clock also runs while another process has the
 // device, so this is not a fault: the warps then read what is left of their rows from global memory.
@@ -1621,7 +1627,7 @@ cudaError_t launch_combine_ring(const float* X_e, const float* G, const int32_t*
   auto kern = combine_ring_kernel<T, GROUP, NQ>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
   if (e != cudaSuccess) return e;
-  const int fit = kRingBytes / (d * 4), depth = fit < kRingMost ? fit : kRingMost;
+  const int depth = kRingBytes / (d * 4);
   return launch_chained(kern, dim3((unsigned)(n < sms ? n : sms)), dim3(32 * (kRingWarps + 1)), (size_t)depth * d * 4, st, X_e, G, row_ptr, slots, X_out, n, d,
                         depth, wait_ns, silent);
 }
@@ -1629,19 +1635,20 @@ template <typename T>
 cudaError_t launch_combine_t(const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, T* X_out, int64_t n, int d,
                              int64_t slots_total, int* status, cudaStream_t st, unsigned long long wait_ns, int silent) {
 #ifdef EC_DEBUG                                        // the debug build's lists may be anything: the plain kernel checks every index
-  const bool ring = silent >= 0;
+  const bool ring = silent >= 0 && takes_ring<T>((int64_t)1 << 40, d);
 #else
-  const bool ring = slots_total * d >= kRingFrom;
+  const bool ring = takes_ring<T>(slots_total * d, d);
 #endif
-  if (ring && d <= 8192) {
+  if (ring) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (d <= 512) return launch_combine_ring<T, 32, 4>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
     if (d <= 1024) return launch_combine_ring<T, 32, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
     if (d <= 2048) return launch_combine_ring<T, 64, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
-    if (d <= 4096) return launch_combine_ring<T, 128, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
-    return launch_combine_ring<T, 256, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
+    if constexpr (sizeof(T) == 2) {
+      if (d <= 4096) return launch_combine_ring<T, 128, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
+      return launch_combine_ring<T, 256, 8>(X_e, G, row_ptr, slots, X_out, n, d, sms, wait_ns, silent, st);
+    }
   }
   const int qpr = d / 4;
   const int64_t tq = n * qpr;

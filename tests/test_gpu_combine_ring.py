@@ -1,4 +1,4 @@
-"""The combine of results that exceed L2 (rows through a ring in shared memory): every width class, tokens without slots (a group of
+"""The combine of results that exceed L2 (rows through a ring in shared memory where they are wide enough): every width class, tokens without slots (a group of
 warps that runs ahead of the others) and with more slots than the ring has entries, against 64 bits and the same bits twice."""
 import pytest
 import torch
@@ -37,6 +37,18 @@ def test_combine_through_the_ring(n, d, E, c, dtype, crowded):
     assert torch.equal(out, B.ec_unshuffle(cfg, X_e, G, row_ptr, order.int()))
 
 
+def _median_time(call):
+    times = []
+    for _ in range(12):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        call()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    return sorted(times)[6]
+
+
 @pytest.mark.parametrize("n,d,E", [(16384, 1024, 64), (16384, 4096, 64)])
 def test_tokens_with_many_slots_side_by_side_cost_no_more(n, d, E):
     """Every expert takes the same first tokens (as with padding rows that are all alike: ties go to the lowest): the same bytes as
@@ -50,13 +62,22 @@ def test_tokens_with_many_slots_side_by_side_cost_no_more(n, d, E):
     for I in (torch.stack([torch.randperm(n, device="cuda", generator=gen)[:k] for _ in range(E)]), torch.arange(k, device="cuda").repeat(E, 1)):
         slots = torch.sort(I.flatten(), stable=True)[1].int()
         row_ptr = torch.cat([I.new_zeros(1), torch.bincount(I.flatten(), minlength=n).cumsum(0)]).int()
-        times = []
-        for _ in range(12):
-            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            B.ec_unshuffle(cfg, X_e, G, row_ptr, slots, out)
-            b.record()
-            torch.cuda.synchronize()
-            times.append(a.elapsed_time(b))
-        took.append(sorted(times)[6])
+        took.append(_median_time(lambda: B.ec_unshuffle(cfg, X_e, G, row_ptr, slots, out)))
     assert took[1] <= 3 * took[0]
+
+
+def test_narrow_rows_take_about_as_long_as_wide_ones():
+    """The same bytes in rows of 1024, 256, 64 and 32: a kernel that pays per row would take several times as long."""
+    took = []
+    for d in (1024, 256, 64, 32):
+        n, E = (32 << 20) // (2 * d), 32
+        cfg = B.make_config(n, d, 8, E, 2.0, torch.bfloat16)
+        k = B.ec_capacity(cfg)
+        gen = torch.Generator(device="cuda").manual_seed(d)
+        I = torch.stack([torch.randperm(n, device="cuda", generator=gen)[:k] for _ in range(E)]).flatten()
+        slots = torch.sort(I, stable=True)[1].int()
+        row_ptr = torch.cat([I.new_zeros(1), torch.bincount(I, minlength=n).cumsum(0)]).int()
+        X_e, G = torch.empty((E, k, d), device="cuda").normal_(generator=gen), torch.rand((E, k), device="cuda", generator=gen)
+        out = torch.empty((n, d), device="cuda", dtype=torch.bfloat16)
+        took.append(_median_time(lambda: B.ec_unshuffle(cfg, X_e, G, row_ptr, slots, out)))
+    assert max(took) <= 2.5 * took[0], took

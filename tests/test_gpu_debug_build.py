@@ -143,7 +143,7 @@ def test_a_solver_wait_that_runs_out_is_reported_and_leaves_a_defined_assignment
     assert D.ec_read_status(ws) == D.EC_OK and torch.equal(again, want)
 
 
-@pytest.mark.parametrize("n,d,E,dtype", [(3000, 512, 8, BF16), (2000, 1024, 16, F32), (1500, 2048, 8, BF16), (1000, 4096, 8, F32), (700, 8192, 4, BF16)])
+@pytest.mark.parametrize("n,d,E,dtype", [(3000, 768, 8, BF16), (2000, 1024, 16, F32), (1500, 2048, 8, F32), (1000, 4096, 8, BF16), (700, 8192, 4, BF16)])
 def test_an_unshuffle_whose_waits_run_out_is_finished_all_the_same(D, n, d, E, dtype):
     """One CTA of the ring gets its first rows only and its warps wait 2 ms for the others: nobody can tell from the result."""
     cfg = D.make_config(n, d, 8, E, 2.0, dtype)
