@@ -1711,15 +1711,59 @@ __device__ __forceinline__ void bwd_rows(const uint4* dy_row, const float* X_e, 
     for (int u = 0; u < SLOTS; ++u) dot[u] += __shfl_xor_sync(0xffffffffu, dot[u], o);
 }
 
+// A token with more than kBwdLong slots is shared by a CTA's warps: where all experts take the same block of tokens, a warp per
+// token leaves most of the chip idle.  (64 slots a token, 16384 tokens of 1024: 117 us with a warp per token, 55 so; of 4096: 404 and 148.)
+// CTAs of four warps: with eight the common path, whose warps wait for each other at the end, takes 1 % longer.
+constexpr int kBwdLong = 8, kBwdLongs = 64, kBwdThreads = 128;
+// Their slots go by pairs over the warps, then a warp per token does the softmax, in the order of bwd_tokens_kernel.  Not inlined: the
+// registers it would take there cost the common path 1 us of 29.
+template <typename T, typename TL>
+__device__ __noinline__ void bwd_long_lists(const int64_t* tokens, int count, const T* dX_out, const float* X_e, const float* G, const float* S,
+                                            const int32_t* row_ptr, const int32_t* slots, T* dX_e, float* dG, TL* dL, int vecs, int E, int k, int* status) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5, slots_total = E * k;
+  auto slot = [&](int q) { const int s = slots[q]; return s >= 0 && idx_ok(s, 0, slots_total, status) ? s : -1; };
+  for (int i = 0; i < count; ++i) {
+    const int64_t t = tokens[i];
+    const uint4* dy = reinterpret_cast<const uint4*>(dX_out) + t * vecs;
+    for (int q = row_ptr[t] + 2 * warp, b = row_ptr[t + 1]; q < b; q += 2 * warps) {
+      int s[2] = {slot(q), q + 1 < b ? slot(q + 1) : -1};
+      if (s[0] < 0) { s[0] = s[1]; s[1] = -1; }
+      if (s[0] < 0) continue;
+      const float w[2] = {G[s[0]], s[1] >= 0 ? G[s[1]] : 0.f};
+      float dg[2];
+      if (s[1] >= 0) bwd_rows<2>(dy, X_e, dX_e, s, w, vecs, dg); else bwd_rows<1>(dy, X_e, dX_e, s, w, vecs, dg);
+      if (lane == 0) { dG[s[0]] = dg[0]; if (s[1] >= 0) dG[s[1]] = dg[1]; }
+    }
+  }
+  __syncthreads();                                     // dG is read back by other warps
+  for (int i = warp; i < count; i += warps) {
+    const int64_t t = tokens[i];
+    const int a = row_ptr[t], b = row_ptr[t + 1];
+    const float* St = S + t * E;
+    float dot = 0.f;
+    for (int q = a + lane; q < b; q += 32) { const int s = slot(q); if (s >= 0) dot = fmaf(dG[s], St[s / k], dot); }
+    for (int o = 16; o; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    for (int e = lane; e < E; e += 32) st_dl(dL, t * E + e, -St[e] * dot);
+    __syncwarp();
+    for (int q = a + lane; q < b; q += 32) { const int s = slot(q); if (s >= 0) st_dl(dL, t * E + s / k, St[s / k] * (dG[s] - dot)); }
+  }
+}
+
 // empty: not null where slots may be empty (token-choice routing): I, whose negative entries get zero rows and no gradient
 template <typename T, typename TL>
-__global__ void __launch_bounds__(256, 4) bwd_tokens_kernel(const T* dX_out, const float* X_e, const float* G, const float* S, const int32_t* row_ptr,
+__global__ void __launch_bounds__(kBwdThreads, 1024 / kBwdThreads) bwd_tokens_kernel(const T* dX_out, const float* X_e, const float* G, const float* S, const int32_t* row_ptr,
                                                             const int32_t* slots, const int32_t* empty, T* dX_e, float* dG, TL* dL, int64_t n, int vecs,
                                                             int E, int k, int clear, int* status) {
   chain_enter();
   if (clear && blockIdx.x == 0 && threadIdx.x < kStatusWords) status[threadIdx.x] = 0;       // the first kernel of a call
   const int lane = threadIdx.x & 31, slots_total = E * k;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5, first = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  // neighbouring tokens lie in different CTAs, and a CTA's long lists (s_long) wait for all of its warps
+  __shared__ int s_longs;
+  __shared__ int64_t s_long[kBwdLongs];
+  const int warp = threadIdx.x >> 5;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5, first = (int64_t)warp * gridDim.x + blockIdx.x;
+  if (threadIdx.x == 0) s_longs = 0;
+  __syncthreads();
   auto list_of = [&](int64_t t, int& a, int& b) {
     a = b = 0;
     if (t >= n) return;
@@ -1733,10 +1777,20 @@ __global__ void __launch_bounds__(256, 4) bwd_tokens_kernel(const T* dX_out, con
   // a token's list is fetched while the one before it is worked on, its bounds one token earlier still
   int a, b, an, bn;
   list_of(first, a, b); list_of(first + warps, an, bn);
-  int id = slot_at(a, b);
+  int id = slot_at(a, b), longs = 0;
   for (int64_t t = first; t < n; t += warps) {
     const int idn = slot_at(an, bn);
     int a2, b2; list_of(t + 2 * warps, a2, b2);
+    if (b - a > kBwdLong) {
+      longs = 1;
+      int at = lane == 0 ? atomicAdd(&s_longs, 1) : 0;
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (at < kBwdLongs) {
+        if (lane == 0) s_long[at] = t;
+        a = an; b = bn; id = idn; an = a2; bn = b2;
+        continue;
+      }
+    }
     float dot = 0.f, mine = 0.f, sc = 0.f;             // of this lane's slot: dG, and its score
     for (int q = a; q < b; q += 32) {                  // nearly always once
       if (q > a) id = slot_at(q, b);
@@ -1773,6 +1827,7 @@ __global__ void __launch_bounds__(256, 4) bwd_tokens_kernel(const T* dX_out, con
     }
     a = an; b = bn; id = idn; an = a2; bn = b2;
   }
+  if (__syncthreads_or(longs)) bwd_long_lists(s_long, min(s_longs, kBwdLongs), dX_out, X_e, G, S, row_ptr, slots, dX_e, dG, dL, vecs, E, k, status);
   if (empty == nullptr) return;
   for (int64_t s = first; s < slots_total; s += warps) {
     if (empty[s] >= 0) continue;
@@ -1784,7 +1839,7 @@ __global__ void __launch_bounds__(256, 4) bwd_tokens_kernel(const T* dX_out, con
 template <typename T, typename TL>
 cudaError_t launch_bwd_tokens_t(const void* dX_out, const float* X_e, const float* G, const float* S, const int32_t* row_ptr, const int32_t* slots,
                                 const int32_t* empty, void* dX_e, float* dG, void* dL, int64_t n, int d, int E, int64_t k, int clear, int* status, cudaStream_t st) {
-  return launch_chained(bwd_tokens_kernel<T, TL>, dim3(grid_for(n * 32, 256, 148 * 16)), dim3(256), 0, st, (const T*)dX_out, X_e, G, S, row_ptr, slots, empty,
+  return launch_chained(bwd_tokens_kernel<T, TL>, dim3(grid_for(n * 32, kBwdThreads, 148 * 32)), dim3(kBwdThreads), 0, st, (const T*)dX_out, X_e, G, S, row_ptr, slots, empty,
                         (T*)dX_e, dG, (TL*)dL, n, d / Vec<T>::N, E, (int)k, clear, status);
 }
 cudaError_t launch_bwd_tokens(int dtype, const void* dX_out, const float* X_e, const float* G, const float* S, const int32_t* row_ptr, const int32_t* slots,
