@@ -188,7 +188,7 @@ ec_status run_gemm(const Dims& D, const BatchedGemm& b, int* status_word, cudaSt
 
 ec_status route_impl(const Dims& D, const void* X, const void* Wg, float* S, int32_t* I, float* G,
                      int32_t* row_ptr, int32_t* slots, char* ws, const WsLayout& W, cudaStream_t st,
-                     int32_t* load = nullptr, int32_t* requested = nullptr) {
+                     int32_t* load = nullptr, int32_t* requested = nullptr, int silent = 0) {
   bool done = false;
   int* status = (int*)(ws + W.status);
   const bool selects = D.router != EC_ROUTER_TOKEN_TOP2;
@@ -199,7 +199,7 @@ ec_status route_impl(const Dims& D, const void* X, const void* Wg, float* S, int
     t.A = X; t.B = Wg; t.a_mn_major = 0; t.b_mn_major = 1;
     t.M = (int)D.n; t.N = D.E; t.K = D.d; t.batches = 1; t.lda = D.d; t.ldb = D.E;
     t.epi = EPI_SOFTMAX; t.S = S; t.ldc = D.E; t.status = status;
-    t.clear = plan.marks.words; t.clear_words = plan.marks.per_token ? plan.marks.per_token : 1;
+    t.clear = plan.marks.words; t.clear_words = plan.marks.per_token ? plan.marks.per_token : 1; t.silent = silent;
     if (tc_gemm_supported(t)) { EC_CUDA(launch_gemm_tc(t, st)); done = true; }
   }
   if (!done) EC_CUDA(launch_gate_softmax_simt(D.dtype, X, Wg, S, D.n, D.d, D.E, plan.marks, status, st));
@@ -624,6 +624,15 @@ ec_status ec_debug_capped_wait(const ec_config* c, const float* S, float* A, voi
   EC_CUDA(launch_capped_assignment(S, D.ng, D.E, D.kg, D.groups, D.cap_b, D.cap_iters, (float)D.cap_lambda, A, (char*)ws + W.capped,
                                    (int*)((char*)ws + W.status), st, (unsigned long long)wait_ns, silent_cta));
   return EC_OK;
+}
+// ec_route in which the gate's first CTA loads nothing, so that its waits run out.
+ec_status ec_debug_gate_wait(const ec_config* c, const void* X, const void* Wg, float* S, int32_t* I, float* G, int32_t* row_ptr, int32_t* slots,
+                             void* ws, size_t ws_bytes, void* stream) {
+  Dims D; ec_status s = check_cfg(c, &D); if (s != EC_OK) return s;
+  if (!X || !Wg || !S || !I || !G || !row_ptr || !slots || !ws || D.router != EC_ROUTER_EXPERT_CHOICE) return EC_ERR_INVALID_ARG;
+  const WsLayout W = ws_layout(D);
+  if (ws_bytes < W.total) return EC_ERR_WORKSPACE;
+  return route_impl(D, X, Wg, S, I, G, row_ptr, slots, (char*)ws, W, (cudaStream_t)stream, nullptr, nullptr, 1);
 }
 // ec_unshuffle through the ring whatever the number of slots (where the width takes it), in which one CTA asks for a few rows only and its waits run out after wait_ns.
 ec_status ec_debug_unshuffle_wait(const ec_config* c, const float* X_e, const float* G, const int32_t* row_ptr, const int32_t* slots, void* X_out,

@@ -93,6 +93,9 @@ struct TcParams {
   int* status;
   int k_split;                                       // batches are cuts of one product along K
   unsigned* clear; int clear_words;                  // EPI_SOFTMAX: words per row to zero
+#ifdef EC_DEBUG
+  int silent;                                        // see ec_debug_gate_wait
+#endif
   int skip_c;                                        // EPI_GELU: only H = GeLU(acc) is stored, the accumulator itself is not
   const int32_t* row_ptr; const int32_t* slots; const bf16* rows; int64_t ld_rows;   // EPI_ADD_SLOTS
   int64_t slots_total;                               // rows of `rows`: what the debug build checks the slot ids against
@@ -181,6 +184,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   chain_enter(p.early);                            // the barriers and tensor memory above are set up while the previous kernel drains
   const uint32_t tmem_base = *tmem_slot;
   const uint32_t smem_base = smem_u32(smem);
+  if constexpr (EPI == EPI_SOFTMAX) {
+    // The first kernel of a call: its status block and the slot marks start at zero.  Before any wait, so that the marks are clear also
+    // when one runs out: the index takes lengths and places from them, and writes where they say.
+    if (p.clear != nullptr && warp >= 2) {
+      const int64_t me = threadIdx.x - 64, words = (int64_t)p.M * p.clear_words;
+      if (blockIdx.x == 0) for (int64_t i = me; i < kStatusWords; i += kEpiWarps * 32) p.status[i] = 0;
+      for (int64_t i = (int64_t)blockIdx.x * kEpiWarps * 32 + me; i < words; i += (int64_t)gridDim.x * kEpiWarps * 32) p.clear[i] = 0u;
+    }
+  }
   bool gave_up = false;
   if (CTAS == 2 && tmem_base != 0) {               // cannot happen with all 512 columns taken; refuse rather than corrupt
     if (threadIdx.x == 0) { atomicExch(p.status + 1, 9); atomicExch(p.status, 5); }
@@ -259,7 +271,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (lane == 0) {
       int stage = 0; uint32_t phase = 0;
       const uint32_t leader_full0 = CTAS == 2 ? map_to_cta(full0, 0) : full0;
-      for (int tile = first_tile; tile < p.total_tiles && !gave_up; tile += tile_step) {
+#ifdef EC_DEBUG
+      const int from = p.silent && blockIdx.x == 0 ? p.total_tiles : first_tile;
+#else
+      const int from = first_tile;
+#endif
+      for (int tile = from; tile < p.total_tiles && !gave_up; tile += tile_step) {
         const int b = tile / (p.tiles_m * p.tiles_n);
         const int mt = p.n_fast ? (tile / p.tiles_n) % p.tiles_m : tile % p.tiles_m;
         const int nt = p.n_fast ? tile % p.tiles_n : (tile / p.tiles_m) % p.tiles_n;
@@ -427,9 +444,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int q = warp & 3;                        // TMEM lane quarter this warp may read
     const int half = (warp - 2) >> 2;              // which half of the tile's columns this warp handles
     int it = 0;
-    if constexpr (EPI == EPI_SOFTMAX) {            // the first kernel of a call: its status block starts at zero
-      if (p.clear != nullptr && blockIdx.x == 0) for (int i = threadIdx.x - 64; i < kStatusWords; i += kEpiWarps * 32) p.status[i] = 0;
-    }
     uint32_t nchunk = 0;                           // chunks this warp has stored so far: picks the staging buffer
     const uint32_t tempty_leader = CTAS == 2 ? map_to_cta(tempty0, 0) : tempty0;
     // EPI_GELU_GRAD: Z comes through the TMA unit, one chunk of 32 rows x 64 columns ahead of its use, into the staging
@@ -549,8 +563,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         const float inv = 1.f / sum;
         const int sw = lane & 7;
-        if (half == 0 && p.clear != nullptr && r0 + lane < p.M)
-          for (int w = 0; w < p.clear_words; ++w) p.clear[(int64_t)(r0 + lane) * p.clear_words + w] = 0u;
         if (active) {
 #pragma unroll 1
           for (int c0 = cbeg; c0 < cbeg + kColsPerWarp && c0 < p.N; c0 += 32, ++nchunk) {
@@ -1033,6 +1045,9 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& g, cudaStream_t st) {
   p.batch_rows = g.batch_rows; p.ragged = g.ragged;
   p.bias = (const bf16*)g.bias; p.early = g.early;
   p.clear = g.clear; p.clear_words = g.clear_words;
+#ifdef EC_DEBUG
+  p.silent = g.silent;
+#endif
   p.a_rows = g.a_rows; p.a_rows_batch = g.a_rows_batch; p.a_rows_total = (int)g.a_rows_total;
   switch (g.epi) {
     case EPI_STORE: return g.c_f32 ? launch_bn<EPI_STORE_F32>(bn, ctas, ta, tb, tc, tc2, p, st)

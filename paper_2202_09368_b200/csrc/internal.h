@@ -258,6 +258,7 @@ struct TcGemmArgs {
   // k_split or batch_rows.
   const int32_t* a_rows; int64_t a_rows_batch, a_rows_total;
   int early;         // see chain_enter()
+  int silent;        // debug build: the first CTA loads nothing, see ec_debug_gate_wait
 };
 constexpr int EPI_SOFTMAX = 4;
 bool tc_gemm_supported(const TcGemmArgs& g);

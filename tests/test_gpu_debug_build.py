@@ -143,6 +143,28 @@ def test_a_solver_wait_that_runs_out_is_reported_and_leaves_a_defined_assignment
     assert D.ec_read_status(ws) == D.EC_OK and torch.equal(again, want)
 
 
+@pytest.mark.parametrize("n,E,groups", [(2000, 8, 1), (500, 16, 3), (9000, 64, 1), (20000, 32, 1), (20000, 48, 1)])
+def test_a_gate_whose_waits_run_out_leaves_an_index_inside_its_buffers(D, n, E, groups):
+    """128 tokens never get scores, on a workspace full of ones (the marks among them): the status says so, the index that the
+    selection of whatever S holds leads to is a whole one, and the next call on the same workspace is the right one."""
+    cfg = D.make_config(n, 128, 8, E, 2.0, BF16, groups=groups)
+    li = IN.make_layer_inputs(n * groups, 128, 8, E, BF16, seed=n)
+    X, Wg = li.X.cuda(), li.Wg.cuda()
+    ws = D.alloc_workspace(cfg)
+    want = D.ec_route(cfg, X, Wg, ws=ws)
+    assert D.ec_read_status(ws) == D.EC_OK
+    ws.fill_(255)
+    fields = ("S", "I", "G", "row_ptr", "slots")
+    r = D.Routing(*(torch.zeros_like(getattr(want, f)) for f in fields))
+    call = D.lib().ec_debug_gate_wait
+    call.argtypes = [ctypes.POINTER(D.ec_config)] + [ctypes.c_void_p] * 8 + [ctypes.c_size_t, ctypes.c_void_p]
+    assert call(ctypes.byref(cfg), X.data_ptr(), Wg.data_ptr(), *(getattr(r, f).data_ptr() for f in fields), ws.data_ptr(), ws.numel(), D._stream()) == D.EC_OK
+    assert D.ec_read_status(ws) == D.EC_ERR_TIMEOUT
+    assert int(r.row_ptr[-1]) == r.I.numel() and D.ec_validate_routing(cfg, r.I, r.row_ptr, r.slots, ws=ws) == 0
+    again = D.ec_route(cfg, X, Wg, ws=ws)
+    assert D.ec_read_status(ws) == D.EC_OK and all(torch.equal(getattr(again, f), getattr(want, f)) for f in fields)
+
+
 @pytest.mark.parametrize("n,d,E,dtype", [(3000, 768, 8, BF16), (2000, 1024, 16, F32), (1500, 2048, 8, F32), (1000, 4096, 8, BF16), (700, 8192, 4, BF16)])
 def test_an_unshuffle_whose_waits_run_out_is_finished_all_the_same(D, n, d, E, dtype):
     """One CTA of the ring gets its first rows only and its warps wait 2 ms for the others: nobody can tell from the result."""
