@@ -249,7 +249,8 @@ ec_status ec_moe_forward(const ec_config* cfg, const void* X, const void* Wg, co
  * derivative to automatic differentiation): gradients of <dX_out, X_out> with I held
  * constant, so the gate receives gradient through G only.
  *   dX_out [n, d] in, `saved` as filled by ec_moe_forward with the same cfg and inputs;
- *   dX [n, d], dWg [d, E], dW1, dW2 [E, d, d'] out, overwritten (not accumulated);
+ *   dX [n, d], dWg [d, E], dW1, dW2 [E, d, d'] out, overwritten (not accumulated).  dX may be X's or dX_out's memory and dW2
+ *   W2's; the other outputs must not overlap an input, nor any output another one;
  *   db1 [E, d'], db2 [E, d] out, the gradients of the bias terms (sums of dZ and of dX_e over an expert's slots,
  *   fp32 in a fixed order, rounded once); either may be NULL (not wanted).  The biases themselves are not needed here:
  *   the saved Z already contains b1.

@@ -109,6 +109,7 @@ WsLayout ws_layout(const Dims& D) {
 }
 
 inline bool misaligned(const void* p, size_t a) { return ((uintptr_t)p & (a - 1)) != 0; }
+inline bool overlap(const void* a, size_t na, const void* b, size_t nb) { return (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na; }
 
 #define EC_CUDA(x) do { if ((x) != cudaSuccess) return EC_ERR_CUDA; } while (0)
 
@@ -497,9 +498,10 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
     prof_mark("bias_grads", st);
   }
   // dW2[i] = dX_e[i]^T . H[i].  Early (here and below): what it reads is older than the last kernel that waits, as it is for dX_in and
-  // dWg behind dW1, which does, and for dX behind the sum of the partials
+  // dWg behind dW1, which does, and for dX behind the sum of the partials.  Written over W2 or Z, which dZ reads, it waits like the others
   BatchedGemm g4 = {dX_e, 1, D.d, kd, H, 1, D.dff, kf, dW2, D.dff, df, D.d, D.dff, (int)D.k, D.E, EPI_STORE, nullptr, nullptr, 0, rag, 2, nullptr};
-  g4.early = early;
+  const size_t dw = (size_t)D.E * df * D.eb;
+  g4.early = early && !overlap(dW2, dw, W2, dw) && !overlap(dW2, dw, Z, (size_t)D.slots * D.dff * D.eb);
   if ((s = run_gemm(D, g4, status, st)) != EC_OK) return s;
   prof_mark("gemm_dW2", st);
   // dW1[i] = X_in[i]^T . dZ[i]
