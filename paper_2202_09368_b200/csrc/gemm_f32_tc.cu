@@ -366,7 +366,10 @@ cudaError_t launch_f32_tc_one(const GemmArgs& g, int sms, cudaStream_t st) {
   cudaFuncAttributes at;                             // the split of the registers relies on what the compiler gave the kernel
   cudaError_t e = cudaFuncGetAttributes(&at, kern);
   if (e != cudaSuccess) return e;
-  if (at.numRegs != kLaunchRegs) return cudaErrorInvalidConfiguration;
+  if (at.numRegs != kLaunchRegs) return cudaErrorNotSupported;
+#ifdef EC_DEBUG
+  if (g.other_regs) return cudaErrorNotSupported;
+#endif
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
   const int tm = (g.M + FM - 1) / FM, tn = (g.N + FN - 1) / FN, total = tm * tn * g.batches;
   return launch_chained(kern, dim3(total < sms ? total : sms), dim3(kF32Threads), smem, st, g, tm, tn, total);

@@ -428,7 +428,10 @@ cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st) {
       // 256 x 512 x 2048 (16 experts), 14.7 against 12.9 at 58 x 584 x 180 (10); with few rows or a short or lonely contraction
       // a tile of multiply-adds is over sooner: 16.3 against 17.0 at 8 x 128 x 384 (24), 21.0 against 23.1 at 40 x 200 x 600 (16).
       const double tc_cycles = c_vec ? plan_gemm_f32_tc(g, sms, &cols) : -1.;
-      if (tc_cycles >= 0. && tc_cycles < fma_cycles) return launch_gemm_f32_tc(g, cols, sms, st);
+      if (tc_cycles >= 0. && tc_cycles < fma_cycles) {
+        const cudaError_t e = launch_gemm_f32_tc(g, cols, sms, st);
+        if (e != cudaErrorNotSupported) return e;    // else nothing was launched
+      }
       switch (g.epi) {
         case EPI_STORE: return launch_f32<EPI_STORE>(g, tile, oa, ob, c_vec, st);
         case EPI_GELU: return launch_f32<EPI_GELU>(g, tile, oa, ob, c_vec, st);

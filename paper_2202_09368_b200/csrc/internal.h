@@ -212,11 +212,14 @@ struct GemmArgs {
   // the product is refused.
   const int32_t* a_rows; int64_t a_rows_batch, a_rows_total; int a_rows_k;
   int early;                           // see chain_enter()
+  int other_regs;                      // debug build: see ec_debug_expert_gemm_registers
 };
 cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t st);
 // ---- fp32 products on the tensor cores (gemm_f32_tc.cu): launch_gemm_simt takes them where they are the faster ones.  Operands
 // and results fp32, every row a whole number of 16-byte groups at a 16-byte aligned address.  The plan gives the columns per
-// tile (64 or 128) and the estimated cycles, or a negative number for a product that this kernel does not take.
+// tile (64 or 128) and the estimated cycles, or a negative number for a product that this kernel does not take.  The launch answers
+// cudaErrorNotSupported, with nothing queued, when the compiler gave the kernel another number of registers than its split among the
+// warps is made for.
 double plan_gemm_f32_tc(const GemmArgs& g, int sms, int* cols);
 cudaError_t launch_gemm_f32_tc(const GemmArgs& g, int cols, int sms, cudaStream_t st);
 

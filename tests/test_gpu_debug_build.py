@@ -165,6 +165,25 @@ def test_a_gate_whose_waits_run_out_leaves_an_index_inside_its_buffers(D, n, E, 
     assert D.ec_read_status(ws) == D.EC_OK and all(torch.equal(getattr(again, f), getattr(want, f)) for f in fields)
 
 
+@pytest.mark.parametrize("kind", [0, 1, 2])
+def test_fp32_products_go_to_the_multiply_adds_where_the_tensor_kernel_cannot_run(D, kind):
+    """As if the compiler had given it other registers than its split among the warps needs."""
+    n, d, dff, E = 2048, 512, 1024, 8
+    cfg = D.make_config(n, d, dff, E, 2.0, F32)
+    k = D.ec_capacity(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(kind)
+    rows, b = {0: ((E, k, d), (E, d, dff)), 1: ((E, k, dff), (E, d, dff)), 2: ((E, k, d), (E, k, dff))}[kind]
+    A, Bm = (torch.empty(s, device="cuda").normal_(generator=gen) for s in (rows, b))
+    want = {0: lambda: A.double() @ Bm.double(), 1: lambda: A.double() @ Bm.double().mT, 2: lambda: A.double().mT @ Bm.double()}[kind]()
+    usual = D.ec_expert_gemm(cfg, kind, A, Bm)
+    ws, out = D.alloc_workspace(cfg), torch.full_like(usual, float("nan"))
+    call = D.lib().ec_debug_expert_gemm_registers
+    call.argtypes = [ctypes.POINTER(D.ec_config), ctypes.c_int] + [ctypes.c_void_p] * 4 + [ctypes.c_size_t, ctypes.c_void_p]
+    assert call(ctypes.byref(cfg), kind, A.data_ptr(), Bm.data_ptr(), out.data_ptr(), ws.data_ptr(), ws.numel(), D._stream()) == D.EC_OK
+    # sums of at most 1024 fp32 products, one after the other: a few 1e-7 of the result in the 2-norm, at most 1024 * 2^-24
+    assert float((out - want).norm() / want.norm()) < 1024 * 2.0 ** -24 and not torch.equal(out, usual)
+
+
 @pytest.mark.parametrize("n,d,E,dtype", [(3000, 768, 8, BF16), (2000, 1024, 16, F32), (1500, 2048, 8, F32), (1000, 4096, 8, BF16), (700, 8192, 4, BF16)])
 def test_an_unshuffle_whose_waits_run_out_is_finished_all_the_same(D, n, d, E, dtype):
     """One CTA of the ring gets its first rows only and its warps wait 2 ms for the others: nobody can tell from the result."""
