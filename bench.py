@@ -487,7 +487,7 @@ def routing_bytes(n, d, E, c, b=2, cap_iters=0):
         "gate_softmax": n * d * b + d * E * b + n * E * 4,
         "topk": n * E * 4 + slots * 8,
         "inverse_index": slots * 4 + (n + 1 + slots) * 4,
-        "topk_index": n * E * 4 + slots * 8 + slots * 4 + (n + 1 + slots) * 4,      # one launch up to 16384 tokens
+        "topk_index": n * E * 4 + slots * 8 + slots * 4 + (n + 1 + slots) * 4,      # one launch up to 4096 tokens, where the index fits a CTA
         "gather": 2 * slots * d * b + slots * 4,
         "combine": slots * d * 4 + slots * 4 + (n + 1 + slots) * 4 + n * d * b,
     }

@@ -314,8 +314,8 @@ ec_status ec_read_status(const void* ws, void* cuda_stream);
 /* Static, NUL-terminated description of a status code. */
 const char* ec_status_string(ec_status s);
 
-/* 1 if the bf16 path of this cfg runs its expert GEMMs on the tcgen05 tensor-core
- * kernels, 0 if it falls back to the plain FMA kernels (fp32 path, odd shapes). */
+/* 1 if this cfg is of the bf16 path and runs its expert GEMMs on the tcgen05 tensor-core kernels, else 0.  (Of the
+ * fp32 path it says 0, although large fp32 products run on the tensor cores too, in three bf16 pieces.) */
 int ec_uses_tensor_cores(const ec_config* cfg);
 
 /* Number of CUDA kernels this library has launched in this process so far (all calls, all
