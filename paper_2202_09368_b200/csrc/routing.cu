@@ -830,8 +830,10 @@ __device__ __forceinline__ void build_index(const int32_t* I, int N, int total, 
 // 33 k; with the third pass, which is hardly ever needed, 24.5 us at 8192 tokens and 32 experts, 22.5 now).  The CTAs of eight experts form a cluster: each reads an eighth of the tokens, all eight scores of a token together, and sends every
 // score to its expert's CTA.
 constexpr int kSmallN = 16384;
-template <bool CLUSTER>
-__global__ void __launch_bounds__(1024)
+// INDEX: with row_ptr.  build_index wants 54 registers, the selection alone gets by with 32, so that an SM holds two CTAs of 1024
+// threads and up to 296 columns need no second round.
+template <bool CLUSTER, bool INDEX>
+__global__ void __launch_bounds__(1024, INDEX ? 1 : 2)
 topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, const SlotMap map, int32_t* I, float* G, int32_t* row_ptr,
                   int32_t* slots, int* done, int* status) {
   if constexpr (CLUSTER) cluster_barrier();            // every CTA of the cluster has started: its shared memory may be written
@@ -970,15 +972,16 @@ topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, co
   __syncthreads();
   sort_keys(sm_keys, kpad, 0, (unsigned)kpad);
   for (int i = tid; i < k; i += nt) emit_slot(sm_keys[i], I, G, map, (int64_t)grp * E + e, i);
-  if (row_ptr == nullptr) return;
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_less = atomicAdd(done, 1) == E * map.groups - 1 ? 1u : 0u;
-  __syncthreads();
-  if (!s_less) return;
-  __threadfence();
-  build_index(I, n * map.groups, E * k * map.groups, k * map.groups, map.marks, row_ptr, slots, reinterpret_cast<int*>(sm_keys),
-              reinterpret_cast<int*>(s_warp), status);
+  if constexpr (INDEX) {
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_less = atomicAdd(done, 1) == E * map.groups - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!s_less) return;
+    __threadfence();
+    build_index(I, n * map.groups, E * k * map.groups, k * map.groups, map.marks, row_ptr, slots, reinterpret_cast<int*>(sm_keys),
+                reinterpret_cast<int*>(s_warp), status);
+  }
 }
 
 // Dynamic shared memory of a launch: the attribute is one per device, whatever threads launch, so it is always set to the most
@@ -1010,7 +1013,7 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
     int smem = (int)(kpad * 8 + n * 4 + kBins * 4);
     if (plan.fused) smem = max(smem, (int)index_smem_words(n * groups, (int64_t)E * k * groups, plan.marks.per_token) * 4);
     const bool cluster = n > 4096 && E >= 8;
-    auto kern = cluster ? topk_small_kernel<true> : topk_small_kernel<false>;
+    auto kern = cluster ? topk_small_kernel<true, false> : plan.fused ? topk_small_kernel<false, true> : topk_small_kernel<false, false>;
     cudaError_t e0 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSelectSmem);
     if (e0 != cudaSuccess) return e0;
     int threads = 128;                                 // at most four keys per thread for the sort (kpad < 2 n)
@@ -1018,7 +1021,7 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
     while (threads < 1024 && threads * 4 < kpad) threads <<= 1;
     while (plan.fused && threads < 1024 && threads * 8 < (int64_t)E * k * groups) threads <<= 1;
     return launch_chained_cluster(cluster ? 8 : 1, kern, dim3(cluster ? (E + 7) / 8 * 8 : E, groups), dim3(threads), smem, st, S, (int)n, E, (int)k, kpad, smap, I, G,
-                                  plan.fused ? row_ptr : nullptr, slots, status + kSelectCounter, status);
+                                  row_ptr, slots, status + kSelectCounter, status);
   }
   const int64_t VE = (int64_t)groups * E;              // independent columns: E per group
   char* base = (char*)scratch;
