@@ -993,11 +993,13 @@ IndexPlan plan_index(int64_t ng, int E, int64_t k, int groups, bool selects, voi
   const int words = (E + 31) / 32;
   IndexPlan p;
   // The selection's last CTA builds the index where everything fits its shared memory (2048 tokens, 8 experts: 24.5 us with two
-  // launches that counted, filled and sorted, 20.5 so); a cluster of eight CTAs up to 16384 tokens (8192 tokens, 32 experts: 18.4 us with
+  // launches that counted, filled and sorted, 20.5 so), the columns are one round of CTAs (1024 threads each, as the index wants them:
+  // sixteen groups of 256 tokens, 64 experts 55.8 us so, 25.6 by a cluster) and a token's marks are two words (2048 tokens, 128
+  // experts: 27.2 so, 24.4 by a cluster; 64 experts, two groups: 26.2 either way); else a cluster of eight CTAs, up to 16384 tokens (8192 tokens, 32 experts: 18.4 us with
   // atomics and sorting, 14.4 from the marks; one CTA alone takes 22).  Their marks may take the place of the large selection's
   // scratch, which such a call does not use.
   const bool one_launch = selects && ng <= kSmallN && k <= kSortTile;
-  p.fused = one_launch && N <= 4096 && index_smem_words(N, total, words) * 4 <= kMostSelectSmem;
+  p.fused = one_launch && N <= 4096 && (int64_t)E * groups <= 148 && words <= 2 && index_smem_words(N, total, words) * 4 <= kMostSelectSmem;
   p.small = p.fused || (N <= kIndexClusterTokens && total <= kIndexClusterSlots && (one_launch || !selects));
   p.marks.per_token = p.small || words == 1 ? words : 0;
   p.marks.words = (unsigned*)(p.marks.per_token > 1 ? topk_scratch : inverse_scratch);

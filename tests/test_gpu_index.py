@@ -58,3 +58,10 @@ def _shortest_us(n, E, groups, stages):
 def test_columns_beyond_one_per_sm_need_no_second_round():
     """16384 tokens: 256 experts take 1.34 times as long as 128 where an SM holds one CTA of the selection, 1.1 times where it holds two."""
     assert _shortest_us(16384, 256, 1, ("topk",)) < 1.22 * _shortest_us(16384, 128, 1, ("topk",))
+
+
+def test_many_small_columns_do_not_wait_for_the_index():
+    """Sixteen groups of 256 tokens with 64 experts and one of 4096: 2.1 times as long where each of the 1024 CTAs has the threads that
+    the index wants."""
+    stages = ("topk", "topk_index", "inverse_index")
+    assert _shortest_us(256, 64, 16, stages) < 1.4 * _shortest_us(4096, 64, 1, stages)
