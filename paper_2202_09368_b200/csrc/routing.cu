@@ -831,9 +831,11 @@ __device__ __forceinline__ void build_index(const int32_t* I, int N, int total, 
 // score to its expert's CTA.
 constexpr int kSmallN = 16384;
 // INDEX: with row_ptr.  build_index wants 54 registers, the selection alone gets by with 32, so that an SM holds two CTAs of 1024
-// threads and up to 296 columns need no second round.
-template <bool CLUSTER, bool INDEX>
-__global__ void __launch_bounds__(1024, INDEX ? 1 : 2)
+// threads (PER_SM) and up to 296 columns need no second round.  Clusters share SMs only where they are many: forward passes, one and
+// two per SM, of 8192 tokens: 32 experts 57.3 and 60.2 us, 64 161.0 and 166.2, 128 63.3 and 60.0; of 16384: 64 87.7 and 101, 128 108
+// and 104, 256 132 and 136; of 6000: 256 88.0 and 83.1.
+template <bool CLUSTER, bool INDEX, int PER_SM>
+__global__ void __launch_bounds__(1024, PER_SM)
 topk_small_kernel(const float* __restrict__ S, int n, int E, int k, int kpad, const SlotMap map, int32_t* I, float* G, int32_t* row_ptr,
                   int32_t* slots, int* done, int* status) {
   if constexpr (CLUSTER) cluster_barrier();            // every CTA of the cluster has started: its shared memory may be written
@@ -1015,7 +1017,8 @@ cudaError_t launch_topk(const float* S, int64_t n, int E, int64_t k, int groups,
     int smem = (int)(kpad * 8 + n * 4 + kBins * 4);
     if (plan.fused) smem = max(smem, (int)index_smem_words(n * groups, (int64_t)E * k * groups, plan.marks.per_token) * 4);
     const bool cluster = n > 4096 && E >= 8;
-    auto kern = cluster ? topk_small_kernel<true, false> : plan.fused ? topk_small_kernel<false, true> : topk_small_kernel<false, false>;
+    auto kern = cluster ? ((int64_t)E * groups > 96 ? topk_small_kernel<true, false, 2> : topk_small_kernel<true, false, 1>)
+                        : plan.fused ? topk_small_kernel<false, true, 1> : topk_small_kernel<false, false, 2>;
     cudaError_t e0 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSelectSmem);
     if (e0 != cudaSuccess) return e0;
     int threads = 128;                                 // at most four keys per thread for the sort (kpad < 2 n)
