@@ -459,7 +459,8 @@ ec_status ec_moe_backward(const ec_config* c, const void* X, const void* Wg, con
   const int64_t kd = D.k * D.d, kf = D.k * D.dff, df = (int64_t)D.d * D.dff;
   // Products that may start beside their predecessor's tail (see chain_enter()) do, up to a TFLOP each: 2048 x 256 step 100.9 -> 88.6 us,
   // 8192 x 768 x 3072 (77 GFLOP) 673 -> 659.  Products of milliseconds win nothing at their tails and two at a time share L2 and the
-  // power cap worse: the 8B step (4.4 TFLOP) takes 28.1 ms without and 28.8 with.
+  // power cap worse: the 8B step (4.4 TFLOP) takes 28.1 ms without and 28.8 with.  Between, ms without and with, runs of one side up to 5 %
+  // apart: 0.14 TFLOP 0.989 0.984, 0.62 3.77 3.61, 0.83 4.48 4.62, 1.1 6.07 6.29, 1.6 9.01 9.27, 2.2 12.06 12.07.
   const int early = 2.0 * (double)D.slots * D.d * D.dff < 1e12 ? 1 : 0;
   // the two gate-gradient products; on tensor cores dL [n, E] is bf16
   const int P = dwg_splits(D);

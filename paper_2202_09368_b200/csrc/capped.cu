@@ -14,16 +14,17 @@
 // A warp owns a token (its e values, a few per lane), so the column and box steps need only warp shuffles; the
 // row step needs a sum over all tokens, which a round prepares for the next: every CTA leaves (max, sum of exp)
 // of its tokens per expert, and the CTAs each combine those in a fixed order (so the result does not depend on
-// scheduling) before they touch their tokens.  Two forms:
+// scheduling) before they touch their tokens.  Three forms:
 //   - resident: one cooperative launch for all rounds; a warp keeps log A and the factors of its (at most 8 /
 //     experts-per-lane) tokens in registers, and only the row partials go through memory, as words that carry their
 //     round's number: a CTA waits for the words it needs, there is no grid barrier (see Exchange).  Used whenever the tokens
-//     fit (up to about 19 k tokens at 64 experts);
+//     fit (up to about 19 k tokens at 64 experts).  Groups that one cluster of 8 or 16 CTAs holds (up to 4096 tokens at 32
+//     experts) pass the partials through the cluster's shared memory instead (see Box);
 //   - resident in shared memory: the same launch with the state in the CTA's shared memory, for up to about
 //     2.4 M entries per device (16384 tokens x 128 experts, 65536 x 32);
 //   - one launch per round with the state (2 x 4 bytes per entry) in global memory, where it stays in L2 at
 //     the layer sizes.  For everything else.
-// Either way a round costs latency (one round trip for the partials or a launch, the reduction trees), not
+// Whichever it is, a round costs latency (one round trip for the partials or a launch, the reduction trees), not
 // bandwidth.  Routing groups are independent problems (grid.y).
 #include "internal.h"
 #include "tc_ptx.cuh"
